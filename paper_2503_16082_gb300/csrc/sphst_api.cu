@@ -202,15 +202,15 @@ int64_t footprint(const sphst_case_params *P, int64_t n) {
     const int64_t tsz = P->precision == 64 ? 8 : 4;
     const int64_t kmax = P->nbr_mode == SPHST_NBR_LIST
                              ? (P->max_neighbors > 0 ? P->max_neighbors : (P->dim == 3 ? 128 : 48)) : 0;
-    // V4 arrays, scalars, ints, list (+ its pair geometry), band + band list
-    const int64_t per = 9 * 4 * tsz + 2 * tsz + 6 * 4 + 4 * kmax + (SPHST_LIST_GEO ? 4 * tsz * kmax : 0) + 4 + 1 + 8 +
+    // V4 arrays, scalars, ints, list, band + band list, cell list
+    const int64_t per = 9 * 4 * tsz + 2 * tsz + 6 * 4 + 4 * kmax + 4 + 1 + 8 + 8 +
                         (P->surface_corr == 1 ? 2 * 4 * tsz : 0);   // own-fluid correction matrices
     // cell table: cells ~ n / 2.6^d per axis padded to a power of two
     const double side = std::pow((double)std::max<int64_t>(n, 1), 1.0 / P->dim) / 2.6 + 2.0 * P->grid_pad + 2.0;
     int bits = 0;
     while ((double)(1 << bits) < side) ++bits;
     const int64_t table = ((int64_t)1 << (P->dim * bits)) * 4 + 4;
-    return per * n + table + 4096 + (int64_t)(DIAG_BLOCKS + 1) * DIAG_Q * 8;
+    return per * n + table + 4096 + 32 * 4 * kmax + (int64_t)(DIAG_BLOCKS + 1) * DIAG_Q * 8;
 }
 
 // Move `cases` into one new engine (copying resident state), release

@@ -20,10 +20,9 @@ namespace sphst {
 enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
 
 // Tile classes: 0 = 3D list, 1 = 2D list, 2 = 3D cell walk, 3 = 2D cell walk.
-// SPH_CLASSES(NCLS, KERN, args...) launches KERN<T, D, LIST> over the tiles of
-// each non-empty class among the first NCLS (2: list classes only);
-// SPH_CLASSES_F over the tiles of fluid ranks.
-#define SPH_CLASSES(NCLS, KERN, ...) SPH_CLASSES_X(NCLS, KERN, sweep_args, cls_n, __VA_ARGS__)
+// SPH_CLASSES_F(NCLS, KERN, args...) launches KERN<T, D, LIST> over the
+// fluid-rank tiles of each non-empty class among the first NCLS (2: list
+// classes only).
 #define SPH_CLASSES_F(NCLS, KERN, ...) SPH_CLASSES_X(NCLS, KERN, fluid_args, cls_fn, __VA_ARGS__)
 #define SPH_CLASSES_X(NCLS, KERN, ARGS, CNT, ...)                                      \
     for (int k_ = 0; k_ < (NCLS); ++k_) {                                              \
@@ -70,7 +69,7 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
     }
 // SPH_CLASSES_BAND: the sweeps over a list class's band list (S, and A of
 // the list classes): a few blocks per SM whose threads stride over the list
-#define SPH_CLASSES_BAND(KERN, LN, ...) SPH_CLASSES_LX(2, KERN, LN, sweep_args, cls_n, band_grid(cls_n[k_], LN), __VA_ARGS__)
+#define SPH_CLASSES_BAND(KERN, LN, ...) SPH_CLASSES_LX(2, KERN, LN, fluid_args, cls_n, band_grid(cls_n[k_], LN), __VA_ARGS__)
 // SPH_CLASSES_LF: the per-substep sweeps over fluid ranks, whose blocks
 // stride over the work list of active tiles in a batch (the grid is then
 // capped), and which take their case's descriptor from the launch parameters
@@ -121,10 +120,12 @@ template <typename T> struct EngineT : Engine {
     // cell table + scan scratch
     uint32_t *starts = nullptr, *block_sums = nullptr;
     uint32_t *nbr = nullptr, *nbr_cnt = nullptr;   // neighbour lists (ELL per case) and counts
-    V4<T> *lgeo = nullptr;                          // (e_ij, W'_ij) of each list entry (SPHST_LIST_GEO)
     uint8_t *band = nullptr;                        // interface band of the frozen configuration
     uint64_t *band_list = nullptr;                  // band particles per list class (case << 32 | index)
     uint32_t *band_count = nullptr;                 // entries of each class's band list
+    uint64_t *cell_list = nullptr;                  // cells with fluid particles per list class (case << 32 | table index)
+    uint32_t *cell_count = nullptr;                 // entries of each class's cell list (after band_count)
+    int64_t lb_blocks[2] = {0, 0};                  // resident list-build blocks per class
     int64_t band_base[2] = {0, 0};                  // first entry of each list class
     int64_t nbr_total = 0;
     bool any_list = false;
@@ -202,6 +203,7 @@ template <typename T> struct EngineT : Engine {
         n_tiles = 0;
         max_case_n = 0;
         loop_mode = SPHST_LOOP_GRAPH;
+        int64_t nf = 0;
         for (int c = 0; c < ncases; ++c) {
             CaseRec *r = cases[c];
             if (!r->gridded) {
@@ -220,12 +222,14 @@ template <typename T> struct EngineT : Engine {
             max_case_n = std::max(max_case_n, r->n);
             any_tvf = any_tvf || d.tvf_on;
             any_corr = any_corr || d.surface_corr == 1;
+            d.f_begin = nf;
+            nf += r->n_fluid;
             if (d.nbr_mode == 0) {
-                d.nbr_base = nbr_total;
-                nbr_total += (int64_t)d.nbr_k * r->n;
+                d.nbr_base = nbr_total;                 // blocks of 32 slots
+                nbr_total += (r->n_fluid + 31) / 32 * 32 * (int64_t)d.nbr_k;
                 any_list = true;
-                h_desc[c] = d;
             }
+            h_desc[c] = d;
             if (r->P.loop_mode == SPHST_LOOP_HOST) loop_mode = SPHST_LOOP_HOST;
         }
         if (any_list && n >= ((int64_t)1 << (32 - NBR_SHIFT))) {
@@ -261,9 +265,8 @@ template <typename T> struct EngineT : Engine {
         size_t o_flag = take(64);
         size_t o_read = take((size_t)std::max<int64_t>(max_case_n, 1) * 3 * sizeof(double));
         size_t o_nbr = take((size_t)std::max<int64_t>(nbr_total, 1) * 4), o_ncnt = take(nn * 4);
-        size_t o_lgeo = take(SPHST_LIST_GEO ? (size_t)std::max<int64_t>(nbr_total, 1) * sizeof(V4<T>) : 0);
         size_t o_band = take(nn);
-        size_t o_blist = take(nn * 8), o_bcount = take(64);
+        size_t o_blist = take(nn * 8), o_bcount = take(64), o_clist = take(nn * 8);
         size_t o_diag = take((size_t)(DIAG_BLOCKS + 1) * DIAG_Q * sizeof(double));
         cudaError_t e = cudaMalloc(&arena, off);
         if (e != cudaSuccess) {
@@ -292,10 +295,11 @@ template <typename T> struct EngineT : Engine {
         d_read = (double *)(b + o_read);
         nbr = (uint32_t *)(b + o_nbr);
         nbr_cnt = (uint32_t *)(b + o_ncnt);
-        lgeo = SPHST_LIST_GEO ? (V4<T> *)(b + o_lgeo) : nullptr;
         band = (uint8_t *)(b + o_band);
         band_list = (uint64_t *)(b + o_blist);
         band_count = (uint32_t *)(b + o_bcount);
+        cell_count = band_count + 2;
+        cell_list = (uint64_t *)(b + o_clist);
         d_diag = (double *)(b + o_diag);
         SPH_CK(cudaMemsetAsync(arena, 0, off, stream));
         // tiles, grouped by class
@@ -360,6 +364,12 @@ template <typename T> struct EngineT : Engine {
             SPH_CK(cudaGetDevice(&dev));
             SPH_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
             sm_count = std::max(sms, 1);
+        }
+        for (int k = 0; k < 2; ++k) {
+            int per_sm = 0;
+            if (k == 0) SPH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_list<T, 3>, LB_WARPS * 32, 0));
+            else SPH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_list<T, 2>, LB_WARPS * 32, 0));
+            lb_blocks[k] = std::max(per_sm, 1) * sm_count;
         }
         SPH_CK(cudaMemcpyAsync(d_desc, h_desc.data(), sizeof(CaseDesc) * ncases, cudaMemcpyHostToDevice, stream));
         // fill each case
@@ -428,7 +438,6 @@ template <typename T> struct EngineT : Engine {
     int surface_lanes() const { return std::max(lanes, (int)SPHST_SURFACE_MIN_LANES); }
 
     static int tile_class(const CaseDesc &d) { return (d.nbr_mode == 0 ? 0 : 2) + (d.dim == 3 ? 0 : 1); }
-    SweepArgs sweep_args(int k) const { return SweepArgs{d_tiles, d_desc, d_state, starts, nbr, nbr_cnt, cls_b[k]}; }
     SweepArgs fluid_args(int k) const {
         SweepArgs a{d_ftiles, d_desc, d_state, starts, nbr, nbr_cnt, cls_fb[k], fidx};
         if (ncases == 1) a.one = h_desc[0];
@@ -464,7 +473,23 @@ template <typename T> struct EngineT : Engine {
         k_scan_reduce<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
         k_scan_blocks<<<1, SCAN_T, 0, stream>>>(block_sums, nbp);
         k_scan_apply<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
-        k_fluid_scatter<T><<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(n, snap, fscan, fidx, gradC, nbr_cnt);
+        k_fluid_scatter<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, snap, fscan, starts, fidx, gradC, nbr_cnt,
+                                                                   band, cell_list, cell_count, band_base[1]);
+    }
+    // neighbour lists: a block per cell, as many blocks as fit the GPU striding
+    // over the cell list (the number of cells with fluid particles is known on
+    // the device only; there are at most as many as fluid particles)
+    void launch_lists() {
+        for (int k = 0; k < 2; ++k) {
+            if (!cls_fn[k]) continue;
+            const SweepArgs a = fluid_args(k);
+            const unsigned g = (unsigned)std::min<int64_t>(lb_blocks[k], cls_fn[k] * block);
+            const uint64_t *cl = cell_list + band_base[k];
+            if (k == 0)
+                k_build_list<T, 3><<<g, LB_WARPS * 32, 0, stream>>>(a, cl, cell_count + k, fscan, snap, nbr, nbr_cnt, band);
+            else
+                k_build_list<T, 2><<<g, LB_WARPS * 32, 0, stream>>>(a, cl, cell_count + k, fscan, snap, nbr, nbr_cnt, band);
+        }
     }
     int n_classes(int upto) const {
         int m = 0;
@@ -491,11 +516,10 @@ template <typename T> struct EngineT : Engine {
         k_cell_sort<<<(unsigned)((table_total + nthr - 1) / nthr), nthr, 0, stream>>>(table_total, starts, id, perm);
         k_gather<T><<<pgrid, nthr, 0, stream>>>(n, perm, pos, vel, drho, id, snap, vel_new, drho_old, rank);
         k_copy_back<T><<<pgrid, nthr, 0, stream>>>(n, snap, vel_new, drho_old, rank, pos, vel, drho, id);
+        SPH_CK(cudaMemsetAsync(band_count, 0, 4 * sizeof(uint32_t), stream));   // band and cell lists
         launch_fluid_ranks();
-        SPH_CLASSES_F(2, k_build_list, snap, nbr, nbr_cnt);
-        if (SPHST_LIST_GEO) SPH_CLASSES(2, k_list_geo, snap, lgeo);
-        SPH_CK(cudaMemsetAsync(band_count, 0, 2 * sizeof(uint32_t), stream));
-        SPH_CLASSES_F(2, k_band, snap, band, band_list + band_base[k_], band_count + k_);
+        launch_lists();
+        SPH_CLASSES_F(2, k_band, band, band_list + band_base[k_], band_count + k_);
         if (any_tvf || any_corr) SPH_CLASSES_F(4, k_sweep_M, snap, drho, bmat, bk);
         SPH_CLASSES_F(4, k_sweep_V, snap, drho, vel, bmat, acc_visc, pos);
         SPH_CK(cudaGetLastError());
@@ -508,7 +532,7 @@ template <typename T> struct EngineT : Engine {
     // cell-walk classes
     void launch_colour() {
         SPH_CLASSES_BAND(k_sweep_A_band, surface_lanes(), band_list + band_base[k_], band_count + k_, snap, drho, gradC);
-        SPH_CLASSES_LFK(2, 4, k_sweep_A, lanes, snap, drho, lgeo, gradC);
+        SPH_CLASSES_LFK(2, 4, k_sweep_A, lanes, snap, drho, gradC);
     }
 
     int launch_body(cudaGraphConditionalHandle h, int use_handle) {
@@ -516,8 +540,8 @@ template <typename T> struct EngineT : Engine {
         launch_work_lists();
         launch_colour();
         SPH_CLASSES_BAND(k_sweep_S, surface_lanes(), band_list + band_base[k_], band_count + k_, band, snap, vel, gradC, acc_surf, bk, drho);
-        SPH_CLASSES_LF(4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, lgeo, bk);
-        SPH_CLASSES_LF(4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos, lgeo);
+        SPH_CLASSES_LF(4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk);
+        SPH_CLASSES_LF(4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos);
         SPH_CK(cudaGetLastError());
         return SPHST_OK;
     }
@@ -634,12 +658,13 @@ template <typename T> struct EngineT : Engine {
             k_gather<T><<<pgrid, nthr, 0, stream>>>(n, perm, pos, vel, drho, id, snap, vel_new, drho_old, rank);
             k_copy_back<T><<<pgrid, nthr, 0, stream>>>(n, snap, vel_new, drho_old, rank, pos, vel, drho, id);
         });
-        timed(0, 5, [&] { launch_fluid_ranks(); });
-        timed(0, (SPHST_LIST_GEO ? 3 : 2) * nlist, [&] {
-            SPH_CLASSES_F(2, k_build_list, snap, nbr, nbr_cnt);
-            if (SPHST_LIST_GEO) SPH_CLASSES(2, k_list_geo, snap, lgeo);
-            cudaMemsetAsync(band_count, 0, 2 * sizeof(uint32_t), stream);
-            SPH_CLASSES_F(2, k_band, snap, band, band_list + band_base[k_], band_count + k_);
+        timed(0, 5, [&] {
+            cudaMemsetAsync(band_count, 0, 4 * sizeof(uint32_t), stream);
+            launch_fluid_ranks();
+        });
+        timed(0, 2 * nlist, [&] {
+            launch_lists();
+            SPH_CLASSES_F(2, k_band, band, band_list + band_base[k_], band_count + k_);
         });
         timed(1, (any_tvf || any_corr) ? 2 * ncls : ncls, [&] {
             if (any_tvf || any_corr) SPH_CLASSES_F(4, k_sweep_M, snap, drho, bmat, bk);
@@ -654,8 +679,8 @@ template <typename T> struct EngineT : Engine {
             timed(6, nlist, [&] {
                 SPH_CLASSES_BAND(k_sweep_S, surface_lanes(), band_list + band_base[k_], band_count + k_, band, snap, vel, gradC, acc_surf, bk, drho);
             });
-            timed(4, ncls, [&] { SPH_CLASSES_LF(4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, lgeo, bk); });
-            timed(5, ncls, [&] { SPH_CLASSES_LF(4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos, lgeo); });
+            timed(4, ncls, [&] { SPH_CLASSES_LF(4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk); });
+            timed(5, ncls, [&] { SPH_CLASSES_LF(4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos); });
             if (rc) break;
             int flag = 0;
             cudaError_t e = cudaMemcpy(&flag, d_loop_flag, sizeof(int), cudaMemcpyDeviceToHost);

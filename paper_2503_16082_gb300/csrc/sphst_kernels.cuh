@@ -53,8 +53,6 @@
 //                      packed two-lane instructions (sm_100 and later)
 //   SPHST_LIST_NOALLOC 1: the list words are read without allocating L1 lines
 //                      (measured +1% on the 3D drop)
-//   SPHST_LIST_SORTED  1: the neighbour list holds each part in increasing j
-//                      (cells by table index); 0: in the cell walk's order
 #ifndef SPHST_LIST_PREFETCH
 #define SPHST_LIST_PREFETCH 2
 #endif
@@ -81,14 +79,6 @@
 #endif
 #ifndef SPHST_LIST_NOALLOC
 #define SPHST_LIST_NOALLOC 1
-#endif
-#ifndef SPHST_LIST_SORTED
-#define SPHST_LIST_SORTED 1
-#endif
-#if SPHST_LIST_SORTED
-#define LIST_WALK walk_sorted
-#else
-#define LIST_WALK walk
 #endif
 #ifndef SPHST_SWEEPB_MINB_ONE
 #define SPHST_SWEEPB_MINB_ONE 5
@@ -336,76 +326,28 @@ __device__ __forceinline__ bool walk(const CaseDesc &d, const CasePhys<T> &cp,
     return coincident;
 }
 
-// Neighbour list of the frozen configuration (ELL layout per case: entry k of
-// particle i at nbr[nbr_base + k * n_case + (i - p_begin)], so a warp's 32
-// lanes read 32 consecutive words).  An entry is j << 6 | cell code, the code
-// holding (o + 1) per axis in 2 bits, o the neighbour cell's offset.  Each
-// list holds the neighbours of the other fluid phase first, then the rest,
-// each part in increasing j (SPHST_LIST_SORTED; else in cell-walk order);
+// Neighbour list of the frozen configuration.  The fluid particle of local
+// rank r (its slot) holds entry k at word ((r / 32) K + k) 32 + r % 32 of its
+// case's lists, K the list capacity: a warp's 32 slots own one contiguous
+// block of K rows, a row of 32 words is one 128-byte line, and consecutive
+// entries are one row apart whatever the case's size.  An entry is
+// j << 6 | cell code, the code holding (o + 1) per axis in 2 bits, o the
+// neighbour cell's offset.  Each list holds the neighbours of the other fluid
+// phase first, then the rest, each part in increasing j;
 // cnt[i] = count | (other-phase count << 16),
 // so the colour-gradient sweep reads only the first part.
 constexpr uint32_t NBR_SHIFT = 6;
 constexpr uint32_t CNT_MASK = 0xffffu;
+constexpr int LROW = 32;                        // words between consecutive entries of a list
+// first word of the list of global fluid rank q
+__device__ __forceinline__ int64_t list_word(const CaseDesc &d, int64_t q) {
+    const int64_t r = q - d.f_begin;
+    return d.nbr_base + (r >> 5) * ((int64_t)d.nbr_k * LROW) + (r & 31);
+}
 enum NbrPart { PART_ALL = 0, PART_OTHER = 1 };
 template <int D>
 __device__ __forceinline__ uint32_t cell_code(int ox, int oy, int oz) {
     return (uint32_t)(ox + 1) | ((uint32_t)(oy + 1) << 2) | (D == 3 ? ((uint32_t)(oz + 1) << 4) : 0u);
-}
-
-// The same neighbours as walk(), visited in increasing index j: the 3^D
-// cells are taken in increasing order of their cell-table index (the cells
-// are stored in that order, each cell's particles in index order).  The
-// neighbour list is built in this order, so that the 32 lanes of a warp,
-// neighbouring particles with largely the same neighbours, gather entries k
-// that lie close together in memory.
-template <typename T, int D, typename F>
-__device__ __forceinline__ bool walk_sorted(const CaseDesc &d, const CasePhys<T> &cp,
-                                            const uint32_t *__restrict__ starts,
-                                            const V4<T> *__restrict__ snap, int64_t i,
-                                            const V4<T> &si, uint32_t pki, F &&f) {
-    constexpr int NC = D == 3 ? 27 : 9;
-    const int cx = cell_x<D>(pki), cy = cell_y<D>(pki), cz = cell_z<D>(pki);
-    const uint32_t toff = (uint32_t)d.table_off;
-    uint32_t cell[NC];
-    uint32_t code[NC];
-    int nc = 0;
-    for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz) {
-        int nz = cz + oz;
-        if (D == 3 && !wrap_cell(d, 2, nz)) continue;
-        for (int oy = -1; oy <= 1; ++oy) {
-            int ny = cy + oy;
-            if (!wrap_cell(d, 1, ny)) continue;
-            for (int ox = -1; ox <= 1; ++ox) {
-                int nx = cx + ox;
-                if (!wrap_cell(d, 0, nx)) continue;
-                // insertion by cell-table index
-                const uint32_t m = toff + morton<D>(nx, ny, nz), c = cell_code<D>(ox, oy, oz);
-                int b = nc++;
-                while (b > 0 && cell[b - 1] > m) { cell[b] = cell[b - 1]; code[b] = code[b - 1]; --b; }
-                cell[b] = m;
-                code[b] = c;
-            }
-        }
-    }
-    const T cs = cp.cs, R2 = cp.four_h2;
-    bool coincident = false;
-    for (int q = 0; q < nc; ++q) {
-        const int ox = (int)(code[q] & 3u) - 1, oy = (int)((code[q] >> 2) & 3u) - 1, oz = (int)((code[q] >> 4) & 3u) - 1;
-        const T sx = sub_rn(si.x, mul_rn(T(ox), cs)), sy = sub_rn(si.y, mul_rn(T(oy), cs));
-        const T sz = D == 3 ? sub_rn(si.z, mul_rn(T(oz), cs)) : T(0);
-        const uint32_t b = __ldg(starts + cell[q]), e = __ldg(starts + cell[q] + 1);
-        for (uint32_t j = b; j < e; ++j) {
-            const V4<T> sj = ld4(snap + j);
-            const T rx = sub_rn(sx, sj.x), ry = sub_rn(sy, sj.y);
-            const T rz = D == 3 ? sub_rn(sz, sj.z) : T(0);
-            const T r2 = norm2<T, D>(rx, ry, rz);
-            if (r2 < R2 && j != (uint32_t)i) {
-                if (r2 > T(0)) f(j, sj, rx, ry, rz, r2);
-                else coincident = true;
-            }
-        }
-    }
-    return coincident;
 }
 
 // With L lanes per particle, lane `sub` of the particle's group takes the
@@ -414,10 +356,10 @@ template <int PART, typename T, int D, int L = 1, typename F>
 __device__ __forceinline__ void walk_list(const CaseDesc &d, const CasePhys<T> &cp,
                                           const uint32_t *__restrict__ nbr,
                                           const uint32_t *__restrict__ cnt,
-                                          const V4<T> *__restrict__ snap, int64_t i,
+                                          const V4<T> *__restrict__ snap, int64_t i, int64_t slot,
                                           const V4<T> &si, F &&f, uint32_t sub = 0) {
-    const int64_t stride = d.p_end - d.p_begin;
-    const uint32_t *p = nbr + d.nbr_base + (i - d.p_begin) + (int64_t)sub * stride;
+    constexpr int stride = LROW;
+    const uint32_t *p = nbr + list_word(d, slot) + (int)sub * stride;
     const uint32_t c = PART == PART_OTHER ? cnt[i] >> 16 : cnt[i] & CNT_MASK;
     const T cs = cp.cs;
 #if SPHST_LIST_PREFETCH >= 2
@@ -461,10 +403,10 @@ __device__ __forceinline__ void walk_list_aux(const CaseDesc &d, const CasePhys<
                                               const uint32_t *__restrict__ nbr,
                                               const uint32_t *__restrict__ cnt,
                                               const V4<T> *__restrict__ snap,
-                                              const V4<T> *__restrict__ aux, int64_t i,
+                                              const V4<T> *__restrict__ aux, int64_t i, int64_t slot,
                                               const V4<T> &si, F &&f, uint32_t sub = 0) {
-    const int64_t stride = d.p_end - d.p_begin;
-    const uint32_t *p = nbr + d.nbr_base + (i - d.p_begin) + (int64_t)sub * stride;
+    constexpr int stride = LROW;
+    const uint32_t *p = nbr + list_word(d, slot) + (int)sub * stride;
     const uint32_t c = cnt[i] & CNT_MASK;
     const T cs = cp.cs;
     const auto pair = [&](uint32_t e, const V4<T> &sj, const V4<T> &aj) {
@@ -509,10 +451,10 @@ template <bool LIST, typename T, int D, int L = 1, typename F>
 __device__ __forceinline__ bool neighbors_aux(const CaseDesc &d, const CasePhys<T> &cp,
                                               const uint32_t *starts, const uint32_t *nbr,
                                               const uint32_t *cnt, const V4<T> *snap, const V4<T> *aux,
-                                              int64_t i, const V4<T> &si, uint32_t pki, F &&f,
+                                              int64_t i, int64_t slot, const V4<T> &si, uint32_t pki, F &&f,
                                               uint32_t sub = 0) {
     if constexpr (LIST) {
-        walk_list_aux<T, D, L>(d, cp, nbr, cnt, snap, aux, i, si, f, sub);
+        walk_list_aux<T, D, L>(d, cp, nbr, cnt, snap, aux, i, slot, si, f, sub);
         return false;
     } else {
         return walk<T, D>(d, cp, starts, snap, i, si, pki,
@@ -526,76 +468,14 @@ __device__ __forceinline__ bool neighbors_aux(const CaseDesc &d, const CasePhys<
 template <bool LIST, typename T, int D, int PART = PART_ALL, int L = 1, typename F>
 __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &cp,
                                           const uint32_t *starts, const uint32_t *nbr,
-                                          const uint32_t *cnt, const V4<T> *snap, int64_t i,
+                                          const uint32_t *cnt, const V4<T> *snap, int64_t i, int64_t slot,
                                           const V4<T> &si, uint32_t pki, F &&f, uint32_t sub = 0) {
     if constexpr (LIST) {
-        walk_list<PART, T, D, L>(d, cp, nbr, cnt, snap, i, si, f, sub);
+        walk_list<PART, T, D, L>(d, cp, nbr, cnt, snap, i, slot, si, f, sub);
         return false;
     } else {
         return walk<T, D>(d, cp, starts, snap, i, si, pki, f);
     }
-}
-
-// ---- stored pair geometry (SPHST_LIST_GEO): entry k of particle i holds
-// (e_ij, W'_ij) of the frozen configuration at the list's own position, so
-// it streams beside the list.  W' < 0 for every pair (0 < q < 2); an entry
-// whose neighbour is a wall particle stores -W' instead, so the sign bit
-// tells walls from fluid without reading the neighbour's packed phase.  The
-// other fluid phase's entries come first (cnt >> 16 of them), so the phase
-// of a fluid neighbour is known from k.
-__device__ __forceinline__ bool geo_wall(float w) { return (__float_as_uint(w) >> 31) == 0u; }
-__device__ __forceinline__ bool geo_wall(double w) { return __double_as_longlong(w) >= 0; }
-template <typename T> __device__ __forceinline__ V4<T> ld_geo(const V4<T> *p) { return *p; }
-template <> __device__ __forceinline__ V4<float> ld_geo<float>(const V4<float> *p) {
-#if SPHST_LIST_LDCS
-    const float4 v = __ldcs(reinterpret_cast<const float4 *>(p));
-    return V4<float>{v.x, v.y, v.z, v.w};
-#else
-    return ld4(p);
-#endif
-}
-
-// f(other, j, G) for the list entries of i with their stored geometry G;
-// other: j belongs to the other fluid phase
-template <int PART, typename T, typename F>
-__device__ __forceinline__ void walk_geo(const CaseDesc &d, const uint32_t *__restrict__ nbr,
-                                         const uint32_t *__restrict__ cnt, const V4<T> *__restrict__ lgeo,
-                                         int64_t i, F &&f) {
-    const int64_t stride = d.p_end - d.p_begin;
-    const int64_t off = d.nbr_base + (i - d.p_begin);
-    const uint32_t *p = nbr + off;
-    const V4<T> *q = lgeo + off;
-    const uint32_t ci = cnt[i];
-    const uint32_t c_other = ci >> 16;
-    const uint32_t c = PART == PART_OTHER ? c_other : ci & CNT_MASK;
-#if SPHST_LIST_PREFETCH
-    uint32_t next = c ? ld_list(p) : 0u;
-#endif
-    V4<T> g1 = c ? ld_geo(q) : V4<T>{};
-#pragma unroll 1
-    for (uint32_t k = 0; k < c; ++k) {
-#if SPHST_LIST_PREFETCH
-        const uint32_t e = next;
-        p += stride;
-        if (k + 1 < c) next = ld_list(p);
-#else
-        const uint32_t e = ld_list(p);
-        p += stride;
-#endif
-        const V4<T> G = g1;                       // geometry one entry ahead
-        if (k + 1 < c) g1 = ld_geo(q + stride);
-        q += stride;
-        f(PART == PART_OTHER || k < c_other, e >> NBR_SHIFT, G);
-    }
-}
-
-// f(other, j, G, aux_j): walk_geo with the neighbour's aux word
-template <typename T, typename F>
-__device__ __forceinline__ void walk_geo_aux(const CaseDesc &d, const uint32_t *__restrict__ nbr,
-                                             const uint32_t *__restrict__ cnt, const V4<T> *__restrict__ lgeo,
-                                             const V4<T> *__restrict__ aux, int64_t i, F &&f) {
-    walk_geo<PART_ALL, T>(d, nbr, cnt, lgeo, i,
-                          [&](bool other, uint32_t j, const V4<T> &G) { f(other, j, G, ld4(aux + j)); });
 }
 
 // Sum over the L lanes that share one particle (L = 1, 2, 4, 8; groups are
@@ -871,18 +751,46 @@ __global__ void k_fluid_flag(int64_t n, const V4<T> *snap, uint32_t *flag) {
     flag[i] = (i < n && phase_of(w_bits(snap[i].w)) != PH_WALL) ? 1u : 0u;
 }
 
-// Wall slots get their fixed values here, since no sweep visits them: a zero
-// colour gradient and an empty neighbour list.
+// Wall particles get their fixed values here, since no sweep visits them: a
+// zero colour gradient and an empty neighbour list.  The first fluid particle
+// of each cell of a list case appends the cell, as (case << 32 | table
+// index), to its class's cell list for the list build (warp-aggregated; the
+// order is irrelevant, neighbouring cells stay close).
 template <typename T>
-__global__ void k_fluid_scatter(int64_t n, const V4<T> *snap, const uint32_t *rank, uint32_t *fidx,
-                                V4<T> *gradC, uint32_t *cnt) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    // the colour gradient starts every advection step at zero: the list
-    // classes' colour sweep then writes only the interface band
-    gradC[i] = V4<T>{T(0), T(0), T(0), T(0)};
-    if (phase_of(w_bits(snap[i].w)) != PH_WALL) fidx[rank[i]] = (uint32_t)i;
-    else cnt[i] = 0u;
+__global__ void k_fluid_scatter(const Tile *__restrict__ tiles, const CaseDesc *__restrict__ desc, const V4<T> *snap,
+                                const uint32_t *rank, const uint32_t *starts, uint32_t *fidx, V4<T> *gradC,
+                                uint32_t *cnt, uint8_t *band, uint64_t *clist, uint32_t *ccount, int64_t base2d) {
+    const Tile t = tiles[blockIdx.x];
+    const CaseDesc &d = desc[t.c];
+    const int64_t i = t.begin + threadIdx.x;
+    bool first = false;
+    uint32_t m = 0;
+    if ((int)threadIdx.x < t.n) {
+        // the colour gradient starts every advection step at zero: the list
+        // classes' colour sweep then writes only the interface band
+        gradC[i] = V4<T>{T(0), T(0), T(0), T(0)};
+        band[i] = 0;                             // the list build marks the interface band
+        const uint32_t pk = w_bits(snap[i].w);
+        if (phase_of(pk) != PH_WALL) {
+            const uint32_t r = rank[i];
+            fidx[r] = (uint32_t)i;
+            if (d.nbr_mode == 0) {
+                m = (uint32_t)d.table_off + (d.dim == 3 ? morton_of_packed<3>(pk) : morton_of_packed<2>(pk));
+                first = rank[starts[m]] == r;
+            }
+        } else {
+            cnt[i] = 0u;
+        }
+    }
+    const unsigned mask = __ballot_sync(0xffffffffu, first);
+    if (!mask) return;
+    const int k = d.dim == 3 ? 0 : 1;
+    const int lane = threadIdx.x & 31, leader = __ffs(mask) - 1;
+    uint32_t base = 0;
+    if (lane == leader) base = atomicAdd(ccount + k, (uint32_t)__popc(mask));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (first)
+        clist[(k ? base2d : 0) + base + __popc(mask & ((1u << lane) - 1u))] = ((uint64_t)(uint32_t)t.c << 32) | m;
 }
 
 // ================================================================ time step
@@ -1061,7 +969,7 @@ __device__ __forceinline__ void store_B(const Moment<T> &M, int64_t i, V4<T> *bm
 }
 
 template <bool LIST, typename T, int D>
-__device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
+__device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp, int64_t i, int64_t slot,
                                         const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap, const T *drho,
                                         V4<T> *bmat, V4<T> *bk, int32_t *status) {
     const V4<T> si = ld4(snap + i);
@@ -1070,7 +978,7 @@ __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp
     if (ki == PH_WALL) return;
     const bool own = bk != nullptr && d.surface_corr == 1;
     Moment<T> M, Mk;
-    const bool coinc = neighbors<LIST, T, D>(d, cp, starts, nbr, cnt, snap, i, si, pki,
+    const bool coinc = neighbors<LIST, T, D>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki,
         [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
             const uint32_t kj = phase_of(w_bits(sj.w));
             M.template add<D>(d, cp, drho, j, kj, rx, ry, rz, r2);
@@ -1084,7 +992,7 @@ __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp
 
 // ---- V: viscous acceleration (Eq. 13) and transport shift (Eq. 14)
 template <bool LIST, typename T, int D>
-__device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
+__device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp, int64_t i, int64_t slot,
                                         const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap, const T *drho,
                                         const V4<T> *vel, const V4<T> *bmat, V4<T> *acc_visc,
                                         V4<T> *pos, int32_t *status) {
@@ -1106,7 +1014,7 @@ __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp
     V4<T> Bi0 = {0, 0, 0, 0}, Bi1 = {0, 0, 0, 0};
     if (tvf) { Bi0 = bmat[2 * i]; Bi1 = bmat[2 * i + 1]; }
     T ax = 0, ay = 0, az = 0, sx = 0, sy = 0, sz = 0;
-    const bool coinc = neighbors_aux<LIST, T, D>(d, cp, starts, nbr, cnt, snap, vel, i, si, pki,
+    const bool coinc = neighbors_aux<LIST, T, D>(d, cp, starts, nbr, cnt, snap, vel, i, slot, si, pki,
         [&](uint32_t j, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
             const PairGeo<T> g = kgeo(r2);
             const uint32_t kj = phase_of(w_bits(sj.w));
@@ -1149,9 +1057,9 @@ __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp
 
 // ---- A: colour gradient, Eq. 22 (only pairs of different fluids contribute)
 template <bool LIST, typename T, int D, int L = 1>
-__device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
+__device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp, int64_t i, int64_t slot,
                                         const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap, const T *drho,
-                                        const V4<T> *lgeo, V4<T> *gradC, uint32_t sub = 0) {
+                                        V4<T> *gradC, uint32_t sub = 0) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
     const uint32_t ki = phase_of(pki);
@@ -1160,15 +1068,7 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
         const uint32_t other = ki ^ 1u;
         const T two_phi = cp.two_phi[ki];
         const T m_o = cp.mass[other], rho0_o = cp.rho0[other];
-        if constexpr (LIST && SPHST_LIST_GEO && L == 1) {
-            walk_geo<PART_OTHER, T>(d, nbr, cnt, lgeo, i, [&](bool, uint32_t j, const V4<T> &G) {
-                const T s = two_phi * G.w * div_fast(m_o, add_rn(rho0_o, drho[j]));
-                g.x = fma_rn(s, G.x, g.x);
-                g.y = fma_rn(s, G.y, g.y);
-                if (D == 3) g.z = fma_rn(s, G.z, g.z);
-            });
-        } else
-        neighbors<LIST, T, D, PART_OTHER, L>(d, cp, starts, nbr, cnt, snap, i, si, pki,
+        neighbors<LIST, T, D, PART_OTHER, L>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki,
             [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
                 if (!LIST && phase_of(w_bits(sj.w)) != other) return;
                 const PairGeo<T> gg = geo(cp, r2);
@@ -1201,11 +1101,11 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
 // stored surface sum (list), 2 = surface sum only (list, band particles).
 template <bool LIST, int PASS, typename T, int D, int L = 1>
 __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &cp, T dt,
-                                          int64_t i, const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt,
+                                          int64_t i, int64_t slot, const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt,
                                           const uint8_t *band, const V4<T> *snap,
                                           const V4<T> *vel, const V4<T> *gradC,
                                           const V4<T> *acc_visc, V4<T> *acc_surf, V4<T> *vel_new,
-                                          const V4<T> *lgeo, uint32_t *phase_out, uint32_t sub = 0,
+                                          uint32_t *phase_out, uint32_t sub = 0,
                                           const V4<T> *bk = nullptr, const T *drho_s = nullptr) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
@@ -1382,23 +1282,14 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
 
     const bool surface_on = d.n_fluid_phases == 2;
     if constexpr (PASS == 2) {
-        if (surface_on) neighbors<LIST, T, D, PART_ALL, L>(d, cp, starts, nbr, cnt, snap, i, si, pki, surface, sub);
+        if (surface_on) neighbors<LIST, T, D, PART_ALL, L>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki, surface, sub);
         asx = group_sum<L>(asx);
         asy = group_sum<L>(asy);
         if (D == 3) asz = group_sum<L>(asz);
         if (sub == 0) acc_surf[i] = V4<T>{asx, asy, asz, T(0)};
         return 0.0;
     } else if constexpr (PASS == 1) {
-        if constexpr (LIST && SPHST_LIST_GEO && L == 1) {
-            const T rho0_o = sel(ki ^ 1u, rho0_0, rho0_1), rho0_s = sel(ki, rho0_0, rho0_1);
-            const T m_o = sel(ki ^ 1u, m_0, m_1), m_s = sel(ki, m_0, m_1);
-            walk_geo_aux<T>(d, nbr, cnt, lgeo, vel, i, [&](bool other, uint32_t, const V4<T> &G, const V4<T> &vj) {
-                const bool wall = geo_wall(G.w);
-                pressure_pair(l2(G.x, G.y), G.z, wall ? -G.w : G.w, wall, other ? rho0_o : rho0_s,
-                              other ? m_o : m_s, vj);
-            });
-        } else
-        neighbors_aux<LIST, T, D, L>(d, cp, starts, nbr, cnt, snap, vel, i, si, pki, pressure, sub);
+        neighbors_aux<LIST, T, D, L>(d, cp, starts, nbr, cnt, snap, vel, i, slot, si, pki, pressure, sub);
         apx = group_sum<L>(apx);
         apy = group_sum<L>(apy);
         if (D == 3) apz = group_sum<L>(apz);
@@ -1411,7 +1302,7 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             asx = as.x; asy = as.y; asz = as.z;
         }
     } else {
-        neighbors<LIST, T, D>(d, cp, starts, nbr, cnt, snap, i, si, pki,
+        neighbors<LIST, T, D>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki,
             [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
                 pressure(j, sj, vel[j], rx, ry, rz, r2);
                 if (surface_on) surface(j, sj, rx, ry, rz, r2);
@@ -1431,10 +1322,10 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
 
 // ---- C: continuity (Eq. 6) with v* (normal component -U*) + drift
 template <bool LIST, typename T, int D, int L = 1>
-__device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp, T dt, int64_t i,
+__device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp, T dt, int64_t i, int64_t slot,
                                         const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap,
                                         const V4<T> *vel_new, T *drho,
-                                        V4<T> *vel, V4<T> *pos, const V4<T> *lgeo, uint32_t sub = 0) {
+                                        V4<T> *vel, V4<T> *pos, uint32_t sub = 0) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
     const uint32_t ki = phase_of(pki);
@@ -1466,18 +1357,7 @@ __device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp
         const T num = fma_rn(rho_j * c0, dve, fma_rn(-sc0sq, drj, sp_i)) * m_j;
         s = fma_rn(div_fast(num, c0 * add_rn(rho_i, rho_j) * rho_j), dW, s);
     };
-    if constexpr (LIST && SPHST_LIST_GEO && L == 1) {
-        const T rho0_o = sel(ki ^ 1u, rho0_0, rho0_1), rho0_s = sel(ki, rho0_0, rho0_1);
-        const T m_o = sel(ki ^ 1u, m_0, m_1), m_s = sel(ki, m_0, m_1);
-        walk_geo_aux<T>(d, nbr, cnt, lgeo, vel_new, i, [&](bool other, uint32_t, const V4<T> &G, const V4<T> &vj) {
-            const L2<T> dvxy = fma2(l2(vj.x, vj.y), l2(T(-1), T(-1)), l2(vi.x, vi.y));
-            const T dve = D == 3 ? fma_rn(dvxy.x, G.x, fma_rn(dvxy.y, G.y, sub_rn(vi.z, vj.z) * G.z))
-                                 : fma_rn(dvxy.x, G.x, dvxy.y * G.y);
-            const bool wall = geo_wall(G.w);
-            pair(dve, wall ? -G.w : G.w, wall, other ? rho0_o : rho0_s, other ? m_o : m_s, vj.w);
-        });
-    } else
-    neighbors_aux<LIST, T, D, L>(d, cp, starts, nbr, cnt, snap, vel_new, i, si, pki,
+    neighbors_aux<LIST, T, D, L>(d, cp, starts, nbr, cnt, snap, vel_new, i, slot, si, pki,
         [&](uint32_t, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
             const PairGeo<T> g = kgeo(r2);
             const uint32_t kj = phase_of(w_bits(sj.w));
@@ -1554,148 +1434,303 @@ __device__ __forceinline__ int64_t particle_at(const SweepArgs &a, int64_t q) {
     return a.fidx ? (int64_t)a.fidx[q] : q;
 }
 
-// offset -1/0/+1 between neighbour cells from their index difference, which
-// is +-(ncell - 1) across the wrap of a periodic axis
-__device__ __forceinline__ int cell_step(const CaseDesc &d, int a, int diff) {
-    if (diff > 1) return diff - d.ncell[a];
-    if (diff < -1) return diff + d.ncell[a];
-    return diff;
+// ---- L: neighbour lists of the frozen configuration (fluid particles only),
+// one block per cell that holds fluid particles.  All particles of a cell
+// share their candidates, the particles of the 3^D cells around it (475 in
+// 3D, of which 80 are neighbours): the block orders those cells by table
+// index, so that candidates come in increasing j, and copies their positions
+// to shared memory once, moved by their cell's offset and in FP32.  Each warp
+// takes one slot (fluid particle) after the other and tests 32 candidates at a
+// time, one per lane; a ballot gives the hits and their places in the slot's
+// list, which is put together in shared memory (the other phase's entries
+// from the end) and written at the end row by row, neighbouring slots side by
+// side.  In FP64 the FP32 test keeps every candidate within 2h (1 + 1e-6) and
+// the hits alone, a sixth of the candidates, are tested again in FP64, whose
+// pipe is 64 times narrower.  It is bound by instruction issue (about 18
+// instructions per 32 candidates of a slot).  Measured, rebuild of an
+// advection step: 1M fluid particles in FP32 1.71 -> 1.09 ms, 64k 0.56 ->
+// 0.18 ms, 6.9M 11.6 -> 6.7 ms, 43k in FP64 1.17 -> 0.31 ms, against a thread
+// per particle that walked its cells alone (lanes in different cells, the
+// ordered cells of each lane in local memory) and a separate pass over all
+// lists for the band; a warp per cell with the slots in its inner loop took
+// 1.76 ms at 1M (58 instructions per 32 candidates of a slot).
+constexpr int LB_WARPS = 4;                     // warps per block
+constexpr int LB_CAND = 576;                    // candidates in shared memory at a time (8^3 on a lattice, and some)
+constexpr int LB_WORDS = 3072;                  // list words of a group of slots in shared memory
+constexpr int LB_SLOTS = 32;                    // slots of a group at most
+struct ListSmem {
+    float4 cand[LB_CAND];                       // x, y, z relative to the cell, list entry
+    uint32_t fluid[2][LB_CAND / 32];            // candidates of each fluid, a word per 32
+    uint32_t begin[32], pre[33], code[32];      // cells around in increasing table index
+    uint32_t own;                               // first candidate of the cell itself
+    uint32_t idx[LB_SLOTS], rest[LB_SLOTS], other[LB_SLOTS];
+    uint32_t list[LB_WORDS];
+};
+// The row length of the shared lists: K + 1 words, so that for the even
+// capacities in use a column of slots lies in different banks; capacities of
+// LB_WORDS or more are not accepted by the library (K <= 1024)
+__device__ __forceinline__ int lb_group(int K) { return min(LB_SLOTS, LB_WORDS / (K + 1)); }
+
+
+// whether list entry e lies within 2h of slot i, by the cell walk's operations
+template <typename T, int D>
+__device__ __forceinline__ bool list_exact(uint32_t e, const CasePhys<T> &cp, const V4<T> &si, uint32_t i,
+                                           const V4<T> *snap, bool &coinc) {
+    const uint32_t j = e >> NBR_SHIFT;
+    const V4<T> sj = ld4(snap + j);
+    const T cs = cp.cs;
+    const T rx = sub_rn(fma_rn(-code_off(e & 3u, T()), cs, si.x), sj.x);
+    const T ry = sub_rn(fma_rn(-code_off((e >> 2) & 3u, T()), cs, si.y), sj.y);
+    const T rz = D == 3 ? sub_rn(fma_rn(-code_off((e >> 4) & 3u, T()), cs, si.z), sj.z) : T(0);
+    const T r2 = norm2<T, D>(rx, ry, rz);
+    const bool near = r2 < cp.four_h2 && j != i;
+    coinc |= near && !(r2 > T(0));
+    return near && r2 > T(0);
 }
 
-// ---- L: neighbour list of the frozen configuration (fluid particles only)
+// keeps the exact neighbours among the n entries row[at], row[at + step], ...;
+// returns their number
 template <typename T, int D>
-__device__ __forceinline__ void build_list(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
-                                           const uint32_t *starts, const V4<T> *snap,
-                                           uint32_t *nbr, uint32_t *cnt, int32_t *status) {
-    const V4<T> si = ld4(snap + i);
-    const uint32_t pki = w_bits(si.w);
-    if (phase_of(pki) == PH_WALL) { cnt[i] = 0; return; }
-    const int cx = cell_x<D>(pki), cy = cell_y<D>(pki), cz = cell_z<D>(pki);
-    const int64_t stride = d.p_end - d.p_begin;
-    uint32_t *base = nbr + d.nbr_base + (i - d.p_begin);
-    const uint32_t kmax = (uint32_t)d.nbr_k;
-    const uint32_t other = phase_of(pki) ^ 1u;
-    const auto entry_of = [&](uint32_t j, uint32_t pkj) {
-        const uint32_t code = cell_code<D>(cell_step(d, 0, cell_x<D>(pkj) - cx),
-                                           cell_step(d, 1, cell_y<D>(pkj) - cy),
-                                           D == 3 ? cell_step(d, 2, cell_z<D>(pkj) - cz) : 0);
-        return (j << NBR_SHIFT) | code;
-    };
-    // one walk: the rest goes straight to the list, other-phase entries to a
-    // small buffer; then, where there are any, the rest moves up and the
-    // buffer goes in front (each part keeps the walk's order)
-    constexpr uint32_t OBUF = 32;
-    uint32_t obuf[OBUF];
-    uint32_t c_rest = 0, c_other = 0;
-    bool coinc = LIST_WALK<T, D>(d, cp, starts, snap, i, si, pki,
-        [&](uint32_t j, const V4<T> &sj, T, T, T, T) {
-            const uint32_t pkj = w_bits(sj.w);
-            if (phase_of(pkj) == other) {
-                if (c_other < OBUF) obuf[c_other] = entry_of(j, pkj);
-                ++c_other;
-            } else {
-                if (c_rest < kmax) base[(int64_t)c_rest * stride] = entry_of(j, pkj);
-                ++c_rest;
-            }
-        });
-    uint32_t c = c_rest + c_other;
-    bool overflow = c > kmax;
-    if (!overflow && c_other > OBUF) {
-        // rare: more other-phase neighbours than the buffer holds; two walks
-        c = 0;
-        for (int part = 0; part < 2; ++part) {
-            coinc |= LIST_WALK<T, D>(d, cp, starts, snap, i, si, pki,
-                [&](uint32_t j, const V4<T> &sj, T, T, T, T) {
-                    const uint32_t pkj = w_bits(sj.w);
-                    if ((phase_of(pkj) == other) != (part == 0)) return;
-                    base[(int64_t)c * stride] = entry_of(j, pkj);
-                    ++c;
-                });
-        }
-    } else if (!overflow && c_other > 0) {
-        for (uint32_t k = c_rest; k-- > 0;) base[(int64_t)(k + c_other) * stride] = base[(int64_t)k * stride];
-        for (uint32_t k = 0; k < c_other; ++k) base[(int64_t)k * stride] = obuf[k];
+__device__ __forceinline__ uint32_t list_keep(uint32_t *row, int at, int step, uint32_t n, const CasePhys<T> &cp,
+                                              const V4<T> &si, uint32_t i, const V4<T> *snap, bool &coinc) {
+    const int lane = threadIdx.x & 31;
+    uint32_t kept = 0;
+    for (uint32_t k0 = 0; k0 < n; k0 += 32) {
+        const uint32_t k = k0 + lane;
+        const uint32_t e = k < n ? row[at + (int)k * step] : 0u;
+        const bool hit = k < n && list_exact<T, D>(e, cp, si, i, snap, coinc);
+        const unsigned h = __ballot_sync(0xffffffffu, hit);   // all of the chunk is read before it is written
+        if (hit) row[at + (int)(kept + __popc(h & ((1u << lane) - 1u))) * step] = e;
+        kept += (uint32_t)__popc(h);
     }
-    if (overflow) c = kmax;
-    cnt[i] = c | (c_other << 16);
+    __syncwarp();
+    return kept;
+}
+
+// tests nc staged candidates (a multiple of 32) against slot i and appends the
+// hits to its shared list.  EXACT: what the test keeps is tested again by the
+// cell walk's operations.  Returns this lane's number of zero distances
+// (FP32; the FP64 and EXACT tests see to those themselves).
+template <typename T, int D, bool MIXED, bool EXACT>
+__device__ __forceinline__ int list_scan(const ListSmem &S, uint32_t *row, int K, int nc, const CasePhys<T> &cp,
+                                         const V4<T> &si, uint32_t i, uint32_t ki, float R2, const V4<T> *snap,
+                                         uint32_t &c_rest, uint32_t &c_other, bool &coinc) {
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const float sx = (float)si.x, sy = (float)si.y, sz = (float)si.z;
+    int zero = 0;
+    uint32_t cr = c_rest, co = c_other;
+#pragma unroll 3
+    for (int q = 0; q < nc; q += 32) {
+        const float4 s = S.cand[q + lane];
+        const float r2 = norm2<float, D>(sub_rn(sx, s.x), sub_rn(sy, s.y), D == 3 ? sub_rn(sz, s.z) : 0.0f);
+        const bool near = r2 < R2;
+        const uint32_t e = __float_as_uint(s.w);
+        bool hit = near && (sizeof(T) == 8 || EXACT || r2 > 0.0f);
+        zero += near && !hit;
+        if (EXACT) hit = hit && list_exact<T, D>(e, cp, si, i, snap, coinc);
+        const unsigned h = __ballot_sync(0xffffffffu, hit);
+        if (MIXED) {
+            const unsigned ho = h & S.fluid[ki ^ 1u][q >> 5], hr = h & ~ho;
+            const uint32_t nr = (uint32_t)__popc(hr), no = (uint32_t)__popc(ho);
+            const uint32_t at = (ho >> lane) & 1u ? K - 1 - (co + __popc(ho & below)) : cr + __popc(hr & below);
+            if (hit && cr + nr + co + no <= (uint32_t)K) row[at] = e;
+            cr += nr;
+            co += no;
+        } else {
+            const uint32_t at = cr + __popc(h & below);
+            if (hit && at + co < (uint32_t)K) row[at] = e;
+            cr += (uint32_t)__popc(h);
+        }
+    }
+    __syncwarp();
+    c_rest = cr;
+    c_other = co;
+    return zero;
+}
+
+template <typename T, int D>
+__device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> &cp, uint32_t m, ListSmem &S,
+                                           const uint32_t *starts, const uint32_t *rank, const uint32_t *fidx,
+                                           const V4<T> *snap, uint32_t *nbr, uint32_t *cnt, uint8_t *band,
+                                           int32_t *status) {
+    constexpr int NC = D == 3 ? 27 : 9;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int K = d.nbr_k, LS = K + 1, G = lb_group(K);
+    const uint32_t b = starts[m];
+    const uint32_t f0 = rank[b], f1 = rank[starts[m + 1]];
+    __syncthreads();                            // the previous cell's shared data is done with
+    if (warp == 0) {
+        // the 3^D cells around, one per lane, in increasing table index
+        const uint32_t pk = w_bits(snap[b].w);
+        uint32_t mq = 0xffffffffu, bq = 0, nq = 0, code = 0;
+        if (lane < NC) {
+            const int ox = lane % 3 - 1, oy = lane / 3 % 3 - 1, oz = D == 3 ? lane / 9 - 1 : 0;
+            int nx = cell_x<D>(pk) + ox, ny = cell_y<D>(pk) + oy, nz = cell_z<D>(pk) + oz;
+            if (wrap_cell(d, 0, nx) && wrap_cell(d, 1, ny) && (D == 2 || wrap_cell(d, 2, nz))) {
+                mq = (uint32_t)d.table_off + morton<D>(nx, ny, nz);
+                bq = starts[mq];
+                nq = starts[mq + 1] - bq;
+                code = cell_code<D>(ox, oy, oz);
+            }
+        }
+        int place = 0;
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+            const uint32_t o = __shfl_sync(0xffffffffu, mq, q);
+            place += o < mq || (o == mq && q < lane);
+        }
+        if (lane < NC) { S.begin[place] = bq; S.pre[place] = nq; S.code[place] = code; }
+        __syncwarp();
+        const uint32_t own = lane < NC ? S.pre[lane] : 0u;
+        uint32_t x = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        __syncwarp();
+        S.pre[lane] = x - own;                  // candidates before cell `lane`
+        if (lane == 31) S.pre[32] = x;          // all of them
+        if (lane < NC && S.code[lane] == cell_code<D>(0, 0, 0) && own) S.own = x - own;
+    }
+    __syncthreads();
+    const uint32_t total = S.pre[32];
+    // coordinates lie within 2 cells of the origin, so in FP32 r^2 is wrong by
+    // less than 1.2e-6 of (2h)^2: 2e-6 more keeps every neighbour
+    const float R2 = (float)cp.four_h2, R2w = R2 * 1.000002f;
+    bool coinc = false, overflow = false, has0 = false, has1 = false;
+    for (uint32_t g0 = f0; g0 < f1; g0 += G) {
+        const int ns = (int)min((uint32_t)G, f1 - g0);
+        // a group with a list that does not fit is built again with every hit
+        // tested by the cell walk's operations: only what they count overflows
+        bool exact = false;
+    again:
+        bool full = false;
+        for (uint32_t c0 = 0; c0 < total; c0 += LB_CAND) {
+            const int nc = ((int)min((uint32_t)LB_CAND, total - c0) + 31) / 32 * 32;
+            if ((g0 == f0 && !exact) || total > LB_CAND) {
+                __syncthreads();
+                bool p0 = false, p1 = false;
+                for (int q = threadIdx.x; q < nc; q += LB_WARPS * 32) {
+                    const uint32_t t = c0 + q;
+                    float4 s = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // beyond every slot
+                    uint32_t pj = PH_WALL;
+                    if (t < total) {
+                        int cell = 0;
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1)
+                            if (cell + o < NC && S.pre[cell + o] <= t) cell += o;
+                        const uint32_t j = S.begin[cell] + (t - S.pre[cell]), cj = S.code[cell];
+                        const V4<T> sj = ld4(snap + j);
+                        pj = phase_of(w_bits(sj.w));
+                        s.x = (float)fma_rn(code_off(cj & 3u, T()), cp.cs, sj.x);
+                        s.y = (float)fma_rn(code_off((cj >> 2) & 3u, T()), cp.cs, sj.y);
+                        if (D == 3) s.z = (float)fma_rn(code_off((cj >> 4) & 3u, T()), cp.cs, sj.z);
+                        s.w = __uint_as_float((j << NBR_SHIFT) | cj);
+                    }
+                    S.cand[q] = s;
+                    const unsigned m0 = __ballot_sync(0xffffffffu, pj == 0), m1 = __ballot_sync(0xffffffffu, pj == 1);
+                    if (lane == 0) { S.fluid[0][q >> 5] = m0; S.fluid[1][q >> 5] = m1; }
+                    p0 |= m0 != 0;
+                    p1 |= m1 != 0;
+                }
+                has0 = __syncthreads_or(p0);
+                has1 = __syncthreads_or(p1);
+            }
+            for (int s = warp; s < ns; s += LB_WARPS) {
+                const uint32_t i = fidx[g0 + s];
+                const V4<T> si = ld4(snap + i);
+                const uint32_t ki = phase_of(w_bits(si.w));
+                const bool mixed = ki == 0 ? has1 : has0;
+                const uint32_t r0 = c0 ? S.rest[s] : 0u, o0 = c0 ? S.other[s] : 0u;
+                uint32_t cr = r0, co = o0;
+                uint32_t *row = S.list + s * LS;
+                if (exact) {
+                    list_scan<T, D, true, true>(S, row, K, nc, cp, si, i, ki, R2w, snap, cr, co, coinc);
+                } else {
+                    const float r2max = sizeof(T) == 8 ? R2w : R2;
+                    int zero = mixed ? list_scan<T, D, true, false>(S, row, K, nc, cp, si, i, ki, r2max, snap, cr, co, coinc)
+                                     : list_scan<T, D, false, false>(S, row, K, nc, cp, si, i, ki, r2max, snap, cr, co, coinc);
+                    if (sizeof(T) == 4) {
+                        // one zero distance is the particle's own, when it is among these candidates
+                        const uint32_t own = S.own + (i - b);
+                        if (lane == (int)((own - c0) & 31u) && own >= c0 && own < c0 + LB_CAND) --zero;
+                        coinc |= zero > 0;
+                    } else if (cr + co <= (uint32_t)K) {
+                        cr = r0 + list_keep<T, D>(row, (int)r0, 1, cr - r0, cp, si, i, snap, coinc);
+                        if (co > o0) co = o0 + list_keep<T, D>(row, K - 1 - (int)o0, -1, co - o0, cp, si, i, snap, coinc);
+                    }
+                }
+                full |= cr + co > (uint32_t)K;
+                if (lane == 0) { S.idx[s] = i; S.rest[s] = cr; S.other[s] = co; }
+            }
+        }
+        if (__syncthreads_or(full) && !exact) {
+            exact = true;
+            goto again;
+        }
+        // rows of 32 slots; a slot with more neighbours than its list holds
+        // keeps none (its case stops).  A particle with neighbours of the
+        // other fluid and all its neighbours form the interface band
+        const int s = lane;
+        if (s < ns) {
+            uint32_t co = S.other[s], c = S.rest[s] + co;
+            if (c > (uint32_t)K) {
+                overflow = true;
+                c = co = 0;
+            }
+            const uint32_t i = S.idx[s], *src = S.list + s * LS;
+            if (warp == 0) {
+                cnt[i] = c | (co << 16);
+                if (co) band[i] = 1;
+            }
+            uint32_t *dst = nbr + list_word(d, (int64_t)g0 + s);
+            for (uint32_t k = warp; k < c; k += LB_WARPS) {
+                const uint32_t e = src[k < co ? K - 1 - k : k - co];
+                dst[k * LROW] = e;
+                if (co) band[e >> NBR_SHIFT] = 1;
+            }
+        }
+        __syncthreads();
+    }
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
     if (overflow) atomicCAS(status, 0, DEV_ERR_NBR_OVERFLOW);
 }
 
-// ---- interface band of the frozen configuration: i, or one of its
-// neighbours, has neighbours of the other fluid phase.  Band particles are
-// also appended, as (case << 32 | index), to the class's list that the
-// surface sweep walks (warp-aggregated atomics; the order is irrelevant
-// because every particle's sum is its own).
-template <typename T, int D, bool LIST>
-__global__ void __launch_bounds__(256) k_band(SweepArgs a, const V4<T> *snap, uint8_t *band,
-                                              uint64_t *blist, uint32_t *bcount) {
-    const Tile t = a.tiles[a.tile0 + blockIdx.x];
-    const bool live = (int)threadIdx.x < t.n && a.st[t.c].active;
-    const int64_t i = live ? particle_at(a, t.begin + threadIdx.x) : 0;
-    bool b = false;
-    if (live) {
-        const CaseDesc &d = a.desc[t.c];
-        const uint32_t ci = a.cnt[i];
-        b = (ci >> 16) != 0;
-        if (!b && d.n_fluid_phases == 2) {
-            const int64_t stride = d.p_end - d.p_begin;
-            const uint32_t *p = a.nbr + d.nbr_base + (i - d.p_begin);
-            const uint32_t c = ci & CNT_MASK;
-            for (uint32_t k = 0; k < c && !b; ++k, p += stride) b = (a.cnt[ld_list(p) >> NBR_SHIFT] >> 16) != 0;
-        }
-        band[i] = b ? 1 : 0;
+template <typename T, int D>
+__global__ void __launch_bounds__(LB_WARPS * 32) k_build_list(SweepArgs a, const uint64_t *clist, const uint32_t *ccount,
+                                                              const uint32_t *rank, const V4<T> *snap,
+                                                              uint32_t *nbr, uint32_t *cnt, uint8_t *band) {
+    __shared__ ListSmem S;
+    const uint32_t cells = *ccount;
+    for (uint32_t e = blockIdx.x; e < cells; e += gridDim.x) {
+        const uint64_t cm = clist[e];
+        const int c = (int)(cm >> 32);
+        if (!a.st[c].active) continue;          // uniform per block
+        const CaseDesc &d = a.desc[c];
+        build_cell<T, D>(d, phys<T>(d), (uint32_t)cm, S, a.starts, rank, a.fidx, snap, nbr, cnt, band, &a.st[c].status);
     }
+}
+
+// ---- interface band of the frozen configuration: the list build has marked
+// the particles that have neighbours of the other fluid phase and all their
+// neighbours.  The marked fluid particles are appended, as
+// (case << 32 | slot), to the class's list that the surface and colour sweeps
+// walk (warp-aggregated atomics; the order is irrelevant because every
+// particle's sum is its own).
+template <typename T, int D, bool LIST>
+__global__ void __launch_bounds__(256) k_band(SweepArgs a, const uint8_t *band, uint64_t *blist, uint32_t *bcount) {
+    const Tile t = a.tiles[a.tile0 + blockIdx.x];
+    const int64_t q = t.begin + threadIdx.x;
+    const bool b = (int)threadIdx.x < t.n && a.st[t.c].active && band[particle_at(a, q)];
     const unsigned m = __ballot_sync(0xffffffffu, b);
     if (!m) return;
     const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
     uint32_t base = 0;
     if (lane == leader) base = atomicAdd(bcount, (uint32_t)__popc(m));
     base = __shfl_sync(0xffffffffu, base, leader);
-    if (b) blist[base + __popc(m & ((1u << lane) - 1u))] = ((uint64_t)(uint32_t)t.c << 32) | (uint64_t)(uint32_t)i;
-}
-
-template <typename T, int D, bool LIST>
-__global__ void __launch_bounds__(256) k_build_list(SweepArgs a, const V4<T> *snap, uint32_t *nbr, uint32_t *cnt) {
-    const Tile t = a.tiles[a.tile0 + blockIdx.x];
-    if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
-    const CaseDesc &d = a.desc[t.c];
-    const int64_t i = particle_at(a, t.begin + threadIdx.x);
-    build_list<T, D>(d, phys<T>(d), i, a.starts, snap, nbr, cnt, &a.st[t.c].status);
-}
-
-// ---- G: the stored pair geometry of the list (SPHST_LIST_GEO), once per
-// advection step after the list build.  e_ij and W'_ij are formed by the
-// same operations as in the list walk, so the sweeps that read them see the
-// values they would have computed.
-template <typename T, int D, bool LIST>
-__global__ void __launch_bounds__(256) k_list_geo(SweepArgs a, const V4<T> *snap, V4<T> *lgeo) {
-    const Tile t = a.tiles[a.tile0 + blockIdx.x];
-    if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
-    const CaseDesc &d = a.desc[t.c];
-    const CasePhys<T> &cp = phys<T>(d);
-    const int64_t i = t.begin + threadIdx.x;
-    const V4<T> si = ld4(snap + i);
-    if (phase_of(w_bits(si.w)) == PH_WALL) return;
-    const int64_t stride = d.p_end - d.p_begin;
-    const int64_t off = d.nbr_base + (i - d.p_begin);
-    const uint32_t *p = a.nbr + off;
-    V4<T> *q = lgeo + off;
-    const uint32_t c = a.cnt[i] & CNT_MASK;
-    const T cs = cp.cs;
-    const KernelGeo<T> kgeo(cp);
-    for (uint32_t k = 0; k < c; ++k, p += stride, q += stride) {
-        const uint32_t e = ld_list(p);
-        const V4<T> sj = ld4(snap + (e >> NBR_SHIFT));
-        const L2<T> tt = fma2(neg_code_off2(e & 3u, (e >> 2) & 3u, T()), l2(cs, cs), l2(si.x, si.y));
-        const L2<T> rxy = fma2(l2(sj.x, sj.y), l2(T(-1), T(-1)), tt);
-        T rz = T(0);
-        if (D == 3) rz = sub_rn(fma_rn(-code_off((e >> 4) & 3u, T()), cs, si.z), sj.z);
-        const PairGeo<T> g = kgeo(norm2<T, D>(rxy.x, rxy.y, rz));
-        const L2<T> exy = mul2(rxy, l2(g.inv_r, g.inv_r));
-        const bool wall = phase_of(w_bits(sj.w)) == PH_WALL;
-        *q = V4<T>{exy.x, exy.y, D == 3 ? rz * g.inv_r : T(0), wall ? -g.dW : g.dW};
-    }
+    if (b) blist[base + __popc(m & ((1u << lane) - 1u))] = ((uint64_t)(uint32_t)t.c << 32) | (uint64_t)(uint32_t)q;
 }
 
 template <typename T, int D, bool LIST>
@@ -1705,8 +1740,8 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const
     if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
     if (!d.tvf_on && d.surface_corr != 1) return;
-    const int64_t i = particle_at(a, t.begin + threadIdx.x);
-    sweep_M<LIST, T, D>(d, phys<T>(d), i, a.starts, a.nbr, a.cnt, snap, drho, bmat, bk, &a.st[t.c].status);
+    const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
+    sweep_M<LIST, T, D>(d, phys<T>(d), i, q, a.starts, a.nbr, a.cnt, snap, drho, bmat, bk, &a.st[t.c].status);
 }
 
 template <typename T, int D, bool LIST>
@@ -1715,8 +1750,8 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
-    const int64_t i = particle_at(a, t.begin + threadIdx.x);
-    sweep_V<LIST, T, D>(d, phys<T>(d), i, a.starts, a.nbr, a.cnt, snap, drho, vel, bmat, acc_visc, pos,
+    const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
+    sweep_V<LIST, T, D>(d, phys<T>(d), i, q, a.starts, a.nbr, a.cnt, snap, drho, vel, bmat, acc_visc, pos,
                         &a.st[t.c].status);
 }
 
@@ -1731,15 +1766,14 @@ template <int L> __device__ __forceinline__ int local_index(int64_t w) {
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
-__global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, const T *drho, const V4<T> *lgeo,
-                                           V4<T> *gradC) {
+__global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, const T *drho, V4<T> *gradC) {
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         const int li = local_index<L>(w);
         if (li >= t.n || !a.st[t.c].active) return;
         const CaseDesc &d = case_desc<MODE>(a, t.c);
-        const int64_t i = particle_at(a, t.begin + li);
-        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, a.starts, a.nbr, a.cnt, snap, drho, lgeo, gradC, threadIdx.x % L);
+        const int64_t q = t.begin + li, i = particle_at(a, q);
+        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, q, a.starts, a.nbr, a.cnt, snap, drho, gradC, threadIdx.x % L);
     };
     if constexpr (MODE == MODE_WORK) {
         const int64_t items = work_items<L, true>(a);
@@ -1762,10 +1796,11 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A_band(SweepArgs a, const uint64_t *b
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t e = blist[t / L];
         const int c = (int)(e >> 32);
-        const int64_t i = (int64_t)(uint32_t)e;
+        const int64_t q = (int64_t)(uint32_t)e;
         if (!a.st[c].active) continue;
         const CaseDesc &d = a.desc[c];
-        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, a.starts, a.nbr, a.cnt, snap, drho, nullptr, gradC, threadIdx.x % L);
+        sweep_A<LIST, T, D, L>(d, phys<T>(d), (int64_t)a.fidx[q], q, a.starts, a.nbr, a.cnt, snap, drho, gradC,
+                               threadIdx.x % L);
     }
 }
 
@@ -1781,19 +1816,19 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_S(SweepArgs a, const uint64_t *blist,
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t e = blist[t / L];
         const int c = (int)(e >> 32);
-        const int64_t i = (int64_t)(uint32_t)e;
+        const int64_t q = (int64_t)(uint32_t)e;
         if (!a.st[c].active) continue;
         const CaseDesc &d = a.desc[c];
         uint32_t ph;
-        sweep_B<LIST, 2, T, D, L>(d, phys<T>(d), T(0), i, a.starts, a.nbr, a.cnt, band, snap, vel, gradC, nullptr,
-                                  acc_surf, nullptr, nullptr, &ph, threadIdx.x % L, bk, drho);
+        sweep_B<LIST, 2, T, D, L>(d, phys<T>(d), T(0), (int64_t)a.fidx[q], q, a.starts, a.nbr, a.cnt, band, snap, vel,
+                                  gradC, nullptr, acc_surf, nullptr, &ph, threadIdx.x % L, bk, drho);
     }
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
 __global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
                                             const V4<T> *gradC, const V4<T> *acc_visc, V4<T> *acc_surf,
-                                            V4<T> *vel_new, const V4<T> *lgeo, const V4<T> *bk) {
+                                            V4<T> *vel_new, const V4<T> *bk) {
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         if (!a.st[t.c].active) return;             // uniform per block
@@ -1802,10 +1837,10 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_
         uint32_t ph = PH_WALL;
         const int li = local_index<L>(w);
         if (li < t.n) {
-            const int64_t i = particle_at(a, t.begin + li);
+            const int64_t q = t.begin + li, i = particle_at(a, q);
             const T dt = (T)a.st[t.c].dt;
-            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L>(d, phys<T>(d), dt, i, a.starts, a.nbr, a.cnt, band, snap, vel,
-                                                      gradC, acc_visc, acc_surf, vel_new, lgeo, &ph, threadIdx.x % L,
+            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L>(d, phys<T>(d), dt, i, q, a.starts, a.nbr, a.cnt, band, snap, vel,
+                                                      gradC, acc_visc, acc_surf, vel_new, &ph, threadIdx.x % L,
                                                       LIST ? nullptr : bk);
         }
         unsigned long long m0 = ph == 0 ? (unsigned long long)__double_as_longlong(v2) : 0ull;
@@ -1827,15 +1862,15 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
 __global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho,
-                                           V4<T> *vel, V4<T> *pos, const V4<T> *lgeo) {
+                                           V4<T> *vel, V4<T> *pos) {
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         const int li = local_index<L>(w);
         if (li >= t.n || !a.st[t.c].active) return;
         const CaseDesc &d = case_desc<MODE>(a, t.c);
-        const int64_t i = particle_at(a, t.begin + li);
+        const int64_t q = t.begin + li, i = particle_at(a, q);
         const T dt = (T)a.st[t.c].dt;
-        sweep_C<LIST, T, D, L>(d, phys<T>(d), dt, i, a.starts, a.nbr, a.cnt, snap, vel_new, drho, vel, pos, lgeo,
+        sweep_C<LIST, T, D, L>(d, phys<T>(d), dt, i, q, a.starts, a.nbr, a.cnt, snap, vel_new, drho, vel, pos,
                                threadIdx.x % L);
     };
     if constexpr (MODE == MODE_WORK) {
