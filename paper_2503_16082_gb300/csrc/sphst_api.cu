@@ -133,6 +133,8 @@ template <typename T> static CasePhys<T> phys_of(const CaseRec *c) {
     p.inv_h = (T)(1.0 / h);
     p.four_h2 = (T)((2.0 * h) * (2.0 * h));
     p.kcoef = (T)(-5.0 * alpha / h);
+    p.mhalf_inv_h = (T)(-0.5 / h);
+    p.kcoef_h = (T)(-5.0 * alpha / h / h);
     p.cs = (T)cell_width(c);
     p.c0 = (T)P.c0;
     p.c0sq = (T)(P.c0 * P.c0);
@@ -147,10 +149,12 @@ template <typename T> static CasePhys<T> phys_of(const CaseRec *c) {
         p.rho0[k] = (T)c->rho0[k];
         p.eta[k] = (T)c->eta[k];
         p.mass[k] = (T)(c->rho0[k] * vol);
+        p.mass_c0[k] = (T)(c->rho0[k] * vol * P.c0);
         p.two_phi[k] = (T)(2.0 * c->rho0[k] / rsum);
     }
     p.four_phi_phi = (T)(4.0 * c->rho0[0] * c->rho0[1] / (rsum * rsum));
     p.vol_wall = (T)vol;
+    p.c0_vol = (T)(P.c0 * vol);
     p.nhat_eps = (T)1e-4;
     p.tvf_coef = (T)(-P.tvf_alpha * h * h);
     return p;

@@ -20,15 +20,13 @@ namespace sphst {
 enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
 
 // Tile classes: 0 = 3D list, 1 = 2D list, 2 = 3D cell walk, 3 = 2D cell walk.
-// SPH_CLASSES_F(NCLS, KERN, args...) launches KERN<T, D, LIST> over the
-// fluid-rank tiles of each non-empty class among the first NCLS (2: list
-// classes only).
-#define SPH_CLASSES_F(NCLS, KERN, ...) SPH_CLASSES_X(NCLS, KERN, fluid_args, cls_fn, __VA_ARGS__)
-#define SPH_CLASSES_X(NCLS, KERN, ARGS, CNT, ...)                                      \
-    for (int k_ = 0; k_ < (NCLS); ++k_) {                                              \
-        if (!CNT[k_]) continue;                                                        \
-        const SweepArgs a_ = ARGS(k_);                                                 \
-        const unsigned g_ = (unsigned)CNT[k_];                                         \
+// SPH_CLASSES_F(K0, NCLS, KERN, args...) launches KERN<T, D, LIST> over the
+// slot tiles of each non-empty class from K0 on.
+#define SPH_CLASSES_F(K0, NCLS, KERN, ...)                                             \
+    for (int k_ = (K0); k_ < (NCLS); ++k_) {                                           \
+        if (!cls_fn[k_]) continue;                                                     \
+        const SweepArgs a_ = fluid_args(k_);                                           \
+        const unsigned g_ = (unsigned)cls_fn[k_];                                      \
         switch (k_) {                                                                  \
         case 0: KERN<T, 3, true><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;    \
         case 1: KERN<T, 2, true><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;    \
@@ -37,17 +35,9 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         }                                                                              \
     }
 
-// SPH_LANES / SPH_CLASSES_LX: the same for the sweeps whose list classes run
-// with LN lanes per particle (L blocks per tile or per grid block).
-#define SPH_LANES(KERN, D, LN, ...)                                                               \
-    switch (LN) {                                                                                 \
-    case 2: KERN<T, D, true, 2><<<g_ * 2, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
-    case 4: KERN<T, D, true, 4><<<g_ * 4, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
-    case 8: KERN<T, D, true, 8><<<g_ * 8, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
-    default: KERN<T, D, true, 1><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;               \
-    }
-// the same for sweeps A, B and C with their tile mode (MODE_TILES, MODE_WORK
-// for the work-list kernels of a batch, MODE_ONE for a one-case engine)
+// SPH_LANES_M: sweeps A, B and C, whose list classes run with LN lanes per
+// particle (L blocks per tile), in their tile mode (MODE_TILES, MODE_WORK for
+// the work-list kernels of a batch, MODE_ONE and MODE_FEW for a one-case engine)
 #define SPH_LANES_M(KERN, D, LN, MODE, ...)                                                             \
     switch (LN) {                                                                                       \
     case 2: KERN<T, D, true, 2, MODE><<<g_ * 2, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
@@ -55,37 +45,15 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
     case 8: KERN<T, D, true, 8, MODE><<<g_ * 8, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
     default: KERN<T, D, true, 1, MODE><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;               \
     }
-#define SPH_CLASSES_LX(NCLS, KERN, LN, ARGS, CNT, GRID, ...)                           \
-    for (int k_ = 0; k_ < (NCLS); ++k_) {                                              \
-        if (!CNT[k_]) continue;                                                        \
-        const SweepArgs a_ = ARGS(k_);                                                 \
-        const unsigned g_ = (unsigned)(GRID);                                          \
-        switch (k_) {                                                                  \
-        case 0: SPH_LANES(KERN, 3, LN, __VA_ARGS__) break;                             \
-        case 1: SPH_LANES(KERN, 2, LN, __VA_ARGS__) break;                             \
-        case 2: KERN<T, 3, false><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;   \
-        default: KERN<T, 2, false><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;  \
-        }                                                                              \
-    }
-// SPH_CLASSES_BAND: the sweeps over a list class's band list (S, and A of
-// the list classes): a few blocks per SM whose threads stride over the list
-#define SPH_CLASSES_BAND(KERN, LN, ...) SPH_CLASSES_LX(2, KERN, LN, fluid_args, cls_n, band_grid(cls_n[k_], LN), __VA_ARGS__)
-// SPH_CLASSES_LF: the per-substep sweeps over fluid ranks, whose blocks
-// stride over the work list of active tiles in a batch (the grid is then
+// SPH_CLASSES_LF: the per-substep sweeps over slots from class K0 on, whose
+// blocks stride over the work list of active tiles in a batch (the grid is then
 // capped), and which take their case's descriptor from the launch parameters
 // in a one-case engine
-#define SPH_CLASSES_LF(NCLS, KERN, LN, ...)                                                            \
-    if (use_work) {                                                                                    \
-        SPH_CLASSES_LXM(NCLS, KERN, LN, work_args, cls_fn, work_grid(cls_fn[k_]), MODE_WORK, __VA_ARGS__) \
-    } else if (ncases == 1) {                                                                          \
-        SPH_CLASSES_LXM(NCLS, KERN, LN, fluid_args, cls_fn, cls_fn[k_], MODE_ONE, __VA_ARGS__)           \
-    } else {                                                                                           \
-        SPH_CLASSES_LXM(NCLS, KERN, LN, fluid_args, cls_fn, cls_fn[k_], MODE_TILES, __VA_ARGS__)         \
-    }
-// the same from class K0 on
-#define SPH_CLASSES_LFK(K0, NCLS, KERN, LN, ...)                                                        \
+#define SPH_CLASSES_LF(K0, NCLS, KERN, LN, ...)                                                         \
     if (use_work) {                                                                                    \
         SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, work_args, cls_fn, work_grid(cls_fn[k_]), MODE_WORK, __VA_ARGS__) \
+    } else if (ncases == 1 && few) {                                                                   \
+        SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, fluid_args, cls_fn, cls_fn[k_], MODE_FEW, __VA_ARGS__)      \
     } else if (ncases == 1) {                                                                          \
         SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, fluid_args, cls_fn, cls_fn[k_], MODE_ONE, __VA_ARGS__)      \
     } else {                                                                                           \
@@ -94,8 +62,7 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
 // the cell-walk classes keep the descriptor array in a one-case engine: their
 // sweep B also evaluates the surface terms, whose sums are left to the
 // compiler's contraction, so only one compiled form of it may exist
-#define CELL_MODE(MODE) ((MODE) == MODE_ONE ? MODE_TILES : (MODE))
-#define SPH_CLASSES_LXM(NCLS, KERN, LN, ARGS, CNT, GRID, MODE, ...) SPH_CLASSES_LXMK(0, NCLS, KERN, LN, ARGS, CNT, GRID, MODE, __VA_ARGS__)
+#define CELL_MODE(MODE) ((MODE) == MODE_ONE || (MODE) == MODE_FEW ? MODE_TILES : (MODE))
 #define SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, ARGS, CNT, GRID, MODE, ...)                              \
     for (int k_ = (K0); k_ < (NCLS); ++k_) {                                                              \
         if (!CNT[k_]) continue;                                                                        \
@@ -109,6 +76,13 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         }                                                                                              \
     }
 
+// Up to this many lanes per SM, the sweeps B and C of a one-case engine take
+// their MODE_FEW form: the SMs hold fewer warps than the registers would allow
+// (B 42 registers: 1,536 lanes), and the latency of the gathers is what a
+// substep waits for.  64k particles (421 per SM): B 35 -> 33 us; 1M (6,580 per
+// SM): B 250 -> 285 us.
+constexpr int64_t FEW_MAX_PER_SM = 1024;
+
 template <typename T> struct EngineT : Engine {
     // particle arrays
     V4<T> *pos = nullptr, *snap = nullptr, *vel = nullptr, *vel_new = nullptr;
@@ -116,14 +90,14 @@ template <typename T> struct EngineT : Engine {
     V4<T> *bk = nullptr;                             // own-fluid correction matrices (surface_corr)
     T *drho = nullptr, *drho_old = nullptr;        // drho_old: rebuild scratch (sorted copy)
     uint32_t *id = nullptr, *key = nullptr, *rank = nullptr, *perm = nullptr;
-    uint32_t *fidx = nullptr, *fscan = nullptr;     // particle of each fluid rank; scan scratch
+    uint32_t *fidx = nullptr, *fscan = nullptr;     // particle of each fluid rank (slot); scan scratch
     // cell table + scan scratch
     uint32_t *starts = nullptr, *block_sums = nullptr;
     uint32_t *nbr = nullptr, *nbr_cnt = nullptr;   // neighbour lists (ELL per case) and counts
     uint8_t *band = nullptr;                        // interface band of the frozen configuration
     uint64_t *band_list = nullptr;                  // band particles per list class (case << 32 | index)
     uint32_t *band_count = nullptr;                 // entries of each class's band list
-    uint64_t *cell_list = nullptr;                  // cells with fluid particles per list class (case << 32 | table index)
+    uint64_t *cell_list = nullptr;                  // cells with fluid particles per list class (case << 32 | first particle)
     uint32_t *cell_count = nullptr;                 // entries of each class's cell list (after band_count)
     int64_t lb_blocks[2] = {0, 0};                  // resident list-build blocks per class
     int64_t band_base[2] = {0, 0};                  // first entry of each list class
@@ -151,6 +125,7 @@ template <typename T> struct EngineT : Engine {
     int64_t cls_fb[4] = {0, 0, 0, 0}, cls_fn[4] = {0, 0, 0, 0}; // the same over fluid ranks
     int64_t n_ftiles = 0;
     int ncases = 0, block = 128, lanes = 1;
+    bool few = false;                               // a one-case engine that leaves the SMs with few warps
     bool any_tvf = false;
     bool any_corr = false;                          // a case takes the own-fluid surface correction
     int loop_mode = SPHST_LOOP_GRAPH;
@@ -203,7 +178,16 @@ template <typename T> struct EngineT : Engine {
         n_tiles = 0;
         max_case_n = 0;
         loop_mode = SPHST_LOOP_GRAPH;
-        int64_t nf = 0;
+        int64_t nf = 0, list_fluid = 0;
+        int dev = 0, sms = 0;
+        SPH_CK(cudaGetDevice(&dev));
+        SPH_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        sm_count = std::max(sms, 1);
+        for (CaseRec *r : cases) {
+            if (r->P.nbr_mode == SPHST_NBR_LIST) list_fluid += r->n_fluid;
+            any_corr = any_corr || r->P.surface_corr == 1;
+        }
+        few = list_fluid * lanes <= sm_count * FEW_MAX_PER_SM;
         for (int c = 0; c < ncases; ++c) {
             CaseRec *r = cases[c];
             if (!r->gridded) {
@@ -218,12 +202,11 @@ template <typename T> struct EngineT : Engine {
             n += r->n;
             table_total += d.table_size;
             n_tiles += (r->n + block - 1) / block;
-            n_ftiles += (r->n_fluid + block - 1) / block;
             max_case_n = std::max(max_case_n, r->n);
             any_tvf = any_tvf || d.tvf_on;
-            any_corr = any_corr || d.surface_corr == 1;
             d.f_begin = nf;
             nf += r->n_fluid;
+            n_ftiles += (r->n_fluid + block - 1) / block;
             if (d.nbr_mode == 0) {
                 d.nbr_base = nbr_total;                 // blocks of 32 slots
                 nbr_total += (r->n_fluid + 31) / 32 * 32 * (int64_t)d.nbr_k;
@@ -320,8 +303,8 @@ template <typename T> struct EngineT : Engine {
         band_base[0] = 0;
         band_base[1] = np0;
         SPH_CK(cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice, stream));
-        // tiles over fluid ranks: case c's fluid particles hold the ranks
-        // after those of cases 0..c-1
+        // tiles over fluid ranks (slots): case c's fluid particles hold the
+        // ranks after those of cases 0..c-1
         std::vector<int64_t> fb(ncases + 1, 0);
         for (int c = 0; c < ncases; ++c) fb[c + 1] = fb[c] + cases[c]->n_fluid;
         std::vector<Tile> ftiles;
@@ -354,21 +337,12 @@ template <typename T> struct EngineT : Engine {
             SPH_CK(cudaMemcpyAsync(d_ftn, ftn.data(), 4 * ncases, cudaMemcpyHostToDevice, stream));
             SPH_CK(cudaMemcpyAsync(d_ft_first, ft_first.data(), 8 * ncases, cudaMemcpyHostToDevice, stream));
             SPH_CK(cudaMemcpyAsync(d_cls0, cls0.data(), 8 * 4, cudaMemcpyHostToDevice, stream));
-            int dev = 0, sms = 0;
-            SPH_CK(cudaGetDevice(&dev));
-            SPH_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-            work_cap = (int64_t)std::max(sms, 1) * 16;
-        }
-        {
-            int dev = 0, sms = 0;
-            SPH_CK(cudaGetDevice(&dev));
-            SPH_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-            sm_count = std::max(sms, 1);
+            work_cap = sm_count * 16;
         }
         for (int k = 0; k < 2; ++k) {
             int per_sm = 0;
-            if (k == 0) SPH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_list<T, 3>, LB_WARPS * 32, 0));
-            else SPH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_list<T, 2>, LB_WARPS * 32, 0));
+            const void *f = k == 0 ? (const void *)k_build_list<T, 3> : (const void *)k_build_list<T, 2>;
+            SPH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, LB_WARPS * 32, 0));
             lb_blocks[k] = std::max(per_sm, 1) * sm_count;
         }
         SPH_CK(cudaMemcpyAsync(d_desc, h_desc.data(), sizeof(CaseDesc) * ncases, cudaMemcpyHostToDevice, stream));
@@ -432,10 +406,10 @@ template <typename T> struct EngineT : Engine {
         return SPHST_OK;
     }
 
-    // The surface sweep covers only the interface band, a few blocks per SM
-    // at most, so it takes at least SPHST_SURFACE_MIN_LANES lanes per band
-    // particle whatever `lanes` is (measured on the 3D drop: 93 -> 60 us with 2)
-    int surface_lanes() const { return std::max(lanes, (int)SPHST_SURFACE_MIN_LANES); }
+    // The band sweeps cover only the interface, a few blocks per SM at most, so
+    // they take at least 2 lanes per band particle whatever `lanes` is
+    // (measured on the 3D drop: S 93 -> 60 us)
+    int surface_lanes() const { return std::max(lanes, 2); }
 
     static int tile_class(const CaseDesc &d) { return (d.nbr_mode == 0 ? 0 : 2) + (d.dim == 3 ? 0 : 1); }
     SweepArgs fluid_args(int k) const {
@@ -473,24 +447,56 @@ template <typename T> struct EngineT : Engine {
         k_scan_reduce<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
         k_scan_blocks<<<1, SCAN_T, 0, stream>>>(block_sums, nbp);
         k_scan_apply<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
-        k_fluid_scatter<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, snap, fscan, starts, fidx, gradC, nbr_cnt,
-                                                                   band, cell_list, cell_count, band_base[1]);
+        k_fluid_scatter<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, snap, fscan, fidx, gradC, band, cell_list,
+                                                                   cell_count, band_base[1]);
     }
     // neighbour lists: a block per cell, as many blocks as fit the GPU striding
     // over the cell list (the number of cells with fluid particles is known on
     // the device only; there are at most as many as fluid particles)
+    template <int D> void launch_list(int k) {
+        if (!cls_fn[k]) return;
+        const unsigned g = (unsigned)std::min<int64_t>(lb_blocks[k], cls_fn[k] * block);
+        k_build_list<T, D><<<g, LB_WARPS * 32, 0, stream>>>(fluid_args(k), cell_list + band_base[k], cell_count + k, fscan, snap,
+                                                            nbr, nbr_cnt, band);
+    }
     void launch_lists() {
-        for (int k = 0; k < 2; ++k) {
-            if (!cls_fn[k]) continue;
-            const SweepArgs a = fluid_args(k);
-            const unsigned g = (unsigned)std::min<int64_t>(lb_blocks[k], cls_fn[k] * block);
-            const uint64_t *cl = cell_list + band_base[k];
-            if (k == 0)
-                k_build_list<T, 3><<<g, LB_WARPS * 32, 0, stream>>>(a, cl, cell_count + k, fscan, snap, nbr, nbr_cnt, band);
-            else
-                k_build_list<T, 2><<<g, LB_WARPS * 32, 0, stream>>>(a, cl, cell_count + k, fscan, snap, nbr, nbr_cnt, band);
+        launch_list<3>(0);
+        launch_list<2>(1);
+    }
+    void launch_band() {
+        for (int k = 0; k < 2; ++k)
+            if (cls_fn[k])
+                k_band<<<(unsigned)cls_fn[k], block, 0, stream>>>(fluid_args(k), band, band_list + band_base[k], band_count + k);
+    }
+    // correction matrices, viscous force and transport shift
+    void launch_setup() {
+        if (any_tvf || any_corr) SPH_CLASSES_F(0, 4, k_sweep_M, snap, drho, bmat, bk);
+        SPH_CLASSES_F(0, 4, k_sweep_V, snap, vel, bmat, acc_visc, pos);
+    }
+    // the band sweeps (A of the list classes, S): a few blocks per SM whose
+    // threads stride over the class's band list
+    template <int D, int L> void launch_band_sweep(int k, bool surface) {
+        const unsigned g = (unsigned)(band_grid(cls_fn[k], L) * L);
+        const uint64_t *bl = band_list + band_base[k];
+        if (surface)
+            k_sweep_S<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, band, snap, vel, gradC, acc_surf, bk, drho);
+        else
+            k_sweep_A_band<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, snap, drho, gradC);
+    }
+    template <int D> void launch_band_class(int k, bool surface) {
+        if (!cls_fn[k]) return;
+        switch (surface_lanes()) {
+        case 4: launch_band_sweep<D, 4>(k, surface); break;
+        case 8: launch_band_sweep<D, 8>(k, surface); break;
+        default: launch_band_sweep<D, 2>(k, surface); break;
         }
     }
+    void launch_surface() {
+        launch_band_class<3>(0, true);
+        launch_band_class<2>(1, true);
+    }
+    void launch_B() { SPH_CLASSES_LF(0, 4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk); }
+    void launch_C() { SPH_CLASSES_LF(0, 4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos); }
     int n_classes(int upto) const {
         int m = 0;
         for (int k = 0; k < upto; ++k) m += cls_n[k] > 0;
@@ -519,29 +525,28 @@ template <typename T> struct EngineT : Engine {
         SPH_CK(cudaMemsetAsync(band_count, 0, 4 * sizeof(uint32_t), stream));   // band and cell lists
         launch_fluid_ranks();
         launch_lists();
-        SPH_CLASSES_F(2, k_band, band, band_list + band_base[k_], band_count + k_);
-        if (any_tvf || any_corr) SPH_CLASSES_F(4, k_sweep_M, snap, drho, bmat, bk);
-        SPH_CLASSES_F(4, k_sweep_V, snap, drho, vel, bmat, acc_visc, pos);
+        launch_band();
+        launch_setup();
         SPH_CK(cudaGetLastError());
         return SPHST_OK;
     }
 
     // colour gradient: over the interface band in the list classes (zero
-    // elsewhere, from the start of the advection step), with the surface
-    // sweep's lanes per band particle; over every fluid particle in the
-    // cell-walk classes
+    // elsewhere, from the start of the advection step); over every fluid
+    // particle in the cell-walk classes
     void launch_colour() {
-        SPH_CLASSES_BAND(k_sweep_A_band, surface_lanes(), band_list + band_base[k_], band_count + k_, snap, drho, gradC);
-        SPH_CLASSES_LFK(2, 4, k_sweep_A, lanes, snap, drho, gradC);
+        launch_band_class<3>(0, false);
+        launch_band_class<2>(1, false);
+        SPH_CLASSES_LF(2, 4, k_sweep_A, lanes, snap, drho, gradC);
     }
 
     int launch_body(cudaGraphConditionalHandle h, int use_handle) {
         k_dt<<<1, 256, 0, stream>>>(ncases, d_desc, d_state, d_loop_flag, h, use_handle);
         launch_work_lists();
         launch_colour();
-        SPH_CLASSES_BAND(k_sweep_S, surface_lanes(), band_list + band_base[k_], band_count + k_, band, snap, vel, gradC, acc_surf, bk, drho);
-        SPH_CLASSES_LF(4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk);
-        SPH_CLASSES_LF(4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos);
+        launch_surface();
+        launch_B();
+        launch_C();
         SPH_CK(cudaGetLastError());
         return SPHST_OK;
     }
@@ -664,11 +669,10 @@ template <typename T> struct EngineT : Engine {
         });
         timed(0, 2 * nlist, [&] {
             launch_lists();
-            SPH_CLASSES_F(2, k_band, band, band_list + band_base[k_], band_count + k_);
+            launch_band();
         });
         timed(1, (any_tvf || any_corr) ? 2 * ncls : ncls, [&] {
-            if (any_tvf || any_corr) SPH_CLASSES_F(4, k_sweep_M, snap, drho, bmat, bk);
-            SPH_CLASSES_F(4, k_sweep_V, snap, drho, vel, bmat, acc_visc, pos);
+            launch_setup();
         });
         for (;;) {
             timed(2, use_work ? 3 : 1, [&] {
@@ -676,11 +680,9 @@ template <typename T> struct EngineT : Engine {
                 launch_work_lists();
             });
             timed(3, ncls, [&] { launch_colour(); });
-            timed(6, nlist, [&] {
-                SPH_CLASSES_BAND(k_sweep_S, surface_lanes(), band_list + band_base[k_], band_count + k_, band, snap, vel, gradC, acc_surf, bk, drho);
-            });
-            timed(4, ncls, [&] { SPH_CLASSES_LF(4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk); });
-            timed(5, ncls, [&] { SPH_CLASSES_LF(4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos); });
+            timed(6, nlist, [&] { launch_surface(); });
+            timed(4, ncls, [&] { launch_B(); });
+            timed(5, ncls, [&] { launch_C(); });
             if (rc) break;
             int flag = 0;
             cudaError_t e = cudaMemcpy(&flag, d_loop_flag, sizeof(int), cudaMemcpyDeviceToHost);

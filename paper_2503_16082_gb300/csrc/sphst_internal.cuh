@@ -79,6 +79,8 @@ template <typename T> struct CasePhys {
     T two_phi[2];              // 2 phi_i of a cross-phase pair, i in fluid k (Eq. 23)
     T four_phi_phi;            // 4 phi_i phi_j of a cross-phase pair
     T vol_wall;                // dp^dim
+    T mhalf_inv_h, kcoef_h;    // -1 / (2h); kcoef / h: W'/r = kcoef_h (1 - q/2)^3
+    T mass_c0[2], c0_vol;      // m c0 per fluid; c0 dp^dim
     T nhat_eps;                // |gradC| h threshold of an interface particle
     T tvf_coef;                // -alpha h^2 (Eq. 14, sign reading)
     T beta_k, beta_lo, beta_hi; // Eq. 11 limiter as min(max(beta_k dU, lo), hi) per reading
@@ -111,7 +113,7 @@ struct CaseDesc {
     int32_t nbr_mode;          // 0: neighbour list built per advection step; 1: cell walk
     int32_t nbr_k;             // list capacity per particle
     int64_t nbr_base;          // first list word of this case
-    int64_t f_begin;           // first fluid rank (list slot) of this case
+    int64_t f_begin;           // first slot of this case
     CasePhys<float> pf;
     CasePhys<double> pd;
 };

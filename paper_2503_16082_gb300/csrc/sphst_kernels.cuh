@@ -38,38 +38,20 @@
 //                      sweeps (caps registers per thread)
 //   SPHST_SWEEPB_MINB  the same for sweep B alone (default 4: 64 registers)
 //   SPHST_SWEEPB_MINB_ONE  the same for the FP32 sweep B of a one-case engine
-//                      (default 5: 48 registers, as its per-case constants are
-//                      not in registers; measured 6 (40) and 4 slower)
-//   SPHST_SURFACE_MIN_LANES  least lanes per band particle of sweep S (1, 2, 4)
-//   SPHST_SWEEPAS_MINB the same for sweeps A and S (default 4: with the
-//                      64-register room the compiler keeps more loads in
-//                      flight; measured: A 35 -> 28 us, S 93 -> 89 us on the
-//                      3D drop)
-//   SPHST_LIST_PREFETCH 1: load list entry k+1 while pair k is evaluated;
-//                      2: entries k+1 and k+2 (measured: a general ring of
-//                      2-4 entries compiles to slower sweeps)
+//                      (default 6: 42 registers, as its per-case constants are
+//                      not in registers; 1M particles: 6 250 us, 5 271, 7 279)
+//   SPHST_SWEEPAS_MINB the same for sweep A of the cell-walk classes
 //   SPHST_FAST_DIV     1: FP32 pair divisions through the SFU reciprocal
-//   SPHST_F32X2        1: x/y components of the FP32 pair geometry and sums in
-//                      packed two-lane instructions (sm_100 and later)
 //   SPHST_LIST_NOALLOC 1: the list words are read without allocating L1 lines
 //                      (measured +1% on the 3D drop)
-#ifndef SPHST_LIST_PREFETCH
-#define SPHST_LIST_PREFETCH 2
-#endif
 #ifndef SPHST_FAST_DIV
 #define SPHST_FAST_DIV 1
-#endif
-#ifndef SPHST_F32X2
-#define SPHST_F32X2 1
 #endif
 #ifndef SPHST_LIST_LDCS
 #define SPHST_LIST_LDCS 1
 #endif
 #ifndef SPHST_SWEEP_MINB
 #define SPHST_SWEEP_MINB 0
-#endif
-#ifndef SPHST_SURFACE_MIN_LANES
-#define SPHST_SURFACE_MIN_LANES 2
 #endif
 #ifndef SPHST_SWEEPAS_MINB
 #define SPHST_SWEEPAS_MINB 4
@@ -81,7 +63,7 @@
 #define SPHST_LIST_NOALLOC 1
 #endif
 #ifndef SPHST_SWEEPB_MINB_ONE
-#define SPHST_SWEEPB_MINB_ONE 5
+#define SPHST_SWEEPB_MINB_ONE 6
 #endif
 #if SPHST_SWEEP_MINB > 0
 #define SPH_SWEEP_BOUNDS __launch_bounds__(256, SPHST_SWEEP_MINB)
@@ -104,19 +86,46 @@
 // sweep B of a one-case engine reads its per-case constants from the
 // parameter block, which leaves it room for more resident blocks
 #define SPH_SWEEPB_BOUNDS_M(T, MODE)                                                          \
-    __launch_bounds__(256, (MODE) == 2 && sizeof(T) == 4 ? SPHST_SWEEPB_MINB_ONE                  \
+    __launch_bounds__(256, (MODE) == 3 ? 1 : sizeof(T) == 8 ? 2 : (MODE) == 2 ? SPHST_SWEEPB_MINB_ONE                  \
                                                          : (SPHST_SWEEPB_MINB > 0 ? SPHST_SWEEPB_MINB : 1))
 
 namespace sphst {
 
 // ------------------------------------------------------------------ helpers
-__device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
+// r^2 of a pair and rho_i + rho_j are normal numbers (a case whose r^2 is not
+// has a kernel derivative beyond FP32), so the flush-to-zero forms give the
+// same values without the scaling of denormal arguments
+__device__ __forceinline__ float rsq(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
 
 template <typename T> __device__ __forceinline__ V4<T> ld4(const V4<T> *p) { return *p; }
 template <> __device__ __forceinline__ V4<float> ld4<float>(const V4<float> *p) {
     float4 v = __ldg(reinterpret_cast<const float4 *>(p));
     return V4<float>{v.x, v.y, v.z, v.w};
+}
+
+// the same, issued where it stands: a gather that is to be in flight while
+// other neighbours are evaluated (a plain load, used behind a branch or in the
+// next iteration only, is moved down to its use by the compiler)
+__device__ __forceinline__ V4<float> ld4_now(const V4<float> *p) {
+    V4<float> v;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ V4<double> ld4_now(const V4<double> *p) {
+    V4<double> v;
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2+16];" : "=d"(v.z), "=d"(v.w) : "l"(p));
+    return v;
 }
 
 // Divisions inside the FP32 pair loops: __fdividef (error <= 2 ulp for
@@ -139,6 +148,10 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
 }
 __device__ __forceinline__ double rsqrt_fast(double x) { return 1.0 / sqrt(x); }
 
+// a / b of the pair sums: in FP32 a times the SFU reciprocal (<= 2 ulp)
+__device__ __forceinline__ float vdiv(float a, float b) { return __fmul_rn(a, rcp_approx(b)); }
+__device__ __forceinline__ double vdiv(double a, double b) { return a / b; }
+
 // b - 1 as a floating-point value for a 2-bit field b (0..2), without an
 // integer conversion: the bit pattern 2^23 + b (2^52 + b) is exact and the
 // subtraction of 2^23 + 1 (2^52 + 1) is exact too
@@ -149,53 +162,15 @@ __device__ __forceinline__ double code_off(uint32_t b, double) {
     return __dsub_rn(__longlong_as_double(0x4330000000000000ll | (long long)b), 4503599627370497.0);
 }
 
-// Two-lane (x, y) arithmetic, each lane rounded once: packed FP32
-// instructions for float, scalar operations for double.
-template <typename T> struct L2 { T x, y; };
-template <typename T> __device__ __forceinline__ L2<T> l2(T x, T y) { return L2<T>{x, y}; }
-__device__ __forceinline__ L2<float> fma2(L2<float> a, L2<float> b, L2<float> c) {
-#if SPHST_F32X2
-    const float2 r = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
-    return L2<float>{r.x, r.y};
-#else
-    return L2<float>{__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y)};
-#endif
-}
-__device__ __forceinline__ L2<float> add2(L2<float> a, L2<float> b) {
-#if SPHST_F32X2
-    const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
-    return L2<float>{r.x, r.y};
-#else
-    return L2<float>{__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)};
-#endif
-}
-__device__ __forceinline__ L2<float> mul2(L2<float> a, L2<float> b) {
-#if SPHST_F32X2
-    const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
-    return L2<float>{r.x, r.y};
-#else
-    return L2<float>{__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)};
-#endif
-}
-__device__ __forceinline__ L2<double> fma2(L2<double> a, L2<double> b, L2<double> c) {
-    return L2<double>{__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y)};
-}
-__device__ __forceinline__ L2<double> add2(L2<double> a, L2<double> b) {
-    return L2<double>{__dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y)};
-}
-__device__ __forceinline__ L2<double> mul2(L2<double> a, L2<double> b) {
-    return L2<double>{__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y)};
-}
-// 1 - b for the 2-bit offset fields (bx, by), exactly: -(2^23 + b) + (2^23 + 1)
-__device__ __forceinline__ L2<float> neg_code_off2(uint32_t bx, uint32_t by, float) {
-    return add2(l2(__uint_as_float(0xCB000000u | bx), __uint_as_float(0xCB000000u | by)),
-                l2(8388609.0f, 8388609.0f));
-}
-__device__ __forceinline__ L2<double> neg_code_off2(uint32_t bx, uint32_t by, double) {
-    return add2(l2(__longlong_as_double((long long)(0xC330000000000000ull | bx)),
-                   __longlong_as_double((long long)(0xC330000000000000ull | by))),
-                l2(4503599627370497.0, 4503599627370497.0));
-}
+// Every operation of the pair sums is explicitly rounded, so a particle's
+// sums have the same bits whichever kernel computes them and whatever its
+// register allocation.
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double vadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
 
 // a ? x1 : x0 for the two fluid phases' constants (no indexed loads)
 template <typename T> __device__ __forceinline__ T sel(uint32_t k, T x0, T x1) { return k ? x1 : x0; }
@@ -261,16 +236,9 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 // printed form (P_L + P_R)/(rho_L + rho_R) of the pair
 __device__ __forceinline__ float clamp_lh(float x, float lo, float hi) { return fminf(fmaxf(x, lo), hi); }
 __device__ __forceinline__ double clamp_lh(double x, double lo, double hi) { return fmin(fmax(x, lo), hi); }
-template <typename T> struct Limiter {
-    T k, lo, hi;
-    bool printed;
-    __device__ __forceinline__ Limiter(const CasePhys<T> &cp, int mode)
-        : k(cp.beta_k), lo(cp.beta_lo), hi(cp.beta_hi), printed(mode == 3) {}
-    __device__ __forceinline__ T operator()(T dU, T psum, T rhosum) const {
-        const T x = printed ? k * dU * div_fast(psum, rhosum) : k * dU;
-        return clamp_lh(x, lo, hi);
-    }
-};
+// the no-suction wall reading's floor
+__device__ __forceinline__ float vpush(float x) { return x > 0.0f ? x : 0.0f; }
+__device__ __forceinline__ double vpush(double x) { return x > 0.0 ? x : 0.0; }
 
 // Neighbour cell index along axis a: wrapped on a periodic axis (the cells
 // tile the period exactly, so the cell at -1 is the last one and lies one
@@ -326,20 +294,20 @@ __device__ __forceinline__ bool walk(const CaseDesc &d, const CasePhys<T> &cp,
     return coincident;
 }
 
-// Neighbour list of the frozen configuration.  The fluid particle of local
-// rank r (its slot) holds entry k at word ((r / 32) K + k) 32 + r % 32 of its
-// case's lists, K the list capacity: a warp's 32 slots own one contiguous
-// block of K rows, a row of 32 words is one 128-byte line, and consecutive
-// entries are one row apart whatever the case's size.  An entry is
-// j << 6 | cell code, the code holding (o + 1) per axis in 2 bits, o the
-// neighbour cell's offset.  Each list holds the neighbours of the other fluid
-// phase first, then the rest, each part in increasing j;
-// cnt[i] = count | (other-phase count << 16),
+// Neighbour list of the frozen configuration.  A slot is one fluid particle,
+// by its rank among them.  The slot of local number r holds entry k at word
+// ((r / 32) K + k) 32 + r % 32 of its case's lists, K the list capacity: a
+// warp's 32 slots own one contiguous block of K rows, a row of 32 words is one
+// 128-byte line, and consecutive entries are one row apart whatever the case's
+// size.  An entry is j << 6 | cell code, the code holding (o + 1) per axis in
+// 2 bits, o the neighbour cell's offset.  Each list holds the neighbours of
+// the other fluid phase first, then the rest, each part in increasing j;
+// cnt[slot] = count | (other-phase count << 16),
 // so the colour-gradient sweep reads only the first part.
 constexpr uint32_t NBR_SHIFT = 6;
 constexpr uint32_t CNT_MASK = 0xffffu;
 constexpr int LROW = 32;                        // words between consecutive entries of a list
-// first word of the list of global fluid rank q
+// first word of the list of global slot q
 __device__ __forceinline__ int64_t list_word(const CaseDesc &d, int64_t q) {
     const int64_t r = q - d.f_begin;
     return d.nbr_base + (r >> 5) * ((int64_t)d.nbr_k * LROW) + (r & 31);
@@ -350,131 +318,114 @@ __device__ __forceinline__ uint32_t cell_code(int ox, int oy, int oz) {
     return (uint32_t)(ox + 1) | ((uint32_t)(oy + 1) << 2) | (D == 3 ? ((uint32_t)(oz + 1) << 4) : 0u);
 }
 
-// With L lanes per particle, lane `sub` of the particle's group takes the
-// entries sub, sub + L, sub + 2L, ... of its list.
-template <int PART, typename T, int D, int L = 1, typename F>
-__device__ __forceinline__ void walk_list(const CaseDesc &d, const CasePhys<T> &cp,
-                                          const uint32_t *__restrict__ nbr,
-                                          const uint32_t *__restrict__ cnt,
-                                          const V4<T> *__restrict__ snap, int64_t i, int64_t slot,
-                                          const V4<T> &si, F &&f, uint32_t sub = 0) {
-    constexpr int stride = LROW;
-    const uint32_t *p = nbr + list_word(d, slot) + (int)sub * stride;
-    const uint32_t c = PART == PART_OTHER ? cnt[i] >> 16 : cnt[i] & CNT_MASK;
-    const T cs = cp.cs;
-#if SPHST_LIST_PREFETCH >= 2
-    uint32_t next = sub < c ? ld_list_walk(p) : 0u;
-    uint32_t next2 = sub + L < c ? ld_list_walk(p + L * stride) : 0u;
-    p += L * stride;
-#elif SPHST_LIST_PREFETCH
-    uint32_t next = sub < c ? ld_list_walk(p) : 0u;
-#endif
+// r_ij = s_i - (s_j + o cs): the neighbour's offset moved into i's cell, once
+// for all particles that look at it (o cs is exact, so the sum rounds once)
+template <typename T, int D> struct Moved { T nx, ny, nz; };   // -(s_j + o cs)
+template <typename T, int D>
+__device__ __forceinline__ Moved<T, D> moved(uint32_t e, const V4<T> &sj, T cs) {
+    return Moved<T, D>{fma_rn(-code_off(e & 3u, T()), cs, -sj.x), fma_rn(-code_off((e >> 2) & 3u, T()), cs, -sj.y),
+                       D == 3 ? fma_rn(-code_off((e >> 4) & 3u, T()), cs, -sj.z) : T(0)};
+}
+
+// How a sweep gathers its neighbours (U of walk_list), by measurement at 1M and
+// 64k particles in 3D and 37k in 2D (FP32; us per launch, PLAIN against the
+// choice):  C 237 -> 213, 33 -> 25 (AHEAD), 16.0 -> 12.7 (4, in 2D);
+// V + M 977 -> 822, 134 -> 107; A 19.3 -> 14.6; S 72 -> 63, 31 -> 27 (4).
+// Sweep B at 1M particles stays PLAIN (250 against 271-300): its arithmetic
+// leaves no registers for a neighbour in flight at the warps it needs.
+constexpr int PLAIN = 1, AHEAD = -1;
+// A list: f(e, s_j, aux_j) for the first c entries from word p on, in order.
+// With L lanes, lane `sub` of the group takes the entries sub, sub + L,
+// sub + 2L, ...  AUX: a second record per neighbour is gathered too.
+// PLAIN keeps two list words in flight and leaves the latency of the gathers
+// to the other warps; AHEAD gathers the next neighbour while the current one
+// is evaluated and reads list words four entries ahead of it (a word comes
+// from HBM and is needed one evaluation earlier); U > 1 gathers U neighbours
+// before the first is evaluated.  The order of the entries, and with it every
+// sum, is the same.
+template <bool AUX, typename T, int L, int U, typename F>
+__device__ __forceinline__ void walk_list(const uint32_t *__restrict__ p, uint32_t c, const V4<T> *__restrict__ snap,
+                                          const V4<T> *__restrict__ aux, F &&f, uint32_t sub) {
+    p += (int)sub * LROW;
+    if constexpr (U == PLAIN) {
+        uint32_t next = sub < c ? ld_list_walk(p) : 0u;
+        uint32_t next2 = sub + L < c ? ld_list_walk(p + L * LROW) : 0u;
+        p += L * LROW;
 #pragma unroll 1
-    for (uint32_t k = sub; k < c; k += L) {
-#if SPHST_LIST_PREFETCH >= 2
-        const uint32_t e = next;            // entries k + L and k + 2L in flight
-        next = next2;
-        p += L * stride;
-        if (k + 2 * L < c) next2 = ld_list_walk(p);
-#elif SPHST_LIST_PREFETCH
-        const uint32_t e = next;
-        p += L * stride;
-        if (k + L < c) next = ld_list_walk(p);
-#else
-        const uint32_t e = ld_list_walk(p);
-        p += L * stride;
-#endif
-        const uint32_t j = e >> NBR_SHIFT;
-        const V4<T> sj = ld4(snap + j);
-        // s_i - o cs with o in {-1, 0, 1}: o cs is exact, so the FMA rounds
-        // once, exactly like the cell walk's subtraction
-        const T rx = sub_rn(fma_rn(-code_off(e & 3u, T()), cs, si.x), sj.x);
-        const T ry = sub_rn(fma_rn(-code_off((e >> 2) & 3u, T()), cs, si.y), sj.y);
-        T rz = T(0);
-        if (D == 3) rz = sub_rn(fma_rn(-code_off((e >> 4) & 3u, T()), cs, si.z), sj.z);
-        const T r2 = norm2<T, D>(rx, ry, rz);
-        f(j, sj, rx, ry, rz, r2);
+        for (uint32_t k = sub; k < c; k += L) {
+            const uint32_t e = next;            // entries k + L and k + 2L in flight
+            next = next2;
+            p += L * LROW;
+            if (k + 2 * L < c) next2 = ld_list_walk(p);
+            const uint32_t j = e >> NBR_SHIFT;
+            const V4<T> sj = ld4(snap + j);
+            f(e, sj, AUX ? ld4(aux + j) : sj);
+        }
+    } else if constexpr (U == AHEAD) {
+        const auto word = [&](uint32_t k) { return k < c ? ld_list_walk(p + (int64_t)(k - sub) * LROW) : 0u; };
+        uint32_t e = word(sub), w1 = word(sub + L), w2 = word(sub + 2 * L), w3 = word(sub + 3 * L);
+        V4<T> sj = ld4_now(snap + (e >> NBR_SHIFT)), aj = AUX ? ld4_now(aux + (e >> NBR_SHIFT)) : sj;
+        p += 4 * L * LROW;
+#pragma unroll 2
+        for (uint32_t k = sub; k < c; k += L) {
+            const V4<T> sn = ld4_now(snap + (w1 >> NBR_SHIFT)), an = AUX ? ld4_now(aux + (w1 >> NBR_SHIFT)) : sn;
+            uint32_t w4 = 0u;
+            if (k + 4 * L < c) w4 = ld_list_walk(p);
+            p += L * LROW;
+            f(e, sj, AUX ? aj : sj);
+            e = w1;
+            w1 = w2;
+            w2 = w3;
+            w3 = w4;
+            sj = sn;
+            aj = an;
+        }
+    } else {
+        uint32_t next[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) next[u] = sub + u * L < c ? ld_list_walk(p + u * L * LROW) : 0u;
+#pragma unroll 1
+        for (uint32_t k = sub; k < c; k += U * L) {
+            uint32_t e[U];
+            V4<T> sj[U], aj[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {       // a missing entry gathers particle 0 and is dropped
+                e[u] = next[u];
+                sj[u] = ld4_now(snap + (e[u] >> NBR_SHIFT));
+                if (AUX) aj[u] = ld4_now(aux + (e[u] >> NBR_SHIFT));
+            }
+            p += U * L * LROW;
+#pragma unroll
+            for (int u = 0; u < U; ++u) next[u] = k + (U + u) * L < c ? ld_list_walk(p + u * L * LROW) : 0u;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (k + u * L < c) f(e[u], sj[u], AUX ? aj[u] : sj[u]);
+        }
     }
 }
 
-// The list walk with one more per-neighbour array: f(j, s_j, aux_j, r_ij, r^2).
-template <typename T, int D, int L = 1, typename F>
-__device__ __forceinline__ void walk_list_aux(const CaseDesc &d, const CasePhys<T> &cp,
-                                              const uint32_t *__restrict__ nbr,
-                                              const uint32_t *__restrict__ cnt,
-                                              const V4<T> *__restrict__ snap,
-                                              const V4<T> *__restrict__ aux, int64_t i, int64_t slot,
-                                              const V4<T> &si, F &&f, uint32_t sub = 0) {
-    constexpr int stride = LROW;
-    const uint32_t *p = nbr + list_word(d, slot) + (int)sub * stride;
-    const uint32_t c = cnt[i] & CNT_MASK;
-    const T cs = cp.cs;
-    const auto pair = [&](uint32_t e, const V4<T> &sj, const V4<T> &aj) {
-        // (s_i - o cs) - s_j per axis, each step rounded once as in the cell walk
-        const L2<T> t = fma2(neg_code_off2(e & 3u, (e >> 2) & 3u, T()), l2(cs, cs), l2(si.x, si.y));
-        const L2<T> rxy = fma2(l2(sj.x, sj.y), l2(T(-1), T(-1)), t);
-        const T rx = rxy.x, ry = rxy.y;
-        T rz = T(0);
-        if (D == 3) rz = sub_rn(fma_rn(-code_off((e >> 4) & 3u, T()), cs, si.z), sj.z);
-        f(e >> NBR_SHIFT, sj, aj, rx, ry, rz, norm2<T, D>(rx, ry, rz));
-    };
-#if SPHST_LIST_PREFETCH >= 2
-    uint32_t next = sub < c ? ld_list_walk(p) : 0u;
-    uint32_t next2 = sub + L < c ? ld_list_walk(p + L * stride) : 0u;
-    p += L * stride;
-#elif SPHST_LIST_PREFETCH
-    uint32_t next = sub < c ? ld_list_walk(p) : 0u;
-#endif
-#pragma unroll 1
-    for (uint32_t k = sub; k < c; k += L) {
-#if SPHST_LIST_PREFETCH >= 2
-        const uint32_t e = next;            // entries k + L and k + 2L in flight
-        next = next2;
-        p += L * stride;
-        if (k + 2 * L < c) next2 = ld_list_walk(p);
-#elif SPHST_LIST_PREFETCH
-        const uint32_t e = next;
-        p += L * stride;
-        if (k + L < c) next = ld_list_walk(p);
-#else
-        const uint32_t e = ld_list_walk(p);
-        p += L * stride;
-#endif
-        const uint32_t j = e >> NBR_SHIFT;
-        pair(e, ld4(snap + j), ld4(aux + j));
-    }
-}
-
-// neighbours of i with aux[j] loaded for f(j, s_j, aux_j, r_ij, r^2), from the
-// list or the cell walk
-template <bool LIST, typename T, int D, int L = 1, typename F>
-__device__ __forceinline__ bool neighbors_aux(const CaseDesc &d, const CasePhys<T> &cp,
-                                              const uint32_t *starts, const uint32_t *nbr,
-                                              const uint32_t *cnt, const V4<T> *snap, const V4<T> *aux,
-                                              int64_t i, int64_t slot, const V4<T> &si, uint32_t pki, F &&f,
-                                              uint32_t sub = 0) {
+// neighbours of particle i as f(j, s_j, aux_j, r_ij, r^2), from the list at
+// word `list` (count as in cnt[]) or from the cell walk, which visits all:
+// PART_OTHER leaves the choice to the caller
+template <bool LIST, bool AUX, typename T, int D, int PART = PART_ALL, int L = 1, int U = PLAIN, typename F>
+__device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &cp, const uint32_t *starts,
+                                          const uint32_t *list, uint32_t count, const V4<T> *snap,
+                                          const V4<T> *aux, int64_t i, const V4<T> &si, uint32_t pki,
+                                          F &&f, uint32_t sub = 0) {
     if constexpr (LIST) {
-        walk_list_aux<T, D, L>(d, cp, nbr, cnt, snap, aux, i, slot, si, f, sub);
+        const T cs = cp.cs;
+        walk_list<AUX, T, L, U>(list, PART == PART_OTHER ? count >> 16 : count & CNT_MASK, snap, aux,
+            [&](uint32_t e, const V4<T> &sj, const V4<T> &aj) {
+                const Moved<T, D> m = moved<T, D>(e, sj, cs);
+                const T rx = vadd(si.x, m.nx), ry = vadd(si.y, m.ny), rz = D == 3 ? vadd(si.z, m.nz) : T(0);
+                f(e >> NBR_SHIFT, sj, aj, rx, ry, rz, norm2<T, D>(rx, ry, rz));
+            }, sub);
         return false;
     } else {
         return walk<T, D>(d, cp, starts, snap, i, si, pki,
-            [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) { f(j, sj, ld4(aux + j), rx, ry, rz, r2); });
-    }
-}
-
-// neighbours of i from the list (LIST) or from the cell walk; PART_OTHER
-// restricts the list to the other fluid phase (the cell walk visits all and
-// the caller filters)
-template <bool LIST, typename T, int D, int PART = PART_ALL, int L = 1, typename F>
-__device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &cp,
-                                          const uint32_t *starts, const uint32_t *nbr,
-                                          const uint32_t *cnt, const V4<T> *snap, int64_t i, int64_t slot,
-                                          const V4<T> &si, uint32_t pki, F &&f, uint32_t sub = 0) {
-    if constexpr (LIST) {
-        walk_list<PART, T, D, L>(d, cp, nbr, cnt, snap, i, slot, si, f, sub);
-        return false;
-    } else {
-        return walk<T, D>(d, cp, starts, snap, i, si, pki, f);
+            [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
+                f(j, sj, AUX ? ld4(aux + j) : sj, rx, ry, rz, r2);
+            });
     }
 }
 
@@ -503,20 +454,63 @@ __device__ __forceinline__ PairGeo<T> geo(const CasePhys<T> &cp, T r2) {
     g.dW = cp.kcoef * q * u * u * u;
     return g;
 }
-// the same with the kernel constants held in registers by the caller
-template <typename T> struct KernelGeo {
-    T inv_h, kcoef;
-    __device__ __forceinline__ explicit KernelGeo(const CasePhys<T> &cp) : inv_h(cp.inv_h), kcoef(cp.kcoef) {}
-    __device__ __forceinline__ PairGeo<T> operator()(T r2) const {
-        PairGeo<T> g;
-        g.inv_r = rsq(r2);
-        g.r = r2 * g.inv_r;
-        const T q = g.r * inv_h;
-        const T u = fma_rn(T(-0.5), q, T(1));
-        g.dW = kcoef * q * u * u * u;
-        return g;
+// the pair geometry the sums need: 1/r, r and W'/r = (kcoef / h) (1 - q/2)^3,
+// so that r_ij itself carries the direction of every pair term.
+template <typename T> struct PairW { T inv, r, w; };
+template <typename T> __device__ __forceinline__ PairW<T> pair_w(const CasePhys<T> &cp, T r2) {
+    PairW<T> g;
+    g.inv = rsq(r2);
+    g.r = vmul(r2, g.inv);
+    const T u = vfma(g.r, cp.mhalf_inv_h, T(1));
+    g.w = vmul(vmul(vmul(cp.kcoef_h, u), u), u);
+    return g;
+}
+// (v_j - v_i) . r_ij, from -v_i
+template <typename T, int D>
+__device__ __forceinline__ T pair_dot(const V4<T> &vj, T nvx, T nvy, T nvz, T rx, T ry, T rz) {
+    const T dx = vadd(vj.x, nvx), dy = vadd(vj.y, nvy);
+    if (D == 2) return vfma(dx, rx, vmul(dy, ry));
+    return vfma(dx, rx, vfma(dy, ry, vmul(vadd(vj.z, nvz), rz)));
+}
+// Pressure (Eqs. 7-12): the factor f of one neighbour's term f r_ij in
+// sum_j P* grad W V_j, for particles of densities rho_i and c0 drho_i = b_i.
+// With p = c0^2 drho, P* = c0 (rho_j (b_i + beta rho_i dU) + rho_i c0 drho_j) /
+// (rho_i + rho_j) (Eqs. 8, 12; beta of Eq. 11) and V_j = m_j / rho_j: one
+// division.  Walls by their mirror state rho_i, p_i, 2 U_w - U_L.
+template <typename T>
+__device__ __forceinline__ T pressure_factor(const CasePhys<T> &cp, bool printed, bool push_only, uint32_t kj, T drj,
+                                             T dot, const PairW<T> &g, T rho_i, T b_i) {
+    T dU = vmul(dot, g.inv);                    // U_L - U_R = (v_j - v_i).e (Eq. 10, U = -v.e)
+    if (kj == PH_WALL) {
+        dU = vmul(T(2), dU);
+        T x = vmul(cp.beta_k, dU);
+        if (printed) x = vmul(x, vdiv(vmul(cp.c0, b_i), rho_i));
+        T ps = vfma(vmul(vmul(clamp_lh(x, cp.beta_lo, cp.beta_hi), rho_i), dU), T(0.5), b_i);   // P* / c0
+        if (push_only) ps = vpush(ps);          // no-suction wall reading
+        return vmul(vmul(ps, cp.c0_vol), g.w);
     }
-};
+    const T rho_j = add_rn(sel(kj, cp.rho0[0], cp.rho0[1]), drj), a_j = mul_rn(cp.c0, drj);
+    const T rs = vadd(rho_i, rho_j);
+    T x = vmul(cp.beta_k, dU);
+    if (printed) x = vmul(x, vdiv(vmul(cp.c0, vadd(b_i, a_j)), rs));
+    const T t = vfma(vmul(clamp_lh(x, cp.beta_lo, cp.beta_hi), dU), rho_i, b_i);
+    const T num = vfma(rho_j, t, vmul(rho_i, a_j));
+    return vmul(vdiv(vmul(num, sel(kj, cp.mass_c0[0], cp.mass_c0[1])), vmul(rs, rho_j)), g.w);
+}
+// Continuity (Eq. 6): (v_i - v*).e V_j of one neighbour, with
+// (v_i - v*).e = U* - U_L = (rho_j (v_i - v_j).e + (b_i - c0 drho_j)) /
+// (rho_i + rho_j); the printed v* takes the other sign of the pressure
+// difference, folded into sb_i and nsc0 = -(+-c0).  v* = v_w at a wall.
+template <typename T>
+__device__ __forceinline__ T continuity_factor(const CasePhys<T> &cp, uint32_t kj, T drj, T dot, const PairW<T> &g,
+                                               T rho_i, T sb_i, T nsc0) {
+    const T dU = vmul(dot, g.inv);
+    if (kj == PH_WALL) return vmul(dU, -cp.vol_wall);
+    const T rho_j = add_rn(sel(kj, cp.rho0[0], cp.rho0[1]), drj);
+    const T num = vfma(-rho_j, dU, vadd(sb_i, mul_rn(nsc0, drj)));
+    return vdiv(vmul(num, sel(kj, cp.mass[0], cp.mass[1])),
+                vmul(vadd(rho_i, rho_j), rho_j));
+}
 
 // ================================================================ rebuild
 // First placement of a freshly uploaded case: absolute FP64 positions ->
@@ -737,12 +731,12 @@ __global__ void k_copy_back(int64_t n, const V4<T> *pos_t, const V4<T> *vel_t, c
     id[d] = id_t[d];
 }
 
-// ---- fluid ranks: after the reorder, the sorted positions of the fluid
-// particles, walls left out (an exclusive scan of the fluid flags, then a
-// scatter).  The list build, the band and sweeps M, V, B and C (and A with
-// the cell walk) run their tiles over these ranks, so no lane of theirs idles on a wall particle (16%
-// of the 3D drop, interleaved with the fluid near the walls by the Morton
-// order).  Each case's fluid particles take the ranks after the previous
+// ---- fluid ranks: after the reorder, the fluid particles in sorted order, walls
+// left out: a particle's slot.  The list build, the band and sweeps M, V, B
+// and C (and A with the cell walk) run their tiles over the slots, so no lane
+// of theirs idles on a wall particle (16% of the 3D drop, interleaved with the
+// fluid near the walls by the Morton order).  Flags, an exclusive scan of them,
+// a scatter.  Each case's fluid particles take the slots after the previous
 // cases' ones, whose count is fixed.
 template <typename T>
 __global__ void k_fluid_flag(int64_t n, const V4<T> *snap, uint32_t *flag) {
@@ -751,35 +745,36 @@ __global__ void k_fluid_flag(int64_t n, const V4<T> *snap, uint32_t *flag) {
     flag[i] = (i < n && phase_of(w_bits(snap[i].w)) != PH_WALL) ? 1u : 0u;
 }
 
-// Wall particles get their fixed values here, since no sweep visits them: a
-// zero colour gradient and an empty neighbour list.  The first fluid particle
-// of each cell of a list case appends the cell, as (case << 32 | table
-// index), to its class's cell list for the list build (warp-aggregated; the
-// order is irrelevant, neighbouring cells stay close).
+// Writes each slot's particle and the values a rebuild starts from: a zero
+// colour gradient (the list classes' colour sweep then writes only the
+// interface band) and an empty band.  The first fluid particle of each cell of
+// a list case appends the cell, as (case << 32 | its first particle), to its
+// class's cell list for the list build (warp-aggregated; the order is
+// irrelevant, neighbouring cells stay close).  A cell's particles are found by
+// their packed cell coordinates: both dimensions share this kernel, which
+// therefore forms no Morton code.
+constexpr uint32_t CELL_BITS = 0x3fffffffu;     // the cell coordinates of a packed word
 template <typename T>
 __global__ void k_fluid_scatter(const Tile *__restrict__ tiles, const CaseDesc *__restrict__ desc, const V4<T> *snap,
-                                const uint32_t *rank, const uint32_t *starts, uint32_t *fidx, V4<T> *gradC,
-                                uint32_t *cnt, uint8_t *band, uint64_t *clist, uint32_t *ccount, int64_t base2d) {
+                                const uint32_t *rank, uint32_t *fidx, V4<T> *gradC, uint8_t *band, uint64_t *clist,
+                                uint32_t *ccount, int64_t base2d) {
     const Tile t = tiles[blockIdx.x];
     const CaseDesc &d = desc[t.c];
     const int64_t i = t.begin + threadIdx.x;
     bool first = false;
-    uint32_t m = 0;
+    uint32_t b = (uint32_t)i;
     if ((int)threadIdx.x < t.n) {
-        // the colour gradient starts every advection step at zero: the list
-        // classes' colour sweep then writes only the interface band
         gradC[i] = V4<T>{T(0), T(0), T(0), T(0)};
-        band[i] = 0;                             // the list build marks the interface band
+        band[i] = 0;
         const uint32_t pk = w_bits(snap[i].w);
         if (phase_of(pk) != PH_WALL) {
-            const uint32_t r = rank[i];
-            fidx[r] = (uint32_t)i;
-            if (d.nbr_mode == 0) {
-                m = (uint32_t)d.table_off + (d.dim == 3 ? morton_of_packed<3>(pk) : morton_of_packed<2>(pk));
-                first = rank[starts[m]] == r;
+            fidx[rank[i]] = (uint32_t)i;
+            first = d.nbr_mode == 0;
+            for (; first && (int64_t)b > d.p_begin; --b) {
+                const uint32_t pk2 = w_bits(snap[b - 1].w);
+                if ((pk2 ^ pk) & CELL_BITS) break;
+                first = phase_of(pk2) == PH_WALL;
             }
-        } else {
-            cnt[i] = 0u;
         }
     }
     const unsigned mask = __ballot_sync(0xffffffffu, first);
@@ -790,7 +785,7 @@ __global__ void k_fluid_scatter(const Tile *__restrict__ tiles, const CaseDesc *
     if (lane == leader) base = atomicAdd(ccount + k, (uint32_t)__popc(mask));
     base = __shfl_sync(0xffffffffu, base, leader);
     if (first)
-        clist[(k ? base2d : 0) + base + __popc(mask & ((1u << lane) - 1u))] = ((uint64_t)(uint32_t)t.c << 32) | m;
+        clist[(k ? base2d : 0) + base + __popc(mask & ((1u << lane) - 1u))] = ((uint64_t)(uint32_t)t.c << 32) | b;
 }
 
 // ================================================================ time step
@@ -930,18 +925,18 @@ static __global__ void k_adv_end(int ncases, CaseState *st) {
 // ================================================================= sweeps
 // ---- M: correction matrix of Eq. 15, B_i = -(sum_j r_ij (x) grad_i W_ij V_j)^-1
 template <typename T> struct Moment {
-    T m00 = 0, m01 = 0, m02 = 0, m11 = 0, m12 = 0, m22 = 0;
-    // adds r (x) dW e V = (dW V / r) r_vec (x) r_vec of one neighbour
-    template <int D>
-    __device__ __forceinline__ void add(const CaseDesc &, const CasePhys<T> &cp, const T *drho, uint32_t j,
-                                        uint32_t kj, T rx, T ry, T rz, T r2) {
-        const PairGeo<T> g = geo(cp, r2);
-        const T Vj = kj == PH_WALL ? cp.vol_wall : div_fast(cp.mass[kj], cp.rho0[kj] + drho[j]);
-        const T s = g.dW * Vj * g.inv_r;
-        m00 += s * rx * rx; m01 += s * rx * ry; m11 += s * ry * ry;
-        if (D == 3) { m02 += s * rx * rz; m12 += s * ry * rz; m22 += s * rz * rz; }
+    T m00, m01, m02, m11, m12, m22;
+    // adds (W' V / r) r_vec (x) r_vec of one neighbour, s = W' V / r
+    template <int D> __device__ __forceinline__ void add(T s, T rx, T ry, T rz) {
+        const T tx = vmul(s, rx), ty = vmul(s, ry);
+        m00 = vfma(tx, rx, m00); m01 = vfma(tx, ry, m01); m11 = vfma(ty, ry, m11);
+        if (D == 3) { m02 = vfma(tx, rz, m02); m12 = vfma(ty, rz, m12); m22 = vfma(vmul(s, rz), rz, m22); }
     }
 };
+template <typename T>
+__device__ __forceinline__ T volume_of(const CasePhys<T> &cp, uint32_t kj, T drj) {
+    return kj == PH_WALL ? cp.vol_wall : vdiv(sel(kj, cp.mass[0], cp.mass[1]), add_rn(sel(kj, cp.rho0[0], cp.rho0[1]), drj));
+}
 
 template <typename T, int D>
 __device__ __forceinline__ void store_B(const Moment<T> &M, int64_t i, V4<T> *bmat) {
@@ -969,21 +964,22 @@ __device__ __forceinline__ void store_B(const Moment<T> &M, int64_t i, V4<T> *bm
 }
 
 template <bool LIST, typename T, int D>
-__device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp, int64_t i, int64_t slot,
-                                        const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap, const T *drho,
+__device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
+                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap, const T *drho,
                                         V4<T> *bmat, V4<T> *bk, int32_t *status) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
     const uint32_t ki = phase_of(pki);
     if (ki == PH_WALL) return;
     const bool own = bk != nullptr && d.surface_corr == 1;
-    Moment<T> M, Mk;
-    const bool coinc = neighbors<LIST, T, D>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki,
-        [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
+    Moment<T> M{}, Mk{};
+    const bool coinc = neighbors<LIST, false, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, list, count, snap, nullptr, i, si, pki,
+        [&](uint32_t j, const V4<T> &sj, const V4<T> &, T rx, T ry, T rz, T r2) {
             const uint32_t kj = phase_of(w_bits(sj.w));
-            M.template add<D>(d, cp, drho, j, kj, rx, ry, rz, r2);
+            const T w = vmul(pair_w<T>(cp, r2).w, volume_of(cp, kj, drho[j]));
+            M.template add<D>(w, rx, ry, rz);
             // the same sum over i's own fluid (surface_corr reading of Eq. 33)
-            if (own && kj == ki) Mk.template add<D>(d, cp, drho, j, kj, rx, ry, rz, r2);
+            if (own && kj == ki) Mk.template add<D>(w, rx, ry, rz);
         });
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
     store_B<T, D>(M, i, bmat);
@@ -991,9 +987,63 @@ __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp
 }
 
 // ---- V: viscous acceleration (Eq. 13) and transport shift (Eq. 14)
+// The sums of one particle: a = sum eta (v_i - v_j) W' V / r
+// (each step from -v_i) and the shift sum (B_i + B_j) grad W V with symmetric
+// B = [b00 b01 b02; b01 b11 b12; b02 b12 b22]
+template <typename T> struct ViscSum {
+    T ax, ay, az, sx, sy, sz;
+    // w = W' V_j / r, neta = -(pair viscosity), (b0, b1) = B_i
+    template <int D>
+    __device__ __forceinline__ void add(T w, T neta, bool tvf, const V4<T> &vj, T nvx, T nvy, T nvz, T rx, T ry, T rz,
+                                        const T (&b)[6], bool wall, const V4<T> &Bj0, const V4<T> &Bj1) {
+        const T f = vmul(neta, w);
+        ax = vfma(f, vadd(vj.x, nvx), ax);
+        ay = vfma(f, vadd(vj.y, nvy), ay);
+        if (D == 3) az = vfma(f, vadd(vj.z, nvz), az);
+        if (!tvf) return;
+        // a wall lends its fluid partner's B_i
+        const T b00 = wall ? b[0] : Bj0.x, b01 = wall ? b[1] : Bj0.y, b11 = wall ? b[3] : Bj0.w;
+        const T gx = vmul(w, rx), gy = vmul(w, ry);
+        sx = vfma(vadd(b[0], b00), gx, vfma(vadd(b[1], b01), gy, sx));
+        sy = vfma(vadd(b[1], b01), gx, vfma(vadd(b[3], b11), gy, sy));
+        if (D == 3) {
+            const T b02 = wall ? b[2] : Bj0.z, b12 = wall ? b[4] : Bj1.x, b22 = wall ? b[5] : Bj1.y;
+            const T gz = vmul(w, rz);
+            sx = vfma(vadd(b[2], b02), gz, sx);
+            sy = vfma(vadd(b[4], b12), gz, sy);
+            sz = vfma(vadd(b[2], b02), gx, vfma(vadd(b[4], b12), gy, vfma(vadd(b[5], b22), gz, sz)));
+        }
+    }
+};
+// the pair viscosity 2 eta_i eta_j / (eta_i + eta_j) takes one value per fluid
+// of j; walls use eta_i.  Negated.
+template <typename T> struct PairEta {
+    T wall, e0, e1;
+    __device__ __forceinline__ PairEta(const CasePhys<T> &cp, uint32_t ki) {
+        const T eta_i = sel(ki, cp.eta[0], cp.eta[1]);
+        wall = -eta_i;
+        e0 = -(T(2) * eta_i * cp.eta[0] / (eta_i + cp.eta[0]));
+        e1 = -(T(2) * eta_i * cp.eta[1] / (eta_i + cp.eta[1]));
+    }
+    __device__ __forceinline__ T operator()(uint32_t kj) const { return kj == PH_WALL ? wall : sel(kj, e0, e1); }
+};
+template <typename T, int D>
+__device__ __forceinline__ void store_V(const CasePhys<T> &cp, bool tvf, int64_t i, T rho_i, T ax, T ay, T az, T sx, T sy,
+                                        T sz, V4<T> *acc_visc, V4<T> *pos) {
+    const T c = T(2) / rho_i;
+    acc_visc[i] = V4<T>{vmul(c, ax), vmul(c, ay), vmul(c, az), T(0)};
+    if (tvf) {
+        V4<T> p = pos[i];
+        p.x = vfma(cp.tvf_coef, sx, p.x);
+        p.y = vfma(cp.tvf_coef, sy, p.y);
+        if (D == 3) p.z = vfma(cp.tvf_coef, sz, p.z);
+        pos[i] = p;
+    }
+}
+
 template <bool LIST, typename T, int D>
-__device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp, int64_t i, int64_t slot,
-                                        const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap, const T *drho,
+__device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
+                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap,
                                         const V4<T> *vel, const V4<T> *bmat, V4<T> *acc_visc,
                                         V4<T> *pos, int32_t *status) {
     const V4<T> si = ld4(snap + i);
@@ -1001,64 +1051,31 @@ __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp
     const uint32_t ki = phase_of(pki);
     if (ki == PH_WALL) return;
     const V4<T> vi = vel[i];
-    const T rho_i = sel(ki, cp.rho0[0], cp.rho0[1]) + vi.w;
-    // the pair viscosity 2 eta_i eta_j / (eta_i + eta_j) takes one value per
-    // fluid of j; walls use eta_i
-    const T eta_i = sel(ki, cp.eta[0], cp.eta[1]);
-    const T etab0 = T(2) * eta_i * cp.eta[0] / (eta_i + cp.eta[0]);
-    const T etab1 = T(2) * eta_i * cp.eta[1] / (eta_i + cp.eta[1]);
-    const T rho0_0 = cp.rho0[0], rho0_1 = cp.rho0[1], m_0 = cp.mass[0], m_1 = cp.mass[1];
-    const T vol_wall = cp.vol_wall;
-    const KernelGeo<T> kgeo(cp);
+    const PairEta<T> eta(cp, ki);
     const bool tvf = d.tvf_on != 0;
-    V4<T> Bi0 = {0, 0, 0, 0}, Bi1 = {0, 0, 0, 0};
-    if (tvf) { Bi0 = bmat[2 * i]; Bi1 = bmat[2 * i + 1]; }
-    T ax = 0, ay = 0, az = 0, sx = 0, sy = 0, sz = 0;
-    const bool coinc = neighbors_aux<LIST, T, D>(d, cp, starts, nbr, cnt, snap, vel, i, slot, si, pki,
+    T b[6] = {0, 0, 0, 0, 0, 0};
+    if (tvf) {
+        const V4<T> b0 = bmat[2 * i], b1 = bmat[2 * i + 1];
+        b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y;
+    }
+    ViscSum<T> S{};
+    const bool coinc = neighbors<LIST, true, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, list, count, snap, vel, i, si, pki,
         [&](uint32_t j, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
-            const PairGeo<T> g = kgeo(r2);
             const uint32_t kj = phase_of(w_bits(sj.w));
-            T eta_bar, Vj;
-            V4<T> Bj0 = Bi0, Bj1 = Bi1;
-            if (kj == PH_WALL) {
-                eta_bar = eta_i;
-                Vj = vol_wall;
-            } else {
-                eta_bar = sel(kj, etab0, etab1);
-                Vj = div_fast(sel(kj, m_0, m_1), sel(kj, rho0_0, rho0_1) + vj.w);
-                if (tvf) { Bj0 = bmat[2 * j]; Bj1 = bmat[2 * j + 1]; }
-            }
-            const T w = g.dW * Vj * g.inv_r;                 // grad W V = w r_vec
-            const T f = eta_bar * w;                          // eta (v_ij / r) dW V
-            ax += f * (vi.x - vj.x);
-            ay += f * (vi.y - vj.y);
-            if (D == 3) az += f * (vi.z - vj.z);
-            if (tvf) {
-                const T gx = w * rx, gy = w * ry, gz = w * rz;
-                // (B_i + B_j) grad W V with symmetric B = [b00 b01 b02; b01 b11 b12; b02 b12 b22]
-                const T s00 = Bi0.x + Bj0.x, s01 = Bi0.y + Bj0.y, s02 = Bi0.z + Bj0.z;
-                const T s11 = Bi0.w + Bj0.w, s12 = Bi1.x + Bj1.x, s22 = Bi1.y + Bj1.y;
-                sx += s00 * gx + s01 * gy + (D == 3 ? s02 * gz : T(0));
-                sy += s01 * gx + s11 * gy + (D == 3 ? s12 * gz : T(0));
-                if (D == 3) sz += s02 * gx + s12 * gy + s22 * gz;
-            }
+            const bool wall = kj == PH_WALL;
+            V4<T> B0{}, B1{};
+            if (tvf && !wall) { B0 = bmat[2 * j]; if (D == 3) B1 = bmat[2 * j + 1]; }
+            S.template add<D>(vmul(pair_w<T>(cp, r2).w, volume_of(cp, kj, vj.w)), eta(kj), tvf, vj, -vi.x, -vi.y, -vi.z,
+                                 rx, ry, rz, b, wall, B0, B1);
         });
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
-    const T c = T(2) / rho_i;
-    acc_visc[i] = V4<T>{c * ax, c * ay, c * az, T(0)};
-    if (tvf) {
-        V4<T> p = pos[i];
-        p.x += cp.tvf_coef * sx;
-        p.y += cp.tvf_coef * sy;
-        if (D == 3) p.z += cp.tvf_coef * sz;
-        pos[i] = p;
-    }
+    store_V<T, D>(cp, tvf, i, sel(ki, cp.rho0[0], cp.rho0[1]) + vi.w, S.ax, S.ay, S.az, S.sx, S.sy, S.sz, acc_visc, pos);
 }
 
 // ---- A: colour gradient, Eq. 22 (only pairs of different fluids contribute)
-template <bool LIST, typename T, int D, int L = 1>
-__device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp, int64_t i, int64_t slot,
-                                        const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap, const T *drho,
+template <bool LIST, typename T, int D, int L = 1, int U = PLAIN>
+__device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
+                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap, const T *drho,
                                         V4<T> *gradC, uint32_t sub = 0) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
@@ -1068,12 +1085,10 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
         const uint32_t other = ki ^ 1u;
         const T two_phi = cp.two_phi[ki];
         const T m_o = cp.mass[other], rho0_o = cp.rho0[other];
-        neighbors<LIST, T, D, PART_OTHER, L>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki,
-            [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
+        neighbors<LIST, false, T, D, PART_OTHER, L, U>(d, cp, starts, list, count, snap, nullptr, i, si, pki,
+            [&](uint32_t j, const V4<T> &sj, const V4<T> &, T rx, T ry, T rz, T r2) {
                 if (!LIST && phase_of(w_bits(sj.w)) != other) return;
-                const PairGeo<T> gg = geo(cp, r2);
-                const T Vj = div_fast(m_o, add_rn(rho0_o, drho[j]));
-                const T s = two_phi * gg.dW * Vj * gg.inv_r;
+                const T s = vmul(vmul(two_phi, pair_w<T>(cp, r2).w), vdiv(m_o, add_rn(rho0_o, drho[j])));
                 g.x = fma_rn(s, rx, g.x);
                 g.y = fma_rn(s, ry, g.y);
                 if (D == 3) g.z = fma_rn(s, rz, g.z);
@@ -1084,6 +1099,20 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
         g.w = sqrt(fma_rn(g.x, g.x, fma_rn(g.y, g.y, g.z * g.z)));
     }
     if (sub == 0) gradC[i] = g;
+}
+
+// v + dt (a^p + a^s + a^v), w = the density deviation for sweep C
+template <typename T, int D>
+__device__ __forceinline__ V4<T> kicked(const V4<T> &vi, T rho_i, T dt, T apx, T apy, T apz, T asx, T asy, T asz,
+                                        const V4<T> &av) {
+    const T inv_rho = T(1) / rho_i;
+    const T m2inv_rho = T(-2) * inv_rho;
+    V4<T> vn;
+    vn.x = fma_rn(dt, fma_rn(inv_rho, asx, fma_rn(m2inv_rho, apx, av.x)), vi.x);
+    vn.y = fma_rn(dt, fma_rn(inv_rho, asy, fma_rn(m2inv_rho, apy, av.y)), vi.y);
+    vn.z = D == 3 ? fma_rn(dt, fma_rn(inv_rho, asz, fma_rn(m2inv_rho, apz, av.z)), vi.z) : T(0);
+    vn.w = vi.w;
+    return vn;
 }
 
 // ---- B: pressure + surface tension + kick
@@ -1097,11 +1126,12 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
 // surface sweep's lanes add them in another order, so the two agree to
 // rounding.
 //
+// neighbours gathered at a time by the surface sweep
 // PASS: 0 = pressure + surface in one walk (cell walk), 1 = pressure and the
 // stored surface sum (list), 2 = surface sum only (list, band particles).
-template <bool LIST, int PASS, typename T, int D, int L = 1>
+template <bool LIST, int PASS, typename T, int D, int L = 1, int U = PLAIN>
 __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &cp, T dt,
-                                          int64_t i, int64_t slot, const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt,
+                                          int64_t i, const uint32_t *starts, const uint32_t *list, uint32_t count,
                                           const uint8_t *band, const V4<T> *snap,
                                           const V4<T> *vel, const V4<T> *gradC,
                                           const V4<T> *acc_visc, V4<T> *acc_surf, V4<T> *vel_new,
@@ -1116,56 +1146,16 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
     const V4<T> vi = vel[i];
     const T dri = vi.w;
     const T rho_i = add_rn(sel(ki, cp.rho0[0], cp.rho0[1]), dri);
-    const T p_i = cp.c0sq * dri;
+    const T b_i = mul_rn(cp.c0, dri);
     T apx = 0, apy = 0, apz = 0, asx = 0, asy = 0, asz = 0;
-    const Limiter<T> limiter_beta(cp, d.limiter);
-    const bool wall_push_only = d.wall_form == 1;
-    const T c0 = cp.c0, c0sq = cp.c0sq, vol_wall = cp.vol_wall;
-    const T rho0_0 = cp.rho0[0], rho0_1 = cp.rho0[1], m_0 = cp.mass[0], m_1 = cp.mass[1];
-    const KernelGeo<T> kgeo(cp);
-
-    // pressure (Eqs. 7-12) of one pair from e_ij, W'_ij, the neighbour's
-    // kind (wall, or fluid of rest density rho0_j and mass m_j) and state
-    // every sum is written as an explicitly rounded add or FMA: the same
-    // source compiled for another launch mode (one case, batch) then rounds
-    // identically whatever the register allocation
-    const T c0rho_i = c0 * rho_i;
-    const auto pressure_pair = [&](L2<T> exy, T ez, T dW, bool wall, T rho0_j, T m_j, const V4<T> &vj) {
-        // U_L - U_R = (v_j - v_i).e  (Eq. 10, U = -v.e)
-        const L2<T> dvxy = fma2(l2(vi.x, vi.y), l2(T(-1), T(-1)), l2(vj.x, vj.y));
-        const T dUe = D == 3 ? fma_rn(dvxy.x, exy.x, fma_rn(dvxy.y, exy.y, sub_rn(vj.z, vi.z) * ez))
-                             : fma_rn(dvxy.x, exy.x, dvxy.y * exy.y);
-        if (wall) {
-            // mirror state behind a wall moving with v_w: rho_i, p_i, 2 U_w - U_L
-            const T dU = T(2) * dUe;
-            const T beta = limiter_beta(dU, p_i, rho_i);       // mirror state: rho_R, p_R = rho_i, p_i
-            T Ps = fma_rn(beta * c0rho_i * dU, T(0.5), p_i);
-            if (wall_push_only) Ps = Ps > T(0) ? Ps : T(0);    // no-suction wall reading
-            const T f = Ps * dW * vol_wall;
-            const L2<T> a = fma2(l2(f, f), exy, l2(apx, apy));
-            apx = a.x; apy = a.y; if (D == 3) apz = fma_rn(f, ez, apz);
-            return;
-        }
-        const T drj = vj.w;
-        const T rho_j = add_rn(rho0_j, drj);
-        const T p_j = c0sq * drj;
-        const T dU = dUe;
-        const T rsum = add_rn(rho_i, rho_j);
-        const T beta = limiter_beta(dU, add_rn(p_i, p_j), rsum);   // Eq. 11
-        // P* V_j with P* = (rho_i p_j + rho_j p_i + beta c0 rho_i rho_j dU) / (rho_i + rho_j)
-        // (Eqs. 8, 12) and V_j = m_j / rho_j: one division
-        const T num = fma_rn(beta * c0rho_i * rho_j, dU, fma_rn(rho_i, p_j, rho_j * p_i));
-        const T f = div_fast(num * m_j, rsum * rho_j) * dW;
-        const L2<T> a = fma2(l2(f, f), exy, l2(apx, apy));
-        apx = a.x; apy = a.y; if (D == 3) apz = fma_rn(f, ez, apz);
-    };
-    // walls by their mirror state
+    const bool printed = d.limiter == 3, push_only = d.wall_form == 1;
     const auto pressure = [&](uint32_t, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
-        const PairGeo<T> g = kgeo(r2);
-        const L2<T> exy = mul2(l2(rx, ry), l2(g.inv_r, g.inv_r));
-        const uint32_t kj = phase_of(w_bits(sj.w));
-        pressure_pair(exy, D == 3 ? rz * g.inv_r : T(0), g.dW, kj == PH_WALL, sel(kj, rho0_0, rho0_1),
-                      sel(kj, m_0, m_1), vj);
+        const PairW<T> g = pair_w<T>(cp, r2);
+        const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, rx, ry, rz);
+        const T f = pressure_factor<T>(cp, printed, push_only, phase_of(w_bits(sj.w)), vj.w, dot, g, rho_i, b_i);
+        apx = vfma(f, rx, apx);
+        apy = vfma(f, ry, apy);
+        if (D == 3) apz = vfma(f, rz, apz);
     };
 
     // surface stress and penalty (Eqs. 24, 26, 30, 33); walls take no part
@@ -1175,10 +1165,9 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
     const bool corr = bk != nullptr && d.surface_corr == 1;
     V4<T> bi0{T(0), T(0), T(0), T(0)}, bi1{T(0), T(0), T(0), T(0)};
     if (corr && PASS != 1) { bi0 = bk[2 * i]; bi1 = bk[2 * i + 1]; }
-    const auto surface = [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
+    const auto surface = [&](uint32_t j, const V4<T> &sj, const V4<T> &gj, T rx, T ry, T rz, T r2) {
         const uint32_t kj = phase_of(w_bits(sj.w));
         if (kj == PH_WALL) return;
-        const V4<T> gj = gradC[j];
         if (gi.w == T(0) && gj.w == T(0)) return;                // every surface term vanishes
         const PairGeo<T> g = geo(cp, r2);
         const T ex = rx * g.inv_r, ey = ry * g.inv_r, ez = D == 3 ? rz * g.inv_r : T(0);
@@ -1282,14 +1271,15 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
 
     const bool surface_on = d.n_fluid_phases == 2;
     if constexpr (PASS == 2) {
-        if (surface_on) neighbors<LIST, T, D, PART_ALL, L>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki, surface, sub);
+        if (surface_on)
+            neighbors<LIST, true, T, D, PART_ALL, L, U>(d, cp, starts, list, count, snap, gradC, i, si, pki, surface, sub);
         asx = group_sum<L>(asx);
         asy = group_sum<L>(asy);
         if (D == 3) asz = group_sum<L>(asz);
         if (sub == 0) acc_surf[i] = V4<T>{asx, asy, asz, T(0)};
         return 0.0;
     } else if constexpr (PASS == 1) {
-        neighbors_aux<LIST, T, D, L>(d, cp, starts, nbr, cnt, snap, vel, i, slot, si, pki, pressure, sub);
+        neighbors<LIST, true, T, D, PART_ALL, L, U>(d, cp, starts, list, count, snap, vel, i, si, pki, pressure, sub);
         apx = group_sum<L>(apx);
         apy = group_sum<L>(apy);
         if (D == 3) apz = group_sum<L>(apz);
@@ -1302,73 +1292,21 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             asx = as.x; asy = as.y; asz = as.z;
         }
     } else {
-        neighbors<LIST, T, D>(d, cp, starts, nbr, cnt, snap, i, slot, si, pki,
-            [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
-                pressure(j, sj, vel[j], rx, ry, rz, r2);
-                if (surface_on) surface(j, sj, rx, ry, rz, r2);
+        neighbors<LIST, true, T, D>(d, cp, starts, list, count, snap, vel, i, si, pki,
+            [&](uint32_t j, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
+                pressure(j, sj, vj, rx, ry, rz, r2);
+                if (surface_on) surface(j, sj, gradC[j], rx, ry, rz, r2);
             });
     }
-    const T inv_rho = T(1) / rho_i;
-    const T m2inv_rho = T(-2) * inv_rho;
-    const V4<T> av = acc_visc[i];
-    V4<T> vn;
-    vn.x = fma_rn(dt, fma_rn(inv_rho, asx, fma_rn(m2inv_rho, apx, av.x)), vi.x);
-    vn.y = fma_rn(dt, fma_rn(inv_rho, asy, fma_rn(m2inv_rho, apy, av.y)), vi.y);
-    vn.z = D == 3 ? fma_rn(dt, fma_rn(inv_rho, asz, fma_rn(m2inv_rho, apz, av.z)), vi.z) : T(0);
-    vn.w = dri;                       // density deviation for sweep C
+    const V4<T> vn = kicked<T, D>(vi, rho_i, dt, apx, apy, apz, asx, asy, asz, acc_visc[i]);
     vel_new[i] = vn;
     return speed2(vn, D);
 }
 
 // ---- C: continuity (Eq. 6) with v* (normal component -U*) + drift
-template <bool LIST, typename T, int D, int L = 1>
-__device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp, T dt, int64_t i, int64_t slot,
-                                        const uint32_t *starts, const uint32_t *nbr, const uint32_t *cnt, const V4<T> *snap,
-                                        const V4<T> *vel_new, T *drho,
-                                        V4<T> *vel, V4<T> *pos, uint32_t sub = 0) {
-    const V4<T> si = ld4(snap + i);
-    const uint32_t pki = w_bits(si.w);
-    const uint32_t ki = phase_of(pki);
-    if (ki == PH_WALL) return;
-    V4<T> vi = vel_new[i];
-    const T dri = vi.w;
-    const T rho0_0 = cp.rho0[0], rho0_1 = cp.rho0[1], m_0 = cp.mass[0], m_1 = cp.mass[1];
-    const T c0 = cp.c0, c0sq = cp.c0sq, vol_wall = cp.vol_wall;
-    const T rho_i = add_rn(sel(ki, rho0_0, rho0_1), dri);
-    const T p_i = c0sq * dri;
-    const KernelGeo<T> kgeo(cp);
-    // the pressure difference enters with the sign of the v* reading; the
-    // sign is folded into p_i and c0^2 once
-    const T psign = d.vstar_printed ? T(-1) : T(1);
-    const T sp_i = psign * p_i, sc0sq = psign * c0sq;
-    T s = 0;
-    // one pair from (v_i - v_j).e = U_R - U_L, W'_ij, the neighbour's kind and
-    // its density deviation
-    const auto pair = [&](T dve, T dW, bool wall, T rho0_j, T m_j, T drj) {
-        if (wall) {                   // v* = v_w
-            s = fma_rn(dve * dW, vol_wall, s);
-            return;
-        }
-        const T rho_j = add_rn(rho0_j, drj);
-        // (v_i - v*).e V_j with (v_i - v*).e = U* - U_L = (Z_R (U_R - U_L) + p_i - p_j)
-        // / (Z_L + Z_R) and V_j = m_j / rho_j: one division.  The printed v*
-        // gives (Z_R (U_R - U_L) - (p_i - p_j)) / (Z_L + Z_R) instead.
-        // (sums explicitly rounded, as in sweep B)
-        const T num = fma_rn(rho_j * c0, dve, fma_rn(-sc0sq, drj, sp_i)) * m_j;
-        s = fma_rn(div_fast(num, c0 * add_rn(rho_i, rho_j) * rho_j), dW, s);
-    };
-    neighbors_aux<LIST, T, D, L>(d, cp, starts, nbr, cnt, snap, vel_new, i, slot, si, pki,
-        [&](uint32_t, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
-            const PairGeo<T> g = kgeo(r2);
-            const uint32_t kj = phase_of(w_bits(sj.w));
-            const L2<T> dvxy = fma2(l2(vj.x, vj.y), l2(T(-1), T(-1)), l2(vi.x, vi.y));
-            const T dvr = D == 3 ? fma_rn(dvxy.x, rx, fma_rn(dvxy.y, ry, sub_rn(vi.z, vj.z) * rz))
-                                 : fma_rn(dvxy.x, rx, dvxy.y * ry);
-            pair(dvr * g.inv_r, g.dW, kj == PH_WALL, sel(kj, rho0_0, rho0_1), sel(kj, m_0, m_1), vj.w);
-        }, sub);
-    s = group_sum<L>(s);
-    if (sub != 0) return;
-    const T dr_new = fma_rn(dt, T(2) * rho_i * s, dri);
+template <typename T, int D>
+__device__ __forceinline__ void store_C(int64_t i, T dt, T rho_i, T sum, V4<T> vi, T *drho, V4<T> *vel, V4<T> *pos) {
+    const T dr_new = fma_rn(dt, T(2) * rho_i * sum, vi.w);
     drho[i] = dr_new;
     V4<T> p = pos[i];
     p.x = fma_rn(dt, vi.x, p.x);
@@ -1377,6 +1315,30 @@ __device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp
     pos[i] = p;
     vi.w = dr_new;
     vel[i] = vi;
+}
+
+template <bool LIST, typename T, int D, int L = 1, int U = PLAIN>
+__device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp, T dt, int64_t i,
+                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap,
+                                        const V4<T> *vel_new, T *drho,
+                                        V4<T> *vel, V4<T> *pos, uint32_t sub = 0) {
+    const V4<T> si = ld4(snap + i);
+    const uint32_t pki = w_bits(si.w);
+    const uint32_t ki = phase_of(pki);
+    if (ki == PH_WALL) return;
+    const V4<T> vi = vel_new[i];
+    const T rho_i = add_rn(sel(ki, cp.rho0[0], cp.rho0[1]), vi.w);
+    const T nsc0 = d.vstar_printed ? cp.c0 : -cp.c0, sb_i = mul_rn(-nsc0, vi.w);
+    T s = 0;
+    neighbors<LIST, true, T, D, PART_ALL, L, U>(d, cp, starts, list, count, snap, vel_new, i, si, pki,
+        [&](uint32_t, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
+            const PairW<T> g = pair_w<T>(cp, r2);
+            const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, rx, ry, rz);
+            const T f = continuity_factor<T>(cp, phase_of(w_bits(sj.w)), vj.w, dot, g, rho_i, sb_i, nsc0);
+            s = vfma(f, vmul(g.w, g.r), s);
+        }, sub);
+    s = group_sum<L>(s);
+    if (sub == 0) store_C<T, D>(i, dt, rho_i, s, vi, drho, vel, pos);
 }
 
 // ---------------------------------------------------------- sweep kernels
@@ -1409,10 +1371,11 @@ struct SweepArgs {
 // How a per-substep sweep finds its tiles and its case: MODE_TILES, block b
 // takes tile tile0 + b / L and reads desc[c]; MODE_WORK, the blocks stride
 // over the batch's work list; MODE_ONE, as MODE_TILES with the one case's
-// descriptor taken from the parameter block.
-enum SweepMode { MODE_TILES = 0, MODE_WORK = 1, MODE_ONE = 2 };
+// descriptor taken from the parameter block; MODE_FEW, as MODE_ONE for a case
+// that leaves the SMs with few warps: four neighbours are gathered at a time.
+enum SweepMode { MODE_TILES = 0, MODE_WORK = 1, MODE_ONE = 2, MODE_FEW = 3 };
 template <int MODE> __device__ __forceinline__ const CaseDesc &case_desc(const SweepArgs &a, int c) {
-    if constexpr (MODE == MODE_ONE) return a.one;
+    if constexpr (MODE == MODE_ONE || MODE == MODE_FEW) return a.one;
     else return a.desc[c];
 }
 
@@ -1433,6 +1396,24 @@ template <int L, bool WORK> __device__ __forceinline__ Tile work_tile(const Swee
 __device__ __forceinline__ int64_t particle_at(const SweepArgs &a, int64_t q) {
     return a.fidx ? (int64_t)a.fidx[q] : q;
 }
+
+template <bool LIST> __device__ __forceinline__ const uint32_t *list_of(const SweepArgs &a, const CaseDesc &d, int64_t q) {
+    return LIST ? a.nbr + list_word(d, q) : nullptr;
+}
+template <bool LIST> __device__ __forceinline__ uint32_t count_of(const SweepArgs &a, int64_t q) {
+    return LIST ? a.cnt[q] : 0u;
+}
+// entry t of the band list: (case << 32 | slot)
+struct BandEntry {
+    int c;
+    int64_t q, i;
+    __device__ __forceinline__ BandEntry(const SweepArgs &a, const uint64_t *blist, int64_t t) {
+        const uint64_t e = blist[t];
+        c = (int)(e >> 32);
+        q = (int64_t)(uint32_t)e;
+        i = (int64_t)a.fidx[q];
+    }
+};
 
 // ---- L: neighbour lists of the frozen configuration (fluid particles only),
 // one block per cell that holds fluid particles.  All particles of a cell
@@ -1463,7 +1444,7 @@ struct ListSmem {
     uint32_t fluid[2][LB_CAND / 32];            // candidates of each fluid, a word per 32
     uint32_t begin[32], pre[33], code[32];      // cells around in increasing table index
     uint32_t own;                               // first candidate of the cell itself
-    uint32_t idx[LB_SLOTS], rest[LB_SLOTS], other[LB_SLOTS];
+    uint32_t idx[LB_SLOTS], rest[LB_SLOTS], other[LB_SLOTS];   // a slot's particle, entries of its list's parts
     uint32_t list[LB_WORDS];
 };
 // The row length of the shared lists: K + 1 words, so that for the even
@@ -1550,19 +1531,18 @@ __device__ __forceinline__ int list_scan(const ListSmem &S, uint32_t *row, int K
 }
 
 template <typename T, int D>
-__device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> &cp, uint32_t m, ListSmem &S,
+__device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> &cp, uint32_t b, ListSmem &S,
                                            const uint32_t *starts, const uint32_t *rank, const uint32_t *fidx,
                                            const V4<T> *snap, uint32_t *nbr, uint32_t *cnt, uint8_t *band,
                                            int32_t *status) {
     constexpr int NC = D == 3 ? 27 : 9;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int K = d.nbr_k, LS = K + 1, G = lb_group(K);
-    const uint32_t b = starts[m];
+    const uint32_t pk = w_bits(snap[b].w), m = (uint32_t)d.table_off + morton_of_packed<D>(pk);
     const uint32_t f0 = rank[b], f1 = rank[starts[m + 1]];
     __syncthreads();                            // the previous cell's shared data is done with
     if (warp == 0) {
         // the 3^D cells around, one per lane, in increasing table index
-        const uint32_t pk = w_bits(snap[b].w);
         uint32_t mq = 0xffffffffu, bq = 0, nq = 0, code = 0;
         if (lane < NC) {
             const int ox = lane % 3 - 1, oy = lane / 3 % 3 - 1, oz = D == 3 ? lane / 9 - 1 : 0;
@@ -1680,10 +1660,10 @@ __device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> 
                 overflow = true;
                 c = co = 0;
             }
-            const uint32_t i = S.idx[s], *src = S.list + s * LS;
+            const uint32_t *src = S.list + s * LS;
             if (warp == 0) {
-                cnt[i] = c | (co << 16);
-                if (co) band[i] = 1;
+                cnt[g0 + s] = c | (co << 16);
+                if (co) band[S.idx[s]] = 1;
             }
             uint32_t *dst = nbr + list_word(d, (int64_t)g0 + s);
             for (uint32_t k = warp; k < c; k += LB_WARPS) {
@@ -1719,8 +1699,7 @@ __global__ void __launch_bounds__(LB_WARPS * 32) k_build_list(SweepArgs a, const
 // (case << 32 | slot), to the class's list that the surface and colour sweeps
 // walk (warp-aggregated atomics; the order is irrelevant because every
 // particle's sum is its own).
-template <typename T, int D, bool LIST>
-__global__ void __launch_bounds__(256) k_band(SweepArgs a, const uint8_t *band, uint64_t *blist, uint32_t *bcount) {
+static __global__ void __launch_bounds__(256) k_band(SweepArgs a, const uint8_t *band, uint64_t *blist, uint32_t *bcount) {
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     const int64_t q = t.begin + threadIdx.x;
     const bool b = (int)threadIdx.x < t.n && a.st[t.c].active && band[particle_at(a, q)];
@@ -1741,17 +1720,17 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const
     const CaseDesc &d = a.desc[t.c];
     if (!d.tvf_on && d.surface_corr != 1) return;
     const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
-    sweep_M<LIST, T, D>(d, phys<T>(d), i, q, a.starts, a.nbr, a.cnt, snap, drho, bmat, bk, &a.st[t.c].status);
+    sweep_M<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q), snap, drho, bmat, bk, &a.st[t.c].status);
 }
 
 template <typename T, int D, bool LIST>
-__global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const T *drho, const V4<T> *vel,
+__global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const V4<T> *vel,
                                            const V4<T> *bmat, V4<T> *acc_visc, V4<T> *pos) {
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
     const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
-    sweep_V<LIST, T, D>(d, phys<T>(d), i, q, a.starts, a.nbr, a.cnt, snap, drho, vel, bmat, acc_visc, pos,
+    sweep_V<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q), snap, vel, bmat, acc_visc, pos,
                         &a.st[t.c].status);
 }
 
@@ -1773,7 +1752,8 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, con
         if (li >= t.n || !a.st[t.c].active) return;
         const CaseDesc &d = case_desc<MODE>(a, t.c);
         const int64_t q = t.begin + li, i = particle_at(a, q);
-        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, q, a.starts, a.nbr, a.cnt, snap, drho, gradC, threadIdx.x % L);
+        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q), snap, drho, gradC,
+                               threadIdx.x % L);
     };
     if constexpr (MODE == MODE_WORK) {
         const int64_t items = work_items<L, true>(a);
@@ -1789,18 +1769,15 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, con
 // list's length is known only on the device).  A particle outside
 // the band has no neighbour of the other fluid, so its colour gradient is the
 // zero written at the start of the advection step.
-template <typename T, int D, bool LIST, int L = 1>
-__global__ void SPH_SWEEPAS_BOUNDS k_sweep_A_band(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
+template <typename T, int D, int L = 1>
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4) k_sweep_A_band(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
                                                 const V4<T> *snap, const T *drho, V4<T> *gradC) {
     const int64_t items = (int64_t)*bcount * L;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t e = blist[t / L];
-        const int c = (int)(e >> 32);
-        const int64_t q = (int64_t)(uint32_t)e;
-        if (!a.st[c].active) continue;
-        const CaseDesc &d = a.desc[c];
-        sweep_A<LIST, T, D, L>(d, phys<T>(d), (int64_t)a.fidx[q], q, a.starts, a.nbr, a.cnt, snap, drho, gradC,
-                               threadIdx.x % L);
+        const BandEntry e(a, blist, t / L);
+        if (!a.st[e.c].active) continue;
+        const CaseDesc &d = a.desc[e.c];
+        sweep_A<true, T, D, L, AHEAD>(d, phys<T>(d), e.i, a.starts, list_of<true>(a, d, e.q), count_of<true>(a, e.q), snap, drho, gradC, threadIdx.x % L);
     }
 }
 
@@ -1808,20 +1785,30 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A_band(SweepArgs a, const uint64_t *b
 // thread (L lanes) per entry of the class's compacted band list, so warps
 // are full of band particles; the threads stride over the list (a group of
 // L lanes stays together: the stride is a multiple of L)
-template <typename T, int D, bool LIST, int L = 1>
-__global__ void SPH_SWEEPAS_BOUNDS k_sweep_S(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
+template <typename T, int D, int L = 1>
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) k_sweep_S(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
                                            const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
                                            const V4<T> *gradC, V4<T> *acc_surf, const V4<T> *bk, const T *drho) {
     const int64_t items = (int64_t)*bcount * L;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t e = blist[t / L];
-        const int c = (int)(e >> 32);
-        const int64_t q = (int64_t)(uint32_t)e;
-        if (!a.st[c].active) continue;
-        const CaseDesc &d = a.desc[c];
+        const BandEntry e(a, blist, t / L);
+        if (!a.st[e.c].active) continue;
+        const CaseDesc &d = a.desc[e.c];
         uint32_t ph;
-        sweep_B<LIST, 2, T, D, L>(d, phys<T>(d), T(0), (int64_t)a.fidx[q], q, a.starts, a.nbr, a.cnt, band, snap, vel,
-                                  gradC, nullptr, acc_surf, nullptr, &ph, threadIdx.x % L, bk, drho);
+        sweep_B<true, 2, T, D, L, 4>(d, phys<T>(d), T(0), e.i, a.starts, list_of<true>(a, d, e.q), count_of<true>(a, e.q), band, snap, vel, gradC,
+                                          nullptr, acc_surf, nullptr, &ph, threadIdx.x % L, bk, drho);
+    }
+}
+
+// largest |v|^2 (its bits) per fluid of a block's case; all threads of a warp
+// take part
+__device__ __forceinline__ void reduce_vmax(const SweepArgs &a, int c, uint32_t ph, unsigned long long v2) {
+    unsigned long long m0 = ph == 0 ? v2 : 0ull, m1 = ph == 1 ? v2 : 0ull;
+    m0 = warp_max_u64(m0);
+    m1 = warp_max_u64(m1);
+    if ((threadIdx.x & 31) == 0) {
+        if (m0) atomicMax(&a.st[c].vmax2_acc[0], m0);
+        if (m1) atomicMax(&a.st[c].vmax2_acc[1], m1);
     }
 }
 
@@ -1839,18 +1826,12 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_
         if (li < t.n) {
             const int64_t q = t.begin + li, i = particle_at(a, q);
             const T dt = (T)a.st[t.c].dt;
-            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L>(d, phys<T>(d), dt, i, q, a.starts, a.nbr, a.cnt, band, snap, vel,
+            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L, MODE == MODE_FEW ? 4 : PLAIN>(d, phys<T>(d), dt, i, a.starts, list_of<LIST>(a, d, q),
+                                                      count_of<LIST>(a, q), band, snap, vel,
                                                       gradC, acc_visc, acc_surf, vel_new, &ph, threadIdx.x % L,
                                                       LIST ? nullptr : bk);
         }
-        unsigned long long m0 = ph == 0 ? (unsigned long long)__double_as_longlong(v2) : 0ull;
-        unsigned long long m1 = ph == 1 ? (unsigned long long)__double_as_longlong(v2) : 0ull;
-        m0 = warp_max_u64(m0);
-        m1 = warp_max_u64(m1);
-        if ((threadIdx.x & 31) == 0) {
-            if (m0) atomicMax(&a.st[t.c].vmax2_acc[0], m0);
-            if (m1) atomicMax(&a.st[t.c].vmax2_acc[1], m1);
-        }
+        reduce_vmax(a, t.c, ph, (unsigned long long)__double_as_longlong(v2));
     };
     if constexpr (MODE == MODE_WORK) {
         const int64_t items = work_items<L, true>(a);
@@ -1870,7 +1851,8 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const
         const CaseDesc &d = case_desc<MODE>(a, t.c);
         const int64_t q = t.begin + li, i = particle_at(a, q);
         const T dt = (T)a.st[t.c].dt;
-        sweep_C<LIST, T, D, L>(d, phys<T>(d), dt, i, q, a.starts, a.nbr, a.cnt, snap, vel_new, drho, vel, pos,
+        sweep_C<LIST, T, D, L, MODE == MODE_FEW && D == 2 ? 4 : AHEAD>(d, phys<T>(d), dt, i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q),
+                               snap, vel_new, drho, vel, pos,
                                threadIdx.x % L);
     };
     if constexpr (MODE == MODE_WORK) {
