@@ -207,7 +207,7 @@ int64_t footprint(const sphst_case_params *P, int64_t n) {
     const int64_t kmax = P->nbr_mode == SPHST_NBR_LIST
                              ? (P->max_neighbors > 0 ? P->max_neighbors : (P->dim == 3 ? 128 : 48)) : 0;
     // V4 arrays, scalars, ints, list, band + band list, cell list
-    const int64_t per = 9 * 4 * tsz + 2 * tsz + 6 * 4 + 4 * kmax + 4 + 1 + 8 + 8 +
+    const int64_t per = 9 * 4 * tsz + (tsz == 8 ? 3 : 2) * tsz + 6 * 4 + 4 * kmax + 4 + 1 + 8 + 8 +
                         (P->surface_corr == 1 ? 2 * 4 * tsz : 0);   // own-fluid correction matrices
     // cell table: cells ~ n / 2.6^d per axis padded to a power of two
     const double side = std::pow((double)std::max<int64_t>(n, 1), 1.0 / P->dim) / 2.6 + 2.0 * P->grid_pad + 2.0;

@@ -83,17 +83,28 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
 // SM): B 250 -> 285 us.
 constexpr int64_t FEW_MAX_PER_SM = 1024;
 
+// FP64 sweeps take smaller blocks than asked for until every SM has this many:
+// their time is the busiest SM's arithmetic, and whole blocks of a small case
+// divide badly (43k particles in blocks of 128 are 2.2 blocks per SM: the
+// busiest has 3).  43k particles in 3D: B 383 -> 282, C 240 -> 190, S 254 ->
+// 172 us; 16 gives the same.  FP32 sweeps, which wait for gathers, lose by it
+// (64k particles: C 26 -> 28 us).
+constexpr int64_t MIN_BLOCKS_PER_SM = 8;
+
 template <typename T> struct EngineT : Engine {
     // particle arrays
     V4<T> *pos = nullptr, *snap = nullptr, *vel = nullptr, *vel_new = nullptr;
     V4<T> *gradC = nullptr, *acc_visc = nullptr, *acc_surf = nullptr, *bmat = nullptr;
     V4<T> *bk = nullptr;                             // own-fluid correction matrices (surface_corr)
-    T *drho = nullptr, *drho_old = nullptr;        // drho_old: rebuild scratch (sorted copy)
+    T *drho = nullptr, *vol = nullptr;              // density deviations; volumes (FP32 forms them from drho)
+    T *drho_old = nullptr;        // drho_old: rebuild scratch (sorted copy)
     uint32_t *id = nullptr, *key = nullptr, *rank = nullptr, *perm = nullptr;
     uint32_t *fidx = nullptr, *fscan = nullptr;     // particle of each fluid rank (slot); scan scratch
     // cell table + scan scratch
     uint32_t *starts = nullptr, *block_sums = nullptr;
     uint32_t *nbr = nullptr, *nbr_cnt = nullptr;   // neighbour lists (ELL per case) and counts
+    V4<T> *lgeo = nullptr;                          // (e_ij, W') and (r, 1/r) of each list entry (FP64)
+    RInv *lrinv = nullptr;
     uint8_t *band = nullptr;                        // interface band of the frozen configuration
     uint64_t *band_list = nullptr;                  // band particles per list class (case << 32 | index)
     uint32_t *band_count = nullptr;                 // entries of each class's band list
@@ -187,6 +198,10 @@ template <typename T> struct EngineT : Engine {
             if (r->P.nbr_mode == SPHST_NBR_LIST) list_fluid += r->n_fluid;
             any_corr = any_corr || r->P.surface_corr == 1;
         }
+        int64_t fluid = 0;
+        for (CaseRec *r : cases) fluid += r->n_fluid;
+        if (sizeof(T) == 8)
+            while (block > 32 && fluid * lanes < sm_count * MIN_BLOCKS_PER_SM * block) block = block / 2 / 32 * 32;
         few = list_fluid * lanes <= sm_count * FEW_MAX_PER_SM;
         for (int c = 0; c < ncases; ++c) {
             CaseRec *r = cases[c];
@@ -234,7 +249,7 @@ template <typename T> struct EngineT : Engine {
         size_t o_as = take(nn * sizeof(V4<T>));
         size_t o_bm = take(2 * nn * sizeof(V4<T>));
         size_t o_bk = take(any_corr ? 2 * nn * sizeof(V4<T>) : 0);
-        size_t o_dr = take(nn * sizeof(T)), o_dro = take(nn * sizeof(T));
+        size_t o_dr = take(nn * sizeof(T)), o_vol = take(sizeof(T) == 8 ? nn * sizeof(T) : 0), o_dro = take(nn * sizeof(T));
         size_t o_id = take(nn * 4), o_key = take(nn * 4), o_rank = take(nn * 4), o_perm = take(nn * 4);
         size_t o_st = take((size_t)(table_total + 1) * 4), o_bs = take((size_t)nb * 4);
         size_t o_desc = take(sizeof(CaseDesc) * ncases), o_state = take(sizeof(CaseState) * ncases);
@@ -247,6 +262,16 @@ template <typename T> struct EngineT : Engine {
         size_t o_ftfirst = take(nc * 8), o_cls0 = take(64);
         size_t o_flag = take(64);
         size_t o_read = take((size_t)std::max<int64_t>(max_case_n, 1) * 3 * sizeof(double));
+        // FP64 keeps the lists' pair geometry where it fits easily: the results
+        // are the same without it
+        bool geo = false;
+        if (sizeof(T) == 8 && any_list) {
+            size_t mem_free = 0, mem_total = 0;
+            SPH_CK(cudaMemGetInfo(&mem_free, &mem_total));
+            const size_t bytes = (size_t)nbr_total * (sizeof(V4<T>) + sizeof(RInv));
+            geo = bytes <= std::min(mem_free / 4, mem_total / 16);
+        }
+        const size_t o_lgeo = take(geo ? (size_t)nbr_total * sizeof(V4<T>) : 0), o_lrinv = take(geo ? (size_t)nbr_total * sizeof(RInv) : 0);
         size_t o_nbr = take((size_t)std::max<int64_t>(nbr_total, 1) * 4), o_ncnt = take(nn * 4);
         size_t o_band = take(nn);
         size_t o_blist = take(nn * 8), o_bcount = take(64), o_clist = take(nn * 8);
@@ -264,7 +289,7 @@ template <typename T> struct EngineT : Engine {
         gradC = (V4<T> *)(b + o_gc); acc_visc = (V4<T> *)(b + o_av);
         acc_surf = (V4<T> *)(b + o_as); bmat = (V4<T> *)(b + o_bm);
         bk = any_corr ? (V4<T> *)(b + o_bk) : nullptr;
-        drho = (T *)(b + o_dr); drho_old = (T *)(b + o_dro);
+        drho = (T *)(b + o_dr); vol = sizeof(T) == 8 ? (T *)(b + o_vol) : drho; drho_old = (T *)(b + o_dro);
         id = (uint32_t *)(b + o_id); key = (uint32_t *)(b + o_key);
         rank = (uint32_t *)(b + o_rank); perm = (uint32_t *)(b + o_perm);
         starts = (uint32_t *)(b + o_st); block_sums = (uint32_t *)(b + o_bs);
@@ -277,6 +302,8 @@ template <typename T> struct EngineT : Engine {
         d_work = (uint32_t *)(b + o_work); d_ft_first = (int64_t *)(b + o_ftfirst); d_cls0 = (int64_t *)(b + o_cls0);
         d_read = (double *)(b + o_read);
         nbr = (uint32_t *)(b + o_nbr);
+        lgeo = geo ? (V4<T> *)(b + o_lgeo) : nullptr;
+        lrinv = geo ? (RInv *)(b + o_lrinv) : nullptr;
         nbr_cnt = (uint32_t *)(b + o_ncnt);
         band = (uint8_t *)(b + o_band);
         band_list = (uint64_t *)(b + o_blist);
@@ -413,7 +440,7 @@ template <typename T> struct EngineT : Engine {
 
     static int tile_class(const CaseDesc &d) { return (d.nbr_mode == 0 ? 0 : 2) + (d.dim == 3 ? 0 : 1); }
     SweepArgs fluid_args(int k) const {
-        SweepArgs a{d_ftiles, d_desc, d_state, starts, nbr, nbr_cnt, cls_fb[k], fidx};
+        SweepArgs a{d_ftiles, d_desc, d_state, starts, nbr, nbr_cnt, cls_fb[k], fidx, lgeo, lrinv};
         if (ncases == 1) a.one = h_desc[0];
         return a;
     }
@@ -430,7 +457,8 @@ template <typename T> struct EngineT : Engine {
     // blocks (per lane) of a band-list sweep: at most one per tile, at most 8
     // blocks of all lanes per SM
     int64_t band_grid(int64_t tiles, int lanes_) const {
-        return std::max<int64_t>(1, std::min<int64_t>(tiles, sm_count * 8 / std::max(lanes_, 1)));
+        const int64_t per_sm = std::max<int64_t>(8, 1024 / block);
+        return std::max<int64_t>(1, std::min<int64_t>(tiles, sm_count * per_sm / std::max(lanes_, 1)));
     }
     // list the active cases' tiles (after the criterion kernel of a substep)
     void launch_work_lists() {
@@ -447,7 +475,7 @@ template <typename T> struct EngineT : Engine {
         k_scan_reduce<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
         k_scan_blocks<<<1, SCAN_T, 0, stream>>>(block_sums, nbp);
         k_scan_apply<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
-        k_fluid_scatter<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, snap, fscan, fidx, gradC, band, cell_list,
+        k_fluid_scatter<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, snap, fscan, drho, vol, fidx, gradC, band, cell_list,
                                                                    cell_count, band_base[1]);
     }
     // neighbour lists: a block per cell, as many blocks as fit the GPU striding
@@ -462,6 +490,11 @@ template <typename T> struct EngineT : Engine {
     void launch_lists() {
         launch_list<3>(0);
         launch_list<2>(1);
+        if constexpr (sizeof(T) == 8) {
+            const dim3 b(32, LG_WARPS);
+            if (lgeo && cls_fn[0]) k_list_geo<3><<<(unsigned)cls_fn[0], b, 0, stream>>>(fluid_args(0), snap, lgeo, lrinv);
+            if (lgeo && cls_fn[1]) k_list_geo<2><<<(unsigned)cls_fn[1], b, 0, stream>>>(fluid_args(1), snap, lgeo, lrinv);
+        }
     }
     void launch_band() {
         for (int k = 0; k < 2; ++k)
@@ -470,8 +503,8 @@ template <typename T> struct EngineT : Engine {
     }
     // correction matrices, viscous force and transport shift
     void launch_setup() {
-        if (any_tvf || any_corr) SPH_CLASSES_F(0, 4, k_sweep_M, snap, drho, bmat, bk);
-        SPH_CLASSES_F(0, 4, k_sweep_V, snap, vel, bmat, acc_visc, pos);
+        if (any_tvf || any_corr) SPH_CLASSES_F(0, 4, k_sweep_M, snap, vol, bmat, bk);
+        SPH_CLASSES_F(0, 4, k_sweep_V, snap, vel, vol, bmat, acc_visc, pos);
     }
     // the band sweeps (A of the list classes, S): a few blocks per SM whose
     // threads stride over the class's band list
@@ -479,9 +512,9 @@ template <typename T> struct EngineT : Engine {
         const unsigned g = (unsigned)(band_grid(cls_fn[k], L) * L);
         const uint64_t *bl = band_list + band_base[k];
         if (surface)
-            k_sweep_S<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, band, snap, vel, gradC, acc_surf, bk, drho);
+            k_sweep_S<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, band, snap, vel, gradC, acc_surf, bk, vol);
         else
-            k_sweep_A_band<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, snap, drho, gradC);
+            k_sweep_A_band<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, snap, vol, gradC);
     }
     template <int D> void launch_band_class(int k, bool surface) {
         if (!cls_fn[k]) return;
@@ -495,8 +528,8 @@ template <typename T> struct EngineT : Engine {
         launch_band_class<3>(0, true);
         launch_band_class<2>(1, true);
     }
-    void launch_B() { SPH_CLASSES_LF(0, 4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk); }
-    void launch_C() { SPH_CLASSES_LF(0, 4, k_sweep_C, lanes, snap, vel_new, drho, vel, pos); }
+    void launch_B() { SPH_CLASSES_LF(0, 4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk, vol); }
+    void launch_C() { SPH_CLASSES_LF(0, 4, k_sweep_C, lanes, snap, vel_new, drho, vol, vel, pos); }
     int n_classes(int upto) const {
         int m = 0;
         for (int k = 0; k < upto; ++k) m += cls_n[k] > 0;
@@ -537,7 +570,7 @@ template <typename T> struct EngineT : Engine {
     void launch_colour() {
         launch_band_class<3>(0, false);
         launch_band_class<2>(1, false);
-        SPH_CLASSES_LF(2, 4, k_sweep_A, lanes, snap, drho, gradC);
+        SPH_CLASSES_LF(2, 4, k_sweep_A, lanes, snap, vol, gradC);
     }
 
     int launch_body(cudaGraphConditionalHandle h, int use_handle) {

@@ -146,7 +146,7 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
     return 1.0f / sqrtf(x);
 #endif
 }
-__device__ __forceinline__ double rsqrt_fast(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_fast(double x) { return rsqrt(x); }
 
 // a / b of the pair sums: in FP32 a times the SFU reciprocal (<= 2 ulp)
 __device__ __forceinline__ float vdiv(float a, float b) { return __fmul_rn(a, rcp_approx(b)); }
@@ -404,27 +404,116 @@ __device__ __forceinline__ void walk_list(const uint32_t *__restrict__ p, uint32
     }
 }
 
-// neighbours of particle i as f(j, s_j, aux_j, r_ij, r^2), from the list at
-// word `list` (count as in cnt[]) or from the cell walk, which visits all:
-// PART_OTHER leaves the choice to the caller
-template <bool LIST, bool AUX, typename T, int D, int PART = PART_ALL, int L = 1, int U = PLAIN, typename F>
+// The geometry of one pair as the sums use it.  FP32: the carrier (x, y, z) is
+// r_ij itself, with W'/r = (kcoef / h) (1 - q/2)^3 as its weight, which saves
+// the unit vector.  FP64: the carrier is the unit vector e_ij with weight W',
+// the form that is stored beside the list (below).
+template <typename T> struct PairG;
+template <> struct PairG<float> {
+    float x, y, z, inv, r, wd;                  // r_ij, 1/r, r, W'/r
+    __device__ __forceinline__ PairG(const CasePhys<float> &cp, float rx, float ry, float rz, float r2) : x(rx), y(ry), z(rz) {
+        inv = rsq(r2);
+        r = vmul(r2, inv);
+        const float u = vfma(r, cp.mhalf_inv_h, 1.0f);
+        wd = vmul(vmul(vmul(cp.kcoef_h, u), u), u);
+    }
+    __device__ __forceinline__ float du(float dot) const { return vmul(dot, inv); }   // carrier product -> along e
+    __device__ __forceinline__ float e(float c) const { return vmul(c, inv); }        // carrier -> unit vector
+    __device__ __forceinline__ float dW() const { return vmul(wd, r); }               // W'
+    __device__ __forceinline__ float dW_r() const { return wd; }                      // W' / r
+    __device__ __forceinline__ float outer() const { return wd; }                     // weight of carrier (x) carrier in r (x) W' e
+};
+template <> struct PairG<double> {
+    double x, y, z, inv, r, wd;                 // e_ij, 1/r, r, W'
+    __device__ __forceinline__ PairG() {}
+    __device__ __forceinline__ PairG(const CasePhys<double> &cp, double rx, double ry, double rz, double r2) {
+        inv = rsq(r2);
+        r = vmul(r2, inv);
+        const double u = vfma(r, cp.mhalf_inv_h, 1.0);
+        wd = vmul(vmul(vmul(vmul(cp.kcoef_h, u), u), u), r);
+        x = vmul(rx, inv); y = vmul(ry, inv); z = vmul(rz, inv);
+    }
+    __device__ __forceinline__ double du(double dot) const { return dot; }
+    __device__ __forceinline__ double e(double c) const { return c; }
+    __device__ __forceinline__ double dW() const { return wd; }
+    __device__ __forceinline__ double dW_r() const { return vmul(wd, inv); }
+    __device__ __forceinline__ double outer() const { return vmul(wd, r); }
+};
+
+// One particle's list: its first word, its count as in cnt[], and (FP64,
+// optional) the stored geometry of its entries: (e_ij, W') and (r, 1/r) of the
+// frozen configuration at the list's own positions.  W' < 0 for every pair; a
+// wall's entry stores -W', and the other fluid's entries come first, so the
+// neighbour's kind is known without its position.
+struct alignas(16) RInv { double r, inv; };
+template <typename T> struct ListRef {
+    const uint32_t *p;
+    uint32_t count;
+    const V4<T> *ge;
+    const RInv *gr;
+};
+// The walk over stored geometry: word, geometry and second record of the next
+// entry are in flight while the current one is evaluated.
+template <bool AUX, bool NEED_R, int L, typename F>
+__device__ __forceinline__ void walk_geo(const ListRef<double> &l, uint32_t c, const V4<double> *__restrict__ aux, uint32_t ki,
+                                         F &&f, uint32_t sub) {
+    const uint32_t c_other = l.count >> 16;
+    const uint32_t *p = l.p + (int)sub * LROW;
+    const V4<double> *ge = l.ge + (int)sub * LROW;
+    const RInv *gr = l.gr + (int)sub * LROW;
+    if (sub >= c) return;
+    uint32_t e = ld_list_walk(p), w1 = sub + L < c ? ld_list_walk(p + L * LROW) : 0u;
+    V4<double> g = ld4_now(ge), aj = AUX ? ld4_now(aux + (e >> NBR_SHIFT)) : g;
+    RInv ri = NEED_R ? *gr : RInv{0.0, 0.0};
+#pragma unroll 1
+    for (uint32_t k = sub; k < c; k += L) {
+        p += L * LROW;
+        ge += L * LROW;
+        gr += L * LROW;
+        const uint32_t ec = e;
+        const V4<double> gc = g, ac = aj;
+        const RInv rc = ri;
+        e = w1;
+        if (k + L < c) {
+            g = ld4_now(ge);
+            if (AUX) aj = ld4_now(aux + (e >> NBR_SHIFT));
+            if (NEED_R) ri = *gr;
+        }
+        if (k + 2 * L < c) w1 = ld_list_walk(p + L * LROW);
+        const bool wall = gc.w >= 0.0;
+        PairG<double> G;
+        G.x = gc.x; G.y = gc.y; G.z = gc.z; G.wd = wall ? -gc.w : gc.w;
+        G.r = rc.r; G.inv = rc.inv;
+        f(ec >> NBR_SHIFT, wall ? PH_WALL : k < c_other ? ki ^ 1u : ki, AUX ? ac : gc, G);
+    }
+}
+
+// neighbours of particle i as f(j, kind of j, aux_j, geometry), from its list
+// or from the cell walk, which visits all: PART_OTHER leaves the choice to the
+// caller.  NEED_R: f reads r or 1/r.
+template <bool LIST, bool AUX, bool NEED_R, typename T, int D, int PART = PART_ALL, int L = 1, int U = PLAIN, typename F>
 __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &cp, const uint32_t *starts,
-                                          const uint32_t *list, uint32_t count, const V4<T> *snap,
-                                          const V4<T> *aux, int64_t i, const V4<T> &si, uint32_t pki,
-                                          F &&f, uint32_t sub = 0) {
+                                          const ListRef<T> &l, const V4<T> *snap, const V4<T> *aux, int64_t i,
+                                          const V4<T> &si, uint32_t pki, F &&f, uint32_t sub = 0) {
     if constexpr (LIST) {
+        const uint32_t c = PART == PART_OTHER ? l.count >> 16 : l.count & CNT_MASK;
+        if constexpr (sizeof(T) == 8)
+            if (l.ge) {
+                walk_geo<AUX, NEED_R, L>(l, c, aux, phase_of(pki), f, sub);
+                return false;
+            }
         const T cs = cp.cs;
-        walk_list<AUX, T, L, U>(list, PART == PART_OTHER ? count >> 16 : count & CNT_MASK, snap, aux,
+        walk_list<AUX, T, L, U>(l.p, c, snap, aux,
             [&](uint32_t e, const V4<T> &sj, const V4<T> &aj) {
                 const Moved<T, D> m = moved<T, D>(e, sj, cs);
                 const T rx = vadd(si.x, m.nx), ry = vadd(si.y, m.ny), rz = D == 3 ? vadd(si.z, m.nz) : T(0);
-                f(e >> NBR_SHIFT, sj, aj, rx, ry, rz, norm2<T, D>(rx, ry, rz));
+                f(e >> NBR_SHIFT, phase_of(w_bits(sj.w)), aj, PairG<T>(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz)));
             }, sub);
         return false;
     } else {
         return walk<T, D>(d, cp, starts, snap, i, si, pki,
             [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
-                f(j, sj, AUX ? ld4(aux + j) : sj, rx, ry, rz, r2);
+                f(j, phase_of(w_bits(sj.w)), AUX ? ld4(aux + j) : sj, PairG<T>(cp, rx, ry, rz, r2));
             });
     }
 }
@@ -442,52 +531,29 @@ template <int L, typename T> __device__ __forceinline__ T group_sum(T v) {
     return v;
 }
 
-// kernel radial derivative and unit vector of one pair
-template <typename T> struct PairGeo { T inv_r, r, dW; };
-template <typename T>
-__device__ __forceinline__ PairGeo<T> geo(const CasePhys<T> &cp, T r2) {
-    PairGeo<T> g;
-    g.inv_r = rsq(r2);
-    g.r = r2 * g.inv_r;
-    const T q = g.r * cp.inv_h;
-    const T u = fma_rn(T(-0.5), q, T(1));
-    g.dW = cp.kcoef * q * u * u * u;
-    return g;
-}
-// the pair geometry the sums need: 1/r, r and W'/r = (kcoef / h) (1 - q/2)^3,
-// so that r_ij itself carries the direction of every pair term.
-template <typename T> struct PairW { T inv, r, w; };
-template <typename T> __device__ __forceinline__ PairW<T> pair_w(const CasePhys<T> &cp, T r2) {
-    PairW<T> g;
-    g.inv = rsq(r2);
-    g.r = vmul(r2, g.inv);
-    const T u = vfma(g.r, cp.mhalf_inv_h, T(1));
-    g.w = vmul(vmul(vmul(cp.kcoef_h, u), u), u);
-    return g;
-}
-// (v_j - v_i) . r_ij, from -v_i
+// (v_j - v_i) . carrier, from -v_i
 template <typename T, int D>
 __device__ __forceinline__ T pair_dot(const V4<T> &vj, T nvx, T nvy, T nvz, T rx, T ry, T rz) {
     const T dx = vadd(vj.x, nvx), dy = vadd(vj.y, nvy);
     if (D == 2) return vfma(dx, rx, vmul(dy, ry));
     return vfma(dx, rx, vfma(dy, ry, vmul(vadd(vj.z, nvz), rz)));
 }
-// Pressure (Eqs. 7-12): the factor f of one neighbour's term f r_ij in
-// sum_j P* grad W V_j, for particles of densities rho_i and c0 drho_i = b_i.
+// Pressure (Eqs. 7-12): the factor f of one neighbour's term f x (x the
+// carrier) in sum_j P* grad W V_j, for particles of densities rho_i and c0 drho_i = b_i.
 // With p = c0^2 drho, P* = c0 (rho_j (b_i + beta rho_i dU) + rho_i c0 drho_j) /
 // (rho_i + rho_j) (Eqs. 8, 12; beta of Eq. 11) and V_j = m_j / rho_j: one
 // division.  Walls by their mirror state rho_i, p_i, 2 U_w - U_L.
 template <typename T>
 __device__ __forceinline__ T pressure_factor(const CasePhys<T> &cp, bool printed, bool push_only, uint32_t kj, T drj,
-                                             T dot, const PairW<T> &g, T rho_i, T b_i) {
-    T dU = vmul(dot, g.inv);                    // U_L - U_R = (v_j - v_i).e (Eq. 10, U = -v.e)
+                                             T dot, const PairG<T> &g, T rho_i, T b_i) {
+    T dU = g.du(dot);                           // U_L - U_R = (v_j - v_i).e (Eq. 10, U = -v.e)
     if (kj == PH_WALL) {
         dU = vmul(T(2), dU);
         T x = vmul(cp.beta_k, dU);
         if (printed) x = vmul(x, vdiv(vmul(cp.c0, b_i), rho_i));
         T ps = vfma(vmul(vmul(clamp_lh(x, cp.beta_lo, cp.beta_hi), rho_i), dU), T(0.5), b_i);   // P* / c0
         if (push_only) ps = vpush(ps);          // no-suction wall reading
-        return vmul(vmul(ps, cp.c0_vol), g.w);
+        return vmul(vmul(ps, cp.c0_vol), g.wd);
     }
     const T rho_j = add_rn(sel(kj, cp.rho0[0], cp.rho0[1]), drj), a_j = mul_rn(cp.c0, drj);
     const T rs = vadd(rho_i, rho_j);
@@ -495,16 +561,16 @@ __device__ __forceinline__ T pressure_factor(const CasePhys<T> &cp, bool printed
     if (printed) x = vmul(x, vdiv(vmul(cp.c0, vadd(b_i, a_j)), rs));
     const T t = vfma(vmul(clamp_lh(x, cp.beta_lo, cp.beta_hi), dU), rho_i, b_i);
     const T num = vfma(rho_j, t, vmul(rho_i, a_j));
-    return vmul(vdiv(vmul(num, sel(kj, cp.mass_c0[0], cp.mass_c0[1])), vmul(rs, rho_j)), g.w);
+    return vmul(vdiv(vmul(num, sel(kj, cp.mass_c0[0], cp.mass_c0[1])), vmul(rs, rho_j)), g.wd);
 }
 // Continuity (Eq. 6): (v_i - v*).e V_j of one neighbour, with
 // (v_i - v*).e = U* - U_L = (rho_j (v_i - v_j).e + (b_i - c0 drho_j)) /
 // (rho_i + rho_j); the printed v* takes the other sign of the pressure
 // difference, folded into sb_i and nsc0 = -(+-c0).  v* = v_w at a wall.
 template <typename T>
-__device__ __forceinline__ T continuity_factor(const CasePhys<T> &cp, uint32_t kj, T drj, T dot, const PairW<T> &g,
+__device__ __forceinline__ T continuity_factor(const CasePhys<T> &cp, uint32_t kj, T drj, T dot, const PairG<T> &g,
                                                T rho_i, T sb_i, T nsc0) {
-    const T dU = vmul(dot, g.inv);
+    const T dU = g.du(dot);
     if (kj == PH_WALL) return vmul(dU, -cp.vol_wall);
     const T rho_j = add_rn(sel(kj, cp.rho0[0], cp.rho0[1]), drj);
     const T num = vfma(-rho_j, dU, vadd(sb_i, mul_rn(nsc0, drj)));
@@ -731,6 +797,19 @@ __global__ void k_copy_back(int64_t n, const V4<T> *pos_t, const V4<T> *vel_t, c
     id[d] = id_t[d];
 }
 
+template <typename T>
+__device__ __forceinline__ T volume_of(const CasePhys<T> &cp, uint32_t kj, T drj) {
+    return kj == PH_WALL ? cp.vol_wall : vdiv(sel(kj, cp.mass[0], cp.mass[1]), add_rn(sel(kj, cp.rho0[0], cp.rho0[1]), drj));
+}
+// Volume of neighbour j.  FP64 reads it: its division takes 10 operations of
+// the narrow pipe per pair, and k_fluid_scatter and sweep C leave the volumes
+// in memory.  FP32 forms it from the density deviation: that write made its
+// sweep C 4% slower and saves two operations per pair here.
+template <typename T>
+__device__ __forceinline__ T volume_at(const CasePhys<T> &cp, uint32_t kj, const T *vd, uint32_t j) {
+    return sizeof(T) == 8 ? vd[j] : volume_of(cp, kj, vd[j]);
+}
+
 // ---- fluid ranks: after the reorder, the fluid particles in sorted order, walls
 // left out: a particle's slot.  The list build, the band and sweeps M, V, B
 // and C (and A with the cell walk) run their tiles over the slots, so no lane
@@ -745,8 +824,8 @@ __global__ void k_fluid_flag(int64_t n, const V4<T> *snap, uint32_t *flag) {
     flag[i] = (i < n && phase_of(w_bits(snap[i].w)) != PH_WALL) ? 1u : 0u;
 }
 
-// Writes each slot's particle and the values a rebuild starts from: a zero
-// colour gradient (the list classes' colour sweep then writes only the
+// Writes each slot's particle and the values a rebuild starts from: the
+// particles' volumes (FP64), a zero colour gradient (the list classes' colour sweep then writes only the
 // interface band) and an empty band.  The first fluid particle of each cell of
 // a list case appends the cell, as (case << 32 | its first particle), to its
 // class's cell list for the list build (warp-aggregated; the order is
@@ -756,7 +835,7 @@ __global__ void k_fluid_flag(int64_t n, const V4<T> *snap, uint32_t *flag) {
 constexpr uint32_t CELL_BITS = 0x3fffffffu;     // the cell coordinates of a packed word
 template <typename T>
 __global__ void k_fluid_scatter(const Tile *__restrict__ tiles, const CaseDesc *__restrict__ desc, const V4<T> *snap,
-                                const uint32_t *rank, uint32_t *fidx, V4<T> *gradC, uint8_t *band, uint64_t *clist,
+                                const uint32_t *rank, const T *drho, T *vol, uint32_t *fidx, V4<T> *gradC, uint8_t *band, uint64_t *clist,
                                 uint32_t *ccount, int64_t base2d) {
     const Tile t = tiles[blockIdx.x];
     const CaseDesc &d = desc[t.c];
@@ -767,6 +846,7 @@ __global__ void k_fluid_scatter(const Tile *__restrict__ tiles, const CaseDesc *
         gradC[i] = V4<T>{T(0), T(0), T(0), T(0)};
         band[i] = 0;
         const uint32_t pk = w_bits(snap[i].w);
+        if (sizeof(T) == 8) vol[i] = volume_of(phys<T>(d), phase_of(pk), drho[i]);
         if (phase_of(pk) != PH_WALL) {
             fidx[rank[i]] = (uint32_t)i;
             first = d.nbr_mode == 0;
@@ -933,10 +1013,6 @@ template <typename T> struct Moment {
         if (D == 3) { m02 = vfma(tx, rz, m02); m12 = vfma(ty, rz, m12); m22 = vfma(vmul(s, rz), rz, m22); }
     }
 };
-template <typename T>
-__device__ __forceinline__ T volume_of(const CasePhys<T> &cp, uint32_t kj, T drj) {
-    return kj == PH_WALL ? cp.vol_wall : vdiv(sel(kj, cp.mass[0], cp.mass[1]), add_rn(sel(kj, cp.rho0[0], cp.rho0[1]), drj));
-}
 
 template <typename T, int D>
 __device__ __forceinline__ void store_B(const Moment<T> &M, int64_t i, V4<T> *bmat) {
@@ -965,7 +1041,7 @@ __device__ __forceinline__ void store_B(const Moment<T> &M, int64_t i, V4<T> *bm
 
 template <bool LIST, typename T, int D>
 __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
-                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap, const T *drho,
+                                        const uint32_t *starts, const ListRef<T> &l, const V4<T> *snap, const T *vol,
                                         V4<T> *bmat, V4<T> *bk, int32_t *status) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
@@ -973,13 +1049,12 @@ __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp
     if (ki == PH_WALL) return;
     const bool own = bk != nullptr && d.surface_corr == 1;
     Moment<T> M{}, Mk{};
-    const bool coinc = neighbors<LIST, false, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, list, count, snap, nullptr, i, si, pki,
-        [&](uint32_t j, const V4<T> &sj, const V4<T> &, T rx, T ry, T rz, T r2) {
-            const uint32_t kj = phase_of(w_bits(sj.w));
-            const T w = vmul(pair_w<T>(cp, r2).w, volume_of(cp, kj, drho[j]));
-            M.template add<D>(w, rx, ry, rz);
+    const bool coinc = neighbors<LIST, false, true, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, l, snap, nullptr, i, si, pki,
+        [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &g) {
+            const T w = vmul(g.outer(), volume_at(cp, kj, vol, j));
+            M.template add<D>(w, g.x, g.y, g.z);
             // the same sum over i's own fluid (surface_corr reading of Eq. 33)
-            if (own && kj == ki) Mk.template add<D>(w, rx, ry, rz);
+            if (own && kj == ki) Mk.template add<D>(w, g.x, g.y, g.z);
         });
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
     store_B<T, D>(M, i, bmat);
@@ -992,11 +1067,12 @@ __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp
 // B = [b00 b01 b02; b01 b11 b12; b02 b12 b22]
 template <typename T> struct ViscSum {
     T ax, ay, az, sx, sy, sz;
-    // w = W' V_j / r, neta = -(pair viscosity), (b0, b1) = B_i
+    // wv = W' V_j / r, w = V_j times the carrier's weight, neta = -(pair
+    // viscosity), b = B_i
     template <int D>
-    __device__ __forceinline__ void add(T w, T neta, bool tvf, const V4<T> &vj, T nvx, T nvy, T nvz, T rx, T ry, T rz,
+    __device__ __forceinline__ void add(T wv, T w, T neta, bool tvf, const V4<T> &vj, T nvx, T nvy, T nvz, T rx, T ry, T rz,
                                         const T (&b)[6], bool wall, const V4<T> &Bj0, const V4<T> &Bj1) {
-        const T f = vmul(neta, w);
+        const T f = vmul(neta, wv);
         ax = vfma(f, vadd(vj.x, nvx), ax);
         ay = vfma(f, vadd(vj.y, nvy), ay);
         if (D == 3) az = vfma(f, vadd(vj.z, nvz), az);
@@ -1043,8 +1119,8 @@ __device__ __forceinline__ void store_V(const CasePhys<T> &cp, bool tvf, int64_t
 
 template <bool LIST, typename T, int D>
 __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
-                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap,
-                                        const V4<T> *vel, const V4<T> *bmat, V4<T> *acc_visc,
+                                        const uint32_t *starts, const ListRef<T> &l, const V4<T> *snap,
+                                        const V4<T> *vel, const T *vol, const V4<T> *bmat, V4<T> *acc_visc,
                                         V4<T> *pos, int32_t *status) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
@@ -1059,23 +1135,24 @@ __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp
         b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y;
     }
     ViscSum<T> S{};
-    const bool coinc = neighbors<LIST, true, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, list, count, snap, vel, i, si, pki,
-        [&](uint32_t j, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
-            const uint32_t kj = phase_of(w_bits(sj.w));
+    const bool coinc = neighbors<LIST, true, true, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, l, snap, vel, i, si, pki,
+        [&](uint32_t j, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
             const bool wall = kj == PH_WALL;
             V4<T> B0{}, B1{};
             if (tvf && !wall) { B0 = bmat[2 * j]; if (D == 3) B1 = bmat[2 * j + 1]; }
-            S.template add<D>(vmul(pair_w<T>(cp, r2).w, volume_of(cp, kj, vj.w)), eta(kj), tvf, vj, -vi.x, -vi.y, -vi.z,
-                                 rx, ry, rz, b, wall, B0, B1);
+            const T V = sizeof(T) == 8 ? vol[j] : volume_of(cp, kj, vj.w);
+            S.template add<D>(vmul(g.dW_r(), V), vmul(g.wd, V), eta(kj), tvf, vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z, b, wall,
+                              B0, B1);
         });
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
     store_V<T, D>(cp, tvf, i, sel(ki, cp.rho0[0], cp.rho0[1]) + vi.w, S.ax, S.ay, S.az, S.sx, S.sy, S.sz, acc_visc, pos);
 }
 
-// ---- A: colour gradient, Eq. 22 (only pairs of different fluids contribute)
+// ---- A: colour gradient, Eq. 22 (only pairs of different fluids contribute),
+// kept as its unit vector and its magnitude (w), the form the surface sum reads
 template <bool LIST, typename T, int D, int L = 1, int U = PLAIN>
 __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
-                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap, const T *drho,
+                                        const uint32_t *starts, const ListRef<T> &l, const V4<T> *snap, const T *vol,
                                         V4<T> *gradC, uint32_t sub = 0) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
@@ -1084,19 +1161,20 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
     if (ki != PH_WALL && d.n_fluid_phases == 2) {
         const uint32_t other = ki ^ 1u;
         const T two_phi = cp.two_phi[ki];
-        const T m_o = cp.mass[other], rho0_o = cp.rho0[other];
-        neighbors<LIST, false, T, D, PART_OTHER, L, U>(d, cp, starts, list, count, snap, nullptr, i, si, pki,
-            [&](uint32_t j, const V4<T> &sj, const V4<T> &, T rx, T ry, T rz, T r2) {
-                if (!LIST && phase_of(w_bits(sj.w)) != other) return;
-                const T s = vmul(vmul(two_phi, pair_w<T>(cp, r2).w), vdiv(m_o, add_rn(rho0_o, drho[j])));
-                g.x = fma_rn(s, rx, g.x);
-                g.y = fma_rn(s, ry, g.y);
-                if (D == 3) g.z = fma_rn(s, rz, g.z);
+        neighbors<LIST, false, false, T, D, PART_OTHER, L, U>(d, cp, starts, l, snap, nullptr, i, si, pki,
+            [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &G) {
+                if (!LIST && kj != other) return;
+                const T s = vmul(vmul(two_phi, G.wd), volume_at(cp, kj, vol, j));
+                g.x = fma_rn(s, G.x, g.x);
+                g.y = fma_rn(s, G.y, g.y);
+                if (D == 3) g.z = fma_rn(s, G.z, g.z);
             }, sub);
         g.x = group_sum<L>(g.x);
         g.y = group_sum<L>(g.y);
         if (D == 3) g.z = group_sum<L>(g.z);
         g.w = sqrt(fma_rn(g.x, g.x, fma_rn(g.y, g.y, g.z * g.z)));
+        const T inv = g.w > T(0) ? T(1) / g.w : T(0);
+        g.x *= inv; g.y *= inv; g.z *= inv;
     }
     if (sub == 0) gradC[i] = g;
 }
@@ -1131,12 +1209,12 @@ __device__ __forceinline__ V4<T> kicked(const V4<T> &vi, T rho_i, T dt, T apx, T
 // stored surface sum (list), 2 = surface sum only (list, band particles).
 template <bool LIST, int PASS, typename T, int D, int L = 1, int U = PLAIN>
 __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &cp, T dt,
-                                          int64_t i, const uint32_t *starts, const uint32_t *list, uint32_t count,
+                                          int64_t i, const uint32_t *starts, const ListRef<T> &l,
                                           const uint8_t *band, const V4<T> *snap,
                                           const V4<T> *vel, const V4<T> *gradC,
                                           const V4<T> *acc_visc, V4<T> *acc_surf, V4<T> *vel_new,
                                           uint32_t *phase_out, uint32_t sub = 0,
-                                          const V4<T> *bk = nullptr, const T *drho_s = nullptr) {
+                                          const V4<T> *bk = nullptr, const T *vol = nullptr) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
     const uint32_t ki = phase_of(pki);
@@ -1149,41 +1227,35 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
     const T b_i = mul_rn(cp.c0, dri);
     T apx = 0, apy = 0, apz = 0, asx = 0, asy = 0, asz = 0;
     const bool printed = d.limiter == 3, push_only = d.wall_form == 1;
-    const auto pressure = [&](uint32_t, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
-        const PairW<T> g = pair_w<T>(cp, r2);
-        const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, rx, ry, rz);
-        const T f = pressure_factor<T>(cp, printed, push_only, phase_of(w_bits(sj.w)), vj.w, dot, g, rho_i, b_i);
-        apx = vfma(f, rx, apx);
-        apy = vfma(f, ry, apy);
-        if (D == 3) apz = vfma(f, rz, apz);
+    const auto pressure = [&](uint32_t, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
+        const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z);
+        const T f = pressure_factor<T>(cp, printed, push_only, kj, vj.w, dot, g, rho_i, b_i);
+        apx = vfma(f, g.x, apx);
+        apy = vfma(f, g.y, apy);
+        if (D == 3) apz = vfma(f, g.z, apz);
     };
 
     // surface stress and penalty (Eqs. 24, 26, 30, 33); walls take no part
-    const V4<T> gi = d.n_fluid_phases == 2 ? gradC[i] : V4<T>{0, 0, 0, 0};
+    // unit normal, magnitude and colour gradient of i; n = 0 off the interface
+    const V4<T> ni = d.n_fluid_phases == 2 ? gradC[i] : V4<T>{0, 0, 0, 0};
+    const V4<T> gi{ni.w * ni.x, ni.w * ni.y, ni.w * ni.z, ni.w};
+    const bool if_i = ni.w * cp.h > cp.nhat_eps;
+    const T nix = if_i ? ni.x : T(0), niy = if_i ? ni.y : T(0), niz = if_i ? ni.z : T(0);
+    const T gam_gi = if_i ? cp.gamma * ni.w : T(0);
     // surface_corr reading: the own-fluid correction matrix of i (Eq. 15
     // over i's fluid), symmetric: (b00, b01, b02, b11), (b12, b22)
     const bool corr = bk != nullptr && d.surface_corr == 1;
     V4<T> bi0{T(0), T(0), T(0), T(0)}, bi1{T(0), T(0), T(0), T(0)};
     if (corr && PASS != 1) { bi0 = bk[2 * i]; bi1 = bk[2 * i + 1]; }
-    const auto surface = [&](uint32_t j, const V4<T> &sj, const V4<T> &gj, T rx, T ry, T rz, T r2) {
-        const uint32_t kj = phase_of(w_bits(sj.w));
+    const auto surface = [&](uint32_t j, uint32_t kj, const V4<T> &nj, const PairG<T> &g) {
         if (kj == PH_WALL) return;
-        if (gi.w == T(0) && gj.w == T(0)) return;                // every surface term vanishes
-        const PairGeo<T> g = geo(cp, r2);
-        const T ex = rx * g.inv_r, ey = ry * g.inv_r, ez = D == 3 ? rz * g.inv_r : T(0);
-        // the density deviation of j: the 4-byte array in the surface sweep
-        // (the same value as vel[j].w, fewer bytes through L1)
-        const T drj_s = PASS == 2 ? drho_s[j] : vel[j].w;
-        const T rho_j = sel(kj, cp.rho0[0], cp.rho0[1]) + drj_s;
-        const T Vj = div_fast(sel(kj, cp.mass[0], cp.mass[1]), rho_j);
-        const bool if_i = gi.w * cp.h > cp.nhat_eps;
-        const T inv_gi = if_i ? div_fast(T(1), gi.w) : T(0);
-        const T nix = gi.x * inv_gi, niy = gi.y * inv_gi, niz = gi.z * inv_gi;
-        const T gam_gi = if_i ? cp.gamma * gi.w : T(0);
-        const bool if_j = gj.w * cp.h > cp.nhat_eps;
-        const T inv_gj = if_j ? div_fast(T(1), gj.w) : T(0);
-        const T njx = gj.x * inv_gj, njy = gj.y * inv_gj, njz = gj.z * inv_gj;
-        const T gam_gj = if_j ? cp.gamma * gj.w : T(0);
+        if (ni.w == T(0) && nj.w == T(0)) return;                // every surface term vanishes
+        const T ex = g.e(g.x), ey = g.e(g.y), ez = D == 3 ? g.e(g.z) : T(0);
+        const T Vj = volume_at(cp, kj, vol, j);
+        const V4<T> gj{nj.w * nj.x, nj.w * nj.y, nj.w * nj.z, nj.w};
+        const bool if_j = nj.w * cp.h > cp.nhat_eps;
+        const T njx = if_j ? nj.x : T(0), njy = if_j ? nj.y : T(0), njz = if_j ? nj.z : T(0);
+        const T gam_gj = if_j ? cp.gamma * nj.w : T(0);
         if (corr && kj == ki) {
             // same-phase line applied to the corrected kernel gradient
             // W' (B^k_i + B^k_j)/2 e = W' v (C_ij = 0): S v with
@@ -1212,11 +1284,11 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             const T nic = nix * cx + niy * cy + niz * cz, njc = njx * cx + njy * cy + njz * cz;
             const T qx = T(0.5) * (nix * nic + njx * njc), qy = T(0.5) * (niy * nic + njy * njc),
                     qz = T(0.5) * (niz * nic + njz * njc);
-            const T pen_s = d.penalty_scope == 1 ? T(0) : cp.xi * cp.gamma * g.inv_r;
+            const T pen_s = d.penalty_scope == 1 ? T(0) : cp.xi * cp.gamma * g.inv;
             const T sx = gam_gi * (vx - nix * niv) + gam_gj * (vx - njx * njv) + pen_s * (cx - qx);
             const T sy = gam_gi * (vy - niy * niv) + gam_gj * (vy - njy * njv) + pen_s * (cy - qy);
             const T sz = gam_gi * (vz - niz * niv) + gam_gj * (vz - njz * njv) + pen_s * (cz - qz);
-            const T w = g.dW * Vj;
+            const T w = g.dW() * Vj;
             asx += sx * w; asy += sy * w; if (D == 3) asz += sz * w;
             return;
         }
@@ -1248,7 +1320,7 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
         const T njc = njx * cx + njy * cy + njz * cz;
         const T qx = T(0.5) * (nix * nic + njx * njc), qy = T(0.5) * (niy * nic + njy * njc),
                 qz = T(0.5) * (niz * nic + njz * njc);
-        const T pen = cp.xi * cp.gamma * g.inv_r;
+        const T pen = cp.xi * cp.gamma * g.inv;
         T sx, sy, sz;
         if (same) {   // Eq. 33, first line; T-bar c = c - N-bar c
             const T pen_s = d.penalty_scope == 1 ? T(0) : pen;
@@ -1265,21 +1337,21 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             sy = a * piy + b * pjy - c * qy;
             sz = a * piz + b * pjz - c * qz;
         }
-        const T w = g.dW * Vj;
+        const T w = g.dW() * Vj;
         asx += sx * w; asy += sy * w; if (D == 3) asz += sz * w;
     };
 
     const bool surface_on = d.n_fluid_phases == 2;
     if constexpr (PASS == 2) {
         if (surface_on)
-            neighbors<LIST, true, T, D, PART_ALL, L, U>(d, cp, starts, list, count, snap, gradC, i, si, pki, surface, sub);
+            neighbors<LIST, true, true, T, D, PART_ALL, L, U>(d, cp, starts, l, snap, gradC, i, si, pki, surface, sub);
         asx = group_sum<L>(asx);
         asy = group_sum<L>(asy);
         if (D == 3) asz = group_sum<L>(asz);
         if (sub == 0) acc_surf[i] = V4<T>{asx, asy, asz, T(0)};
         return 0.0;
     } else if constexpr (PASS == 1) {
-        neighbors<LIST, true, T, D, PART_ALL, L, U>(d, cp, starts, list, count, snap, vel, i, si, pki, pressure, sub);
+        neighbors<LIST, true, false, T, D, PART_ALL, L, U>(d, cp, starts, l, snap, vel, i, si, pki, pressure, sub);
         apx = group_sum<L>(apx);
         apy = group_sum<L>(apy);
         if (D == 3) apz = group_sum<L>(apz);
@@ -1292,10 +1364,10 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             asx = as.x; asy = as.y; asz = as.z;
         }
     } else {
-        neighbors<LIST, true, T, D>(d, cp, starts, list, count, snap, vel, i, si, pki,
-            [&](uint32_t j, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
-                pressure(j, sj, vj, rx, ry, rz, r2);
-                if (surface_on) surface(j, sj, gradC[j], rx, ry, rz, r2);
+        neighbors<LIST, true, true, T, D>(d, cp, starts, l, snap, vel, i, si, pki,
+            [&](uint32_t j, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
+                pressure(j, kj, vj, g);
+                if (surface_on) surface(j, kj, gradC[j], g);
             });
     }
     const V4<T> vn = kicked<T, D>(vi, rho_i, dt, apx, apy, apz, asx, asy, asz, acc_visc[i]);
@@ -1305,9 +1377,11 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
 
 // ---- C: continuity (Eq. 6) with v* (normal component -U*) + drift
 template <typename T, int D>
-__device__ __forceinline__ void store_C(int64_t i, T dt, T rho_i, T sum, V4<T> vi, T *drho, V4<T> *vel, V4<T> *pos) {
+__device__ __forceinline__ void store_C(const CasePhys<T> &cp, uint32_t ki, int64_t i, T dt, T rho_i, T sum, V4<T> vi, T *drho,
+                                        T *vol, V4<T> *vel, V4<T> *pos) {
     const T dr_new = fma_rn(dt, T(2) * rho_i * sum, vi.w);
     drho[i] = dr_new;
+    if (sizeof(T) == 8) vol[i] = volume_of(cp, ki, dr_new);
     V4<T> p = pos[i];
     p.x = fma_rn(dt, vi.x, p.x);
     p.y = fma_rn(dt, vi.y, p.y);
@@ -1319,8 +1393,8 @@ __device__ __forceinline__ void store_C(int64_t i, T dt, T rho_i, T sum, V4<T> v
 
 template <bool LIST, typename T, int D, int L = 1, int U = PLAIN>
 __device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp, T dt, int64_t i,
-                                        const uint32_t *starts, const uint32_t *list, uint32_t count, const V4<T> *snap,
-                                        const V4<T> *vel_new, T *drho,
+                                        const uint32_t *starts, const ListRef<T> &l, const V4<T> *snap,
+                                        const V4<T> *vel_new, T *drho, T *vol,
                                         V4<T> *vel, V4<T> *pos, uint32_t sub = 0) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
@@ -1330,15 +1404,13 @@ __device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp
     const T rho_i = add_rn(sel(ki, cp.rho0[0], cp.rho0[1]), vi.w);
     const T nsc0 = d.vstar_printed ? cp.c0 : -cp.c0, sb_i = mul_rn(-nsc0, vi.w);
     T s = 0;
-    neighbors<LIST, true, T, D, PART_ALL, L, U>(d, cp, starts, list, count, snap, vel_new, i, si, pki,
-        [&](uint32_t, const V4<T> &sj, const V4<T> &vj, T rx, T ry, T rz, T r2) {
-            const PairW<T> g = pair_w<T>(cp, r2);
-            const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, rx, ry, rz);
-            const T f = continuity_factor<T>(cp, phase_of(w_bits(sj.w)), vj.w, dot, g, rho_i, sb_i, nsc0);
-            s = vfma(f, vmul(g.w, g.r), s);
+    neighbors<LIST, true, false, T, D, PART_ALL, L, U>(d, cp, starts, l, snap, vel_new, i, si, pki,
+        [&](uint32_t, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
+            const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z);
+            s = vfma(continuity_factor<T>(cp, kj, vj.w, dot, g, rho_i, sb_i, nsc0), g.dW(), s);
         }, sub);
     s = group_sum<L>(s);
-    if (sub == 0) store_C<T, D>(i, dt, rho_i, s, vi, drho, vel, pos);
+    if (sub == 0) store_C<T, D>(cp, ki, i, dt, rho_i, s, vi, drho, vol, vel, pos);
 }
 
 // ---------------------------------------------------------- sweep kernels
@@ -1356,6 +1428,8 @@ struct SweepArgs {
     // nullptr: tile entries are particle indices; else the tiles run over
     // fluid ranks and fidx maps a rank to the particle (sweeps B and C)
     const uint32_t *fidx = nullptr;
+    // stored pair geometry of the lists (FP64, where it is kept)
+    const void *ge = nullptr, *gr = nullptr;
     // batches: the tiles of the cases active in this substep, compacted per
     // class after the criterion kernel (work[tile0 + k] is a tile index,
     // *work_count of them); the launch's blocks stride over them.  nullptr:
@@ -1397,12 +1471,14 @@ __device__ __forceinline__ int64_t particle_at(const SweepArgs &a, int64_t q) {
     return a.fidx ? (int64_t)a.fidx[q] : q;
 }
 
-template <bool LIST> __device__ __forceinline__ const uint32_t *list_of(const SweepArgs &a, const CaseDesc &d, int64_t q) {
-    return LIST ? a.nbr + list_word(d, q) : nullptr;
+template <bool LIST, typename T> __device__ __forceinline__ ListRef<T> list_of(const SweepArgs &a, const CaseDesc &d, int64_t q) {
+    if (!LIST) return ListRef<T>{nullptr, 0u, nullptr, nullptr};
+    const int64_t w = list_word(d, q);
+    if (sizeof(T) == 8 && a.ge)
+        return ListRef<T>{a.nbr + w, a.cnt[q], static_cast<const V4<T> *>(a.ge) + w, static_cast<const RInv *>(a.gr) + w};
+    return ListRef<T>{a.nbr + w, a.cnt[q], nullptr, nullptr};
 }
-template <bool LIST> __device__ __forceinline__ uint32_t count_of(const SweepArgs &a, int64_t q) {
-    return LIST ? a.cnt[q] : 0u;
-}
+
 // entry t of the band list: (case << 32 | slot)
 struct BandEntry {
     int c;
@@ -1712,25 +1788,54 @@ static __global__ void __launch_bounds__(256) k_band(SweepArgs a, const uint8_t 
     if (b) blist[base + __popc(m & ((1u << lane) - 1u))] = ((uint64_t)(uint32_t)t.c << 32) | (uint64_t)(uint32_t)q;
 }
 
+// ---- G: the stored geometry of the lists (FP64), once per advection step.  A
+// block takes a tile's slots 32 at a time, its warps the rows.  FP64 sweeps
+// are bound by their arithmetic (2 FP64 lanes per clock and SM), of which the
+// pair geometry is half: 26 of 59 operations in B, of 49 in C; reading 32 bytes
+// per pair instead costs 1/10 of that time.
+constexpr int LG_WARPS = 8;
+template <int D>
+__global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V4<double> *snap, V4<double> *ge, RInv *gr) {
+    const Tile t = a.tiles[a.tile0 + blockIdx.x];
+    if (!a.st[t.c].active) return;
+    const CaseDesc &d = a.desc[t.c];
+    const CasePhys<double> &cp = d.pd;
+    for (int s = threadIdx.x; s < t.n; s += 32) {
+        const int64_t q = t.begin + s, i = particle_at(a, q), w = list_word(d, q);
+        const V4<double> si = ld4(snap + i);
+        const uint32_t c = a.cnt[q] & CNT_MASK;
+        for (uint32_t k = threadIdx.y; k < c; k += LG_WARPS) {
+            const int64_t at = w + (int64_t)k * LROW;
+            const uint32_t e = ld_list(a.nbr + at);
+            const V4<double> sj = ld4(snap + (e >> NBR_SHIFT));
+            const Moved<double, D> m = moved<double, D>(e, sj, cp.cs);
+            const double rx = vadd(si.x, m.nx), ry = vadd(si.y, m.ny), rz = D == 3 ? vadd(si.z, m.nz) : 0.0;
+            const PairG<double> g(cp, rx, ry, rz, norm2<double, D>(rx, ry, rz));
+            ge[at] = V4<double>{g.x, g.y, g.z, phase_of(w_bits(sj.w)) == PH_WALL ? -g.wd : g.wd};
+            gr[at] = RInv{g.r, g.inv};
+        }
+    }
+}
+
 template <typename T, int D, bool LIST>
-__global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const T *drho, V4<T> *bmat,
+__global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const T *vol, V4<T> *bmat,
                                            V4<T> *bk) {
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
     if (!d.tvf_on && d.surface_corr != 1) return;
     const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
-    sweep_M<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q), snap, drho, bmat, bk, &a.st[t.c].status);
+    sweep_M<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, bmat, bk, &a.st[t.c].status);
 }
 
 template <typename T, int D, bool LIST>
-__global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const V4<T> *vel,
+__global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const V4<T> *vel, const T *vol,
                                            const V4<T> *bmat, V4<T> *acc_visc, V4<T> *pos) {
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
     const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
-    sweep_V<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q), snap, vel, bmat, acc_visc, pos,
+    sweep_V<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vel, vol, bmat, acc_visc, pos,
                         &a.st[t.c].status);
 }
 
@@ -1745,14 +1850,14 @@ template <int L> __device__ __forceinline__ int local_index(int64_t w) {
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
-__global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, const T *drho, V4<T> *gradC) {
+__global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, const T *vol, V4<T> *gradC) {
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         const int li = local_index<L>(w);
         if (li >= t.n || !a.st[t.c].active) return;
         const CaseDesc &d = case_desc<MODE>(a, t.c);
         const int64_t q = t.begin + li, i = particle_at(a, q);
-        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q), snap, drho, gradC,
+        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, gradC,
                                threadIdx.x % L);
     };
     if constexpr (MODE == MODE_WORK) {
@@ -1771,13 +1876,13 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, con
 // zero written at the start of the advection step.
 template <typename T, int D, int L = 1>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4) k_sweep_A_band(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
-                                                const V4<T> *snap, const T *drho, V4<T> *gradC) {
+                                                const V4<T> *snap, const T *vol, V4<T> *gradC) {
     const int64_t items = (int64_t)*bcount * L;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
         const BandEntry e(a, blist, t / L);
         if (!a.st[e.c].active) continue;
         const CaseDesc &d = a.desc[e.c];
-        sweep_A<true, T, D, L, AHEAD>(d, phys<T>(d), e.i, a.starts, list_of<true>(a, d, e.q), count_of<true>(a, e.q), snap, drho, gradC, threadIdx.x % L);
+        sweep_A<true, T, D, L, AHEAD>(d, phys<T>(d), e.i, a.starts, list_of<true, T>(a, d, e.q), snap, vol, gradC, threadIdx.x % L);
     }
 }
 
@@ -1788,15 +1893,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4) k_sweep_A_band(Sw
 template <typename T, int D, int L = 1>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) k_sweep_S(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
                                            const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
-                                           const V4<T> *gradC, V4<T> *acc_surf, const V4<T> *bk, const T *drho) {
+                                           const V4<T> *gradC, V4<T> *acc_surf, const V4<T> *bk, const T *vol) {
     const int64_t items = (int64_t)*bcount * L;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
         const BandEntry e(a, blist, t / L);
         if (!a.st[e.c].active) continue;
         const CaseDesc &d = a.desc[e.c];
         uint32_t ph;
-        sweep_B<true, 2, T, D, L, 4>(d, phys<T>(d), T(0), e.i, a.starts, list_of<true>(a, d, e.q), count_of<true>(a, e.q), band, snap, vel, gradC,
-                                          nullptr, acc_surf, nullptr, &ph, threadIdx.x % L, bk, drho);
+        sweep_B<true, 2, T, D, L, 4>(d, phys<T>(d), T(0), e.i, a.starts, list_of<true, T>(a, d, e.q), band, snap, vel, gradC,
+                                          nullptr, acc_surf, nullptr, &ph, threadIdx.x % L, bk, vol);
     }
 }
 
@@ -1815,7 +1920,7 @@ __device__ __forceinline__ void reduce_vmax(const SweepArgs &a, int c, uint32_t 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
 __global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
                                             const V4<T> *gradC, const V4<T> *acc_visc, V4<T> *acc_surf,
-                                            V4<T> *vel_new, const V4<T> *bk) {
+                                            V4<T> *vel_new, const V4<T> *bk, const T *vol) {
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         if (!a.st[t.c].active) return;             // uniform per block
@@ -1826,10 +1931,9 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_
         if (li < t.n) {
             const int64_t q = t.begin + li, i = particle_at(a, q);
             const T dt = (T)a.st[t.c].dt;
-            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L, MODE == MODE_FEW ? 4 : PLAIN>(d, phys<T>(d), dt, i, a.starts, list_of<LIST>(a, d, q),
-                                                      count_of<LIST>(a, q), band, snap, vel,
+            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L, MODE == MODE_FEW ? 4 : PLAIN>(d, phys<T>(d), dt, i, a.starts, list_of<LIST, T>(a, d, q), band, snap, vel,
                                                       gradC, acc_visc, acc_surf, vel_new, &ph, threadIdx.x % L,
-                                                      LIST ? nullptr : bk);
+                                                      LIST ? nullptr : bk, vol);
         }
         reduce_vmax(a, t.c, ph, (unsigned long long)__double_as_longlong(v2));
     };
@@ -1842,7 +1946,7 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
-__global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho,
+__global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho, T *vol,
                                            V4<T> *vel, V4<T> *pos) {
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
@@ -1851,8 +1955,8 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const
         const CaseDesc &d = case_desc<MODE>(a, t.c);
         const int64_t q = t.begin + li, i = particle_at(a, q);
         const T dt = (T)a.st[t.c].dt;
-        sweep_C<LIST, T, D, L, MODE == MODE_FEW && D == 2 ? 4 : AHEAD>(d, phys<T>(d), dt, i, a.starts, list_of<LIST>(a, d, q), count_of<LIST>(a, q),
-                               snap, vel_new, drho, vel, pos,
+        sweep_C<LIST, T, D, L, MODE == MODE_FEW && D == 2 ? 4 : AHEAD>(d, phys<T>(d), dt, i, a.starts, list_of<LIST, T>(a, d, q),
+                               snap, vel_new, drho, vol, vel, pos,
                                threadIdx.x % L);
     };
     if constexpr (MODE == MODE_WORK) {
@@ -2013,8 +2117,8 @@ __global__ void k_read_field(const CaseDesc *desc, int c, int field, const V4<T>
         case 3: out[o] = ph < 2 ? d.c0 * d.c0 * (double)drho[i] : 0.0; break;
         case 5: {
             const V4<T> g = gradC[i];
-            const double gg[3] = {(double)g.x, (double)g.y, (double)g.z};
-            for (int a = 0; a < dim; ++a) out[o * dim + a] = gg[a];
+            const double gg[3] = {(double)g.x, (double)g.y, (double)g.z};   // unit vector; w the magnitude
+            for (int a = 0; a < dim; ++a) out[o * dim + a] = (double)g.w * gg[a];
             break;
         }
         case 6: {
