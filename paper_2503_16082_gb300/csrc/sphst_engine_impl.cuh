@@ -30,8 +30,8 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         switch (k_) {                                                                  \
         case 0: KERN<T, 3, true><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;    \
         case 1: KERN<T, 2, true><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;    \
-        case 2: KERN<T, 3, false><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;   \
-        default: KERN<T, 2, false><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;  \
+        case 2: KERN<T, 3, false, CELL_LANES><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break;   \
+        default: KERN<T, 2, false, CELL_LANES><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break;  \
         }                                                                              \
     }
 
@@ -71,8 +71,8 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         switch (k_) {                                                                                  \
         case 0: SPH_LANES_M(KERN, 3, LN, MODE, __VA_ARGS__) break;                                     \
         case 1: SPH_LANES_M(KERN, 2, LN, MODE, __VA_ARGS__) break;                                     \
-        case 2: KERN<T, 3, false, 1, CELL_MODE(MODE)><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break; \
-        default: KERN<T, 2, false, 1, CELL_MODE(MODE)><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;\
+        case 2: KERN<T, 3, false, CELL_LANES, CELL_MODE(MODE)><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break; \
+        default: KERN<T, 2, false, CELL_LANES, CELL_MODE(MODE)><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break;\
         }                                                                                              \
     }
 

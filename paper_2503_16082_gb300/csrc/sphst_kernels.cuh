@@ -7,8 +7,8 @@
 // frozen configuration and the interface band.
 //
 // Pair sweeps (gather-only: every particle's sum is owned by one thread, or by
-// a group of 2-8 lanes that split its list and add their parts in a fixed
-// order, so there are no atomics on particle data):
+// a group of 2-8 lanes that split its list, or its cells, and add their parts
+// in a fixed order, so there are no atomics on particle data):
 //   M  correction matrix B_i (Eq. 15; also over the own fluid for the
 //      surface_corr reading)                             once per advection step
 //   V  viscous acceleration (Eq. 13) + transport shift (Eq. 14)  once per advection step
@@ -85,8 +85,8 @@
 #endif
 // sweep B of a one-case engine reads its per-case constants from the
 // parameter block, which leaves it room for more resident blocks
-#define SPH_SWEEPB_BOUNDS_M(T, MODE)                                                          \
-    __launch_bounds__(256, (MODE) == 3 ? 1 : sizeof(T) == 8 ? 2 : (MODE) == 2 ? SPHST_SWEEPB_MINB_ONE                  \
+#define SPH_SWEEPB_BOUNDS_M(T, LIST, MODE)                                                          \
+    __launch_bounds__(256, (MODE) == 3 || !(LIST) ? 1 : sizeof(T) == 8 ? 2 : (MODE) == 2 ? SPHST_SWEEPB_MINB_ONE                  \
                                                          : (SPHST_SWEEPB_MINB > 0 ? SPHST_SWEEPB_MINB : 1))
 
 namespace sphst {
@@ -260,34 +260,27 @@ __device__ __forceinline__ bool walk(const CaseDesc &d, const CasePhys<T> &cp,
                                      const uint32_t *__restrict__ starts,
                                      const V4<T> *__restrict__ snap, int64_t i,
                                      const V4<T> &si, uint32_t pki, F &&f) {
+    constexpr int NC = D == 3 ? 27 : 9;
     const int cx = cell_x<D>(pki), cy = cell_y<D>(pki), cz = cell_z<D>(pki);
     const uint32_t toff = (uint32_t)d.table_off;
     const T cs = cp.cs, R2 = cp.four_h2;
     bool coincident = false;
-    for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz) {
-        int nz = cz + oz;
-        if (D == 3 && !wrap_cell(d, 2, nz)) continue;
+    for (int q = 0; q < NC; ++q) {
+        const int ox = q % 3 - 1, oy = q / 3 % 3 - 1, oz = D == 3 ? q / 9 - 1 : 0;
+        int nx = cx + ox, ny = cy + oy, nz = cz + oz;
+        if (!wrap_cell(d, 0, nx) || !wrap_cell(d, 1, ny) || (D == 3 && !wrap_cell(d, 2, nz))) continue;
+        const T sx = sub_rn(si.x, mul_rn(T(ox), cs)), sy = sub_rn(si.y, mul_rn(T(oy), cs));
         const T sz = D == 3 ? sub_rn(si.z, mul_rn(T(oz), cs)) : T(0);
-        for (int oy = -1; oy <= 1; ++oy) {
-            int ny = cy + oy;
-            if (!wrap_cell(d, 1, ny)) continue;
-            const T sy = sub_rn(si.y, mul_rn(T(oy), cs));
-            for (int ox = -1; ox <= 1; ++ox) {
-                int nx = cx + ox;
-                if (!wrap_cell(d, 0, nx)) continue;
-                const T sx = sub_rn(si.x, mul_rn(T(ox), cs));
-                const uint32_t m = toff + morton<D>(nx, ny, nz);
-                const uint32_t b = __ldg(starts + m), e = __ldg(starts + m + 1);
-                for (uint32_t j = b; j < e; ++j) {
-                    const V4<T> sj = ld4(snap + j);
-                    const T rx = sub_rn(sx, sj.x), ry = sub_rn(sy, sj.y);
-                    const T rz = D == 3 ? sub_rn(sz, sj.z) : T(0);
-                    const T r2 = norm2<T, D>(rx, ry, rz);
-                    if (r2 < R2 && j != (uint32_t)i) {
-                        if (r2 > T(0)) f(j, sj, rx, ry, rz, r2);
-                        else coincident = true;
-                    }
-                }
+        const uint32_t m = toff + morton<D>(nx, ny, nz);
+        const uint32_t b = __ldg(starts + m), e = __ldg(starts + m + 1);
+        for (uint32_t j = b; j < e; ++j) {
+            const V4<T> sj = ld4(snap + j);
+            const T rx = sub_rn(sx, sj.x), ry = sub_rn(sy, sj.y);
+            const T rz = D == 3 ? sub_rn(sz, sj.z) : T(0);
+            const T r2 = norm2<T, D>(rx, ry, rz);
+            if (r2 < R2 && j != (uint32_t)i) {
+                if (r2 > T(0)) f(j, sj, rx, ry, rz, r2);
+                else coincident = true;
             }
         }
     }
@@ -488,10 +481,136 @@ __device__ __forceinline__ void walk_geo(const ListRef<double> &l, uint32_t c, c
     }
 }
 
+// The cell walk of a sweep (cases without a list).  Only a sixth of the
+// candidates of the 3^D cells are neighbours, and which ones differs from lane
+// to lane: evaluated where they are found, nearly every candidate cost its
+// warp the whole pair with few lanes at work.  So each thread puts its hits
+// aside in shared memory, and when a lane of the warp might run out of places
+// all lanes evaluate what they have, in the walk's order (the same sums).
+// With two lanes per particle, 30k particles in 3D: FP32 A 76 -> 52, B 308 ->
+// 92, C 150 -> 68 us; FP64 A 614 -> 388, B 4381 -> 1118, C 1689 -> 703.  125k:
+// A 87 -> 101, B 376 -> 257, C 187 -> 168; at 1M, where one lane per particle
+// filled the chip as well, A 458 -> 600, B 1789 -> 1775, C 1001 -> 1043.
+// Lanes per particle: lane `sub` takes the cells sub, sub + L, ... of the 3^D,
+// and the lanes add their sums in a fixed order.  One lane leaves a case of 30k
+// particles 6 warps per SM, each waiting for its candidates.
+constexpr int CELL_LANES = 2;
+// Places of a thread, a word and a byte each.  More make the evaluations
+// fuller, fewer leave shared memory to more warps, which the cheap pairs of
+// FP32 sweeps A (which puts only the other fluid aside) and C need more: at
+// 125k particles C 168 us with 32, 175 with 38, 195 with 56; B 257 with 56,
+// 272 with 48, 283 with 38.  FP64 pairs are dear: C 703 with 56, 838 with 38.
+constexpr int CELL_PLACES_MAX = 56;
+constexpr int CELL_PLACES_k_sweep_A = 20, CELL_PLACES_k_sweep_C = 32;
+constexpr int CELL_PLACES_k_sweep_B = 56, CELL_PLACES_k_sweep_V = 56, CELL_PLACES_k_sweep_M = 32;
+// at most 48 KB per block, so that no block size asks for an opt-in
+template <typename T> __host__ __device__ inline int cell_places(int threads, int want) {
+    return min(sizeof(T) == 8 ? CELL_PLACES_MAX : want, 49152 / (threads * 5));
+}
+template <typename T> __host__ __device__ inline size_t cell_walk_bytes(int threads, int want) {
+    return (size_t)threads * cell_places<T>(threads, want) * 5;
+}
+constexpr int CELL_STEP = 16;                   // candidates between two looks at the free places
+template <int PLACES, bool AUX, bool AUX2, bool OTHER, typename T, int D, int L, typename F>
+__device__ __forceinline__ bool walk_cells(const CaseDesc &d, const CasePhys<T> &cp, const uint32_t *__restrict__ starts,
+                                           const V4<T> *__restrict__ snap, const V4<T> *__restrict__ aux,
+                                           const V4<T> *__restrict__ aux2, int64_t i, const V4<T> &si, uint32_t pki, uint32_t sub, F &&f) {
+    constexpr int NC = D == 3 ? 27 : 9;
+    constexpr int U = sizeof(T) == 8 ? 2 : 4;   // gathers in flight
+    extern __shared__ __align__(16) unsigned char sph_cells[];
+    const int threads = blockDim.x, places = cell_places<T>(threads, PLACES), step = min(CELL_STEP, places);
+    const uint32_t other = phase_of(pki) ^ 1u;
+    uint32_t *const word = reinterpret_cast<uint32_t *>(sph_cells) + threadIdx.x;
+    uint8_t *const codes = sph_cells + (size_t)threads * places * 4 + threadIdx.x;
+    const unsigned lanes = __activemask();
+    const int cx = cell_x<D>(pki), cy = cell_y<D>(pki), cz = cell_z<D>(pki);
+    const T cs = cp.cs, R2 = cp.four_h2;
+    bool coincident = false;
+    int held = 0;
+    const auto evaluate = [&]() {
+        for (int k0 = 0; k0 < held; k0 += U) {
+            uint32_t j[U];
+            V4<T> sj[U], aj[U], bj[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {        // past the end: the last one again, not evaluated
+                j[u] = word[min(k0 + u, held - 1) * threads];
+                sj[u] = ld4_now(snap + j[u]);
+                aj[u] = AUX ? ld4_now(aux + j[u]) : sj[u];
+                bj[u] = AUX2 ? ld4_now(aux2 + j[u]) : sj[u];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (k0 + u >= held) break;
+                const uint32_t c = codes[(k0 + u) * threads];
+                const T rx = sub_rn(fma_rn(-code_off(c & 3u, T()), cs, si.x), sj[u].x);
+                const T ry = sub_rn(fma_rn(-code_off((c >> 2) & 3u, T()), cs, si.y), sj[u].y);
+                const T rz = D == 3 ? sub_rn(fma_rn(-code_off((c >> 4) & 3u, T()), cs, si.z), sj[u].z) : T(0);
+                const PairG<T> g(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz));
+                if constexpr (AUX2) f(j[u], phase_of(w_bits(sj[u].w)), aj[u], bj[u], g);
+                else f(j[u], phase_of(w_bits(sj[u].w)), aj[u], g);
+            }
+        }
+        held = 0;
+        __syncwarp(lanes);
+    };
+    // particles of the q-th cell around, none past the last or off the grid
+    const auto range = [&](int q, uint32_t &b, uint32_t &e) {
+        int nx = cx + q % 3 - 1, ny = cy + q / 3 % 3 - 1, nz = D == 3 ? cz + q / 9 - 1 : 0;
+        b = e = 0;
+        if (q < NC && wrap_cell(d, 0, nx) && wrap_cell(d, 1, ny) && (D == 2 || wrap_cell(d, 2, nz))) {
+            const uint32_t m = (uint32_t)d.table_off + morton<D>(nx, ny, nz);
+            b = __ldg(starts + m);
+            e = __ldg(starts + m + 1);
+        }
+    };
+    uint32_t nb, ne;                             // the next cell's, read one cell ahead
+    range((int)sub, nb, ne);
+#pragma unroll 1
+    for (int q = (int)sub; __any_sync(lanes, q < NC); q += L) {
+        uint32_t b = nb;
+        const uint32_t e = ne;
+        const int ox = q % 3 - 1, oy = q / 3 % 3 - 1, oz = D == 3 ? q / 9 - 1 : 0;
+        const T sx = sub_rn(si.x, mul_rn(T(ox), cs)), sy = sub_rn(si.y, mul_rn(T(oy), cs));
+        const T sz = D == 3 ? sub_rn(si.z, mul_rn(T(oz), cs)) : T(0);
+        const uint8_t code = (uint8_t)cell_code<D>(ox, oy, oz);
+        range(q + L, nb, ne);
+        while (__any_sync(lanes, b < e)) {
+            const uint32_t end = min(e, b + step);
+            if (__any_sync(lanes, held + (int)(end - min(b, end)) > places)) evaluate();
+            const auto test = [&](uint32_t k, const V4<T> &sj) {
+                const T rx = sub_rn(sx, sj.x), ry = sub_rn(sy, sj.y);
+                const T rz = D == 3 ? sub_rn(sz, sj.z) : T(0);
+                const T r2 = norm2<T, D>(rx, ry, rz);
+                if (r2 < R2) {
+                    if (!(r2 > T(0))) {
+                        coincident |= k != (uint32_t)i;
+                    } else if (!OTHER || phase_of(w_bits(sj.w)) == other) {
+                        word[held * threads] = k;
+                        codes[held * threads] = code;
+                        ++held;
+                    }
+                }
+            };
+            for (; b + U <= end; b += U) {
+                V4<T> sj[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) sj[u] = ld4_now(snap + b + u);
+#pragma unroll
+                for (int u = 0; u < U; ++u) test(b + u, sj[u]);
+            }
+            for (; b < end; ++b) test(b, ld4_now(snap + b));
+            b = max(b, end);
+            __syncwarp(lanes);
+        }
+    }
+    evaluate();
+    return coincident;
+}
+
 // neighbours of particle i as f(j, kind of j, aux_j, geometry), from its list
-// or from the cell walk, which visits all: PART_OTHER leaves the choice to the
-// caller.  NEED_R: f reads r or 1/r.
-template <bool LIST, bool AUX, bool NEED_R, typename T, int D, int PART = PART_ALL, int L = 1, int U = PLAIN, typename F>
+// or from the cell walk.  NEED_R: f reads r or 1/r.
+template <bool LIST, bool AUX, bool NEED_R, typename T, int D, int PART = PART_ALL, int L = 1, int U = PLAIN, int PLACES = 0,
+          typename F>
 __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &cp, const uint32_t *starts,
                                           const ListRef<T> &l, const V4<T> *snap, const V4<T> *aux, int64_t i,
                                           const V4<T> &si, uint32_t pki, F &&f, uint32_t sub = 0) {
@@ -511,10 +630,7 @@ __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &
             }, sub);
         return false;
     } else {
-        return walk<T, D>(d, cp, starts, snap, i, si, pki,
-            [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
-                f(j, phase_of(w_bits(sj.w)), AUX ? ld4(aux + j) : sj, PairG<T>(cp, rx, ry, rz, r2));
-            });
+        return walk_cells<PLACES, AUX, false, PART == PART_OTHER, T, D, L>(d, cp, starts, snap, aux, nullptr, i, si, pki, sub, f);
     }
 }
 
@@ -1012,6 +1128,10 @@ template <typename T> struct Moment {
         m00 = vfma(tx, rx, m00); m01 = vfma(tx, ry, m01); m11 = vfma(ty, ry, m11);
         if (D == 3) { m02 = vfma(tx, rz, m02); m12 = vfma(ty, rz, m12); m22 = vfma(vmul(s, rz), rz, m22); }
     }
+    template <int L> __device__ __forceinline__ void group() {
+        m00 = group_sum<L>(m00); m01 = group_sum<L>(m01); m02 = group_sum<L>(m02);
+        m11 = group_sum<L>(m11); m12 = group_sum<L>(m12); m22 = group_sum<L>(m22);
+    }
 };
 
 template <typename T, int D>
@@ -1039,24 +1159,27 @@ __device__ __forceinline__ void store_B(const Moment<T> &M, int64_t i, V4<T> *bm
     bmat[2 * i + 1] = V4<T>{b12, b22, T(0), T(0)};
 }
 
-template <bool LIST, typename T, int D>
+template <bool LIST, typename T, int D, int L = 1>
 __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
                                         const uint32_t *starts, const ListRef<T> &l, const V4<T> *snap, const T *vol,
-                                        V4<T> *bmat, V4<T> *bk, int32_t *status) {
+                                        V4<T> *bmat, V4<T> *bk, int32_t *status, uint32_t sub = 0) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
     const uint32_t ki = phase_of(pki);
     if (ki == PH_WALL) return;
     const bool own = bk != nullptr && d.surface_corr == 1;
     Moment<T> M{}, Mk{};
-    const bool coinc = neighbors<LIST, false, true, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, l, snap, nullptr, i, si, pki,
+    const bool coinc = neighbors<LIST, false, true, T, D, PART_ALL, L, AHEAD, CELL_PLACES_k_sweep_M>(d, cp, starts, l, snap, nullptr, i, si, pki,
         [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &g) {
             const T w = vmul(g.outer(), volume_at(cp, kj, vol, j));
             M.template add<D>(w, g.x, g.y, g.z);
             // the same sum over i's own fluid (surface_corr reading of Eq. 33)
             if (own && kj == ki) Mk.template add<D>(w, g.x, g.y, g.z);
-        });
+        }, sub);
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
+    M.template group<L>();
+    if (own) Mk.template group<L>();
+    if (sub != 0) return;
     store_B<T, D>(M, i, bmat);
     if (own) store_B<T, D>(Mk, i, bk);
 }
@@ -1090,6 +1213,10 @@ template <typename T> struct ViscSum {
             sz = vfma(vadd(b[2], b02), gx, vfma(vadd(b[4], b12), gy, vfma(vadd(b[5], b22), gz, sz)));
         }
     }
+    template <int L> __device__ __forceinline__ void group() {
+        ax = group_sum<L>(ax); ay = group_sum<L>(ay); az = group_sum<L>(az);
+        sx = group_sum<L>(sx); sy = group_sum<L>(sy); sz = group_sum<L>(sz);
+    }
 };
 // the pair viscosity 2 eta_i eta_j / (eta_i + eta_j) takes one value per fluid
 // of j; walls use eta_i.  Negated.
@@ -1117,11 +1244,11 @@ __device__ __forceinline__ void store_V(const CasePhys<T> &cp, bool tvf, int64_t
     }
 }
 
-template <bool LIST, typename T, int D>
+template <bool LIST, typename T, int D, int L = 1>
 __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp, int64_t i,
                                         const uint32_t *starts, const ListRef<T> &l, const V4<T> *snap,
                                         const V4<T> *vel, const T *vol, const V4<T> *bmat, V4<T> *acc_visc,
-                                        V4<T> *pos, int32_t *status) {
+                                        V4<T> *pos, int32_t *status, uint32_t sub = 0) {
     const V4<T> si = ld4(snap + i);
     const uint32_t pki = w_bits(si.w);
     const uint32_t ki = phase_of(pki);
@@ -1135,7 +1262,7 @@ __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp
         b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y;
     }
     ViscSum<T> S{};
-    const bool coinc = neighbors<LIST, true, true, T, D, PART_ALL, 1, AHEAD>(d, cp, starts, l, snap, vel, i, si, pki,
+    const bool coinc = neighbors<LIST, true, true, T, D, PART_ALL, L, AHEAD, CELL_PLACES_k_sweep_V>(d, cp, starts, l, snap, vel, i, si, pki,
         [&](uint32_t j, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
             const bool wall = kj == PH_WALL;
             V4<T> B0{}, B1{};
@@ -1143,8 +1270,10 @@ __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp
             const T V = sizeof(T) == 8 ? vol[j] : volume_of(cp, kj, vj.w);
             S.template add<D>(vmul(g.dW_r(), V), vmul(g.wd, V), eta(kj), tvf, vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z, b, wall,
                               B0, B1);
-        });
+        }, sub);
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
+    S.template group<L>();
+    if (sub != 0) return;
     store_V<T, D>(cp, tvf, i, sel(ki, cp.rho0[0], cp.rho0[1]) + vi.w, S.ax, S.ay, S.az, S.sx, S.sy, S.sz, acc_visc, pos);
 }
 
@@ -1159,11 +1288,9 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
     const uint32_t ki = phase_of(pki);
     V4<T> g = {0, 0, 0, 0};
     if (ki != PH_WALL && d.n_fluid_phases == 2) {
-        const uint32_t other = ki ^ 1u;
         const T two_phi = cp.two_phi[ki];
-        neighbors<LIST, false, false, T, D, PART_OTHER, L, U>(d, cp, starts, l, snap, nullptr, i, si, pki,
+        neighbors<LIST, false, false, T, D, PART_OTHER, L, U, CELL_PLACES_k_sweep_A>(d, cp, starts, l, snap, nullptr, i, si, pki,
             [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &G) {
-                if (!LIST && kj != other) return;
                 const T s = vmul(vmul(two_phi, G.wd), volume_at(cp, kj, vol, j));
                 g.x = fma_rn(s, G.x, g.x);
                 g.y = fma_rn(s, G.y, g.y);
@@ -1344,14 +1471,14 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
     const bool surface_on = d.n_fluid_phases == 2;
     if constexpr (PASS == 2) {
         if (surface_on)
-            neighbors<LIST, true, true, T, D, PART_ALL, L, U>(d, cp, starts, l, snap, gradC, i, si, pki, surface, sub);
+            neighbors<LIST, true, true, T, D, PART_ALL, L, U, CELL_PLACES_k_sweep_B>(d, cp, starts, l, snap, gradC, i, si, pki, surface, sub);
         asx = group_sum<L>(asx);
         asy = group_sum<L>(asy);
         if (D == 3) asz = group_sum<L>(asz);
         if (sub == 0) acc_surf[i] = V4<T>{asx, asy, asz, T(0)};
         return 0.0;
     } else if constexpr (PASS == 1) {
-        neighbors<LIST, true, false, T, D, PART_ALL, L, U>(d, cp, starts, l, snap, vel, i, si, pki, pressure, sub);
+        neighbors<LIST, true, false, T, D, PART_ALL, L, U, CELL_PLACES_k_sweep_B>(d, cp, starts, l, snap, vel, i, si, pki, pressure, sub);
         apx = group_sum<L>(apx);
         apy = group_sum<L>(apy);
         if (D == 3) apz = group_sum<L>(apz);
@@ -1364,11 +1491,23 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             asx = as.x; asy = as.y; asz = as.z;
         }
     } else {
-        neighbors<LIST, true, true, T, D>(d, cp, starts, l, snap, vel, i, si, pki,
-            [&](uint32_t j, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
-                pressure(j, kj, vj, g);
-                if (surface_on) surface(j, kj, gradC[j], g);
-            });
+        if (surface_on)
+            walk_cells<CELL_PLACES_k_sweep_B, true, true, false, T, D, L>(d, cp, starts, snap, vel, gradC, i, si, pki, sub,
+                [&](uint32_t j, uint32_t kj, const V4<T> &vj, const V4<T> &nj, const PairG<T> &g) {
+                    pressure(j, kj, vj, g);
+                    surface(j, kj, nj, g);
+                });
+        else
+            walk_cells<CELL_PLACES_k_sweep_B, true, false, false, T, D, L>(d, cp, starts, snap, vel, nullptr, i, si, pki, sub, pressure);
+        apx = group_sum<L>(apx);
+        apy = group_sum<L>(apy);
+        asx = group_sum<L>(asx);
+        asy = group_sum<L>(asy);
+        if (D == 3) { apz = group_sum<L>(apz); asz = group_sum<L>(asz); }
+        if (sub != 0) {
+            *phase_out = PH_WALL;
+            return 0.0;
+        }
     }
     const V4<T> vn = kicked<T, D>(vi, rho_i, dt, apx, apy, apz, asx, asy, asz, acc_visc[i]);
     vel_new[i] = vn;
@@ -1404,7 +1543,7 @@ __device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp
     const T rho_i = add_rn(sel(ki, cp.rho0[0], cp.rho0[1]), vi.w);
     const T nsc0 = d.vstar_printed ? cp.c0 : -cp.c0, sb_i = mul_rn(-nsc0, vi.w);
     T s = 0;
-    neighbors<LIST, true, false, T, D, PART_ALL, L, U>(d, cp, starts, l, snap, vel_new, i, si, pki,
+    neighbors<LIST, true, false, T, D, PART_ALL, L, U, CELL_PLACES_k_sweep_C>(d, cp, starts, l, snap, vel_new, i, si, pki,
         [&](uint32_t, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
             const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z);
             s = vfma(continuity_factor<T>(cp, kj, vj.w, dot, g, rho_i, sb_i, nsc0), g.dW(), s);
@@ -1463,6 +1602,11 @@ template <int L, bool WORK> __device__ __forceinline__ int64_t work_items(const 
 }
 template <int L, bool WORK> __device__ __forceinline__ Tile work_tile(const SweepArgs &a, int64_t w) {
     return a.tiles[WORK ? (int64_t)a.work[a.tile0 + w / L] : a.tile0 + w / L];
+}
+
+// particle of a thread within its tile: with L lanes a block covers 1/L of it
+template <int L> __device__ __forceinline__ int local_index(int64_t w) {
+    return L == 1 ? (int)threadIdx.x : (int)((w % L) * (blockDim.x / L) + threadIdx.x / L);
 }
 
 // particle of tile position q: the position itself, or the fluid particle of
@@ -1817,26 +1961,28 @@ __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V
     }
 }
 
-template <typename T, int D, bool LIST>
+template <typename T, int D, bool LIST, int L = 1>
 __global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const T *vol, V4<T> *bmat,
                                            V4<T> *bk) {
-    const Tile t = a.tiles[a.tile0 + blockIdx.x];
-    if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
+    const Tile t = work_tile<L, false>(a, blockIdx.x);
+    const int li = local_index<L>(blockIdx.x);
+    if (li >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
     if (!d.tvf_on && d.surface_corr != 1) return;
-    const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
-    sweep_M<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, bmat, bk, &a.st[t.c].status);
+    const int64_t q = t.begin + li, i = particle_at(a, q);
+    sweep_M<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, bmat, bk, &a.st[t.c].status, threadIdx.x % L);
 }
 
-template <typename T, int D, bool LIST>
+template <typename T, int D, bool LIST, int L = 1>
 __global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const V4<T> *vel, const T *vol,
                                            const V4<T> *bmat, V4<T> *acc_visc, V4<T> *pos) {
-    const Tile t = a.tiles[a.tile0 + blockIdx.x];
-    if ((int)threadIdx.x >= t.n || !a.st[t.c].active) return;
+    const Tile t = work_tile<L, false>(a, blockIdx.x);
+    const int li = local_index<L>(blockIdx.x);
+    if (li >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
-    const int64_t q = t.begin + threadIdx.x, i = particle_at(a, q);
-    sweep_V<LIST, T, D>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vel, vol, bmat, acc_visc, pos,
-                        &a.st[t.c].status);
+    const int64_t q = t.begin + li, i = particle_at(a, q);
+    sweep_V<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vel, vol, bmat, acc_visc, pos,
+                        &a.st[t.c].status, threadIdx.x % L);
 }
 
 // Sweeps B and C (and A with the cell walk) take L lanes per particle (L = 1,
@@ -1845,9 +1991,6 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const
 // group walks every L-th list entry.  local_index gives the particle's index
 // within its tile.  Sweeps S and A of the list classes do the same per entry
 // of their band list.
-template <int L> __device__ __forceinline__ int local_index(int64_t w) {
-    return L == 1 ? (int)threadIdx.x : (int)((w % L) * (blockDim.x / L) + threadIdx.x / L);
-}
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
 __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, const T *vol, V4<T> *gradC) {
@@ -1918,7 +2061,7 @@ __device__ __forceinline__ void reduce_vmax(const SweepArgs &a, int c, uint32_t 
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
-__global__ void SPH_SWEEPB_BOUNDS_M(T, MODE) k_sweep_B(SweepArgs a, const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
+__global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, MODE) k_sweep_B(SweepArgs a, const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
                                             const V4<T> *gradC, const V4<T> *acc_visc, V4<T> *acc_surf,
                                             V4<T> *vel_new, const V4<T> *bk, const T *vol) {
     const auto item = [&](int64_t w) {
