@@ -28,10 +28,10 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         const SweepArgs a_ = fluid_args(k_);                                           \
         const unsigned g_ = (unsigned)cls_fn[k_];                                      \
         switch (k_) {                                                                  \
-        case 0: KERN<T, 3, true><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;    \
-        case 1: KERN<T, 2, true><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;    \
-        case 2: KERN<T, 3, false, CELL_LANES><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break;   \
-        default: KERN<T, 2, false, CELL_LANES><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break;  \
+        case 0: launch_next(KERN<T, 3, true>, g_, block, 0, stream, a_, __VA_ARGS__); break;    \
+        case 1: launch_next(KERN<T, 2, true>, g_, block, 0, stream, a_, __VA_ARGS__); break;    \
+        case 2: launch_next(KERN<T, 3, false, CELL_LANES>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break;   \
+        default: launch_next(KERN<T, 2, false, CELL_LANES>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break;  \
         }                                                                              \
     }
 
@@ -40,10 +40,10 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
 // the work-list kernels of a batch, MODE_ONE and MODE_FEW for a one-case engine)
 #define SPH_LANES_M(KERN, D, LN, MODE, ...)                                                             \
     switch (LN) {                                                                                       \
-    case 2: KERN<T, D, true, 2, MODE><<<g_ * 2, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
-    case 4: KERN<T, D, true, 4, MODE><<<g_ * 4, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
-    case 8: KERN<T, D, true, 8, MODE><<<g_ * 8, block, 0, stream>>>(a_, __VA_ARGS__); break;            \
-    default: KERN<T, D, true, 1, MODE><<<g_, block, 0, stream>>>(a_, __VA_ARGS__); break;               \
+    case 2: launch_next(KERN<T, D, true, 2, MODE>, g_ * 2, block, 0, stream, a_, __VA_ARGS__); break;            \
+    case 4: launch_next(KERN<T, D, true, 4, MODE>, g_ * 4, block, 0, stream, a_, __VA_ARGS__); break;            \
+    case 8: launch_next(KERN<T, D, true, 8, MODE>, g_ * 8, block, 0, stream, a_, __VA_ARGS__); break;            \
+    default: launch_next(KERN<T, D, true, 1, MODE>, g_, block, 0, stream, a_, __VA_ARGS__); break;               \
     }
 // SPH_CLASSES_LF: the per-substep sweeps over slots from class K0 on, whose
 // blocks stride over the work list of active tiles in a batch (the grid is then
@@ -71,8 +71,8 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         switch (k_) {                                                                                  \
         case 0: SPH_LANES_M(KERN, 3, LN, MODE, __VA_ARGS__) break;                                     \
         case 1: SPH_LANES_M(KERN, 2, LN, MODE, __VA_ARGS__) break;                                     \
-        case 2: KERN<T, 3, false, CELL_LANES, CELL_MODE(MODE)><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break; \
-        default: KERN<T, 2, false, CELL_LANES, CELL_MODE(MODE)><<<g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream>>>(a_, __VA_ARGS__); break;\
+        case 2: launch_next(KERN<T, 3, false, CELL_LANES, CELL_MODE(MODE)>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break; \
+        default: launch_next(KERN<T, 2, false, CELL_LANES, CELL_MODE(MODE)>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break;\
         }                                                                                              \
     }
 
@@ -463,19 +463,19 @@ template <typename T> struct EngineT : Engine {
     // list the active cases' tiles (after the criterion kernel of a substep)
     void launch_work_lists() {
         if (!use_work) return;
-        k_work_scan<<<1, 1024, 0, stream>>>(ncases, d_cls_of, d_ftn, d_state, d_woff, d_wcount);
-        k_work_fill<<<(unsigned)((n_ftiles + 255) / 256), 256, 0, stream>>>(n_ftiles, d_ftiles, d_ft_first, d_cls0,
+        launch_next(k_work_scan, 1, 1024, 0, stream, ncases, d_cls_of, d_ftn, d_state, d_woff, d_wcount);
+        launch_next(k_work_fill, (unsigned)((n_ftiles + 255) / 256), 256, 0, stream, n_ftiles, d_ftiles, d_ft_first, d_cls0,
                                                                           d_cls_of, d_woff, d_state, d_work);
     }
     // fluid ranks of the reordered particles (after the gather)
     void launch_fluid_ranks() {
         const int64_t np1 = n + 1;
         const unsigned nbp = (unsigned)((np1 + SCAN_ITEMS - 1) / SCAN_ITEMS);
-        k_fluid_flag<T><<<(unsigned)((np1 + 255) / 256), 256, 0, stream>>>(n, snap, fscan);
-        k_scan_reduce<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
-        k_scan_blocks<<<1, SCAN_T, 0, stream>>>(block_sums, nbp);
-        k_scan_apply<<<nbp, SCAN_T, 0, stream>>>(fscan, np1, block_sums);
-        k_fluid_scatter<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, snap, fscan, drho, vol, fidx, gradC, band, cell_list,
+        launch_next(k_fluid_flag<T>, (unsigned)((np1 + 255) / 256), 256, 0, stream, n, snap, fscan, band_count);
+        launch_next(k_scan_reduce, nbp, SCAN_T, 0, stream, fscan, np1, block_sums);
+        launch_next(k_scan_blocks, 1, SCAN_T, 0, stream, block_sums, nbp);
+        launch_next(k_scan_apply, nbp, SCAN_T, 0, stream, fscan, np1, block_sums);
+        launch_next(k_fluid_scatter<T>, (unsigned)n_tiles, block, 0, stream, d_tiles, d_desc, snap, fscan, drho, vol, fidx, gradC, band, cell_list,
                                                                    cell_count, band_base[1]);
     }
     // neighbour lists: a block per cell, as many blocks as fit the GPU striding
@@ -484,7 +484,7 @@ template <typename T> struct EngineT : Engine {
     template <int D> void launch_list(int k) {
         if (!cls_fn[k]) return;
         const unsigned g = (unsigned)std::min<int64_t>(lb_blocks[k], cls_fn[k] * block);
-        k_build_list<T, D><<<g, LB_WARPS * 32, 0, stream>>>(fluid_args(k), cell_list + band_base[k], cell_count + k, fscan, snap,
+        launch_next(k_build_list<T, D>, g, LB_WARPS * 32, 0, stream, fluid_args(k), cell_list + band_base[k], cell_count + k, fscan, snap,
                                                             nbr, nbr_cnt, band);
     }
     void launch_lists() {
@@ -492,14 +492,14 @@ template <typename T> struct EngineT : Engine {
         launch_list<2>(1);
         if constexpr (sizeof(T) == 8) {
             const dim3 b(32, LG_WARPS);
-            if (lgeo && cls_fn[0]) k_list_geo<3><<<(unsigned)cls_fn[0], b, 0, stream>>>(fluid_args(0), snap, lgeo, lrinv);
-            if (lgeo && cls_fn[1]) k_list_geo<2><<<(unsigned)cls_fn[1], b, 0, stream>>>(fluid_args(1), snap, lgeo, lrinv);
+            if (lgeo && cls_fn[0]) launch_next(k_list_geo<3>, (unsigned)cls_fn[0], b, 0, stream, fluid_args(0), snap, lgeo, lrinv);
+            if (lgeo && cls_fn[1]) launch_next(k_list_geo<2>, (unsigned)cls_fn[1], b, 0, stream, fluid_args(1), snap, lgeo, lrinv);
         }
     }
     void launch_band() {
         for (int k = 0; k < 2; ++k)
             if (cls_fn[k])
-                k_band<<<(unsigned)cls_fn[k], block, 0, stream>>>(fluid_args(k), band, band_list + band_base[k], band_count + k);
+                launch_next(k_band, (unsigned)cls_fn[k], block, 0, stream, fluid_args(k), band, band_list + band_base[k], band_count + k);
     }
     // correction matrices, viscous force and transport shift
     void launch_setup() {
@@ -512,9 +512,9 @@ template <typename T> struct EngineT : Engine {
         const unsigned g = (unsigned)(band_grid(cls_fn[k], L) * L);
         const uint64_t *bl = band_list + band_base[k];
         if (surface)
-            k_sweep_S<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, band, snap, vel, gradC, acc_surf, bk, vol);
+            launch_next(k_sweep_S<T, D, L>, g, block, 0, stream, fluid_args(k), bl, band_count + k, band, snap, vel, gradC, acc_surf, bk, vol);
         else
-            k_sweep_A_band<T, D, L><<<g, block, 0, stream>>>(fluid_args(k), bl, band_count + k, snap, vol, gradC);
+            launch_next(k_sweep_A_band<T, D, L>, g, block, 0, stream, fluid_args(k), bl, band_count + k, snap, vol, gradC);
     }
     template <int D> void launch_band_class(int k, bool surface) {
         if (!cls_fn[k]) return;
@@ -543,19 +543,18 @@ template <typename T> struct EngineT : Engine {
         const int pgrid = (int)((n + nthr - 1) / nthr);
         SPH_CK(cudaMemsetAsync(starts, 0, (size_t)(table_total + 1) * 4, stream));
         k_reset_vmax<<<cgrid, 128, 0, stream>>>(ncases, d_state);
-        k_vmax<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, d_state, pos, vel);
-        k_adv_begin<<<cgrid, 128, 0, stream>>>(ncases, d_desc, d_state);
-        k_cell_assign<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, d_state, pos, key, rank, starts);
+        launch_next(k_vmax<T>, (unsigned)n_tiles, block, 0, stream, d_tiles, d_desc, d_state, pos, vel);
+        launch_next(k_adv_begin, cgrid, 128, 0, stream, ncases, d_desc, d_state);
+        launch_next(k_cell_assign<T>, (unsigned)n_tiles, block, 0, stream, d_tiles, d_desc, d_state, pos, key, rank, starts);
         const int64_t ns = table_total + 1;
         const unsigned nb = (unsigned)((ns + SCAN_ITEMS - 1) / SCAN_ITEMS);
-        k_scan_reduce<<<nb, SCAN_T, 0, stream>>>(starts, ns, block_sums);
-        k_scan_blocks<<<1, SCAN_T, 0, stream>>>(block_sums, nb);
-        k_scan_apply<<<nb, SCAN_T, 0, stream>>>(starts, ns, block_sums);
-        k_scatter<<<pgrid, nthr, 0, stream>>>(n, key, rank, starts, perm);
-        k_cell_sort<<<(unsigned)((table_total + nthr - 1) / nthr), nthr, 0, stream>>>(table_total, starts, id, perm);
-        k_gather<T><<<pgrid, nthr, 0, stream>>>(n, perm, pos, vel, drho, id, snap, vel_new, drho_old, rank);
-        k_copy_back<T><<<pgrid, nthr, 0, stream>>>(n, snap, vel_new, drho_old, rank, pos, vel, drho, id);
-        SPH_CK(cudaMemsetAsync(band_count, 0, 4 * sizeof(uint32_t), stream));   // band and cell lists
+        launch_next(k_scan_reduce, nb, SCAN_T, 0, stream, starts, ns, block_sums);
+        launch_next(k_scan_blocks, 1, SCAN_T, 0, stream, block_sums, nb);
+        launch_next(k_scan_apply, nb, SCAN_T, 0, stream, starts, ns, block_sums);
+        launch_next(k_scatter, pgrid, nthr, 0, stream, n, key, rank, starts, perm);
+        launch_next(k_cell_sort, (unsigned)((table_total + nthr - 1) / nthr), nthr, 0, stream, table_total, starts, id, perm);
+        launch_next(k_gather<T>, pgrid, nthr, 0, stream, n, perm, pos, vel, drho, id, snap, vel_new, drho_old, rank);
+        launch_next(k_copy_back<T>, pgrid, nthr, 0, stream, n, snap, vel_new, drho_old, rank, pos, vel, drho, id);
         launch_fluid_ranks();
         launch_lists();
         launch_band();
@@ -682,22 +681,21 @@ template <typename T> struct EngineT : Engine {
         const int ncls = n_classes(4), nlist = n_classes(2);
         timed(1, 3, [&] {
             k_reset_vmax<<<cgrid, 128, 0, stream>>>(ncases, d_state);
-            k_vmax<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, d_state, pos, vel);
-            k_adv_begin<<<cgrid, 128, 0, stream>>>(ncases, d_desc, d_state);
+            launch_next(k_vmax<T>, (unsigned)n_tiles, block, 0, stream, d_tiles, d_desc, d_state, pos, vel);
+            launch_next(k_adv_begin, cgrid, 128, 0, stream, ncases, d_desc, d_state);
         });
         timed(0, 8, [&] {
             cudaMemsetAsync(starts, 0, (size_t)ns * 4, stream);
             k_cell_assign<T><<<(unsigned)n_tiles, block, 0, stream>>>(d_tiles, d_desc, d_state, pos, key, rank, starts);
-            k_scan_reduce<<<nb, SCAN_T, 0, stream>>>(starts, ns, block_sums);
-            k_scan_blocks<<<1, SCAN_T, 0, stream>>>(block_sums, nb);
-            k_scan_apply<<<nb, SCAN_T, 0, stream>>>(starts, ns, block_sums);
-            k_scatter<<<pgrid, nthr, 0, stream>>>(n, key, rank, starts, perm);
-            k_cell_sort<<<(unsigned)((table_total + nthr - 1) / nthr), nthr, 0, stream>>>(table_total, starts, id, perm);
-            k_gather<T><<<pgrid, nthr, 0, stream>>>(n, perm, pos, vel, drho, id, snap, vel_new, drho_old, rank);
-            k_copy_back<T><<<pgrid, nthr, 0, stream>>>(n, snap, vel_new, drho_old, rank, pos, vel, drho, id);
+            launch_next(k_scan_reduce, nb, SCAN_T, 0, stream, starts, ns, block_sums);
+            launch_next(k_scan_blocks, 1, SCAN_T, 0, stream, block_sums, nb);
+            launch_next(k_scan_apply, nb, SCAN_T, 0, stream, starts, ns, block_sums);
+            launch_next(k_scatter, pgrid, nthr, 0, stream, n, key, rank, starts, perm);
+            launch_next(k_cell_sort, (unsigned)((table_total + nthr - 1) / nthr), nthr, 0, stream, table_total, starts, id, perm);
+            launch_next(k_gather<T>, pgrid, nthr, 0, stream, n, perm, pos, vel, drho, id, snap, vel_new, drho_old, rank);
+            launch_next(k_copy_back<T>, pgrid, nthr, 0, stream, n, snap, vel_new, drho_old, rank, pos, vel, drho, id);
         });
         timed(0, 5, [&] {
-            cudaMemsetAsync(band_count, 0, 4 * sizeof(uint32_t), stream);
             launch_fluid_ranks();
         });
         timed(0, 2 * nlist, [&] {

@@ -28,6 +28,8 @@
 // on that choice.
 #pragma once
 
+#include <utility>
+
 #include <cuda_runtime.h>
 #include "sphst_internal.cuh"
 
@@ -248,6 +250,36 @@ __device__ __forceinline__ bool wrap_cell(const CaseDesc &d, int a, int &c) {
     if (!((d.periodic >> a) & 1)) return false;
     c += c < 0 ? d.ncell[a] : -d.ncell[a];
     return true;
+}
+
+// First statement of every kernel of a step, which is launched while the one
+// before it still runs out (programmatic dependent launch): waits until that
+// one has finished and its writes are visible.  Nothing is read or written
+// before the wait, so a kernel that has finished had all before it finished.
+__device__ __forceinline__ void follow() { cudaGridDependencySynchronize(); }
+// In the kernels of one or a few blocks: the next kernel's blocks may take
+// their places at once.  Not in the others: blocks placed around a running
+// kernel's leave the SMs unevenly filled (in every kernel, FP64 2D 6k
+// particles 643 -> 817, 64k 1912 -> 2243 us a pass; in these alone 672 -> 542,
+// 1775 -> 1735).
+__device__ __forceinline__ void lead() { cudaTriggerProgrammaticLaunchCompletion(); }
+
+// Launches a kernel that starts with follow() behind the kernel before it in
+// the stream.  Plain launches against these: 2D 576 particles 319 -> 313 us a pass, FP64 2D 6k 643
+// -> 635, shear flow of 37k 499 -> 474, 1M 12.74 -> 12.66 ms.
+template <typename... P, typename... A>
+void launch_next(void (*kernel)(P...), unsigned grid, dim3 block, size_t shared, cudaStream_t stream, A &&...args) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = shared;
+    cfg.stream = stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);   // a failure stays for the caller's cudaGetLastError
 }
 
 // --------------------------------------------------------------- cell walk
@@ -792,6 +824,7 @@ template <typename T>
 __global__ void k_cell_assign(const Tile *__restrict__ tiles, const CaseDesc *__restrict__ desc,
                               CaseState *st, V4<T> *pos, uint32_t *key, uint32_t *rank,
                               uint32_t *counts) {
+    follow();
     const Tile t = tiles[blockIdx.x];
     if ((int)threadIdx.x >= t.n) return;
     const CaseDesc &d = desc[t.c];
@@ -832,6 +865,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *t
 }
 
 static __global__ void k_scan_reduce(const uint32_t *data, int64_t n, uint32_t *block_sums) {
+    follow();
     const int64_t base = (int64_t)blockIdx.x * SCAN_ITEMS + 2 * threadIdx.x;
     uint32_t v = 0;
     if (base < n) v += data[base];
@@ -842,6 +876,8 @@ static __global__ void k_scan_reduce(const uint32_t *data, int64_t n, uint32_t *
 }
 
 static __global__ void k_scan_blocks(uint32_t *block_sums, int64_t nb) {
+    lead();
+    follow();
     uint32_t carry = 0;
     for (int64_t base = 0; base < nb; base += SCAN_T) {
         const int64_t k = base + threadIdx.x;
@@ -854,6 +890,7 @@ static __global__ void k_scan_blocks(uint32_t *block_sums, int64_t nb) {
 }
 
 static __global__ void k_scan_apply(uint32_t *data, int64_t n, const uint32_t *block_sums) {
+    follow();
     const int64_t base = (int64_t)blockIdx.x * SCAN_ITEMS + 2 * threadIdx.x;
     const uint32_t a = base < n ? data[base] : 0u;
     const uint32_t b = base + 1 < n ? data[base + 1] : 0u;
@@ -865,6 +902,7 @@ static __global__ void k_scan_apply(uint32_t *data, int64_t n, const uint32_t *b
 
 static __global__ void k_scatter(int64_t n, const uint32_t *key, const uint32_t *rank,
                           const uint32_t *starts, uint32_t *perm) {
+    follow();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     perm[starts[key[i]] + rank[i]] = (uint32_t)i;
@@ -873,6 +911,7 @@ static __global__ void k_scatter(int64_t n, const uint32_t *key, const uint32_t 
 // canonical order inside each cell: ascending insertion index
 static __global__ void k_cell_sort(int64_t ncells, const uint32_t *starts, const uint32_t *id,
                             uint32_t *perm) {
+    follow();
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (c >= ncells) return;
     const uint32_t b = starts[c], e = starts[c + 1];
@@ -893,6 +932,7 @@ template <typename T>
 __global__ void k_gather(int64_t n, const uint32_t *perm, const V4<T> *pos, const V4<T> *vel,
                          const T *drho, const uint32_t *id, V4<T> *pos_t, V4<T> *vel_t,
                          T *drho_t, uint32_t *id_t) {
+    follow();
     const int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (d >= n) return;
     const uint32_t s = perm[d];
@@ -905,6 +945,7 @@ __global__ void k_gather(int64_t n, const uint32_t *perm, const V4<T> *pos, cons
 template <typename T>
 __global__ void k_copy_back(int64_t n, const V4<T> *pos_t, const V4<T> *vel_t, const T *drho_t,
                             const uint32_t *id_t, V4<T> *pos, V4<T> *vel, T *drho, uint32_t *id) {
+    follow();
     const int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (d >= n) return;
     pos[d] = pos_t[d];
@@ -934,7 +975,9 @@ __device__ __forceinline__ T volume_at(const CasePhys<T> &cp, uint32_t kj, const
 // a scatter.  Each case's fluid particles take the slots after the previous
 // cases' ones, whose count is fixed.
 template <typename T>
-__global__ void k_fluid_flag(int64_t n, const V4<T> *snap, uint32_t *flag) {
+__global__ void k_fluid_flag(int64_t n, const V4<T> *snap, uint32_t *flag, uint32_t *counts) {
+    follow();
+    if (blockIdx.x == 0 && threadIdx.x < 4) counts[threadIdx.x] = 0;   // of the band and cell lists
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i > n) return;
     flag[i] = (i < n && phase_of(w_bits(snap[i].w)) != PH_WALL) ? 1u : 0u;
@@ -953,6 +996,7 @@ template <typename T>
 __global__ void k_fluid_scatter(const Tile *__restrict__ tiles, const CaseDesc *__restrict__ desc, const V4<T> *snap,
                                 const uint32_t *rank, const T *drho, T *vol, uint32_t *fidx, V4<T> *gradC, uint8_t *band, uint64_t *clist,
                                 uint32_t *ccount, int64_t base2d) {
+    follow();
     const Tile t = tiles[blockIdx.x];
     const CaseDesc &d = desc[t.c];
     const int64_t i = t.begin + threadIdx.x;
@@ -986,6 +1030,8 @@ __global__ void k_fluid_scatter(const Tile *__restrict__ tiles, const CaseDesc *
 
 // ================================================================ time step
 static __global__ void k_reset_vmax(int ncases, CaseState *st) {
+    lead();
+    follow();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncases) return;
     st[c].vmax2_acc[0] = 0ull;
@@ -995,6 +1041,7 @@ static __global__ void k_reset_vmax(int ncases, CaseState *st) {
 template <typename T>
 __global__ void k_vmax(const Tile *__restrict__ tiles, const CaseDesc *__restrict__ desc,
                        CaseState *st, const V4<T> *pos, const V4<T> *vel) {
+    follow();
     const Tile t = tiles[blockIdx.x];
     const int dim = desc[t.c].dim;
     unsigned long long m[2] = {0ull, 0ull};
@@ -1014,6 +1061,8 @@ __global__ void k_vmax(const Tile *__restrict__ tiles, const CaseDesc *__restric
 // Eq. 16 per fluid (factor cfl_ad), Eq. 18 minimum; speed terms with
 // |v|max = 0 are dropped.
 static __global__ void k_adv_begin(int ncases, const CaseDesc *desc, CaseState *st) {
+    lead();
+    follow();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncases) return;
     const CaseDesc &d = desc[c];
@@ -1048,6 +1097,8 @@ static __global__ void k_adv_begin(int ncases, const CaseDesc *desc, CaseState *
 // still has a substep after this one".
 static __global__ void k_dt(int ncases, const CaseDesc *desc, CaseState *st, int *loop_flag,
                      cudaGraphConditionalHandle handle, int use_handle) {
+    lead();
+    follow();
     int more = 0;
     for (int c = threadIdx.x; c < ncases; c += blockDim.x) {
         const CaseDesc &d = desc[c];
@@ -1108,6 +1159,7 @@ static __global__ void k_dt(int ncases, const CaseDesc *desc, CaseState *st, int
 // closes the advection step of the cases that ended it in the final substep
 // (the others were closed by k_dt when they went idle)
 static __global__ void k_adv_end(int ncases, CaseState *st) {
+    follow();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncases) return;
     CaseState &s = st[c];
@@ -1902,6 +1954,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(LB_WARPS * 32) k_build_list(SweepArgs a, const uint64_t *clist, const uint32_t *ccount,
                                                               const uint32_t *rank, const V4<T> *snap,
                                                               uint32_t *nbr, uint32_t *cnt, uint8_t *band) {
+    follow();
     __shared__ ListSmem S;
     const uint32_t cells = *ccount;
     for (uint32_t e = blockIdx.x; e < cells; e += gridDim.x) {
@@ -1920,6 +1973,7 @@ __global__ void __launch_bounds__(LB_WARPS * 32) k_build_list(SweepArgs a, const
 // walk (warp-aggregated atomics; the order is irrelevant because every
 // particle's sum is its own).
 static __global__ void __launch_bounds__(256) k_band(SweepArgs a, const uint8_t *band, uint64_t *blist, uint32_t *bcount) {
+    follow();
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     const int64_t q = t.begin + threadIdx.x;
     const bool b = (int)threadIdx.x < t.n && a.st[t.c].active && band[particle_at(a, q)];
@@ -1940,6 +1994,7 @@ static __global__ void __launch_bounds__(256) k_band(SweepArgs a, const uint8_t 
 constexpr int LG_WARPS = 8;
 template <int D>
 __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V4<double> *snap, V4<double> *ge, RInv *gr) {
+    follow();
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     if (!a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
@@ -1964,6 +2019,7 @@ __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V
 template <typename T, int D, bool LIST, int L = 1>
 __global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const T *vol, V4<T> *bmat,
                                            V4<T> *bk) {
+    follow();
     const Tile t = work_tile<L, false>(a, blockIdx.x);
     const int li = local_index<L>(blockIdx.x);
     if (li >= t.n || !a.st[t.c].active) return;
@@ -1976,6 +2032,7 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const
 template <typename T, int D, bool LIST, int L = 1>
 __global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const V4<T> *vel, const T *vol,
                                            const V4<T> *bmat, V4<T> *acc_visc, V4<T> *pos) {
+    follow();
     const Tile t = work_tile<L, false>(a, blockIdx.x);
     const int li = local_index<L>(blockIdx.x);
     if (li >= t.n || !a.st[t.c].active) return;
@@ -1994,6 +2051,7 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
 __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, const T *vol, V4<T> *gradC) {
+    follow();
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         const int li = local_index<L>(w);
@@ -2020,6 +2078,7 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, con
 template <typename T, int D, int L = 1>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4) k_sweep_A_band(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
                                                 const V4<T> *snap, const T *vol, V4<T> *gradC) {
+    follow();
     const int64_t items = (int64_t)*bcount * L;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
         const BandEntry e(a, blist, t / L);
@@ -2037,6 +2096,7 @@ template <typename T, int D, int L = 1>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) k_sweep_S(SweepArgs a, const uint64_t *blist, const uint32_t *bcount,
                                            const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
                                            const V4<T> *gradC, V4<T> *acc_surf, const V4<T> *bk, const T *vol) {
+    follow();
     const int64_t items = (int64_t)*bcount * L;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (int64_t)gridDim.x * blockDim.x) {
         const BandEntry e(a, blist, t / L);
@@ -2064,6 +2124,7 @@ template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
 __global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, MODE) k_sweep_B(SweepArgs a, const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
                                             const V4<T> *gradC, const V4<T> *acc_visc, V4<T> *acc_surf,
                                             V4<T> *vel_new, const V4<T> *bk, const T *vol) {
+    follow();
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         if (!a.st[t.c].active) return;             // uniform per block
@@ -2091,6 +2152,7 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, MODE) k_sweep_B(SweepArgs a, const 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
 __global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho, T *vol,
                                            V4<T> *vel, V4<T> *pos) {
+    follow();
     const auto item = [&](int64_t w) {
         const Tile t = work_tile<L, MODE == MODE_WORK>(a, w);
         const int li = local_index<L>(w);
@@ -2119,6 +2181,8 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const
 // in the tile array and in the list alike.
 static __global__ void k_work_scan(int ncases, const int32_t *cls_of, const uint32_t *ftn, const CaseState *st,
                                    uint32_t *off, uint32_t *count) {
+    lead();
+    follow();
     uint32_t base[4] = {0u, 0u, 0u, 0u};
     for (int c0 = 0; c0 < ncases; c0 += (int)blockDim.x) {
         const int c = c0 + (int)threadIdx.x;
@@ -2137,6 +2201,7 @@ static __global__ void k_work_scan(int ncases, const int32_t *cls_of, const uint
 static __global__ void k_work_fill(int64_t n_ftiles, const Tile *ftiles, const int64_t *ft_first,
                                    const int64_t *cls0, const int32_t *cls_of, const uint32_t *off,
                                    const CaseState *st, uint32_t *work) {
+    follow();
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= n_ftiles) return;
     const int c = ftiles[t].c;

@@ -99,6 +99,7 @@ __global__ void na_zero(uint32_t *counts, int64_t m, uint32_t *flag) {
 template <int D>
 __global__ void na_keys(int64_t n, const double *pos, Grid g, uint32_t *counts, uint32_t *keys,
                         uint32_t *ranks, uint32_t *flag) {
+    follow();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     int cc[3] = {0, 0, 0};
@@ -118,6 +119,7 @@ __global__ void na_keys(int64_t n, const double *pos, Grid g, uint32_t *counts, 
 
 __global__ void na_scatter(int64_t n, const uint32_t *keys, const uint32_t *ranks,
                            const uint32_t *starts, uint32_t *perm) {
+    follow();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     perm[starts[keys[i]] + ranks[i]] = (uint32_t)i;
@@ -130,6 +132,7 @@ __global__ void na_scatter(int64_t n, const uint32_t *keys, const uint32_t *rank
 // so the work is bounded and no thread waits on another.
 __global__ void na_cell_rank(int64_t n, const uint32_t *keys, const uint32_t *starts,
                              const uint32_t *perm, uint32_t *order, uint32_t *flag) {
+    follow();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const uint32_t k = keys[i];
@@ -147,6 +150,7 @@ __global__ void na_cell_rank(int64_t n, const uint32_t *keys, const uint32_t *st
 // (its order entries were not filled)
 __global__ void na_output(int64_t n, const uint32_t *order, const uint32_t *keys, const uint32_t *flag,
                           unsigned long long *keys_out, long long *order_out) {
+    follow();
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n || (*flag & NA_FLAG_CROWDED)) return;
     const uint32_t i = order[k];
@@ -208,15 +212,15 @@ extern "C" int sphst_cell_order_noalloc(int32_t dim, int64_t n, const double *po
     const unsigned pgrid = (unsigned)((n + nthr - 1) / nthr);
     const unsigned nb = (unsigned)((ns + SCAN_ITEMS - 1) / SCAN_ITEMS);
     na_zero<<<(unsigned)std::min<int64_t>((ns + nthr - 1) / nthr, 4096), nthr, 0, st>>>(s.counts, ns, s.flag);
-    if (dim == 3) na_keys<3><<<pgrid, nthr, 0, st>>>(n, pos_dev, g, s.counts, s.keys, s.ranks, s.flag);
-    else na_keys<2><<<pgrid, nthr, 0, st>>>(n, pos_dev, g, s.counts, s.keys, s.ranks, s.flag);
-    k_scan_reduce<<<nb, SCAN_T, 0, st>>>(s.counts, ns, s.block_sums);
-    k_scan_blocks<<<1, SCAN_T, 0, st>>>(s.block_sums, nb);
-    k_scan_apply<<<nb, SCAN_T, 0, st>>>(s.counts, ns, s.block_sums);
-    na_scatter<<<pgrid, nthr, 0, st>>>(n, s.keys, s.ranks, s.counts, s.perm);
+    if (dim == 3) launch_next(na_keys<3>, pgrid, nthr, 0, st, n, pos_dev, g, s.counts, s.keys, s.ranks, s.flag);
+    else launch_next(na_keys<2>, pgrid, nthr, 0, st, n, pos_dev, g, s.counts, s.keys, s.ranks, s.flag);
+    launch_next(k_scan_reduce, nb, SCAN_T, 0, st, s.counts, ns, s.block_sums);
+    launch_next(k_scan_blocks, 1, SCAN_T, 0, st, s.block_sums, nb);
+    launch_next(k_scan_apply, nb, SCAN_T, 0, st, s.counts, ns, s.block_sums);
+    launch_next(na_scatter, pgrid, nthr, 0, st, n, s.keys, s.ranks, s.counts, s.perm);
     // the ranks are not needed after the scatter: their words take the final order
-    na_cell_rank<<<pgrid, nthr, 0, st>>>(n, s.keys, s.counts, s.perm, s.ranks, s.flag);
-    na_output<<<pgrid, nthr, 0, st>>>(n, s.ranks, s.keys, s.flag, (unsigned long long *)keys_dev,
+    launch_next(na_cell_rank, pgrid, nthr, 0, st, n, s.keys, s.counts, s.perm, s.ranks, s.flag);
+    launch_next(na_output, pgrid, nthr, 0, st, n, s.ranks, s.keys, s.flag, (unsigned long long *)keys_dev,
                                       (long long *)order_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "launch of the cell-order kernels");
