@@ -111,13 +111,23 @@ int make_grid(CaseRec *c) {
     return SPHST_OK;
 }
 
+// Exponent e of the unit 2^e in which a case's volumes and masses are kept: 0,
+// or, where kcoef_h ~ 1 / h^(dim + 2) would leave the type's range (FP32: 3D
+// spacings below 1e-6), the power of two that brings it to the range's inner
+// part.  The sums hold kcoef_h and a volume or a mass as one product, so the
+// unit cancels and, being a power of two, changes no bit.
+template <typename T> static int volume_exponent(int kcoef_exponent) {
+    const int room = sizeof(T) == 4 ? 100 : 800;
+    return kcoef_exponent > room ? room - kcoef_exponent : kcoef_exponent < -room ? -room - kcoef_exponent : 0;
+}
+
 template <typename T> static CasePhys<T> phys_of(const CaseRec *c) {
     const sphst_case_params &P = c->P;
     const int dim = P.dim;
     const double h = P.h_factor * P.dx;
     const double pi = 3.14159265358979323846;
     const double alpha = dim == 2 ? 7.0 / (4.0 * pi * h * h) : 21.0 / (16.0 * pi * h * h * h);
-    const double vol = dim == 2 ? P.dx * P.dx : P.dx * P.dx * P.dx;
+    const double volume = dim == 2 ? P.dx * P.dx : P.dx * P.dx * P.dx;
     double xi = P.xi;
     if (xi < 0.0) {
         if (c->n_fluid_phases == 2) {
@@ -134,7 +144,12 @@ template <typename T> static CasePhys<T> phys_of(const CaseRec *c) {
     p.four_h2 = (T)((2.0 * h) * (2.0 * h));
     p.kcoef = (T)(-5.0 * alpha / h);
     p.mhalf_inv_h = (T)(-0.5 / h);
-    p.kcoef_h = (T)(-5.0 * alpha / h / h);
+    // kcoef / h as fraction and exponent: 1 / h^(dim + 2) may leave even FP64
+    int ek = 0, eh = 0;
+    const double fk = std::frexp(-5.0 * alpha / h, &ek) / std::frexp(h, &eh);
+    const int ev = volume_exponent<T>(ek - eh);
+    const double vol = std::ldexp(volume, -ev);
+    p.kcoef_h = (T)std::ldexp(fk, ek - eh + ev);
     p.cs = (T)cell_width(c);
     p.c0 = (T)P.c0;
     p.c0sq = (T)(P.c0 * P.c0);
@@ -180,7 +195,8 @@ CaseDesc make_desc(const CaseRec *c) {
     d.h = c->P.h_factor * c->P.dx;
     d.c0 = c->P.c0;
     d.gamma = c->P.gamma;
-    for (int k = 0; k < 2; ++k) { d.rho0[k] = c->rho0[k]; d.eta[k] = c->eta[k]; }
+    const double volume = c->P.dim == 2 ? c->P.dx * c->P.dx : c->P.dx * c->P.dx * c->P.dx;
+    for (int k = 0; k < 2; ++k) { d.rho0[k] = c->rho0[k]; d.eta[k] = c->eta[k]; d.mass[k] = c->rho0[k] * volume; }
     d.max_substeps = c->P.max_substeps > 0 ? c->P.max_substeps : 1000000;
     d.cfl_ad = c->P.cfl_ad;
     d.cfl_ac = c->P.cfl_ac;

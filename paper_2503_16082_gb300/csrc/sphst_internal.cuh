@@ -81,6 +81,8 @@ template <typename T> struct CasePhys {
     T vol_wall;                // dp^dim
     T mhalf_inv_h, kcoef_h;    // -1 / (2h); kcoef / h: W'/r = kcoef_h (1 - q/2)^3
     T mass_c0[2], c0_vol;      // m c0 per fluid; c0 dp^dim
+    // (volumes and masses in a unit that kcoef_h is the reciprocal of: 1, or a
+    // power of two where 1 would take kcoef_h out of the type's range)
     T nhat_eps;                // |gradC| h threshold of an interface particle
     T tvf_coef;                // -alpha h^2 (Eq. 14, sign reading)
     T beta_k, beta_lo, beta_hi; // Eq. 11 limiter as min(max(beta_k dU, lo), hi) per reading
@@ -106,7 +108,7 @@ struct CaseDesc {
     double origin[3];
     double cs;
     double h, c0, gamma;
-    double rho0[2], eta[2];
+    double rho0[2], eta[2], mass[2];
     int64_t max_substeps;
     double cfl_ad, cfl_ac;
     double dt_surf[2];         // the surface-tension bound of Eq. 17 per fluid (0: none)

@@ -2247,7 +2247,7 @@ __global__ void __launch_bounds__(256) k_diag_partial(const CaseDesc *desc, int 
         const V4<T> v4 = vel[i];
         const double v[3] = {(double)v4.x, (double)v4.y, dim == 3 ? (double)v4.z : 0.0};
         const double dr = (double)drho[i];
-        const double m = d.pd.mass[ph];
+        const double m = d.mass[ph];
         const bool finite = isfinite(x[0]) && isfinite(x[1]) && isfinite(x[2]) && isfinite(v[0]) &&
                             isfinite(v[1]) && isfinite(v[2]) && isfinite(dr);
         if (!finite) { q[19] += 1.0; continue; }

@@ -1,0 +1,46 @@
+"""A case does not know its unit of length.  Scaled by a power of two (with
+c0, velocities, viscosity and surface tension to match, time unchanged) every
+operation scales exactly, so the results are the same bits after scaling back,
+as long as nothing leaves the type's range.  The scales below keep h within
+the range of the kernel's constants (FP32: -5 alpha_d / h finite in 3D down to
+h = 2.8e-10, in 2D down to 2e-13); densities are scaled by the reciprocal, so
+that products of two viscosities stay normal numbers too."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import sphcases
+
+pytestmark = pytest.mark.gpu
+
+S = pytest.importorskip("paper_2503_16082_gb300")
+
+
+def scaled(case, s):
+    phases = [dataclasses.replace(p, pos=p.pos * s, rho0=p.rho0 / s, eta=p.eta * s, vel=None if p.vel is None else p.vel * s)
+              for p in case.phases]
+    return dataclasses.replace(case, lo=[x * s for x in case.lo], hi=[x * s for x in case.hi], dx=case.dx * s,
+                               c0=case.c0 * s, gamma=case.gamma * s**2, phases=phases)
+
+
+def fields(case, precision, s, **kw):
+    h = S.case_from_spec(scaled(case, s), precision=precision, **kw)
+    info = S.step(h, 2, check=False)
+    unit = {S.FIELD_POS: s, S.FIELD_VEL: s, S.FIELD_RHO: 1.0 / s, S.FIELD_GRADC: 1.0 / s, S.FIELD_ACC_VISC: s}
+    out = [S.read_fields(h, f, case.dim) / u for f, u in unit.items()]
+    q = S.diagnose(h, center=[0.5 * s] * case.dim)
+    out.append(np.array(q["momentum"]) / s**case.dim)
+    S.destroy(h)
+    return info["rc"], info["n_sub"], out
+
+
+@pytest.mark.parametrize("dim,precision,exponent", [(3, 32, -28), (2, 32, -36), (3, 32, 20), (3, 64, -50)])
+@pytest.mark.parametrize("nbr_mode", [S.NBR_LIST, S.NBR_CELLS])
+def test_the_bits_do_not_follow_the_unit_of_length(dim, precision, exponent, nbr_mode):
+    case = sphcases.small_droplet(dim, 20 if dim == 2 else 12, seed=2, jitter=0.1, vel_amp=0.02)
+    rc0, n0, a = fields(case, precision, 1.0, nbr_mode=nbr_mode)
+    rc1, n1, b = fields(case, precision, 2.0**exponent, nbr_mode=nbr_mode)
+    assert (rc0, rc1) == (S.OK, S.OK) and n0 == n1
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
