@@ -212,6 +212,7 @@ CaseDesc make_desc(const CaseRec *c) {
     d.vstar_printed = c->P.vstar_form == SPHST_VSTAR_PRINTED;
     for (int a = 0; a < 3; ++a)
         d.period_len[a] = ((c->P.periodic >> a) & 1) ? c->P.period_hi[a] - c->P.period_lo[a] : 0.0;
+    d.list_unit = std::ldexp(1.0, -std::ilogb(c->cs));
     d.nbr_k = c->P.max_neighbors > 0 ? c->P.max_neighbors : (c->P.dim == 3 ? 128 : 48);
     d.pf = phys_of<float>(c);
     d.pd = phys_of<double>(c);

@@ -116,6 +116,7 @@ struct CaseDesc {
     int32_t nbr_k;             // list capacity per particle
     int64_t nbr_base;          // first list word of this case
     int64_t f_begin;           // first slot of this case
+    double list_unit;          // power of two that brings cs into [1, 2) (FP32 test of the FP64 list build)
     CasePhys<float> pf;
     CasePhys<double> pd;
 };

@@ -31,6 +31,7 @@
 #include <utility>
 
 #include <cuda_runtime.h>
+#include <math_constants.h>
 #include "sphst_internal.cuh"
 
 // Tuning switches of the pair sweeps (compile-time):
@@ -1760,17 +1761,23 @@ __device__ __forceinline__ uint32_t list_keep(uint32_t *row, int at, int step, u
     return kept;
 }
 
+// a coordinate as the test in FP32 takes it: FP64 coordinates in the unit
+// list_unit, so that they and their squares lie within FP32 whatever the
+// case's unit of length is
+__device__ __forceinline__ float list_coord(float x, float) { return x; }
+__device__ __forceinline__ float list_coord(double x, double unit) { return (float)(x * unit); }
+
 // tests nc staged candidates (a multiple of 32) against slot i and appends the
 // hits to its shared list.  EXACT: what the test keeps is tested again by the
 // cell walk's operations.  Returns this lane's number of zero distances
 // (FP32; the FP64 and EXACT tests see to those themselves).
 template <typename T, int D, bool MIXED, bool EXACT>
 __device__ __forceinline__ int list_scan(const ListSmem &S, uint32_t *row, int K, int nc, const CasePhys<T> &cp,
-                                         const V4<T> &si, uint32_t i, uint32_t ki, float R2, const V4<T> *snap,
+                                         const V4<T> &si, T unit, uint32_t i, uint32_t ki, float R2, const V4<T> *snap,
                                          uint32_t &c_rest, uint32_t &c_other, bool &coinc) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    const float sx = (float)si.x, sy = (float)si.y, sz = (float)si.z;
+    const float sx = list_coord(si.x, unit), sy = list_coord(si.y, unit), sz = list_coord(si.z, unit);
     int zero = 0;
     uint32_t cr = c_rest, co = c_other;
 #pragma unroll 3
@@ -1850,7 +1857,8 @@ __device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> 
     const uint32_t total = S.pre[32];
     // coordinates lie within 2 cells of the origin, so in FP32 r^2 is wrong by
     // less than 1.2e-6 of (2h)^2: 2e-6 more keeps every neighbour
-    const float R2 = (float)cp.four_h2, R2w = R2 * 1.000002f;
+    const T unit = sizeof(T) == 8 ? (T)d.list_unit : T(1);
+    const float R2 = (float)(cp.four_h2 * unit * unit), R2w = R2 * 1.000002f;
     bool coinc = false, overflow = false, has0 = false, has1 = false;
     for (uint32_t g0 = f0; g0 < f1; g0 += G) {
         const int ns = (int)min((uint32_t)G, f1 - g0);
@@ -1866,7 +1874,7 @@ __device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> 
                 bool p0 = false, p1 = false;
                 for (int q = threadIdx.x; q < nc; q += LB_WARPS * 32) {
                     const uint32_t t = c0 + q;
-                    float4 s = make_float4(1e18f, 1e18f, 1e18f, 0.0f);   // beyond every slot
+                    float4 s = make_float4(CUDART_NAN_F, CUDART_NAN_F, CUDART_NAN_F, 0.0f);   // near no slot
                     uint32_t pj = PH_WALL;
                     if (t < total) {
                         int cell = 0;
@@ -1876,9 +1884,9 @@ __device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> 
                         const uint32_t j = S.begin[cell] + (t - S.pre[cell]), cj = S.code[cell];
                         const V4<T> sj = ld4(snap + j);
                         pj = phase_of(w_bits(sj.w));
-                        s.x = (float)fma_rn(code_off(cj & 3u, T()), cp.cs, sj.x);
-                        s.y = (float)fma_rn(code_off((cj >> 2) & 3u, T()), cp.cs, sj.y);
-                        if (D == 3) s.z = (float)fma_rn(code_off((cj >> 4) & 3u, T()), cp.cs, sj.z);
+                        s.x = list_coord(fma_rn(code_off(cj & 3u, T()), cp.cs, sj.x), unit);
+                        s.y = list_coord(fma_rn(code_off((cj >> 2) & 3u, T()), cp.cs, sj.y), unit);
+                        if (D == 3) s.z = list_coord(fma_rn(code_off((cj >> 4) & 3u, T()), cp.cs, sj.z), unit);
                         s.w = __uint_as_float((j << NBR_SHIFT) | cj);
                     }
                     S.cand[q] = s;
@@ -1899,11 +1907,11 @@ __device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> 
                 uint32_t cr = r0, co = o0;
                 uint32_t *row = S.list + s * LS;
                 if (exact) {
-                    list_scan<T, D, true, true>(S, row, K, nc, cp, si, i, ki, R2w, snap, cr, co, coinc);
+                    list_scan<T, D, true, true>(S, row, K, nc, cp, si, unit, i, ki, R2w, snap, cr, co, coinc);
                 } else {
                     const float r2max = sizeof(T) == 8 ? R2w : R2;
-                    int zero = mixed ? list_scan<T, D, true, false>(S, row, K, nc, cp, si, i, ki, r2max, snap, cr, co, coinc)
-                                     : list_scan<T, D, false, false>(S, row, K, nc, cp, si, i, ki, r2max, snap, cr, co, coinc);
+                    int zero = mixed ? list_scan<T, D, true, false>(S, row, K, nc, cp, si, unit, i, ki, r2max, snap, cr, co, coinc)
+                                     : list_scan<T, D, false, false>(S, row, K, nc, cp, si, unit, i, ki, r2max, snap, cr, co, coinc);
                     if (sizeof(T) == 4) {
                         // one zero distance is the particle's own, when it is among these candidates
                         const uint32_t own = S.own + (i - b);

@@ -44,3 +44,16 @@ def test_the_bits_do_not_follow_the_unit_of_length(dim, precision, exponent, nbr
     assert (rc0, rc1) == (S.OK, S.OK) and n0 == n1
     for x, y in zip(a, b):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("exponent", [-100, 62, 100])
+def test_fp64_lists_hold_beyond_the_range_of_fp32(dim, exponent):
+    # the list build tests candidates in FP32 first: lengths whose squares
+    # FP32 cannot hold, and lengths around 1e18
+    case = sphcases.small_droplet(dim, 20 if dim == 2 else 12, seed=2, jitter=0.1, vel_amp=0.02)
+    rc0, n0, a = fields(case, 64, 1.0)
+    rc1, n1, b = fields(case, 64, 2.0**exponent)
+    assert (rc0, rc1) == (S.OK, S.OK) and n0 == n1
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
