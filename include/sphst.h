@@ -282,6 +282,15 @@ int sphst_debug_keys(sphst_case c, uint64_t *keys, int64_t *ids, int64_t capacit
  * in insertion order (walls included). */
 int sphst_debug_neighbor_counts(sphst_case c, int32_t *counts, int64_t capacity);
 
+/* Neighbours of each fluid particle at the last rebuild as the sweeps of the
+ * last step found them: the case's neighbour lists, or the buffered cell walk
+ * (sphst_debug_neighbor_counts counts by a plain walk of its own, walls too).
+ * In insertion order: counts[i], and the insertion indices of the first
+ * `width` (0..65535) of them in ids[i * width ...], -1 beyond (walls: 0 and
+ * -1).  capacity counts particles.  Errors: STATE (the case has failed, or
+ * has not been stepped, alone or in its present batch), CAPACITY, CUDA. */
+int sphst_debug_neighbors(sphst_case c, int64_t width, int32_t *counts, int64_t *ids, int64_t capacity);
+
 /* Run the case's kernels on the caller's CUDA stream (a cudaStream_t passed
  * as void*, e.g. torch.cuda.current_stream().cuda_stream) instead of a
  * library-owned stream.  Must be called before the first step; NULL keeps

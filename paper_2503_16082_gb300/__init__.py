@@ -103,6 +103,7 @@ EXPORTS = {
     "sphst_debug_grid": (C.c_int, [C.c_void_p, C.c_void_p, C.POINTER(C.c_double), C.c_void_p]),
     "sphst_debug_keys": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64]),
     "sphst_debug_neighbor_counts": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64]),
+    "sphst_debug_neighbors": (C.c_int, [C.c_void_p, C.c_int64, C.c_void_p, C.c_void_p, C.c_int64]),
     "sphst_set_stream": (C.c_int, [C.c_void_p, C.c_void_p]),
     "sphst_profile_step": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p]),
     "sphst_cell_order_noalloc": (C.c_int, [C.c_int32, C.c_int64, C.c_void_p, C.c_void_p, C.c_double,
@@ -256,6 +257,16 @@ def debug_neighbor_counts(case):
     cnt = np.zeros(max(n, 1), dtype=np.int32)
     _check(load().sphst_debug_neighbor_counts(case, cnt.ctypes.data, n), "debug_neighbor_counts")
     return cnt[:n]
+
+
+def debug_neighbors(case, width: int = 0):
+    """(counts, ids) of the fluid particles' neighbours as the sweeps find
+    them: ids (n, width) holds the first `width` insertion indices, -1 beyond."""
+    n, _ = num_particles(case)
+    cnt = np.zeros(max(n, 1), dtype=np.int32)
+    ids = np.full((max(n, 1), width), -1, dtype=np.int64)
+    _check(load().sphst_debug_neighbors(case, width, cnt.ctypes.data, ids.ctypes.data, n), "debug_neighbors")
+    return cnt[:n], ids[:n]
 
 
 def diagnose(case, center=(0.0, 0.0, 0.0), r_in: float = 0.0, r_out: float = float("inf")) -> dict:

@@ -600,6 +600,15 @@ int sphst_debug_neighbor_counts(sphst_case c, int32_t *counts, int64_t capacity)
     return c->r.engine->debug_counts(c->r.slot, counts);
 }
 
+int sphst_debug_neighbors(sphst_case c, int64_t width, int32_t *counts, int64_t *ids, int64_t capacity) {
+    if (!c || !counts || (!ids && width > 0)) { set_error("NULL argument"); return SPHST_ERR_INVALID_ARG; }
+    if (width < 0 || width > 65535) { set_error("width must be 0..65535"); return SPHST_ERR_INVALID_ARG; }
+    if (!c->r.engine) { set_error("case not stepped yet"); return SPHST_ERR_STATE; }
+    if (c->r.info.status) { set_error(status_text(c->r.info.status)); return SPHST_ERR_STATE; }
+    if (capacity < c->r.n) { set_error("destination buffer too small"); return SPHST_ERR_CAPACITY; }
+    return c->r.engine->debug_neighbors(c->r.slot, width, counts, ids);
+}
+
 int sphst_struct_sizes(int64_t *params_bytes, int64_t *phase_props_bytes, int64_t *step_info_bytes) {
     if (params_bytes) *params_bytes = (int64_t)sizeof(sphst_case_params);
     if (phase_props_bytes) *phase_props_bytes = (int64_t)sizeof(sphst_phase_props);

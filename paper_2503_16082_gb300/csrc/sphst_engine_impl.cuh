@@ -144,6 +144,7 @@ template <typename T> struct EngineT : Engine {
     std::vector<CaseState> h_state;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    bool rebuilt = false;                           // a step has placed the cells and lists of its members
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 
@@ -630,6 +631,7 @@ template <typename T> struct EngineT : Engine {
     }
 
     int step(int64_t n_adv) override {
+        rebuilt = rebuilt || n_adv > 0;
         for (int64_t s = 0; s < n_adv; ++s) {
             if (loop_mode == SPHST_LOOP_GRAPH) {
                 SPH_CK(cudaGraphLaunch(exec, stream));
@@ -656,6 +658,7 @@ template <typename T> struct EngineT : Engine {
     int profile_step(double *kernel_ms, int64_t *launches) override {
         const int G = SPHST_PROFILE_GROUPS;
         for (int k = 0; k < G; ++k) { kernel_ms[k] = 0.0; launches[k] = 0; }
+        rebuilt = true;
         cudaEvent_t ev[2];
         SPH_CK(cudaEventCreate(&ev[0]));
         SPH_CK(cudaEventCreate(&ev[1]));
@@ -799,6 +802,28 @@ template <typename T> struct EngineT : Engine {
         SPH_CK(cudaMemcpyAsync(counts, dc, m * 4, cudaMemcpyDeviceToHost, stream));
         SPH_CK(cudaStreamSynchronize(stream));
         return SPHST_OK;
+    }
+
+    int debug_neighbors(int slot, int64_t width, int32_t *counts, int64_t *ids) override {
+        const int64_t m = h_desc[slot].p_end - h_desc[slot].p_begin;
+        if (m == 0) return SPHST_OK;
+        if (!rebuilt) { set_error("case not stepped since it came to its engine"); return SPHST_ERR_STATE; }
+        const size_t id_bytes = (size_t)(m * width) * 8, bytes = id_bytes + (size_t)m * 4;
+        char *tmp = nullptr;
+        SPH_CK(cudaMalloc(&tmp, bytes));
+        long long *di = (long long *)tmp;
+        int *dc = (int *)(tmp + id_bytes);
+        cudaError_t e = cudaMemsetAsync(tmp, 0xff, id_bytes, stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(dc, 0, (size_t)m * 4, stream);
+        if (e == cudaSuccess) {
+            SPH_CLASSES_F(0, 4, k_debug_neighbors, slot, snap, id, width, dc, di);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(counts, dc, (size_t)m * 4, cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess && width) e = cudaMemcpyAsync(ids, di, id_bytes, cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        cudaFree(tmp);
+        return e == cudaSuccess ? SPHST_OK : cuda_fail(e, "debug_neighbors");
     }
 };
 

@@ -535,7 +535,7 @@ constexpr int CELL_LANES = 2;
 // 272 with 48, 283 with 38.  FP64 pairs are dear: C 703 with 56, 838 with 38.
 constexpr int CELL_PLACES_MAX = 56;
 constexpr int CELL_PLACES_k_sweep_A = 20, CELL_PLACES_k_sweep_C = 32;
-constexpr int CELL_PLACES_k_sweep_B = 56, CELL_PLACES_k_sweep_V = 56, CELL_PLACES_k_sweep_M = 32;
+constexpr int CELL_PLACES_k_sweep_B = 56, CELL_PLACES_k_sweep_V = 56, CELL_PLACES_k_sweep_M = 32, CELL_PLACES_k_debug_neighbors = 32;
 // at most 48 KB per block, so that no block size asks for an opt-in
 template <typename T> __host__ __device__ inline int cell_places(int threads, int want) {
     return min(sizeof(T) == 8 ? CELL_PLACES_MAX : want, 49152 / (threads * 5));
@@ -2383,6 +2383,26 @@ __global__ void k_debug_counts(const CaseDesc *desc, int c, const uint32_t *star
     if (k >= n) return;
     if (d.dim == 3) count_nbrs<T, 3>(d, d.p_begin + k, starts, snap, id, out);
     else count_nbrs<T, 2>(d, d.p_begin + k, starts, snap, id, out);
+}
+
+// neighbours of case c's fluid particles as the sweeps find them (its lists,
+// or the cell walk), by insertion index: counts and the first `width` of each
+template <typename T, int D, bool LIST, int L = 1>
+__global__ void __launch_bounds__(256) k_debug_neighbors(SweepArgs a, int c, const V4<T> *snap, const uint32_t *id, int64_t width,
+                                                         int *counts, long long *ids) {
+    follow();
+    const Tile t = work_tile<L, false>(a, blockIdx.x);
+    const int li = local_index<L>(blockIdx.x);
+    if (li >= t.n || t.c != c) return;
+    const CaseDesc &d = a.desc[c];
+    const int64_t q = t.begin + li, i = particle_at(a, q), o = id[i];
+    const V4<T> si = ld4(snap + i);
+    neighbors<LIST, false, false, T, D, PART_ALL, L, PLAIN, CELL_PLACES_k_debug_neighbors>(
+        d, phys<T>(d), a.starts, list_of<LIST, T>(a, d, q), snap, nullptr, i, si, w_bits(si.w),
+        [&](uint32_t j, uint32_t, const V4<T> &, const PairG<T> &) {
+            const int k = atomicAdd(counts + o, 1);
+            if (k < width) ids[o * width + k] = id[j];
+        }, threadIdx.x % L);
 }
 
 }  // namespace sphst

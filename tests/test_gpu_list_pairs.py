@@ -1,0 +1,60 @@
+"""The neighbours that the sweeps sum over, read back pair by pair: those of the
+lists, of the cell walk, and of the definition 0 < r_ij < 2h."""
+import numpy as np
+import pytest
+
+import sphcases
+
+pytestmark = pytest.mark.gpu
+
+S = pytest.importorskip("paper_2503_16082_gb300")
+
+
+def held(case, precision, **kw):
+    """(neighbour sets as rows of sorted insertion indices, counts of the plain
+    walk) of the fluid particles, at the initial positions."""
+    h = S.case_from_spec(case, precision=precision, **kw)
+    S.step(h, 1)
+    width = 200
+    counts, ids = S.debug_neighbors(h, width)
+    walked = S.debug_neighbor_counts(h)
+    S.destroy(h)
+    fluid = case.flat()[3] < 2
+    assert counts.max() <= width and (counts[~fluid] == 0).all()
+    assert ((ids >= 0).sum(axis=1) == counts).all()
+    return np.sort(ids[fluid], axis=1), counts[fluid], walked[fluid]
+
+
+def defined(case, slack):
+    """Rows of neighbours of each fluid particle with r < 2h (1 + slack)."""
+    pos, _, _, kind = case.flat()
+    hh = 2.0 * case.h_factor * case.dx * (1.0 + slack)
+    out = np.full(((kind < 2).sum(), 200), -1)
+    for row, i in enumerate(np.flatnonzero(kind < 2)):
+        d = pos - pos[i]
+        for a in range(case.dim):
+            if (case.periodic >> a) & 1:
+                L = case.hi[a] - case.lo[a]
+                d[:, a] -= L * np.round(d[:, a] / L)
+        r2 = (d * d).sum(axis=1)
+        j = np.flatnonzero(r2 < hh * hh)
+        j = j[j != i]
+        out[row, len(out[row]) - len(j):] = np.sort(j)
+    return out
+
+
+def cases():
+    return {"walls_2d": sphcases.small_droplet(2, 21, seed=4, jitter=0.1), "walls_3d": sphcases.small_droplet(3, 11, seed=5, jitter=0.1),
+            "periodic_2d": sphcases.periodic_blob(2, 17, seed=6), "free_3d": sphcases.free_blob(3, 9, seed=7)}
+
+
+@pytest.mark.parametrize("name", sorted(cases()))
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("nbr_mode", [S.NBR_LIST, S.NBR_CELLS])
+def test_the_sweeps_hold_the_defined_neighbours(name, precision, nbr_mode):
+    # FP32 offsets are good to 2^-24 of two cells, so r is to 1e-6 of 2h; no
+    # pair of these seeded cases lies within that of 2h in either reading
+    case = cases()[name]
+    rows, counts, walked = held(case, precision, nbr_mode=nbr_mode)
+    assert np.array_equal(defined(case, -1e-6), defined(case, 1e-6))
+    assert np.array_equal(rows, defined(case, 0.0)) and np.array_equal(counts, walked)
