@@ -344,13 +344,14 @@ __device__ __forceinline__ uint32_t cell_code(int ox, int oy, int oz) {
     return (uint32_t)(ox + 1) | ((uint32_t)(oy + 1) << 2) | (D == 3 ? ((uint32_t)(oz + 1) << 4) : 0u);
 }
 
-// r_ij = s_i - (s_j + o cs): the neighbour's offset moved into i's cell, once
-// for all particles that look at it (o cs is exact, so the sum rounds once)
-template <typename T, int D> struct Moved { T nx, ny, nz; };   // -(s_j + o cs)
+// r_ij = (s_i - o cs) - s_j of list entry e: the operations of the cell walk
+// (o cs is exact), so every test of a pair and every sum sees the same r_ij and
+// r^2, whichever way the pair was found
 template <typename T, int D>
-__device__ __forceinline__ Moved<T, D> moved(uint32_t e, const V4<T> &sj, T cs) {
-    return Moved<T, D>{fma_rn(-code_off(e & 3u, T()), cs, -sj.x), fma_rn(-code_off((e >> 2) & 3u, T()), cs, -sj.y),
-                       D == 3 ? fma_rn(-code_off((e >> 4) & 3u, T()), cs, -sj.z) : T(0)};
+__device__ __forceinline__ void pair_offset(uint32_t e, const V4<T> &si, const V4<T> &sj, T cs, T &rx, T &ry, T &rz) {
+    rx = sub_rn(fma_rn(-code_off(e & 3u, T()), cs, si.x), sj.x);
+    ry = sub_rn(fma_rn(-code_off((e >> 2) & 3u, T()), cs, si.y), sj.y);
+    rz = D == 3 ? sub_rn(fma_rn(-code_off((e >> 4) & 3u, T()), cs, si.z), sj.z) : T(0);
 }
 
 // How a sweep gathers its neighbours (U of walk_list), by measurement at 1M and
@@ -575,9 +576,8 @@ __device__ __forceinline__ bool walk_cells(const CaseDesc &d, const CasePhys<T> 
             for (int u = 0; u < U; ++u) {
                 if (k0 + u >= held) break;
                 const uint32_t c = codes[(k0 + u) * threads];
-                const T rx = sub_rn(fma_rn(-code_off(c & 3u, T()), cs, si.x), sj[u].x);
-                const T ry = sub_rn(fma_rn(-code_off((c >> 2) & 3u, T()), cs, si.y), sj[u].y);
-                const T rz = D == 3 ? sub_rn(fma_rn(-code_off((c >> 4) & 3u, T()), cs, si.z), sj[u].z) : T(0);
+                T rx, ry, rz;
+                pair_offset<T, D>(c, si, sj[u], cs, rx, ry, rz);
                 const PairG<T> g(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz));
                 if constexpr (AUX2) f(j[u], phase_of(w_bits(sj[u].w)), aj[u], bj[u], g);
                 else f(j[u], phase_of(w_bits(sj[u].w)), aj[u], g);
@@ -657,8 +657,8 @@ __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &
         const T cs = cp.cs;
         walk_list<AUX, T, L, U>(l.p, c, snap, aux,
             [&](uint32_t e, const V4<T> &sj, const V4<T> &aj) {
-                const Moved<T, D> m = moved<T, D>(e, sj, cs);
-                const T rx = vadd(si.x, m.nx), ry = vadd(si.y, m.ny), rz = D == 3 ? vadd(si.z, m.nz) : T(0);
+                T rx, ry, rz;
+                pair_offset<T, D>(e, si, sj, cs, rx, ry, rz);
                 f(e >> NBR_SHIFT, phase_of(w_bits(sj.w)), aj, PairG<T>(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz)));
             }, sub);
         return false;
@@ -1698,8 +1698,10 @@ struct BandEntry {
 // time, one per lane; a ballot gives the hits and their places in the slot's
 // list, which is put together in shared memory (the other phase's entries
 // from the end) and written at the end row by row, neighbouring slots side by
-// side.  In FP64 the FP32 test keeps every candidate within 2h (1 + 1e-6) and
-// the hits alone, a sixth of the candidates, are tested again in FP64, whose
+// side.  Which candidates are neighbours is decided by the cell walk's own
+// operations, so list and walk hold the same pairs: in FP32 for the few that
+// the first test cannot settle, in FP64 for its hits, a sixth of the
+// candidates: the FP64
 // pipe is 64 times narrower.  It is bound by instruction issue (about 18
 // instructions per 32 candidates of a slot).  Measured, rebuild of an
 // advection step: 1M fluid particles in FP32 1.71 -> 1.09 ms, 64k 0.56 ->
@@ -1716,7 +1718,6 @@ struct ListSmem {
     float4 cand[LB_CAND];                       // x, y, z relative to the cell, list entry
     uint32_t fluid[2][LB_CAND / 32];            // candidates of each fluid, a word per 32
     uint32_t begin[32], pre[33], code[32];      // cells around in increasing table index
-    uint32_t own;                               // first candidate of the cell itself
     uint32_t idx[LB_SLOTS], rest[LB_SLOTS], other[LB_SLOTS];   // a slot's particle, entries of its list's parts
     uint32_t list[LB_WORDS];
 };
@@ -1732,10 +1733,8 @@ __device__ __forceinline__ bool list_exact(uint32_t e, const CasePhys<T> &cp, co
                                            const V4<T> *snap, bool &coinc) {
     const uint32_t j = e >> NBR_SHIFT;
     const V4<T> sj = ld4(snap + j);
-    const T cs = cp.cs;
-    const T rx = sub_rn(fma_rn(-code_off(e & 3u, T()), cs, si.x), sj.x);
-    const T ry = sub_rn(fma_rn(-code_off((e >> 2) & 3u, T()), cs, si.y), sj.y);
-    const T rz = D == 3 ? sub_rn(fma_rn(-code_off((e >> 4) & 3u, T()), cs, si.z), sj.z) : T(0);
+    T rx, ry, rz;
+    pair_offset<T, D>(e, si, sj, cp.cs, rx, ry, rz);
     const T r2 = norm2<T, D>(rx, ry, rz);
     const bool near = r2 < cp.four_h2 && j != i;
     coinc |= near && !(r2 > T(0));
@@ -1767,28 +1766,40 @@ __device__ __forceinline__ uint32_t list_keep(uint32_t *row, int at, int step, u
 __device__ __forceinline__ float list_coord(float x, float) { return x; }
 __device__ __forceinline__ float list_coord(double x, double unit) { return (float)(x * unit); }
 
+// Margin of the first test's r^2 against the cell walk's, of (2h)^2: it takes
+// s_i - (s_j + o cs), with coordinates up to 2 cs <= 8/3 (2h) in FP32, which
+// moves r^2 by less than 1.7e-6
+constexpr float LIST_MARGIN = 4e-6f;
+
 // tests nc staged candidates (a multiple of 32) against slot i and appends the
-// hits to its shared list.  EXACT: what the test keeps is tested again by the
-// cell walk's operations.  Returns this lane's number of zero distances
-// (FP32; the FP64 and EXACT tests see to those themselves).
+// hits to its shared list.  The first test settles all but the candidates
+// within its margin of 2h or of 0; in FP32 those (about one in 10^5, and the
+// slot's own particle) are tested by the cell walk's operations at once, in
+// FP64 the caller tests all hits.  EXACT: every hit is tested so.
 template <typename T, int D, bool MIXED, bool EXACT>
-__device__ __forceinline__ int list_scan(const ListSmem &S, uint32_t *row, int K, int nc, const CasePhys<T> &cp,
-                                         const V4<T> &si, T unit, uint32_t i, uint32_t ki, float R2, const V4<T> *snap,
-                                         uint32_t &c_rest, uint32_t &c_other, bool &coinc) {
+__device__ __forceinline__ void list_scan(const ListSmem &S, uint32_t *row, int K, int nc, const CasePhys<T> &cp,
+                                          const V4<T> &si, T unit, uint32_t i, uint32_t ki, float R2, const V4<T> *snap,
+                                          uint32_t &c_rest, uint32_t &c_other, bool &coinc) {
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
     const float sx = list_coord(si.x, unit), sy = list_coord(si.y, unit), sz = list_coord(si.z, unit);
-    int zero = 0;
+    const float R2w = R2 * (1.0f + LIST_MARGIN), mid = R2 * 0.5f, half = mid * (1.0f - 2.0f * LIST_MARGIN);
     uint32_t cr = c_rest, co = c_other;
 #pragma unroll 3
     for (int q = 0; q < nc; q += 32) {
         const float4 s = S.cand[q + lane];
         const float r2 = norm2<float, D>(sub_rn(sx, s.x), sub_rn(sy, s.y), D == 3 ? sub_rn(sz, s.z) : 0.0f);
-        const bool near = r2 < R2;
         const uint32_t e = __float_as_uint(s.w);
-        bool hit = near && (sizeof(T) == 8 || EXACT || r2 > 0.0f);
-        zero += near && !hit;
-        if (EXACT) hit = hit && list_exact<T, D>(e, cp, si, i, snap, coinc);
+        bool hit = r2 < R2w;
+        if (EXACT) {
+            hit = hit && list_exact<T, D>(e, cp, si, i, snap, coinc);
+        } else if (sizeof(T) == 4) {
+            const bool open = hit && !(fabsf(r2 - mid) < half);
+            if (__any_sync(0xffffffffu, open)) {
+                if (open) hit = (e >> NBR_SHIFT) != i && list_exact<T, D>(e, cp, si, i, snap, coinc);
+                __syncwarp();
+            }
+        }
         const unsigned h = __ballot_sync(0xffffffffu, hit);
         if (MIXED) {
             const unsigned ho = h & S.fluid[ki ^ 1u][q >> 5], hr = h & ~ho;
@@ -1806,7 +1817,6 @@ __device__ __forceinline__ int list_scan(const ListSmem &S, uint32_t *row, int K
     __syncwarp();
     c_rest = cr;
     c_other = co;
-    return zero;
 }
 
 template <typename T, int D>
@@ -1851,14 +1861,11 @@ __device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> 
         __syncwarp();
         S.pre[lane] = x - own;                  // candidates before cell `lane`
         if (lane == 31) S.pre[32] = x;          // all of them
-        if (lane < NC && S.code[lane] == cell_code<D>(0, 0, 0) && own) S.own = x - own;
     }
     __syncthreads();
     const uint32_t total = S.pre[32];
-    // coordinates lie within 2 cells of the origin, so in FP32 r^2 is wrong by
-    // less than 1.2e-6 of (2h)^2: 2e-6 more keeps every neighbour
     const T unit = sizeof(T) == 8 ? (T)d.list_unit : T(1);
-    const float R2 = (float)(cp.four_h2 * unit * unit), R2w = R2 * 1.000002f;
+    const float R2 = (float)(cp.four_h2 * unit * unit);
     bool coinc = false, overflow = false, has0 = false, has1 = false;
     for (uint32_t g0 = f0; g0 < f1; g0 += G) {
         const int ns = (int)min((uint32_t)G, f1 - g0);
@@ -1907,17 +1914,11 @@ __device__ __forceinline__ void build_cell(const CaseDesc &d, const CasePhys<T> 
                 uint32_t cr = r0, co = o0;
                 uint32_t *row = S.list + s * LS;
                 if (exact) {
-                    list_scan<T, D, true, true>(S, row, K, nc, cp, si, unit, i, ki, R2w, snap, cr, co, coinc);
+                    list_scan<T, D, true, true>(S, row, K, nc, cp, si, unit, i, ki, R2, snap, cr, co, coinc);
                 } else {
-                    const float r2max = sizeof(T) == 8 ? R2w : R2;
-                    int zero = mixed ? list_scan<T, D, true, false>(S, row, K, nc, cp, si, unit, i, ki, r2max, snap, cr, co, coinc)
-                                     : list_scan<T, D, false, false>(S, row, K, nc, cp, si, unit, i, ki, r2max, snap, cr, co, coinc);
-                    if (sizeof(T) == 4) {
-                        // one zero distance is the particle's own, when it is among these candidates
-                        const uint32_t own = S.own + (i - b);
-                        if (lane == (int)((own - c0) & 31u) && own >= c0 && own < c0 + LB_CAND) --zero;
-                        coinc |= zero > 0;
-                    } else if (cr + co <= (uint32_t)K) {
+                    if (mixed) list_scan<T, D, true, false>(S, row, K, nc, cp, si, unit, i, ki, R2, snap, cr, co, coinc);
+                    else list_scan<T, D, false, false>(S, row, K, nc, cp, si, unit, i, ki, R2, snap, cr, co, coinc);
+                    if (sizeof(T) == 8 && cr + co <= (uint32_t)K) {
                         cr = r0 + list_keep<T, D>(row, (int)r0, 1, cr - r0, cp, si, i, snap, coinc);
                         if (co > o0) co = o0 + list_keep<T, D>(row, K - 1 - (int)o0, -1, co - o0, cp, si, i, snap, coinc);
                     }
@@ -2015,8 +2016,8 @@ __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V
             const int64_t at = w + (int64_t)k * LROW;
             const uint32_t e = ld_list(a.nbr + at);
             const V4<double> sj = ld4(snap + (e >> NBR_SHIFT));
-            const Moved<double, D> m = moved<double, D>(e, sj, cp.cs);
-            const double rx = vadd(si.x, m.nx), ry = vadd(si.y, m.ny), rz = D == 3 ? vadd(si.z, m.nz) : 0.0;
+            double rx, ry, rz;
+            pair_offset<double, D>(e, si, sj, cp.cs, rx, ry, rz);
             const PairG<double> g(cp, rx, ry, rz, norm2<double, D>(rx, ry, rz));
             ge[at] = V4<double>{g.x, g.y, g.z, phase_of(w_bits(sj.w)) == PH_WALL ? -g.wd : g.wd};
             gr[at] = RInv{g.r, g.inv};

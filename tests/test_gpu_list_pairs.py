@@ -58,3 +58,20 @@ def test_the_sweeps_hold_the_defined_neighbours(name, precision, nbr_mode):
     rows, counts, walked = held(case, precision, nbr_mode=nbr_mode)
     assert np.array_equal(defined(case, -1e-6), defined(case, 1e-6))
     assert np.array_equal(rows, defined(case, 0.0)) and np.array_equal(counts, walked)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("cap", [0, 1])
+def test_list_and_walk_hold_the_same_pairs_at_2h(dim, precision, cap):
+    # on the lattice with h = 3/2 dx a whole shell of neighbours lies at 2h, in
+    # or out by the rounding of r^2 alone: the same in the list, whichever way
+    # it was built (cap 1: a capacity that just fits, so that the lists that do
+    # not fit at first are built again), in the buffered and in the plain walk
+    case = sphcases.small_droplet(dim, 23 if dim == 2 else 11)
+    case.h_factor = 1.5
+    cells = held(case, precision, nbr_mode=S.NBR_CELLS)
+    lists = held(case, precision, max_neighbors=int(cells[1].max()) if cap else 160)
+    assert cells[2].max() > cells[2].min()
+    for rows, counts, walked in (cells, lists):
+        assert np.array_equal(counts, walked) and np.array_equal(rows, cells[0])
