@@ -28,6 +28,8 @@
 // on that choice.
 #pragma once
 
+#include <cfloat>
+#include <type_traits>
 #include <utility>
 
 #include <cuda_runtime.h>
@@ -95,14 +97,16 @@
 namespace sphst {
 
 // ------------------------------------------------------------------ helpers
-// r^2 of a pair and rho_i + rho_j are normal numbers (a case whose r^2 is not
-// has a kernel derivative beyond FP32), so the flush-to-zero forms give the
-// same values without the scaling of denormal arguments
+// rho_i + rho_j and its product with rho_j are normal numbers, so the
+// flush-to-zero reciprocal gives the same value without the scaling of
+// denormal arguments.  So does the root for a normal r^2; for the others (r
+// below 1.1e-19, where r_ij is cut off by FP32's range itself) there is rsq_full.
 __device__ __forceinline__ float rsq(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float rsq_full(float x) { return rsqrtf(x); }
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -438,8 +442,16 @@ __device__ __forceinline__ void walk_list(const uint32_t *__restrict__ p, uint32
 template <typename T> struct PairG;
 template <> struct PairG<float> {
     float x, y, z, inv, r, wd;                  // r_ij, 1/r, r, W'/r
-    __device__ __forceinline__ PairG(const CasePhys<float> &cp, float rx, float ry, float rz, float r2) : x(rx), y(ry), z(rz) {
-        inv = rsq(r2);
+    // FULL: 1/r also of a denormal r^2 (r < 1.1e-19).  The sums that weigh
+    // e_ij by W' or r_ij by W'/r take the least normal r^2 instead: such a pair
+    // gives them less than their rounding (its r is below 4e-10 h at the least h
+    // FP32 holds), and the full form costs sweep C 3.4% and B 1.4% at 1M
+    // particles.  The penalty of sweep S, where e_ij W'/r counts, needs it.
+    template <bool FULL>
+    __device__ __forceinline__ PairG(const CasePhys<float> &cp, float rx, float ry, float rz, float r2, std::bool_constant<FULL>)
+        : x(rx), y(ry), z(rz) {
+        r2 = FULL ? r2 : fmaxf(r2, FLT_MIN);
+        inv = FULL ? rsq_full(r2) : rsq(r2);
         r = vmul(r2, inv);
         const float u = vfma(r, cp.mhalf_inv_h, 1.0f);
         wd = vmul(vmul(vmul(cp.kcoef_h, u), u), u);
@@ -453,7 +465,8 @@ template <> struct PairG<float> {
 template <> struct PairG<double> {
     double x, y, z, inv, r, wd;                 // e_ij, 1/r, r, W'
     __device__ __forceinline__ PairG() {}
-    __device__ __forceinline__ PairG(const CasePhys<double> &cp, double rx, double ry, double rz, double r2) {
+    template <bool FULL>
+    __device__ __forceinline__ PairG(const CasePhys<double> &cp, double rx, double ry, double rz, double r2, std::bool_constant<FULL>) {
         inv = rsq(r2);
         r = vmul(r2, inv);
         const double u = vfma(r, cp.mhalf_inv_h, 1.0);
@@ -545,7 +558,7 @@ template <typename T> __host__ __device__ inline size_t cell_walk_bytes(int thre
     return (size_t)threads * cell_places<T>(threads, want) * 5;
 }
 constexpr int CELL_STEP = 16;                   // candidates between two looks at the free places
-template <int PLACES, bool AUX, bool AUX2, bool OTHER, typename T, int D, int L, typename F>
+template <int PLACES, bool AUX, bool AUX2, bool OTHER, bool FULL, typename T, int D, int L, typename F>
 __device__ __forceinline__ bool walk_cells(const CaseDesc &d, const CasePhys<T> &cp, const uint32_t *__restrict__ starts,
                                            const V4<T> *__restrict__ snap, const V4<T> *__restrict__ aux,
                                            const V4<T> *__restrict__ aux2, int64_t i, const V4<T> &si, uint32_t pki, uint32_t sub, F &&f) {
@@ -578,7 +591,7 @@ __device__ __forceinline__ bool walk_cells(const CaseDesc &d, const CasePhys<T> 
                 const uint32_t c = codes[(k0 + u) * threads];
                 T rx, ry, rz;
                 pair_offset<T, D>(c, si, sj[u], cs, rx, ry, rz);
-                const PairG<T> g(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz));
+                const PairG<T> g(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz), std::bool_constant<FULL>());
                 if constexpr (AUX2) f(j[u], phase_of(w_bits(sj[u].w)), aj[u], bj[u], g);
                 else f(j[u], phase_of(w_bits(sj[u].w)), aj[u], g);
             }
@@ -641,7 +654,7 @@ __device__ __forceinline__ bool walk_cells(const CaseDesc &d, const CasePhys<T> 
 }
 
 // neighbours of particle i as f(j, kind of j, aux_j, geometry), from its list
-// or from the cell walk.  NEED_R: f reads r or 1/r.
+// or from the cell walk.  NEED_R: f reads r or 1/r (FULL of PairG).
 template <bool LIST, bool AUX, bool NEED_R, typename T, int D, int PART = PART_ALL, int L = 1, int U = PLAIN, int PLACES = 0,
           typename F>
 __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &cp, const uint32_t *starts,
@@ -659,11 +672,11 @@ __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &
             [&](uint32_t e, const V4<T> &sj, const V4<T> &aj) {
                 T rx, ry, rz;
                 pair_offset<T, D>(e, si, sj, cs, rx, ry, rz);
-                f(e >> NBR_SHIFT, phase_of(w_bits(sj.w)), aj, PairG<T>(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz)));
+                f(e >> NBR_SHIFT, phase_of(w_bits(sj.w)), aj, PairG<T>(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz), std::bool_constant<NEED_R>()));
             }, sub);
         return false;
     } else {
-        return walk_cells<PLACES, AUX, false, PART == PART_OTHER, T, D, L>(d, cp, starts, snap, aux, nullptr, i, si, pki, sub, f);
+        return walk_cells<PLACES, AUX, false, PART == PART_OTHER, NEED_R, T, D, L>(d, cp, starts, snap, aux, nullptr, i, si, pki, sub, f);
     }
 }
 
@@ -1545,13 +1558,13 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
         }
     } else {
         if (surface_on)
-            walk_cells<CELL_PLACES_k_sweep_B, true, true, false, T, D, L>(d, cp, starts, snap, vel, gradC, i, si, pki, sub,
+            walk_cells<CELL_PLACES_k_sweep_B, true, true, false, true, T, D, L>(d, cp, starts, snap, vel, gradC, i, si, pki, sub,
                 [&](uint32_t j, uint32_t kj, const V4<T> &vj, const V4<T> &nj, const PairG<T> &g) {
                     pressure(j, kj, vj, g);
                     surface(j, kj, nj, g);
                 });
         else
-            walk_cells<CELL_PLACES_k_sweep_B, true, false, false, T, D, L>(d, cp, starts, snap, vel, nullptr, i, si, pki, sub, pressure);
+            walk_cells<CELL_PLACES_k_sweep_B, true, false, false, false, T, D, L>(d, cp, starts, snap, vel, nullptr, i, si, pki, sub, pressure);
         apx = group_sum<L>(apx);
         apy = group_sum<L>(apy);
         asx = group_sum<L>(asx);
@@ -2018,7 +2031,7 @@ __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V
             const V4<double> sj = ld4(snap + (e >> NBR_SHIFT));
             double rx, ry, rz;
             pair_offset<double, D>(e, si, sj, cp.cs, rx, ry, rz);
-            const PairG<double> g(cp, rx, ry, rz, norm2<double, D>(rx, ry, rz));
+            const PairG<double> g(cp, rx, ry, rz, norm2<double, D>(rx, ry, rz), std::true_type());
             ge[at] = V4<double>{g.x, g.y, g.z, phase_of(w_bits(sj.w)) == PH_WALL ? -g.wd : g.wd};
             gr[at] = RInv{g.r, g.inv};
         }

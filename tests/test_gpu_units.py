@@ -24,9 +24,9 @@ def scaled(case, s):
                                c0=case.c0 * s, gamma=case.gamma * s**2, phases=phases)
 
 
-def fields(case, precision, s, **kw):
+def fields(case, precision, s, steps=2, **kw):
     h = S.case_from_spec(scaled(case, s), precision=precision, **kw)
-    info = S.step(h, 2, check=False)
+    info = S.step(h, steps, check=False)
     unit = {S.FIELD_POS: s, S.FIELD_VEL: s, S.FIELD_RHO: 1.0 / s, S.FIELD_GRADC: 1.0 / s, S.FIELD_ACC_VISC: s}
     out = [S.read_fields(h, f, case.dim) / u for f, u in unit.items()]
     q = S.diagnose(h, center=[0.5 * s] * case.dim)
@@ -57,3 +57,30 @@ def test_fp64_lists_hold_beyond_the_range_of_fp32(dim, exponent):
     assert (rc0, rc1) == (S.OK, S.OK) and n0 == n1
     for x, y in zip(a, b):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("nbr_mode", [S.NBR_LIST, S.NBR_CELLS])
+@pytest.mark.parametrize("second", [0, 1])
+def test_fp32_pair_whose_squared_distance_is_denormal(nbr_mode, second):
+    # two fluid particles 2^-38 apart next to a cell's corner (h = 1/4, so the
+    # grid's lines are exact), among their neighbours: scaled by 2^-28 their
+    # r^2 = 2^-132 is a denormal.  Finite, and the same results: the pair's e_ij
+    # is weighed by W' or r everywhere but in the penalty, where 1/r is taken in
+    # full, so its error stays below the rounding of a sum (2^-24 of its terms);
+    # the bar is 16 of these after one step, of each field's maximum (in a second
+    # one the offsets, no longer next to the corner, would round together)
+    cs = 0.5 * (1 + 2.0**-16)
+    corner = 4 * cs
+    rng = np.random.default_rng(3)
+    p = sphcases.lattice([0.0, 0.0], [4.0, 4.0], 0.25) + rng.uniform(-0.02, 0.02, (256, 2))
+    p = p[np.abs(p - corner).max(axis=1) > 0.2]
+    p = np.concatenate([[[0.0, 0.0]], p[(p > 0.05).any(axis=1)], [[corner, corner], [corner + 2.0**-38, corner]]])
+    kind = np.hypot(*(p - corner).T) < 0.8
+    kind[-1] = not second
+    phases = [sphcases.Phase("fluid", p[k], rho0=r, eta=0.1, vel=np.full((k.sum(), 2), 0.01)) for k, r in ((kind, 2.0), (~kind, 1.0))]
+    case = sphcases.Case(name="close", dim=2, lo=[0.0, 0.0], hi=[4.0, 4.0], dx=0.25, gamma=1.0, c0=10.0, h_factor=1.0, phases=phases)
+    rc0, n0, a = fields(case, 32, 1.0, steps=1, nbr_mode=nbr_mode)
+    rc1, n1, b = fields(case, 32, 2.0**-28, steps=1, nbr_mode=nbr_mode)
+    assert (rc0, rc1) == (S.OK, S.OK) and n0 == n1
+    for x, y in zip(a[:5], b[:5]):
+        assert np.isfinite(x).all() and np.abs(x - y).max() <= 2.0**-20 * np.abs(x).max()
