@@ -411,10 +411,22 @@ int sphst_fma_peak(int32_t precision, double *tflops, double *kernel_ms);
 int sphst_device_info(int32_t *sm_count, int32_t *max_sm_clock_khz, int32_t *cc_major,
                       int32_t *cc_minor);
 
-/* Device bytes one case of n particles needs (particle arrays, cell table,
- * scratch), for admission control.  Errors: INVALID_ARG. */
+/* Device bytes one case of n particles takes (particle arrays, cell table,
+ * scratch, the stored pair geometry), for admission control.  Errors:
+ * INVALID_ARG. */
 int sphst_footprint_bytes(const sphst_case_params *params, int64_t n_particles,
                           int64_t *bytes_out);
+
+/* The part of it that FP64 neighbour-list cases can do without: the geometry
+ * of the lists' pairs, kept from one substep to the next for speed (48 bytes
+ * per list entry; the results are the same bits without it).  An engine keeps
+ * it for its cases in order up to 16 GiB, all engines of the process together
+ * up to 32 GiB, and only where a quarter of the free memory holds it; a case
+ * whose own geometry is more than 16 GiB never keeps it (0 bytes).
+ * sphst_set_pair_geometry(c, 0), before the first step, has a case go without
+ * it in every engine.  Errors: INVALID_ARG, STATE after the first step. */
+int sphst_pair_geometry_bytes(const sphst_case_params *params, int64_t n_particles, int64_t *bytes_out);
+int sphst_set_pair_geometry(sphst_case c, int32_t keep);
 
 /* sizeof of the three structures of this header as the library was built,
  * so a binding can check its layout before the first call.  Any pointer may

@@ -115,6 +115,8 @@ EXPORTS = {
     "sphst_batch_size": (C.c_int, [C.c_void_p, C.POINTER(C.c_int64)]),
     "sphst_batch_destroy": (C.c_int, [C.c_void_p]),
     "sphst_footprint_bytes": (C.c_int, [C.POINTER(CaseParams), C.c_int64, C.POINTER(C.c_int64)]),
+    "sphst_pair_geometry_bytes": (C.c_int, [C.POINTER(CaseParams), C.c_int64, C.POINTER(C.c_int64)]),
+    "sphst_set_pair_geometry": (C.c_int, [C.c_void_p, C.c_int32]),
     "sphst_diagnose": (C.c_int, [C.c_void_p, C.c_void_p, C.c_double, C.c_double, C.POINTER(Diagnostics)]),
     "sphst_fma_peak": (C.c_int, [C.c_int32, C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     "sphst_device_info": (C.c_int, [C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32),
@@ -365,6 +367,19 @@ def footprint_bytes(params: CaseParams, n: int) -> int:
     out = C.c_int64()
     _check(load().sphst_footprint_bytes(C.byref(params), n, C.byref(out)), "footprint_bytes")
     return out.value
+
+
+def pair_geometry_bytes(params: CaseParams, n: int) -> int:
+    """The part of footprint_bytes that an FP64 list case can do without."""
+    out = C.c_int64()
+    _check(load().sphst_pair_geometry_bytes(C.byref(params), n, C.byref(out)), "pair_geometry_bytes")
+    return out.value
+
+
+def set_pair_geometry(case, keep: bool) -> None:
+    """Whether the case's FP64 lists may keep their pair geometry (speed
+    only); before the first step."""
+    _check(load().sphst_set_pair_geometry(case, int(keep)), "set_pair_geometry")
 
 
 # --------------------------------------------------------------------------

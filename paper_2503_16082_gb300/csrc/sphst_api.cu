@@ -219,10 +219,18 @@ CaseDesc make_desc(const CaseRec *c) {
     return d;
 }
 
+static int64_t list_capacity(const sphst_case_params *P) {
+    return P->nbr_mode == SPHST_NBR_LIST ? (P->max_neighbors > 0 ? P->max_neighbors : (P->dim == 3 ? 128 : 48)) : 0;
+}
+
+int64_t geometry_bytes(const sphst_case_params *P, int64_t n) {
+    const int64_t bytes = P->precision == 64 ? geometry_entries(list_capacity(P), n) * PAIR_GEOMETRY_BYTES : 0;
+    return bytes <= PAIR_GEOMETRY_MAX ? bytes : 0;
+}
+
 int64_t footprint(const sphst_case_params *P, int64_t n) {
     const int64_t tsz = P->precision == 64 ? 8 : 4;
-    const int64_t kmax = P->nbr_mode == SPHST_NBR_LIST
-                             ? (P->max_neighbors > 0 ? P->max_neighbors : (P->dim == 3 ? 128 : 48)) : 0;
+    const int64_t kmax = list_capacity(P);
     // V4 arrays, scalars, ints, list, band + band list, cell list
     const int64_t per = 9 * 4 * tsz + (tsz == 8 ? 3 : 2) * tsz + 6 * 4 + 4 * kmax + 4 + 1 + 8 + 8 +
                         (P->surface_corr == 1 ? 2 * 4 * tsz : 0);   // own-fluid correction matrices
@@ -231,7 +239,7 @@ int64_t footprint(const sphst_case_params *P, int64_t n) {
     int bits = 0;
     while ((double)(1 << bits) < side) ++bits;
     const int64_t table = ((int64_t)1 << (P->dim * bits)) * 4 + 4;
-    return per * n + table + 4096 + 32 * 4 * kmax + (int64_t)(DIAG_BLOCKS + 1) * DIAG_Q * 8;
+    return per * n + table + 4096 + 32 * 4 * kmax + (int64_t)(DIAG_BLOCKS + 1) * DIAG_Q * 8 + geometry_bytes(P, n);
 }
 
 // Move `cases` into one new engine (copying resident state), release
@@ -622,6 +630,22 @@ int sphst_footprint_bytes(const sphst_case_params *params, int64_t n, int64_t *b
         return SPHST_ERR_INVALID_ARG;
     }
     *bytes_out = footprint(params, n);
+    return SPHST_OK;
+}
+
+int sphst_pair_geometry_bytes(const sphst_case_params *params, int64_t n, int64_t *bytes_out) {
+    if (!params || !bytes_out || n < 0 || (params->dim != 2 && params->dim != 3)) {
+        set_error("bad argument");
+        return SPHST_ERR_INVALID_ARG;
+    }
+    *bytes_out = geometry_bytes(params, n);
+    return SPHST_OK;
+}
+
+int sphst_set_pair_geometry(sphst_case c, int32_t keep) {
+    if (!c || keep < 0 || keep > 1) { set_error("NULL case, or keep is not 0 or 1"); return SPHST_ERR_INVALID_ARG; }
+    if (c->r.engine) { set_error("pair geometry must be set before the first step"); return SPHST_ERR_STATE; }
+    c->r.keep_geometry = keep != 0;
     return SPHST_OK;
 }
 

@@ -40,8 +40,17 @@ struct CaseRec {
     int32_t slot = -1;                     // index in the engine
     struct sphst_batch_s *batch = nullptr;
     cudaStream_t user_stream = nullptr;   // caller's stream, or null
+    bool keep_geometry = true;             // FP64 lists may keep their pair geometry
     sphst_step_info info{};
 };
+
+// Stored pair geometry of FP64 lists: bytes per list entry, the most that one
+// engine keeps (its speed is worth it, its memory is not needed), and the most
+// of all engines of the process: two at the first limit, as while a batch
+// moves to a new engine.
+constexpr int64_t PAIR_GEOMETRY_BYTES = 48;
+constexpr int64_t PAIR_GEOMETRY_MAX = (int64_t)16 << 30, PAIR_GEOMETRY_PROCESS_MAX = (int64_t)32 << 30;
+inline int64_t geometry_entries(int64_t nbr_k, int64_t n_fluid) { return (n_fluid + 31) / 32 * 32 * nbr_k; }
 
 // Fills the grid fields of a case from its staged positions (first step).
 int make_grid(CaseRec *c);
@@ -74,6 +83,7 @@ struct Engine {
 
 Engine *new_engine_f32();
 Engine *new_engine_f64();
-int64_t footprint(const sphst_case_params *P, int64_t n);
+int64_t footprint(const sphst_case_params *P, int64_t n);       // with the geometry's bytes
+int64_t geometry_bytes(const sphst_case_params *P, int64_t n);
 
 }  // namespace sphst

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <vector>
 
@@ -104,6 +105,7 @@ template <typename T> struct EngineT : Engine {
     uint32_t *starts = nullptr, *block_sums = nullptr;
     uint32_t *nbr = nullptr, *nbr_cnt = nullptr;   // neighbour lists (ELL per case) and counts
     V4<T> *lgeo = nullptr;                          // (e_ij, W') and (r, 1/r) of each list entry (FP64)
+    int64_t geo_bytes = 0;
     RInv *lrinv = nullptr;
     uint8_t *band = nullptr;                        // interface band of the frozen configuration
     uint64_t *band_list = nullptr;                  // band particles per list class (case << 32 | index)
@@ -154,6 +156,43 @@ template <typename T> struct EngineT : Engine {
         if (graph) cudaGraphDestroy(graph);
         if (stream && own_stream) cudaStreamDestroy(stream);
         if (arena) cudaFree(arena);
+        if (lgeo) {
+            cudaFree(lgeo);
+            geometry_in_use -= geo_bytes;
+        }
+    }
+
+    // FP64 keeps the lists' pair geometry where memory is plentiful: the results
+    // are the same without it.  An allocation of its own, after everything an
+    // engine needs, so that no case fails for it; within one engine the cases
+    // take it in order until PAIR_GEOMETRY_MAX.  Nothing past a list's count is
+    // read, so it is not cleared.
+    static inline std::atomic<int64_t> geometry_in_use{0};
+    void place_geometry(const std::vector<CaseRec *> &cases) {
+        if (sizeof(T) == 4) return;
+        int64_t entries = 0;
+        for (int c = 0; c < ncases; ++c) {
+            const int64_t e = geometry_entries(h_desc[c].nbr_k, cases[c]->n_fluid);
+            if (h_desc[c].nbr_mode != 0 || !cases[c]->keep_geometry || (entries + e) * PAIR_GEOMETRY_BYTES > PAIR_GEOMETRY_MAX) continue;
+            h_desc[c].geo_base = entries;
+            entries += e;
+        }
+        if (!entries) return;
+        geo_bytes = entries * PAIR_GEOMETRY_BYTES;
+        size_t mem_free = 0, mem_total = 0;
+        const int64_t used = geometry_in_use.fetch_add(geo_bytes) + geo_bytes;
+        // a quarter of what is free at most; small ones are not worth the question
+        bool ok = used <= PAIR_GEOMETRY_PROCESS_MAX;
+        if (ok && geo_bytes > ((int64_t)64 << 20))
+            ok = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && (size_t)geo_bytes <= mem_free / 4;
+        if (ok && cudaMalloc(&lgeo, (size_t)geo_bytes) == cudaSuccess) {
+            lrinv = (RInv *)(lgeo + entries);
+            return;
+        }
+        cudaGetLastError();
+        lgeo = nullptr;
+        geometry_in_use -= geo_bytes;
+        for (CaseDesc &d : h_desc) d.geo_base = -1;
     }
 
     void *dev_array(int which) override {
@@ -228,6 +267,7 @@ template <typename T> struct EngineT : Engine {
                 nbr_total += (r->n_fluid + 31) / 32 * 32 * (int64_t)d.nbr_k;
                 any_list = true;
             }
+            d.geo_base = -1;
             h_desc[c] = d;
             if (r->P.loop_mode == SPHST_LOOP_HOST) loop_mode = SPHST_LOOP_HOST;
         }
@@ -263,16 +303,6 @@ template <typename T> struct EngineT : Engine {
         size_t o_ftfirst = take(nc * 8), o_cls0 = take(64);
         size_t o_flag = take(64);
         size_t o_read = take((size_t)std::max<int64_t>(max_case_n, 1) * 3 * sizeof(double));
-        // FP64 keeps the lists' pair geometry where it fits easily: the results
-        // are the same without it
-        bool geo = false;
-        if (sizeof(T) == 8 && any_list) {
-            size_t mem_free = 0, mem_total = 0;
-            SPH_CK(cudaMemGetInfo(&mem_free, &mem_total));
-            const size_t bytes = (size_t)nbr_total * (sizeof(V4<T>) + sizeof(RInv));
-            geo = bytes <= std::min(mem_free / 4, mem_total / 16);
-        }
-        const size_t o_lgeo = take(geo ? (size_t)nbr_total * sizeof(V4<T>) : 0), o_lrinv = take(geo ? (size_t)nbr_total * sizeof(RInv) : 0);
         size_t o_nbr = take((size_t)std::max<int64_t>(nbr_total, 1) * 4), o_ncnt = take(nn * 4);
         size_t o_band = take(nn);
         size_t o_blist = take(nn * 8), o_bcount = take(64), o_clist = take(nn * 8);
@@ -303,8 +333,6 @@ template <typename T> struct EngineT : Engine {
         d_work = (uint32_t *)(b + o_work); d_ft_first = (int64_t *)(b + o_ftfirst); d_cls0 = (int64_t *)(b + o_cls0);
         d_read = (double *)(b + o_read);
         nbr = (uint32_t *)(b + o_nbr);
-        lgeo = geo ? (V4<T> *)(b + o_lgeo) : nullptr;
-        lrinv = geo ? (RInv *)(b + o_lrinv) : nullptr;
         nbr_cnt = (uint32_t *)(b + o_ncnt);
         band = (uint8_t *)(b + o_band);
         band_list = (uint64_t *)(b + o_blist);
@@ -313,6 +341,7 @@ template <typename T> struct EngineT : Engine {
         cell_list = (uint64_t *)(b + o_clist);
         d_diag = (double *)(b + o_diag);
         SPH_CK(cudaMemsetAsync(arena, 0, off, stream));
+        place_geometry(cases);
         // tiles, grouped by class
         std::vector<Tile> tiles;
         tiles.reserve(n_tiles);

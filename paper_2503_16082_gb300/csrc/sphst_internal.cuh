@@ -115,6 +115,7 @@ struct CaseDesc {
     int32_t nbr_mode;          // 0: neighbour list built per advection step; 1: cell walk
     int32_t nbr_k;             // list capacity per particle
     int64_t nbr_base;          // first list word of this case
+    int64_t geo_base;          // first entry of its lists' stored pair geometry; -1: none is kept
     int64_t f_begin;           // first slot of this case
     double list_unit;          // power of two that brings cs into [1, 2) (FP32 test of the FP64 list build)
     CasePhys<float> pf;

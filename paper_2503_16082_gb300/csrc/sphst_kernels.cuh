@@ -1633,7 +1633,7 @@ struct SweepArgs {
     // nullptr: tile entries are particle indices; else the tiles run over
     // fluid ranks and fidx maps a rank to the particle (sweeps B and C)
     const uint32_t *fidx = nullptr;
-    // stored pair geometry of the lists (FP64, where it is kept)
+    // stored pair geometry of the lists (FP64, of the cases that keep it)
     const void *ge = nullptr, *gr = nullptr;
     // batches: the tiles of the cases active in this substep, compacted per
     // class after the criterion kernel (work[tile0 + k] is a tile index,
@@ -1684,8 +1684,10 @@ __device__ __forceinline__ int64_t particle_at(const SweepArgs &a, int64_t q) {
 template <bool LIST, typename T> __device__ __forceinline__ ListRef<T> list_of(const SweepArgs &a, const CaseDesc &d, int64_t q) {
     if (!LIST) return ListRef<T>{nullptr, 0u, nullptr, nullptr};
     const int64_t w = list_word(d, q);
-    if (sizeof(T) == 8 && a.ge)
-        return ListRef<T>{a.nbr + w, a.cnt[q], static_cast<const V4<T> *>(a.ge) + w, static_cast<const RInv *>(a.gr) + w};
+    if (sizeof(T) == 8 && d.geo_base >= 0) {
+        const int64_t g = d.geo_base + (w - d.nbr_base);
+        return ListRef<T>{a.nbr + w, a.cnt[q], static_cast<const V4<T> *>(a.ge) + g, static_cast<const RInv *>(a.gr) + g};
+    }
     return ListRef<T>{a.nbr + w, a.cnt[q], nullptr, nullptr};
 }
 
@@ -2020,7 +2022,10 @@ __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V
     const Tile t = a.tiles[a.tile0 + blockIdx.x];
     if (!a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
+    if (d.geo_base < 0) return;
     const CasePhys<double> &cp = d.pd;
+    ge += d.geo_base - d.nbr_base;
+    gr += d.geo_base - d.nbr_base;
     for (int s = threadIdx.x; s < t.n; s += 32) {
         const int64_t q = t.begin + s, i = particle_at(a, q), w = list_word(d, q);
         const V4<double> si = ld4(snap + i);

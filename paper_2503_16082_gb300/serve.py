@@ -29,7 +29,7 @@ import numpy as np
 
 from . import (FIELD_POS, FIELD_RHO, FIELD_VEL, MAX_LIST_ENGINE_PARTICLES, OK, SphstError, batch_add, batch_create,
                batch_destroy, batch_remove, batch_step, case_from_spec, case_info, default_params,
-               destroy, footprint_bytes, read_fields)
+               destroy, footprint_bytes, pair_geometry_bytes, read_fields, set_pair_geometry)
 
 
 @dataclasses.dataclass
@@ -62,6 +62,7 @@ class _Request:
     submitted: float
     future: concurrent.futures.Future
     footprint: int = 0
+    keep_geometry: bool = True
     handle: object = None
     admitted: float = 0.0
     done_steps: int = 0
@@ -96,11 +97,14 @@ class Server:
         self._stop = threading.Event()
 
     # ------------------------------------------------------------ requests
-    def footprint(self, spec, params: Optional[dict] = None) -> int:
+    def _params(self, spec, params: Optional[dict] = None):
         p = default_params(dim=spec.dim, precision=self.precision, dx=spec.dx)
         for k, v in (params or {}).items():
             setattr(p, k, v)
-        return footprint_bytes(p, spec.n)
+        return p
+
+    def footprint(self, spec, params: Optional[dict] = None) -> int:
+        return footprint_bytes(self._params(spec, params), spec.n)
 
     def submit(self, spec, n_adv: Optional[int] = None, t_end: Optional[float] = None,
                n_sub: Optional[int] = None, **params) -> concurrent.futures.Future:
@@ -113,6 +117,9 @@ class Server:
         with self.lock:
             r = _Request(self.next_id, spec, n_adv, t_end, n_sub, params, time.perf_counter(), fut)
             r.footprint = self.footprint(spec, params)
+            if r.footprint > self.budget:       # go without what only speeds it up
+                r.footprint -= pair_geometry_bytes(self._params(spec, params), spec.n)
+                r.keep_geometry = False
             if r.footprint > self.budget:
                 fut.set_exception(SphstError(-8, f"request needs {r.footprint} B, budget {self.budget:.0f} B"))
                 return fut
@@ -163,6 +170,7 @@ class Server:
                 r = self.queue.popleft()
                 try:
                     r.handle = case_from_spec(r.spec, precision=self.precision, **r.params)
+                    set_pair_geometry(r.handle, r.keep_geometry)
                     batch_add(self.batch, r.handle)
                 except Exception as e:          # noqa: BLE001 - report to the caller
                     r.future.set_exception(e)
