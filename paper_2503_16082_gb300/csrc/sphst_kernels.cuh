@@ -470,7 +470,8 @@ template <> struct PairG<double> {
         inv = rsq(r2);
         r = vmul(r2, inv);
         const double u = vfma(r, cp.mhalf_inv_h, 1.0);
-        wd = vmul(vmul(vmul(vmul(cp.kcoef_h, u), u), u), r);
+        // W' <= 0: at 2h u may round to 0 or below, which is 0 for W'
+        wd = -fabs(vmul(vmul(vmul(vmul(cp.kcoef_h, u), u), u), r));
         x = vmul(rx, inv); y = vmul(ry, inv); z = vmul(rz, inv);
     }
     __device__ __forceinline__ double du(double dot) const { return dot; }
@@ -482,8 +483,9 @@ template <> struct PairG<double> {
 
 // One particle's list: its first word, its count as in cnt[], and (FP64,
 // optional) the stored geometry of its entries: (e_ij, W') and (r, 1/r) of the
-// frozen configuration at the list's own positions.  W' < 0 for every pair; a
-// wall's entry stores -W', and the other fluid's entries come first, so the
+// frozen configuration at the list's own positions.  W' = -|W'| for every
+// pair, with the sign bit set also where it is 0; a wall's entry stores |W'|,
+// with the bit clear, and the other fluid's entries come first, so the
 // neighbour's kind is known without its position.
 struct alignas(16) RInv { double r, inv; };
 template <typename T> struct ListRef {
@@ -520,9 +522,9 @@ __device__ __forceinline__ void walk_geo(const ListRef<double> &l, uint32_t c, c
             if (NEED_R) ri = *gr;
         }
         if (k + 2 * L < c) w1 = ld_list_walk(p + L * LROW);
-        const bool wall = gc.w >= 0.0;
+        const bool wall = __double_as_longlong(gc.w) >= 0;
         PairG<double> G;
-        G.x = gc.x; G.y = gc.y; G.z = gc.z; G.wd = wall ? -gc.w : gc.w;
+        G.x = gc.x; G.y = gc.y; G.z = gc.z; G.wd = -fabs(gc.w);
         G.r = rc.r; G.inv = rc.inv;
         f(ec >> NBR_SHIFT, wall ? PH_WALL : k < c_other ? ki ^ 1u : ki, AUX ? ac : gc, G);
     }
@@ -2037,7 +2039,7 @@ __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V
             double rx, ry, rz;
             pair_offset<double, D>(e, si, sj, cp.cs, rx, ry, rz);
             const PairG<double> g(cp, rx, ry, rz, norm2<double, D>(rx, ry, rz), std::true_type());
-            ge[at] = V4<double>{g.x, g.y, g.z, phase_of(w_bits(sj.w)) == PH_WALL ? -g.wd : g.wd};
+            ge[at] = V4<double>{g.x, g.y, g.z, phase_of(w_bits(sj.w)) == PH_WALL ? fabs(g.wd) : g.wd};
             gr[at] = RInv{g.r, g.inv};
         }
     }

@@ -114,3 +114,36 @@ def test_a_batch_holds_members_with_and_without(work_lists):
         S.batch_remove(batch, h)
         S.destroy(h)
     S.batch_destroy(batch)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("partner", ["wall", "fluid"])
+def test_pairs_at_the_cutoff_keep_their_kind(partner):
+    # isolated pairs at 2h less a few units in the last place: 1 - q/2 rounds
+    # to 0 or to either side of it, so W' is 0 or about 1e-48 and of either sign
+    # by the formula.  The pair's sums are that one term, which tells a wall
+    # partner (viscosity eta_i, volume dp^2) from a fluid one
+    dx = 0.139                          # 0.5 / h rounds up, so one pair in six is past 2h by 1 - q/2
+    h = 1.3 * dx
+    n = 400
+    a = np.stack(np.meshgrid(np.arange(20.0), np.arange(20.0), indexing="ij"), axis=-1).reshape(-1, 2) * (8 * h)
+    ang = np.linspace(0.05, 3.0, n)
+    b = a + 2 * h * (1 - np.arange(n)[:, None] % 8 * 2.0**-53) * np.stack([np.cos(ang), np.sin(ang)], axis=1)
+    phases = [sphcases.Phase("fluid", a, rho0=1.0, eta=0.1, vel=np.full((n, 2), 0.01)),
+              sphcases.Phase("fluid", np.array([[-8 * h, -8 * h]]), rho0=3.0, eta=0.01),
+              sphcases.Phase("wall", b) if partner == "wall" else sphcases.Phase("wall", np.array([[-8 * h, 0.0]]))]
+    if partner == "fluid":
+        phases[1].pos = np.concatenate([phases[1].pos, b])
+    case = sphcases.Case(name="cutoff", dim=2, lo=[-8 * h] * 2, hi=[160 * h] * 2, dx=dx, gamma=0.0, c0=10.0, phases=phases)
+    out, held = [], []
+    for keep in (True, False):
+        c = S.case_from_spec(case, precision=64)
+        S.set_pair_geometry(c, keep)
+        S.step(c, 1)
+        held.append(S.debug_neighbors(c)[0].sum())
+        out.append([S.read_fields(c, f, 2) for f in FIELDS])
+        S.destroy(c)
+    assert held[0] == held[1] > 50
+    assert (np.abs(out[0][4][:n]) > 0).any() and np.abs(out[0][4][:n]).max() < 1e-30
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
