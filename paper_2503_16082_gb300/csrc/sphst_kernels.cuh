@@ -93,6 +93,13 @@
 #define SPH_SWEEPB_BOUNDS_M(T, LIST, MODE)                                                          \
     __launch_bounds__(256, (MODE) == 3 || !(LIST) ? 1 : sizeof(T) == 8 ? 2 : (MODE) == 2 ? SPHST_SWEEPB_MINB_ONE                  \
                                                          : (SPHST_SWEEPB_MINB > 0 ? SPHST_SWEEPB_MINB : 1))
+// sweep C of a batch with lists (FP32): with the constants in registers the
+// compiler left its gathers no room (52 to 55 registers); at 64 (4 blocks per
+// SM) a batch of 6M particles takes 582 us per launch in 3D against 719, with
+// work lists 585 against 604 (2D 154 against 178; the tiled 2D form is better
+// without, 147 against 167)
+#define SPH_SWEEPC_BOUNDS_M(T, D, LIST, MODE)                                                       \
+    __launch_bounds__(256, (LIST) && sizeof(T) == 4 && ((MODE) == 1 || ((MODE) == 0 && (D) == 3)) ? 4 : SPHST_SWEEP_MINB)
 
 namespace sphst {
 
@@ -1356,7 +1363,7 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
     const uint32_t ki = phase_of(pki);
     V4<T> g = {0, 0, 0, 0};
     if (ki != PH_WALL && d.n_fluid_phases == 2) {
-        const T two_phi = cp.two_phi[ki];
+        const T two_phi = sel(ki, cp.two_phi[0], cp.two_phi[1]);
         neighbors<LIST, false, false, T, D, PART_OTHER, L, U, CELL_PLACES_k_sweep_A>(d, cp, starts, l, snap, nullptr, i, si, pki,
             [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &G) {
                 const T s = vmul(vmul(two_phi, G.wd), volume_at(cp, kj, vol, j));
@@ -1659,6 +1666,16 @@ template <int MODE> __device__ __forceinline__ const CaseDesc &case_desc(const S
     if constexpr (MODE == MODE_ONE || MODE == MODE_FEW) return a.one;
     else return a.desc[c];
 }
+
+// A sweep's per-case constants: of the parameter block where the launch has
+// them; else, with the list, copied from memory before the pair loop.  Read
+// through a reference they were loaded again for every pair: per launch of a
+// batch of 6M particles B 876 us against 798, S 347 against 329, A 61 against
+// 57, V 1436 against 1244 (M, 658 against 790, keeps the reference).  The cell
+// walk, whose registers are short, reads them again (3D, 125k particles: B 259
+// us, with copies 321).
+template <bool LIST, int MODE, typename T>
+using Phys = std::conditional_t<!LIST || MODE == MODE_ONE || MODE == MODE_FEW, const CasePhys<T> &, const CasePhys<T>>;
 
 // Work items of a sweep launch: (tile, block of the tile) pairs; with L
 // lanes per particle a tile takes L blocks.  Without a work list (WORK
@@ -2054,8 +2071,9 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_M(SweepArgs a, const V4<T> *snap, const
     if (li >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
     if (!d.tvf_on && d.surface_corr != 1) return;
+    const CasePhys<T> &cp = phys<T>(d);
     const int64_t q = t.begin + li, i = particle_at(a, q);
-    sweep_M<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, bmat, bk, &a.st[t.c].status, threadIdx.x % L);
+    sweep_M<LIST, T, D, L>(d, cp, i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, bmat, bk, &a.st[t.c].status, threadIdx.x % L);
 }
 
 template <typename T, int D, bool LIST, int L = 1>
@@ -2066,8 +2084,9 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_V(SweepArgs a, const V4<T> *snap, const
     const int li = local_index<L>(blockIdx.x);
     if (li >= t.n || !a.st[t.c].active) return;
     const CaseDesc &d = a.desc[t.c];
+    Phys<LIST, MODE_TILES, T> cp = phys<T>(d);
     const int64_t q = t.begin + li, i = particle_at(a, q);
-    sweep_V<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vel, vol, bmat, acc_visc, pos,
+    sweep_V<LIST, T, D, L>(d, cp, i, a.starts, list_of<LIST, T>(a, d, q), snap, vel, vol, bmat, acc_visc, pos,
                         &a.st[t.c].status, threadIdx.x % L);
 }
 
@@ -2086,8 +2105,9 @@ __global__ void SPH_SWEEPAS_BOUNDS k_sweep_A(SweepArgs a, const V4<T> *snap, con
         const int li = local_index<L>(w);
         if (li >= t.n || !a.st[t.c].active) return;
         const CaseDesc &d = case_desc<MODE>(a, t.c);
+        Phys<LIST, MODE, T> cp = phys<T>(d);
         const int64_t q = t.begin + li, i = particle_at(a, q);
-        sweep_A<LIST, T, D, L>(d, phys<T>(d), i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, gradC,
+        sweep_A<LIST, T, D, L>(d, cp, i, a.starts, list_of<LIST, T>(a, d, q), snap, vol, gradC,
                                threadIdx.x % L);
     };
     if constexpr (MODE == MODE_WORK) {
@@ -2113,7 +2133,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4) k_sweep_A_band(Sw
         const BandEntry e(a, blist, t / L);
         if (!a.st[e.c].active) continue;
         const CaseDesc &d = a.desc[e.c];
-        sweep_A<true, T, D, L, AHEAD>(d, phys<T>(d), e.i, a.starts, list_of<true, T>(a, d, e.q), snap, vol, gradC, threadIdx.x % L);
+        const CasePhys<T> cp = phys<T>(d);
+        sweep_A<true, T, D, L, AHEAD>(d, cp, e.i, a.starts, list_of<true, T>(a, d, e.q), snap, vol, gradC, threadIdx.x % L);
     }
 }
 
@@ -2131,8 +2152,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) k_sweep_S(SweepAr
         const BandEntry e(a, blist, t / L);
         if (!a.st[e.c].active) continue;
         const CaseDesc &d = a.desc[e.c];
+        const CasePhys<T> cp = phys<T>(d);
         uint32_t ph;
-        sweep_B<true, 2, T, D, L, 4>(d, phys<T>(d), T(0), e.i, a.starts, list_of<true, T>(a, d, e.q), band, snap, vel, gradC,
+        sweep_B<true, 2, T, D, L, 4>(d, cp, T(0), e.i, a.starts, list_of<true, T>(a, d, e.q), band, snap, vel, gradC,
                                           nullptr, acc_surf, nullptr, &ph, threadIdx.x % L, bk, vol);
     }
 }
@@ -2162,9 +2184,10 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, MODE) k_sweep_B(SweepArgs a, const 
         uint32_t ph = PH_WALL;
         const int li = local_index<L>(w);
         if (li < t.n) {
+            Phys<LIST, MODE, T> cp = phys<T>(d);
             const int64_t q = t.begin + li, i = particle_at(a, q);
             const T dt = (T)a.st[t.c].dt;
-            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L, MODE == MODE_FEW ? 4 : PLAIN>(d, phys<T>(d), dt, i, a.starts, list_of<LIST, T>(a, d, q), band, snap, vel,
+            v2 = sweep_B<LIST, LIST ? 1 : 0, T, D, L, MODE == MODE_FEW ? 4 : PLAIN>(d, cp, dt, i, a.starts, list_of<LIST, T>(a, d, q), band, snap, vel,
                                                       gradC, acc_visc, acc_surf, vel_new, &ph, threadIdx.x % L,
                                                       LIST ? nullptr : bk, vol);
         }
@@ -2179,7 +2202,7 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, MODE) k_sweep_B(SweepArgs a, const 
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
-__global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho, T *vol,
+__global__ void SPH_SWEEPC_BOUNDS_M(T, D, LIST, MODE) k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho, T *vol,
                                            V4<T> *vel, V4<T> *pos) {
     follow();
     const auto item = [&](int64_t w) {
@@ -2187,9 +2210,10 @@ __global__ void SPH_SWEEP_BOUNDS k_sweep_C(SweepArgs a, const V4<T> *snap, const
         const int li = local_index<L>(w);
         if (li >= t.n || !a.st[t.c].active) return;
         const CaseDesc &d = case_desc<MODE>(a, t.c);
+        Phys<LIST, MODE, T> cp = phys<T>(d);
         const int64_t q = t.begin + li, i = particle_at(a, q);
         const T dt = (T)a.st[t.c].dt;
-        sweep_C<LIST, T, D, L, MODE == MODE_FEW && D == 2 ? 4 : AHEAD>(d, phys<T>(d), dt, i, a.starts, list_of<LIST, T>(a, d, q),
+        sweep_C<LIST, T, D, L, MODE == MODE_FEW && D == 2 ? 4 : AHEAD>(d, cp, dt, i, a.starts, list_of<LIST, T>(a, d, q),
                                snap, vel_new, drho, vol, vel, pos,
                                threadIdx.x % L);
     };
