@@ -213,8 +213,8 @@ __device__ __forceinline__ uint32_t ld_list(const uint32_t *p) {
 
 __device__ __forceinline__ double bits_to_d(unsigned long long b) { return __longlong_as_double((long long)b); }
 
-// explicitly rounded operations for the pair geometry, so that the cell walk
-// and the neighbour list produce bitwise-identical r_ij and r^2 for a pair
+// explicitly rounded operations for the pair geometry, so that every test of
+// a pair, by the cell walk and by the list build, finds the same r^2
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
@@ -355,14 +355,26 @@ __device__ __forceinline__ uint32_t cell_code(int ox, int oy, int oz) {
     return (uint32_t)(ox + 1) | ((uint32_t)(oy + 1) << 2) | (D == 3 ? ((uint32_t)(oz + 1) << 4) : 0u);
 }
 
-// r_ij = (s_i - o cs) - s_j of list entry e: the operations of the cell walk
-// (o cs is exact), so every test of a pair and every sum sees the same r_ij and
-// r^2, whichever way the pair was found
+// r_ij = (s_i - o cs) - s_j of an entry or cell code e (o cs is exact): the
+// operations of the cell walk.  Every test of a pair takes them, and the sums
+// of the cell walk, so list and walk hold the same pairs.
 template <typename T, int D>
 __device__ __forceinline__ void pair_offset(uint32_t e, const V4<T> &si, const V4<T> &sj, T cs, T &rx, T &ry, T &rz) {
     rx = sub_rn(fma_rn(-code_off(e & 3u, T()), cs, si.x), sj.x);
     ry = sub_rn(fma_rn(-code_off((e >> 2) & 3u, T()), cs, si.y), sj.y);
     rz = D == 3 ? sub_rn(fma_rn(-code_off((e >> 4) & 3u, T()), cs, si.z), sj.z) : T(0);
+}
+// r_ij = s_i - (s_j + o cs) of list entry e: the form of the list's sums, equal
+// to rounding.  Its rounding differs from neighbour to neighbour, where that
+// of s_i - o cs is common to a cell's: FP32 results lie 10% nearer to those
+// in 64 bits (1M particles, one step: 4.5e-7 against 5.0e-7).  Never zero for
+// a pair of the list: offsets lie in [0, cs), and s_j + o cs does not round
+// into that range unless o = 0, where both forms are one.
+template <typename T, int D>
+__device__ __forceinline__ void moved_offset(uint32_t e, const V4<T> &si, const V4<T> &sj, T cs, T &rx, T &ry, T &rz) {
+    rx = add_rn(si.x, fma_rn(-code_off(e & 3u, T()), cs, -sj.x));
+    ry = add_rn(si.y, fma_rn(-code_off((e >> 2) & 3u, T()), cs, -sj.y));
+    rz = D == 3 ? add_rn(si.z, fma_rn(-code_off((e >> 4) & 3u, T()), cs, -sj.z)) : T(0);
 }
 
 // How a sweep gathers its neighbours (U of walk_list), by measurement at 1M and
@@ -680,7 +692,7 @@ __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &
         walk_list<AUX, T, L, U>(l.p, c, snap, aux,
             [&](uint32_t e, const V4<T> &sj, const V4<T> &aj) {
                 T rx, ry, rz;
-                pair_offset<T, D>(e, si, sj, cs, rx, ry, rz);
+                moved_offset<T, D>(e, si, sj, cs, rx, ry, rz);
                 f(e >> NBR_SHIFT, phase_of(w_bits(sj.w)), aj, PairG<T>(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz), std::bool_constant<NEED_R>()));
             }, sub);
         return false;
@@ -2054,7 +2066,7 @@ __global__ void __launch_bounds__(32 * LG_WARPS) k_list_geo(SweepArgs a, const V
             const uint32_t e = ld_list(a.nbr + at);
             const V4<double> sj = ld4(snap + (e >> NBR_SHIFT));
             double rx, ry, rz;
-            pair_offset<double, D>(e, si, sj, cp.cs, rx, ry, rz);
+            moved_offset<double, D>(e, si, sj, cp.cs, rx, ry, rz);
             const PairG<double> g(cp, rx, ry, rz, norm2<double, D>(rx, ry, rz), std::true_type());
             ge[at] = V4<double>{g.x, g.y, g.z, phase_of(w_bits(sj.w)) == PH_WALL ? fabs(g.wd) : g.wd};
             gr[at] = RInv{g.r, g.inv};
