@@ -147,7 +147,8 @@ typedef struct {
     int32_t grid_pad;       /* spare cells around the initial bounding box (>= 1) */
     int32_t block;          /* threads per block of the pair sweeps: a multiple
                                of 32 in 32..256 (FP64 engines too small to
-                               fill the GPU with them take smaller ones; no
+                               fill the GPU with them take smaller ones, and
+                               engines with a cell-walk case 128 at most; no
                                result depends on it)                          */
     int64_t max_substeps;   /* per advection step before SPHST_ERR_STALLED     */
     double  cfl_ad;         /* factor of the advection criterion, Eq. 16 (0.1) */
@@ -177,7 +178,8 @@ typedef struct {
                                by the rounding of the reordered sum).  More
                                lanes spread small cases over more of the GPU.
                                Speed only; a batch uses its first case's
-                               value.  The cell walk always takes 2.         */
+                               value.  The cell walk takes 2, or 1 with the
+                               same bits where that fills the GPU.           */
     int32_t penalty_scope;  /* SPHST_PENALTY_SCOPE_*                           */
     int32_t wall_form;      /* SPHST_WALL_* (pressure of wall pairs)           */
     int32_t work_lists;     /* batches only (the first case's value counts):

@@ -20,6 +20,21 @@ namespace sphst {
 
 enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
 
+// SPH_CELLS: a cell-walk class's launch, with one thread or CELL_LANES lanes per
+// particle by the class's population
+#define SPH_CELLS(KERN, D, ALONE, LANED, ...)                                                                        \
+    {                                                                                                                \
+        bool alone_ = false;                                                                                         \
+        if constexpr (CELL_ALONE_##KERN<T, D> < CELL_NEVER) {                                                        \
+            alone_ = cls_fluid[k_] >= sm_count * CELL_ALONE_##KERN<T, D>;                                            \
+            if (alone_) launch_next(SPH_KERNEL ALONE, g_, block, 0, stream, a_, __VA_ARGS__);                        \
+        }                                                                                                            \
+        if (!alone_)                                                                                                 \
+            launch_next(SPH_KERNEL LANED, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, \
+                        a_, __VA_ARGS__);                                                                            \
+    }
+#define SPH_KERNEL(...) __VA_ARGS__
+
 // Tile classes: 0 = 3D list, 1 = 2D list, 2 = 3D cell walk, 3 = 2D cell walk.
 // SPH_CLASSES_F(K0, NCLS, KERN, args...) launches KERN<T, D, LIST> over the
 // slot tiles of each non-empty class from K0 on.
@@ -31,8 +46,8 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         switch (k_) {                                                                  \
         case 0: launch_next(KERN<T, 3, true>, g_, block, 0, stream, a_, __VA_ARGS__); break;    \
         case 1: launch_next(KERN<T, 2, true>, g_, block, 0, stream, a_, __VA_ARGS__); break;    \
-        case 2: launch_next(KERN<T, 3, false, CELL_LANES>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break;   \
-        default: launch_next(KERN<T, 2, false, CELL_LANES>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break;  \
+        case 2: SPH_CELLS(KERN, 3, (KERN<T, 3, false, 1>), (KERN<T, 3, false, CELL_LANES>), __VA_ARGS__) break;   \
+        default: SPH_CELLS(KERN, 2, (KERN<T, 2, false, 1>), (KERN<T, 2, false, CELL_LANES>), __VA_ARGS__) break;  \
         }                                                                              \
     }
 
@@ -72,8 +87,8 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         switch (k_) {                                                                                  \
         case 0: SPH_LANES_M(KERN, 3, LN, MODE, __VA_ARGS__) break;                                     \
         case 1: SPH_LANES_M(KERN, 2, LN, MODE, __VA_ARGS__) break;                                     \
-        case 2: launch_next(KERN<T, 3, false, CELL_LANES, CELL_MODE(MODE)>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break; \
-        default: launch_next(KERN<T, 2, false, CELL_LANES, CELL_MODE(MODE)>, g_ * CELL_LANES, block, cell_walk_bytes<T>(block, CELL_PLACES_##KERN), stream, a_, __VA_ARGS__); break;\
+        case 2: SPH_CELLS(KERN, 3, (KERN<T, 3, false, 1, CELL_MODE(MODE)>), (KERN<T, 3, false, CELL_LANES, CELL_MODE(MODE)>), __VA_ARGS__) break; \
+        default: SPH_CELLS(KERN, 2, (KERN<T, 2, false, 1, CELL_MODE(MODE)>), (KERN<T, 2, false, CELL_LANES, CELL_MODE(MODE)>), __VA_ARGS__) break;\
         }                                                                                              \
     }
 
@@ -136,6 +151,7 @@ template <typename T> struct EngineT : Engine {
     int64_t n = 0, table_total = 0, n_tiles = 0, max_case_n = 0;
     int64_t cls_b[4] = {0, 0, 0, 0}, cls_n[4] = {0, 0, 0, 0};   // tile range of each class
     int64_t cls_fb[4] = {0, 0, 0, 0}, cls_fn[4] = {0, 0, 0, 0}; // the same over fluid ranks
+    int64_t cls_fluid[4] = {0, 0, 0, 0};                         // fluid particles of each class
     int64_t n_ftiles = 0;
     int ncases = 0, block = 128, lanes = 1;
     bool few = false;                               // a one-case engine that leaves the SMs with few warps
@@ -242,6 +258,9 @@ template <typename T> struct EngineT : Engine {
         for (CaseRec *r : cases) fluid += r->n_fluid;
         if (sizeof(T) == 8)
             while (block > 32 && fluid * lanes < sm_count * MIN_BLOCKS_PER_SM * block) block = block / 2 / 32 * 32;
+        // the cell walk's places are shared memory per thread: blocks of more than
+        // CELL_BLOCK_MAX would leave a thread fewer than it wants
+        if (list_fluid < fluid) block = std::min(block, CELL_BLOCK_MAX);
         few = list_fluid * lanes <= sm_count * FEW_MAX_PER_SM;
         for (int c = 0; c < ncases; ++c) {
             CaseRec *r = cases[c];
@@ -269,6 +288,7 @@ template <typename T> struct EngineT : Engine {
             }
             d.geo_base = -1;
             h_desc[c] = d;
+            cls_fluid[tile_class(d)] += r->n_fluid;
             if (r->P.loop_mode == SPHST_LOOP_HOST) loop_mode = SPHST_LOOP_HOST;
         }
         if (any_list && n >= ((int64_t)1 << (32 - NBR_SHIFT))) {

@@ -90,8 +90,8 @@
 #endif
 // sweep B of a one-case engine reads its per-case constants from the
 // parameter block, which leaves it room for more resident blocks
-#define SPH_SWEEPB_BOUNDS_M(T, LIST, MODE)                                                          \
-    __launch_bounds__(256, (MODE) == 3 || !(LIST) ? 1 : sizeof(T) == 8 ? 2 : (MODE) == 2 ? SPHST_SWEEPB_MINB_ONE                  \
+#define SPH_SWEEPB_BOUNDS_M(T, LIST, L, MODE)                                                          \
+    __launch_bounds__(256, (MODE) == 3 || (!(LIST) && (L) > 1) ? 1 : !(LIST) ? 4 : sizeof(T) == 8 ? 2 : (MODE) == 2 ? SPHST_SWEEPB_MINB_ONE                  \
                                                          : (SPHST_SWEEPB_MINB > 0 ? SPHST_SWEEPB_MINB : 1))
 // sweep C of a batch with lists (FP32): with the constants in registers the
 // compiler left its gathers no room (52 to 55 registers); at 64 (4 blocks per
@@ -296,40 +296,53 @@ void launch_next(void (*kernel)(P...), unsigned grid, dim3 block, size_t shared,
 
 // --------------------------------------------------------------- cell walk
 // Calls f(j, snap_j, r_ij vector, r^2) for every j != i with 0 < r_ij < 2h in
-// the 3^D cells around i's cell.  r_ij = s_i - s_j - o cs, where o is the
-// neighbour cell's offset, because both offsets are taken from their own
-// cell origins.  Returns true when a coincident particle was met.
-template <typename T, int D, typename F>
+// the 3^D cells around i's cell, x fastest, and next() after each cell (once
+// for an odd number of cells that are off the grid).  r_ij = s_i - s_j - o cs,
+// where o is the neighbour cell's offset, because both offsets are taken from
+// their own cell origins.  OTHER: only particles of the other fluid, which is
+// asked first (most of the fluid has none around).  Returns true when a
+// coincident particle was met.
+template <bool OTHER, typename T, int D, typename F, typename N>
 __device__ __forceinline__ bool walk(const CaseDesc &d, const CasePhys<T> &cp,
                                      const uint32_t *__restrict__ starts,
                                      const V4<T> *__restrict__ snap, int64_t i,
-                                     const V4<T> &si, uint32_t pki, F &&f) {
-    constexpr int NC = D == 3 ? 27 : 9;
+                                     const V4<T> &si, uint32_t pki, F &&f, N &&next) {
     const int cx = cell_x<D>(pki), cy = cell_y<D>(pki), cz = cell_z<D>(pki);
-    const uint32_t toff = (uint32_t)d.table_off;
+    const uint32_t toff = (uint32_t)d.table_off, other = phase_of(pki) ^ 1u;
     const T cs = cp.cs, R2 = cp.four_h2;
     bool coincident = false;
-    for (int q = 0; q < NC; ++q) {
-        const int ox = q % 3 - 1, oy = q / 3 % 3 - 1, oz = D == 3 ? q / 9 - 1 : 0;
-        int nx = cx + ox, ny = cy + oy, nz = cz + oz;
-        if (!wrap_cell(d, 0, nx) || !wrap_cell(d, 1, ny) || (D == 3 && !wrap_cell(d, 2, nz))) continue;
-        const T sx = sub_rn(si.x, mul_rn(T(ox), cs)), sy = sub_rn(si.y, mul_rn(T(oy), cs));
+    for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz) {
+        int nz = cz + oz;
+        if (D == 3 && !wrap_cell(d, 2, nz)) { next(); continue; }
         const T sz = D == 3 ? sub_rn(si.z, mul_rn(T(oz), cs)) : T(0);
-        const uint32_t m = toff + morton<D>(nx, ny, nz);
-        const uint32_t b = __ldg(starts + m), e = __ldg(starts + m + 1);
-        for (uint32_t j = b; j < e; ++j) {
-            const V4<T> sj = ld4(snap + j);
-            const T rx = sub_rn(sx, sj.x), ry = sub_rn(sy, sj.y);
-            const T rz = D == 3 ? sub_rn(sz, sj.z) : T(0);
-            const T r2 = norm2<T, D>(rx, ry, rz);
-            if (r2 < R2 && j != (uint32_t)i) {
-                if (r2 > T(0)) f(j, sj, rx, ry, rz, r2);
-                else coincident = true;
+        for (int oy = -1; oy <= 1; ++oy) {
+            int ny = cy + oy;
+            if (!wrap_cell(d, 1, ny)) { next(); continue; }
+            const T sy = sub_rn(si.y, mul_rn(T(oy), cs));
+            for (int ox = -1; ox <= 1; ++ox) {
+                int nx = cx + ox;
+                if (wrap_cell(d, 0, nx)) {
+                    const T sx = sub_rn(si.x, mul_rn(T(ox), cs));
+                    const uint32_t m = toff + morton<D>(nx, ny, nz);
+                    const uint32_t b = __ldg(starts + m), e = __ldg(starts + m + 1);
+                    for (uint32_t j = b; j < e; ++j) {
+                        const V4<T> sj = ld4(snap + j);
+                        const T rx = sub_rn(sx, sj.x), ry = sub_rn(sy, sj.y);
+                        const T rz = D == 3 ? sub_rn(sz, sj.z) : T(0);
+                        const T r2 = norm2<T, D>(rx, ry, rz);
+                        if ((!OTHER || phase_of(w_bits(sj.w)) == other) && r2 < R2 && j != (uint32_t)i) {
+                            if (r2 > T(0)) f(j, sj, rx, ry, rz, r2);
+                            else coincident = true;
+                        }
+                    }
+                }
+                next();
             }
         }
     }
     return coincident;
 }
+struct Nothing { __device__ __forceinline__ void operator()() const {} };
 
 // Neighbour list of the frozen configuration.  A slot is one fluid particle,
 // by its rank among them.  The slot of local number r holds entry k at word
@@ -557,8 +570,7 @@ __device__ __forceinline__ void walk_geo(const ListRef<double> &l, uint32_t c, c
 // all lanes evaluate what they have, in the walk's order (the same sums).
 // With two lanes per particle, 30k particles in 3D: FP32 A 76 -> 52, B 308 ->
 // 92, C 150 -> 68 us; FP64 A 614 -> 388, B 4381 -> 1118, C 1689 -> 703.  125k:
-// A 87 -> 101, B 376 -> 257, C 187 -> 168; at 1M, where one lane per particle
-// filled the chip as well, A 458 -> 600, B 1789 -> 1775, C 1001 -> 1043.
+// A 87 -> 101, B 376 -> 257, C 187 -> 168.
 // Lanes per particle: lane `sub` takes the cells sub, sub + L, ... of the 3^D,
 // and the lanes add their sums in a fixed order.  One lane leaves a case of 30k
 // particles 6 warps per SM, each waiting for its candidates.
@@ -571,6 +583,26 @@ constexpr int CELL_LANES = 2;
 constexpr int CELL_PLACES_MAX = 56;
 constexpr int CELL_PLACES_k_sweep_A = 20, CELL_PLACES_k_sweep_C = 32;
 constexpr int CELL_PLACES_k_sweep_B = 56, CELL_PLACES_k_sweep_V = 56, CELL_PLACES_k_sweep_M = 32, CELL_PLACES_k_debug_neighbors = 32;
+// From this many particles per SM on a sweep takes one thread per particle,
+// which evaluates its pairs where it finds them: the chip is full then, and
+// what lanes and places spare no longer pays for their own work.  Two lanes
+// against one thread, us per launch (FP32): A in 3D at 822 particles per SM 100
+// and 101, 2775 267 and 235, in 2D at 592 22 and 22, 2368 51 and 41; C in 3D at
+// 822 166 and 186, 2775 460 and 439, 6578 1046 and 905, in 2D at 1332 46 and
+// 55, 2368 73 and 69, 6578 188 and 166; B in 2D at 1332 92 and 99, 2368 155 and
+// 133, 6578 426 and 324 (M and V alike); B in 3D and FP64 pairs, which are
+// dear, stay with the lanes, but for A in 3D (177: 428 and 446, 822: 1777 and
+// 1370).
+constexpr int64_t CELL_NEVER = (int64_t)1 << 40;
+template <typename T, int D> constexpr int64_t CELL_ALONE_k_sweep_A = sizeof(T) == 4 ? 1024 : D == 3 ? 512 : CELL_NEVER;
+template <typename T, int D> constexpr int64_t CELL_ALONE_k_sweep_C = sizeof(T) == 4 ? 2048 : CELL_NEVER;
+template <typename T, int D> constexpr int64_t CELL_ALONE_k_sweep_B = sizeof(T) == 4 && D == 2 ? 2048 : CELL_NEVER;
+template <typename T, int D> constexpr int64_t CELL_ALONE_k_sweep_V = CELL_ALONE_k_sweep_B<T, D>;
+template <typename T, int D> constexpr int64_t CELL_ALONE_k_sweep_M = CELL_ALONE_k_sweep_B<T, D>;
+template <typename T, int D> constexpr int64_t CELL_ALONE_k_debug_neighbors = CELL_NEVER;
+// 1M particles in 3D: B 1784 us in blocks of 128, 2040 of 160 (5 instead of 6
+// blocks per SM), 2680 of 256 (38 places); 2D: 426 and 604
+constexpr int CELL_BLOCK_MAX = 128;
 // at most 48 KB per block, so that no block size asks for an opt-in
 template <typename T> __host__ __device__ inline int cell_places(int threads, int want) {
     return min(sizeof(T) == 8 ? CELL_PLACES_MAX : want, 49152 / (threads * 5));
@@ -677,10 +709,10 @@ __device__ __forceinline__ bool walk_cells(const CaseDesc &d, const CasePhys<T> 
 // neighbours of particle i as f(j, kind of j, aux_j, geometry), from its list
 // or from the cell walk.  NEED_R: f reads r or 1/r (FULL of PairG).
 template <bool LIST, bool AUX, bool NEED_R, typename T, int D, int PART = PART_ALL, int L = 1, int U = PLAIN, int PLACES = 0,
-          typename F>
+          typename F, typename N = Nothing>
 __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &cp, const uint32_t *starts,
                                           const ListRef<T> &l, const V4<T> *snap, const V4<T> *aux, int64_t i,
-                                          const V4<T> &si, uint32_t pki, F &&f, uint32_t sub = 0) {
+                                          const V4<T> &si, uint32_t pki, F &&f, uint32_t sub = 0, N &&next = N()) {
     if constexpr (LIST) {
         const uint32_t c = PART == PART_OTHER ? l.count >> 16 : l.count & CNT_MASK;
         if constexpr (sizeof(T) == 8)
@@ -696,6 +728,11 @@ __device__ __forceinline__ bool neighbors(const CaseDesc &d, const CasePhys<T> &
                 f(e >> NBR_SHIFT, phase_of(w_bits(sj.w)), aj, PairG<T>(cp, rx, ry, rz, norm2<T, D>(rx, ry, rz), std::bool_constant<NEED_R>()));
             }, sub);
         return false;
+    } else if constexpr (L == 1) {
+        return walk<PART == PART_OTHER, T, D>(d, cp, starts, snap, i, si, pki,
+            [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
+                f(j, phase_of(w_bits(sj.w)), AUX ? ld4(aux + j) : sj, PairG<T>(cp, rx, ry, rz, r2, std::bool_constant<NEED_R>()));
+            }, next);
     } else {
         return walk_cells<PLACES, AUX, false, PART == PART_OTHER, NEED_R, T, D, L>(d, cp, starts, snap, aux, nullptr, i, si, pki, sub, f);
     }
@@ -713,6 +750,28 @@ template <int L, typename T> __device__ __forceinline__ T group_sum(T v) {
     }
     return v;
 }
+
+// Where CELL_LANES = 2 lanes share a particle in the cell walk, one takes the
+// even cells and the other the odd ones.  A thread that takes them all keeps the
+// two sums apart, exchanging them from cell to cell, and adds them at the end:
+// the same bits.  walk(next): the walk, which calls next() between cells.
+template <bool LIST, int L, typename T, int N> struct Sums {
+    T *const now[N];
+    T apart[N] = {};
+    template <typename W> __device__ __forceinline__ void over(W &&walk) {
+        static_assert(CELL_LANES == 2);
+        if constexpr (!LIST && L == 1) {
+            walk([&]() {
+#pragma unroll
+                for (int k = 0; k < N; ++k) { const T v = *now[k]; *now[k] = apart[k]; apart[k] = v; }
+            });
+#pragma unroll
+            for (int k = 0; k < N; ++k) *now[k] = add_rn(*now[k], apart[k]);
+        } else {
+            walk(Nothing());
+        }
+    }
+};
 
 // (v_j - v_i) . carrier, from -v_i
 template <typename T, int D>
@@ -1256,13 +1315,16 @@ __device__ __forceinline__ void sweep_M(const CaseDesc &d, const CasePhys<T> &cp
     if (ki == PH_WALL) return;
     const bool own = bk != nullptr && d.surface_corr == 1;
     Moment<T> M{}, Mk{};
-    const bool coinc = neighbors<LIST, false, true, T, D, PART_ALL, L, AHEAD, CELL_PLACES_k_sweep_M>(d, cp, starts, l, snap, nullptr, i, si, pki,
-        [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &g) {
-            const T w = vmul(g.outer(), volume_at(cp, kj, vol, j));
-            M.template add<D>(w, g.x, g.y, g.z);
-            // the same sum over i's own fluid (surface_corr reading of Eq. 33)
-            if (own && kj == ki) Mk.template add<D>(w, g.x, g.y, g.z);
-        }, sub);
+    bool coinc = false;
+    Sums<LIST, L, T, 12>{{&M.m00, &M.m01, &M.m02, &M.m11, &M.m12, &M.m22, &Mk.m00, &Mk.m01, &Mk.m02, &Mk.m11, &Mk.m12, &Mk.m22}}.over([&](auto &&next) {
+        coinc = neighbors<LIST, false, true, T, D, PART_ALL, L, AHEAD, CELL_PLACES_k_sweep_M>(d, cp, starts, l, snap, nullptr, i, si, pki,
+            [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &g) {
+                const T w = vmul(g.outer(), volume_at(cp, kj, vol, j));
+                M.template add<D>(w, g.x, g.y, g.z);
+                // the same sum over i's own fluid (surface_corr reading of Eq. 33)
+                if (own && kj == ki) Mk.template add<D>(w, g.x, g.y, g.z);
+            }, sub, next);
+    });
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
     M.template group<L>();
     if (own) Mk.template group<L>();
@@ -1349,15 +1411,18 @@ __device__ __forceinline__ void sweep_V(const CaseDesc &d, const CasePhys<T> &cp
         b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y;
     }
     ViscSum<T> S{};
-    const bool coinc = neighbors<LIST, true, true, T, D, PART_ALL, L, AHEAD, CELL_PLACES_k_sweep_V>(d, cp, starts, l, snap, vel, i, si, pki,
-        [&](uint32_t j, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
-            const bool wall = kj == PH_WALL;
-            V4<T> B0{}, B1{};
-            if (tvf && !wall) { B0 = bmat[2 * j]; if (D == 3) B1 = bmat[2 * j + 1]; }
-            const T V = sizeof(T) == 8 ? vol[j] : volume_of(cp, kj, vj.w);
-            S.template add<D>(vmul(g.dW_r(), V), vmul(g.wd, V), eta(kj), tvf, vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z, b, wall,
-                              B0, B1);
-        }, sub);
+    bool coinc = false;
+    Sums<LIST, L, T, 6>{{&S.ax, &S.ay, &S.az, &S.sx, &S.sy, &S.sz}}.over([&](auto &&next) {
+        coinc = neighbors<LIST, true, true, T, D, PART_ALL, L, AHEAD, CELL_PLACES_k_sweep_V>(d, cp, starts, l, snap, vel, i, si, pki,
+            [&](uint32_t j, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
+                const bool wall = kj == PH_WALL;
+                V4<T> B0{}, B1{};
+                if (tvf && !wall) { B0 = bmat[2 * j]; if (D == 3) B1 = bmat[2 * j + 1]; }
+                const T V = sizeof(T) == 8 ? vol[j] : volume_of(cp, kj, vj.w);
+                S.template add<D>(vmul(g.dW_r(), V), vmul(g.wd, V), eta(kj), tvf, vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z, b, wall,
+                                  B0, B1);
+            }, sub, next);
+    });
     if (coinc) atomicCAS(status, 0, DEV_ERR_COINCIDENT);
     S.template group<L>();
     if (sub != 0) return;
@@ -1376,13 +1441,15 @@ __device__ __forceinline__ void sweep_A(const CaseDesc &d, const CasePhys<T> &cp
     V4<T> g = {0, 0, 0, 0};
     if (ki != PH_WALL && d.n_fluid_phases == 2) {
         const T two_phi = sel(ki, cp.two_phi[0], cp.two_phi[1]);
-        neighbors<LIST, false, false, T, D, PART_OTHER, L, U, CELL_PLACES_k_sweep_A>(d, cp, starts, l, snap, nullptr, i, si, pki,
-            [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &G) {
-                const T s = vmul(vmul(two_phi, G.wd), volume_at(cp, kj, vol, j));
-                g.x = fma_rn(s, G.x, g.x);
-                g.y = fma_rn(s, G.y, g.y);
-                if (D == 3) g.z = fma_rn(s, G.z, g.z);
-            }, sub);
+        Sums<LIST, L, T, 3>{{&g.x, &g.y, &g.z}}.over([&](auto &&next) {
+            neighbors<LIST, false, false, T, D, PART_OTHER, L, U, CELL_PLACES_k_sweep_A>(d, cp, starts, l, snap, nullptr, i, si, pki,
+                [&](uint32_t j, uint32_t kj, const V4<T> &, const PairG<T> &G) {
+                    const T s = vmul(vmul(two_phi, G.wd), volume_at(cp, kj, vol, j));
+                    g.x = fma_rn(s, G.x, g.x);
+                    g.y = fma_rn(s, G.y, g.y);
+                    if (D == 3) g.z = fma_rn(s, G.z, g.z);
+                }, sub, next);
+        });
         g.x = group_sum<L>(g.x);
         g.y = group_sum<L>(g.y);
         if (D == 3) g.z = group_sum<L>(g.z);
@@ -1578,12 +1645,22 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             asx = as.x; asy = as.y; asz = as.z;
         }
     } else {
-        if (surface_on)
-            walk_cells<CELL_PLACES_k_sweep_B, true, true, false, true, T, D, L>(d, cp, starts, snap, vel, gradC, i, si, pki, sub,
-                [&](uint32_t j, uint32_t kj, const V4<T> &vj, const V4<T> &nj, const PairG<T> &g) {
-                    pressure(j, kj, vj, g);
-                    surface(j, kj, nj, g);
-                });
+        const auto both = [&](uint32_t j, uint32_t kj, const V4<T> &vj, const V4<T> &nj, const PairG<T> &g) {
+            pressure(j, kj, vj, g);
+            surface(j, kj, nj, g);
+        };
+        if constexpr (L == 1)
+            Sums<LIST, L, T, 6>{{&apx, &apy, &apz, &asx, &asy, &asz}}.over([&](auto &&next) {
+                walk<false, T, D>(d, cp, starts, snap, i, si, pki,
+                    [&](uint32_t j, const V4<T> &sj, T rx, T ry, T rz, T r2) {
+                        const uint32_t kj = phase_of(w_bits(sj.w));
+                        const PairG<T> g(cp, rx, ry, rz, r2, std::true_type());
+                        pressure(j, kj, ld4(vel + j), g);
+                        if (surface_on) surface(j, kj, ld4(gradC + j), g);
+                    }, next);
+            });
+        else if (surface_on)
+            walk_cells<CELL_PLACES_k_sweep_B, true, true, false, true, T, D, L>(d, cp, starts, snap, vel, gradC, i, si, pki, sub, both);
         else
             walk_cells<CELL_PLACES_k_sweep_B, true, false, false, false, T, D, L>(d, cp, starts, snap, vel, nullptr, i, si, pki, sub, pressure);
         apx = group_sum<L>(apx);
@@ -1630,11 +1707,13 @@ __device__ __forceinline__ void sweep_C(const CaseDesc &d, const CasePhys<T> &cp
     const T rho_i = add_rn(sel(ki, cp.rho0[0], cp.rho0[1]), vi.w);
     const T nsc0 = d.vstar_printed ? cp.c0 : -cp.c0, sb_i = mul_rn(-nsc0, vi.w);
     T s = 0;
-    neighbors<LIST, true, false, T, D, PART_ALL, L, U, CELL_PLACES_k_sweep_C>(d, cp, starts, l, snap, vel_new, i, si, pki,
-        [&](uint32_t, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
-            const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z);
-            s = vfma(continuity_factor<T>(cp, kj, vj.w, dot, g, rho_i, sb_i, nsc0), g.dW(), s);
-        }, sub);
+    Sums<LIST, L, T, 1>{{&s}}.over([&](auto &&next) {
+        neighbors<LIST, true, false, T, D, PART_ALL, L, U, CELL_PLACES_k_sweep_C>(d, cp, starts, l, snap, vel_new, i, si, pki,
+            [&](uint32_t, uint32_t kj, const V4<T> &vj, const PairG<T> &g) {
+                const T dot = pair_dot<T, D>(vj, -vi.x, -vi.y, -vi.z, g.x, g.y, g.z);
+                s = vfma(continuity_factor<T>(cp, kj, vj.w, dot, g, rho_i, sb_i, nsc0), g.dW(), s);
+            }, sub, next);
+    });
     s = group_sum<L>(s);
     if (sub == 0) store_C<T, D>(cp, ki, i, dt, rho_i, s, vi, drho, vol, vel, pos);
 }
@@ -2184,7 +2263,7 @@ __device__ __forceinline__ void reduce_vmax(const SweepArgs &a, int c, uint32_t 
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
-__global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, MODE) k_sweep_B(SweepArgs a, const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
+__global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, L, MODE) k_sweep_B(SweepArgs a, const uint8_t *band, const V4<T> *snap, const V4<T> *vel,
                                             const V4<T> *gradC, const V4<T> *acc_visc, V4<T> *acc_surf,
                                             V4<T> *vel_new, const V4<T> *bk, const T *vol) {
     follow();
@@ -2426,8 +2505,8 @@ __device__ void count_nbrs(const CaseDesc &d, int64_t i, const uint32_t *starts,
                            const uint32_t *id, int *out) {
     const V4<T> si = ld4(snap + i);
     int cnt = 0;
-    walk<T, D>(d, phys<T>(d), starts, snap, i, si, w_bits(si.w),
-               [&](uint32_t, const V4<T> &, T, T, T, T) { ++cnt; });
+    walk<false, T, D>(d, phys<T>(d), starts, snap, i, si, w_bits(si.w),
+               [&](uint32_t, const V4<T> &, T, T, T, T) { ++cnt; }, Nothing());
     out[id[i]] = cnt;
 }
 
