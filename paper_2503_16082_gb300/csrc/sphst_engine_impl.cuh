@@ -120,7 +120,7 @@ template <typename T> struct EngineT : Engine {
     uint32_t *starts = nullptr, *block_sums = nullptr;
     uint32_t *nbr = nullptr, *nbr_cnt = nullptr;   // neighbour lists (ELL per case) and counts
     V4<T> *lgeo = nullptr;                          // (e_ij, W') and (r, 1/r) of each list entry (FP64)
-    int64_t geo_bytes = 0;
+    int64_t geo_entries = 0, geo_bytes = 0;
     RInv *lrinv = nullptr;
     uint8_t *band = nullptr;                        // interface band of the frozen configuration
     uint64_t *band_list = nullptr;                  // band particles per list class (case << 32 | index)
@@ -172,43 +172,47 @@ template <typename T> struct EngineT : Engine {
         if (graph) cudaGraphDestroy(graph);
         if (stream && own_stream) cudaStreamDestroy(stream);
         if (arena) cudaFree(arena);
-        if (lgeo) {
-            cudaFree(lgeo);
-            geometry_in_use -= geo_bytes;
-        }
+        geometry_in_use -= geo_bytes;
     }
 
     // FP64 keeps the lists' pair geometry where memory is plentiful: the results
-    // are the same without it.  An allocation of its own, after everything an
-    // engine needs, so that no case fails for it; within one engine the cases
-    // take it in order until PAIR_GEOMETRY_MAX.  Nothing past a list's count is
-    // read, so it is not cleared.
+    // are the same without it.  Within one engine the cases take it in order
+    // until PAIR_GEOMETRY_MAX; it lies behind everything an engine needs, in the
+    // same allocation (one of its own cost 50 us of set-up and 40 of release),
+    // which is tried again without it.  Nothing past a list's count is read, so
+    // it is not cleared.
     static inline std::atomic<int64_t> geometry_in_use{0};
-    void place_geometry(const std::vector<CaseRec *> &cases) {
-        if (sizeof(T) == 4) return;
+    void plan_geometry(const std::vector<CaseRec *> &cases) {
         int64_t entries = 0;
-        for (int c = 0; c < ncases; ++c) {
-            const int64_t e = geometry_entries(h_desc[c].nbr_k, cases[c]->n_fluid);
-            if (h_desc[c].nbr_mode != 0 || !cases[c]->keep_geometry || (entries + e) * PAIR_GEOMETRY_BYTES > PAIR_GEOMETRY_MAX) continue;
-            h_desc[c].geo_base = entries;
-            entries += e;
-        }
-        if (!entries) return;
+        if (sizeof(T) == 8)
+            for (int c = 0; c < ncases; ++c) {
+                const int64_t e = geometry_entries(h_desc[c].nbr_k, cases[c]->n_fluid);
+                if (h_desc[c].nbr_mode != 0 || !cases[c]->keep_geometry || (entries + e) * PAIR_GEOMETRY_BYTES > PAIR_GEOMETRY_MAX) continue;
+                h_desc[c].geo_base = entries;
+                entries += e;
+            }
+        geo_entries = entries;
         geo_bytes = entries * PAIR_GEOMETRY_BYTES;
-        size_t mem_free = 0, mem_total = 0;
+        if (!entries) return;
         const int64_t used = geometry_in_use.fetch_add(geo_bytes) + geo_bytes;
         // a quarter of what is free at most; small ones are not worth the question
+        size_t mem_free = 0, mem_total = 0;
         bool ok = used <= PAIR_GEOMETRY_PROCESS_MAX;
         if (ok && geo_bytes > ((int64_t)64 << 20))
             ok = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && (size_t)geo_bytes <= mem_free / 4;
-        if (ok && cudaMalloc(&lgeo, (size_t)geo_bytes) == cudaSuccess) {
-            lrinv = (RInv *)(lgeo + entries);
-            return;
-        }
-        cudaGetLastError();
-        lgeo = nullptr;
+        if (!ok) drop_geometry();
+    }
+    void drop_geometry() {
         geometry_in_use -= geo_bytes;
+        geo_bytes = geo_entries = 0;
         for (CaseDesc &d : h_desc) d.geo_base = -1;
+    }
+
+    // blocks of a kernel that are resident on one SM; asked once per process
+    template <typename F> static int resident_blocks(F *kernel, int threads) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)kernel, threads, 0) != cudaSuccess) cudaGetLastError();
+        return std::max(per_sm, 1);
     }
 
     void *dev_array(int which) override {
@@ -327,7 +331,13 @@ template <typename T> struct EngineT : Engine {
         size_t o_band = take(nn);
         size_t o_blist = take(nn * 8), o_bcount = take(64), o_clist = take(nn * 8);
         size_t o_diag = take((size_t)(DIAG_BLOCKS + 1) * DIAG_Q * sizeof(double));
-        cudaError_t e = cudaMalloc(&arena, off);
+        plan_geometry(cases);
+        cudaError_t e = cudaMalloc(&arena, off + (size_t)geo_bytes);
+        if (e != cudaSuccess && geo_bytes) {
+            cudaGetLastError();
+            drop_geometry();
+            e = cudaMalloc(&arena, off);
+        }
         if (e != cudaSuccess) {
             arena = nullptr;
             cudaGetLastError();
@@ -361,7 +371,10 @@ template <typename T> struct EngineT : Engine {
         cell_list = (uint64_t *)(b + o_clist);
         d_diag = (double *)(b + o_diag);
         SPH_CK(cudaMemsetAsync(arena, 0, off, stream));
-        place_geometry(cases);
+        if (geo_bytes) {
+            lgeo = (V4<T> *)(b + off);
+            lrinv = (RInv *)(lgeo + geo_entries);
+        }
         // tiles, grouped by class
         std::vector<Tile> tiles;
         tiles.reserve(n_tiles);
@@ -416,12 +429,8 @@ template <typename T> struct EngineT : Engine {
             SPH_CK(cudaMemcpyAsync(d_cls0, cls0.data(), 8 * 4, cudaMemcpyHostToDevice, stream));
             work_cap = sm_count * 16;
         }
-        for (int k = 0; k < 2; ++k) {
-            int per_sm = 0;
-            const void *f = k == 0 ? (const void *)k_build_list<T, 3> : (const void *)k_build_list<T, 2>;
-            SPH_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, LB_WARPS * 32, 0));
-            lb_blocks[k] = std::max(per_sm, 1) * sm_count;
-        }
+        static const int resident[2] = {resident_blocks(k_build_list<T, 3>, LB_WARPS * 32), resident_blocks(k_build_list<T, 2>, LB_WARPS * 32)};
+        for (int k = 0; k < 2; ++k) lb_blocks[k] = resident[k] * sm_count;
         SPH_CK(cudaMemcpyAsync(d_desc, h_desc.data(), sizeof(CaseDesc) * ncases, cudaMemcpyHostToDevice, stream));
         // fill each case
         for (int c = 0; c < ncases; ++c) {
