@@ -303,7 +303,7 @@ int sphst_set_stream(sphst_case c, void *cuda_stream);
  * graph) and bracketed by CUDA events on the case's stream.  kernel_ms[k]
  * receives the summed device time of kernel group k and launches[k] its
  * launch count, for k = 0 rebuild (keys, scan, sort, gather, neighbour
- * list, interface band), 1 set-up (speed reduction, criteria, correction
+ * list, its pair geometry, interface band), 1 set-up (speed reduction, criteria, correction
  * matrix, viscous + shift), 2 criterion per substep, 3 sweep A (colour
  * gradient), 4 sweep B (pressure + kick), 5 sweep C (continuity + drift),
  * 6 sweep S (surface sum of the interface band; neighbour-list cases only).

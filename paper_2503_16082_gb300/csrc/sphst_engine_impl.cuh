@@ -759,7 +759,7 @@ template <typename T> struct EngineT : Engine {
         timed(0, 5, [&] {
             launch_fluid_ranks();
         });
-        timed(0, 2 * nlist, [&] {
+        timed(0, (lgeo ? 3 : 2) * nlist, [&] {
             launch_lists();
             launch_band();
         });

@@ -147,3 +147,16 @@ def test_pairs_at_the_cutoff_keep_their_kind(partner):
     assert (np.abs(out[0][4][:n]) > 0).any() and np.abs(out[0][4][:n]).max() < 1e-30
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.gpu
+def test_a_profiled_step_counts_its_launches():
+    # rebuild: 8 of the cell order, 5 of the slots, then per list class the
+    # lists, the stored geometry (FP64) and the band
+    case = sphcases.small_droplet(2, 16, seed=3, jitter=0.1)
+    want = {(32, S.NBR_LIST, True): 15, (64, S.NBR_LIST, True): 16, (64, S.NBR_LIST, False): 15, (64, S.NBR_CELLS, True): 13}
+    for (precision, mode, keep), n in want.items():
+        h = S.case_from_spec(case, precision=precision, nbr_mode=mode)
+        S.set_pair_geometry(h, keep)
+        assert S.profile_step(h)["rebuild"][1] == n
+        S.destroy(h)
