@@ -92,12 +92,20 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         }                                                                                              \
     }
 
-// Up to this many lanes per SM, the sweeps B and C of a one-case engine take
-// their MODE_FEW form: the SMs hold fewer warps than the registers would allow
-// (B 42 registers: 1,536 lanes), and the latency of the gathers is what a
-// substep waits for.  64k particles (421 per SM): B 35 -> 33 us; 1M (6,580 per
-// SM): B 250 -> 285 us.
-constexpr int64_t FEW_MAX_PER_SM = 1024;
+// Whether the sweeps B and C of a one-case engine take their MODE_FEW form.  In
+// FP32: while all lanes are resident at once at B's registers there (80: 768
+// lanes per SM, 88 with several lanes per particle: 640), so that what a
+// substep waits for is the latency of the gathers.  B, one neighbour at a time
+// against four, us per launch at lanes per SM: 3D 421 38.7 and 32.8, 727 45.5
+// and 41.8, 822 49.9 and 56.2, 6578 257 and 285; 2D 592 15.7 and 14.3, 760 16.8
+// and 15.6, 1052 18.4 and 22.3; four lanes per particle 710 20.6 and 21.6.
+// FP64 reads stored geometry, so only the registers differ (B 128 and more):
+// 3D 421 376 and 449, 487 426 and 530, 599 593 and 586, 822 832 and 778; 2D 592
+// 121 and 130, 1052 199 and 215.
+template <typename T> bool few_lanes(int dim, int lanes, int64_t per_sm) {
+    if (sizeof(T) == 4) return per_sm <= (lanes == 1 ? 768 : 640);
+    return dim == 3 && per_sm > 512 && per_sm <= 1024;
+}
 
 // FP64 sweeps take smaller blocks than asked for until every SM has this many:
 // their time is the busiest SM's arithmetic, and whole blocks of a small case
@@ -265,7 +273,7 @@ template <typename T> struct EngineT : Engine {
         // the cell walk's places are shared memory per thread: blocks of more than
         // CELL_BLOCK_MAX would leave a thread fewer than it wants
         if (list_fluid < fluid) block = std::min(block, CELL_BLOCK_MAX);
-        few = list_fluid * lanes <= sm_count * FEW_MAX_PER_SM;
+        few = ncases == 1 && few_lanes<T>(cases[0]->P.dim, lanes, (list_fluid * lanes + sm_count - 1) / sm_count);
         for (int c = 0; c < ncases; ++c) {
             CaseRec *r = cases[c];
             if (!r->gridded) {
