@@ -140,11 +140,9 @@ template <typename T> static CasePhys<T> phys_of(const CaseRec *c) {
     const double rsum = c->rho0[0] + c->rho0[1];
     CasePhys<T> p;
     p.h = (T)h;
-    p.inv_h = (T)(1.0 / h);
     p.four_h2 = (T)((2.0 * h) * (2.0 * h));
-    p.kcoef = (T)(-5.0 * alpha / h);
     p.mhalf_inv_h = (T)(-0.5 / h);
-    // kcoef / h as fraction and exponent: 1 / h^(dim + 2) may leave even FP64
+    // -5 alpha / h^2 as fraction and exponent: 1 / h^(dim + 2) may leave even FP64
     int ek = 0, eh = 0;
     const double fk = std::frexp(-5.0 * alpha / h, &ek) / std::frexp(h, &eh);
     const int ev = volume_exponent<T>(ek - eh);
@@ -152,8 +150,6 @@ template <typename T> static CasePhys<T> phys_of(const CaseRec *c) {
     p.kcoef_h = (T)std::ldexp(fk, ek - eh + ev);
     p.cs = (T)cell_width(c);
     p.c0 = (T)P.c0;
-    p.c0sq = (T)(P.c0 * P.c0);
-    p.inv_c0 = (T)(1.0 / P.c0);
     p.gamma = (T)P.gamma;
     // limiter (Eq. 11): density reading min(max(3 dU / c0, 0), 1); beta = 1; beta = 0
     p.beta_k = (T)((P.limiter == SPHST_LIMITER_DENSITY || P.limiter == SPHST_LIMITER_PRINTED) ? 3.0 / P.c0 : 0.0);

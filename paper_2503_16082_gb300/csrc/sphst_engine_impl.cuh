@@ -51,7 +51,20 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
         }                                                                              \
     }
 
-// SPH_LANES_M: sweeps A, B and C, whose list classes run with LN lanes per
+// SPH_CELL_CLASSES: the per-substep sweeps of the cell-walk classes, in the
+// work list's mode or by tiles: a one-case engine keeps the descriptor array
+// too, as their sweep B also evaluates the surface terms, whose sums are left
+// to the compiler's contraction
+#define SPH_CELL_CLASSES(KERN, MODE, ARGS, GRID, ...)                                                                \
+    for (int k_ = 2; k_ < 4; ++k_) {                                                                                 \
+        if (!cls_fn[k_]) continue;                                                                                   \
+        const SweepArgs a_ = ARGS(k_);                                                                               \
+        const unsigned g_ = (unsigned)(GRID);                                                                        \
+        if (k_ == 2) SPH_CELLS(KERN, 3, (KERN<T, 3, false, 1, MODE>), (KERN<T, 3, false, CELL_LANES, MODE>), __VA_ARGS__) \
+        else SPH_CELLS(KERN, 2, (KERN<T, 2, false, 1, MODE>), (KERN<T, 2, false, CELL_LANES, MODE>), __VA_ARGS__)    \
+    }
+
+// SPH_LANES_M: sweeps B and C, whose list classes run with LN lanes per
 // particle (L blocks per tile), in their tile mode (MODE_TILES, MODE_WORK for
 // the work-list kernels of a batch, MODE_ONE and MODE_FEW for a one-case engine)
 #define SPH_LANES_M(KERN, D, LN, MODE, ...)                                                             \
@@ -61,35 +74,31 @@ enum ArrayId { A_POS = 0, A_VEL, A_DRHO, A_ID, A_GRADC, A_ACCV };
     case 8: launch_next(KERN<T, D, true, 8, MODE>, g_ * 8, block, 0, stream, a_, __VA_ARGS__); break;            \
     default: launch_next(KERN<T, D, true, 1, MODE>, g_, block, 0, stream, a_, __VA_ARGS__); break;               \
     }
-// SPH_CLASSES_LF: the per-substep sweeps over slots from class K0 on, whose
-// blocks stride over the work list of active tiles in a batch (the grid is then
-// capped), and which take their case's descriptor from the launch parameters
-// in a one-case engine
-#define SPH_CLASSES_LF(K0, NCLS, KERN, LN, ...)                                                         \
-    if (use_work) {                                                                                    \
-        SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, work_args, cls_fn, work_grid(cls_fn[k_]), MODE_WORK, __VA_ARGS__) \
-    } else if (ncases == 1 && few) {                                                                   \
-        SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, fluid_args, cls_fn, cls_fn[k_], MODE_FEW, __VA_ARGS__)      \
-    } else if (ncases == 1) {                                                                          \
-        SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, fluid_args, cls_fn, cls_fn[k_], MODE_ONE, __VA_ARGS__)      \
-    } else {                                                                                           \
-        SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, fluid_args, cls_fn, cls_fn[k_], MODE_TILES, __VA_ARGS__)    \
+// SPH_SWEEPS: a per-substep sweep over the slots, whose blocks stride over the
+// work list of active tiles in a batch (the grid is then capped), and whose
+// list classes take their case's descriptor from the launch parameters in a
+// one-case engine
+#define SPH_SWEEPS(KERN, LN, ...)                                                                        \
+    if (use_work) {                                                                                     \
+        SPH_LIST_CLASSES(KERN, LN, work_args, work_grid(cls_fn[k_]), MODE_WORK, __VA_ARGS__)            \
+        SPH_CELL_CLASSES(KERN, MODE_WORK, work_args, work_grid(cls_fn[k_]), __VA_ARGS__)                \
+    } else {                                                                                            \
+        if (ncases == 1 && few) {                                                                       \
+            SPH_LIST_CLASSES(KERN, LN, fluid_args, cls_fn[k_], MODE_FEW, __VA_ARGS__)                   \
+        } else if (ncases == 1) {                                                                       \
+            SPH_LIST_CLASSES(KERN, LN, fluid_args, cls_fn[k_], MODE_ONE, __VA_ARGS__)                   \
+        } else {                                                                                        \
+            SPH_LIST_CLASSES(KERN, LN, fluid_args, cls_fn[k_], MODE_TILES, __VA_ARGS__)                 \
+        }                                                                                               \
+        SPH_CELL_CLASSES(KERN, MODE_TILES, fluid_args, cls_fn[k_], __VA_ARGS__)                         \
     }
-// the cell-walk classes keep the descriptor array in a one-case engine: their
-// sweep B also evaluates the surface terms, whose sums are left to the
-// compiler's contraction, so only one compiled form of it may exist
-#define CELL_MODE(MODE) ((MODE) == MODE_ONE || (MODE) == MODE_FEW ? MODE_TILES : (MODE))
-#define SPH_CLASSES_LXMK(K0, NCLS, KERN, LN, ARGS, CNT, GRID, MODE, ...)                              \
-    for (int k_ = (K0); k_ < (NCLS); ++k_) {                                                              \
-        if (!CNT[k_]) continue;                                                                        \
-        const SweepArgs a_ = ARGS(k_);                                                                 \
-        const unsigned g_ = (unsigned)(GRID);                                                          \
-        switch (k_) {                                                                                  \
-        case 0: SPH_LANES_M(KERN, 3, LN, MODE, __VA_ARGS__) break;                                     \
-        case 1: SPH_LANES_M(KERN, 2, LN, MODE, __VA_ARGS__) break;                                     \
-        case 2: SPH_CELLS(KERN, 3, (KERN<T, 3, false, 1, CELL_MODE(MODE)>), (KERN<T, 3, false, CELL_LANES, CELL_MODE(MODE)>), __VA_ARGS__) break; \
-        default: SPH_CELLS(KERN, 2, (KERN<T, 2, false, 1, CELL_MODE(MODE)>), (KERN<T, 2, false, CELL_LANES, CELL_MODE(MODE)>), __VA_ARGS__) break;\
-        }                                                                                              \
+#define SPH_LIST_CLASSES(KERN, LN, ARGS, GRID, MODE, ...)                                                \
+    for (int k_ = 0; k_ < 2; ++k_) {                                                                    \
+        if (!cls_fn[k_]) continue;                                                                      \
+        const SweepArgs a_ = ARGS(k_);                                                                  \
+        const unsigned g_ = (unsigned)(GRID);                                                           \
+        if (k_ == 0) { SPH_LANES_M(KERN, 3, LN, MODE, __VA_ARGS__) }                                    \
+        else { SPH_LANES_M(KERN, 2, LN, MODE, __VA_ARGS__) }                                            \
     }
 
 // Whether the sweeps B and C of a one-case engine take their MODE_FEW form.  In
@@ -521,8 +530,8 @@ template <typename T> struct EngineT : Engine {
         return a;
     }
     int64_t work_grid(int64_t tiles) const { return use_work ? std::min(tiles, work_cap) : tiles; }
-    // blocks (per lane) of a band-list sweep: at most one per tile, at most 8
-    // blocks of all lanes per SM
+    // blocks (per lane) of a band-list sweep: at most one per tile, at most
+    // 1024 threads, or 8 blocks, of all lanes per SM
     int64_t band_grid(int64_t tiles, int lanes_) const {
         const int64_t per_sm = std::max<int64_t>(8, 1024 / block);
         return std::max<int64_t>(1, std::min<int64_t>(tiles, sm_count * per_sm / std::max(lanes_, 1)));
@@ -595,8 +604,8 @@ template <typename T> struct EngineT : Engine {
         launch_band_class<3>(0, true);
         launch_band_class<2>(1, true);
     }
-    void launch_B() { SPH_CLASSES_LF(0, 4, k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk, vol); }
-    void launch_C() { SPH_CLASSES_LF(0, 4, k_sweep_C, lanes, snap, vel_new, drho, vol, vel, pos); }
+    void launch_B() { SPH_SWEEPS(k_sweep_B, lanes, band, snap, vel, gradC, acc_visc, acc_surf, vel_new, bk, vol); }
+    void launch_C() { SPH_SWEEPS(k_sweep_C, lanes, snap, vel_new, drho, vol, vel, pos); }
     int n_classes(int upto) const {
         int m = 0;
         for (int k = 0; k < upto; ++k) m += cls_n[k] > 0;
@@ -636,7 +645,8 @@ template <typename T> struct EngineT : Engine {
     void launch_colour() {
         launch_band_class<3>(0, false);
         launch_band_class<2>(1, false);
-        SPH_CLASSES_LF(2, 4, k_sweep_A, lanes, snap, vol, gradC);
+        if (use_work) SPH_CELL_CLASSES(k_sweep_A, MODE_WORK, work_args, work_grid(cls_fn[k_]), snap, vol, gradC)
+        else SPH_CELL_CLASSES(k_sweep_A, MODE_TILES, fluid_args, cls_fn[k_], snap, vol, gradC)
     }
 
     int launch_body(cudaGraphConditionalHandle h, int use_handle) {

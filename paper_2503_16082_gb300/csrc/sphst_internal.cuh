@@ -71,15 +71,14 @@ template <int D> __host__ __device__ inline uint32_t morton_of_packed(uint32_t p
 // ------------------------------------------------------- per-case constants
 // Problem statement of one case, in both precisions; read-only on device.
 template <typename T> struct CasePhys {
-    T h, inv_h, four_h2;       // smoothing length, 1/h, (2h)^2
-    T kcoef;                   // dW/dr = kcoef * q (1 - q/2)^3, kcoef = -5 alpha_d / h
+    T h, four_h2;              // smoothing length, (2h)^2
     T cs;                      // cell width
-    T c0, c0sq, inv_c0, gamma, xi;
+    T c0, gamma, xi;
     T rho0[2], eta[2], mass[2];
     T two_phi[2];              // 2 phi_i of a cross-phase pair, i in fluid k (Eq. 23)
     T four_phi_phi;            // 4 phi_i phi_j of a cross-phase pair
     T vol_wall;                // dp^dim
-    T mhalf_inv_h, kcoef_h;    // -1 / (2h); kcoef / h: W'/r = kcoef_h (1 - q/2)^3
+    T mhalf_inv_h, kcoef_h;    // -1 / (2h); -5 alpha_d / h^2: W'/r = kcoef_h (1 - q/2)^3
     T mass_c0[2], c0_vol;      // m c0 per fluid; c0 dp^dim
     // (volumes and masses in a unit that kcoef_h is the reciprocal of: 1, or a
     // power of two where 1 would take kcoef_h out of the type's range)

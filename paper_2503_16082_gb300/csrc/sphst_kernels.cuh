@@ -23,9 +23,9 @@
 // over the fluid particles only (their ranks after each reorder); A and S of
 // the list classes stride over the band list.  Time-step control (Eqs.
 // 16-18) runs in FP64 in one-thread-per-case kernels.  A one-case engine
-// launches A, B and C with the case's constants in the launch parameters
-// (MODE_ONE); their sums are explicitly rounded, so the results do not depend
-// on that choice.
+// launches B and C of the list classes with the case's constants in the launch
+// parameters (MODE_ONE); their sums are explicitly rounded, so the results do
+// not depend on that choice.
 #pragma once
 
 #include <cfloat>
@@ -46,12 +46,8 @@
 //                      (default 6: 42 registers, as its per-case constants are
 //                      not in registers; 1M particles: 6 250 us, 5 271, 7 279)
 //   SPHST_SWEEPAS_MINB the same for sweep A of the cell-walk classes
-//   SPHST_FAST_DIV     1: FP32 pair divisions through the SFU reciprocal
 //   SPHST_LIST_NOALLOC 1: the list words are read without allocating L1 lines
 //                      (measured +1% on the 3D drop)
-#ifndef SPHST_FAST_DIV
-#define SPHST_FAST_DIV 1
-#endif
 #ifndef SPHST_LIST_LDCS
 #define SPHST_LIST_LDCS 1
 #endif
@@ -82,11 +78,6 @@
 #define SPH_SWEEPAS_BOUNDS __launch_bounds__(256, SPHST_SWEEPAS_MINB)
 #else
 #define SPH_SWEEPAS_BOUNDS __launch_bounds__(256)
-#endif
-#if SPHST_SWEEPB_MINB > 0
-#define SPH_SWEEPB_BOUNDS __launch_bounds__(256, SPHST_SWEEPB_MINB)
-#else
-#define SPH_SWEEPB_BOUNDS __launch_bounds__(256)
 #endif
 // sweep B of a one-case engine reads its per-case constants from the
 // parameter block, which leaves it room for more resident blocks
@@ -120,6 +111,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rsq_full(double x) { return rsqrt(x); }
 
 template <typename T> __device__ __forceinline__ V4<T> ld4(const V4<T> *p) { return *p; }
 template <> __device__ __forceinline__ V4<float> ld4<float>(const V4<float> *p) {
@@ -142,27 +134,9 @@ __device__ __forceinline__ V4<double> ld4_now(const V4<double> *p) {
     return v;
 }
 
-// Divisions inside the FP32 pair loops: __fdividef (error <= 2 ulp for
-// divisors below 2^126, which densities and |grad C| are) instead of the
-// IEEE sequence; FP64 keeps IEEE division.  1/sqrt likewise.
-__device__ __forceinline__ float div_fast(float a, float b) {
-#if SPHST_FAST_DIV
-    return __fdividef(a, b);
-#else
-    return a / b;
-#endif
-}
-__device__ __forceinline__ double div_fast(double a, double b) { return a / b; }
-__device__ __forceinline__ float rsqrt_fast(float x) {
-#if SPHST_FAST_DIV
-    return rsqrtf(x);
-#else
-    return 1.0f / sqrtf(x);
-#endif
-}
-__device__ __forceinline__ double rsqrt_fast(double x) { return rsqrt(x); }
-
-// a / b of the pair sums: in FP32 a times the SFU reciprocal (<= 2 ulp)
+// a / b of the pair sums: in FP32 a times the SFU reciprocal (<= 2 ulp, for
+// divisors below 2^126, which products of densities are) instead of the IEEE
+// sequence; FP64 keeps IEEE division
 __device__ __forceinline__ float vdiv(float a, float b) { return __fmul_rn(a, rcp_approx(b)); }
 __device__ __forceinline__ double vdiv(double a, double b) { return a / b; }
 
@@ -1485,7 +1459,6 @@ __device__ __forceinline__ V4<T> kicked(const V4<T> &vi, T rho_i, T dt, T apx, T
 // surface sweep's lanes add them in another order, so the two agree to
 // rounding.
 //
-// neighbours gathered at a time by the surface sweep
 // PASS: 0 = pressure + surface in one walk (cell walk), 1 = pressure and the
 // stored surface sum (list), 2 = surface sum only (list, band particles).
 template <bool LIST, int PASS, typename T, int D, int L = 1, int U = PLAIN>
@@ -1550,7 +1523,7 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
             const T niv = nix * vx + niy * vy + niz * vz, njv = njx * vx + njy * vy + njz * vz;
             const T bx = T(0.5) * (gi.x + gj.x), by = T(0.5) * (gi.y + gj.y), bz = T(0.5) * (gi.z + gj.z);
             const T b2 = bx * bx + by * by + bz * bz;
-            const T inv_bn = b2 > T(0) ? rsqrt_fast(b2) : T(0);
+            const T inv_bn = b2 > T(0) ? rsq_full(b2) : T(0);
             T cx, cy, cz;
             if (d.penalty_form == 0) {            // -|gradCbar| r nbar (nbar.v)
                 const T fac = g.r * (bx * vx + by * vy + bz * vz) * inv_bn;
@@ -1583,7 +1556,7 @@ __device__ __forceinline__ double sweep_B(const CaseDesc &d, const CasePhys<T> &
         const T bx = T(0.5) * (gi.x + sg * gj.x), by = T(0.5) * (gi.y + sg * gj.y),
                 bz = T(0.5) * (gi.z + sg * gj.z);
         const T b2 = bx * bx + by * by + bz * bz;
-        const T inv_bn = b2 > T(0) ? rsqrt_fast(b2) : T(0);
+        const T inv_bn = b2 > T(0) ? rsq_full(b2) : T(0);
         const T Cij = same ? T(0) : T(1);
         // C-hat e (Eq. 30 with the selected contraction)
         T cx, cy, cz;
