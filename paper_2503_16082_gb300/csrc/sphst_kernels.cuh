@@ -88,9 +88,12 @@
 // compiler left its gathers no room (52 to 55 registers); at 64 (4 blocks per
 // SM) a batch of 6M particles takes 582 us per launch in 3D against 719, with
 // work lists 585 against 604 (2D 154 against 178; the tiled 2D form is better
-// without, 147 against 167)
-#define SPH_SWEEPC_BOUNDS_M(T, D, LIST, MODE)                                                       \
-    __launch_bounds__(256, (LIST) && sizeof(T) == 4 && ((MODE) == 1 || ((MODE) == 0 && (D) == 3)) ? 4 : SPHST_SWEEP_MINB)
+// without, 147 against 167).  The two-lane cell walk in 3D (FP32) likewise
+// takes what it asks for (76 instead of 58): 30k particles 60.4 us against
+// 66.2, 125k 170 against 166.
+#define SPH_SWEEPC_BOUNDS_M(T, D, LIST, L, MODE)                                                       \
+    __launch_bounds__(256, (LIST) && sizeof(T) == 4 && ((MODE) == 1 || ((MODE) == 0 && (D) == 3)) ? 4                \
+                         : !(LIST) && (L) > 1 && sizeof(T) == 4 && (D) == 3 ? 1 : SPHST_SWEEP_MINB)
 
 namespace sphst {
 
@@ -2266,7 +2269,7 @@ __global__ void SPH_SWEEPB_BOUNDS_M(T, LIST, L, MODE) k_sweep_B(SweepArgs a, con
 }
 
 template <typename T, int D, bool LIST, int L = 1, int MODE = MODE_TILES>
-__global__ void SPH_SWEEPC_BOUNDS_M(T, D, LIST, MODE) k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho, T *vol,
+__global__ void SPH_SWEEPC_BOUNDS_M(T, D, LIST, L, MODE) k_sweep_C(SweepArgs a, const V4<T> *snap, const V4<T> *vel_new, T *drho, T *vol,
                                            V4<T> *vel, V4<T> *pos) {
     follow();
     const auto item = [&](int64_t w) {
