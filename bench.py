@@ -126,10 +126,11 @@ def device_roofs():
 # particle-substeps/s against 1.516e9 with 128 (sweep C 0.244 against
 # 0.255 ms per launch, B the same), 160: 1.532e9, 192: 1.517e9.
 TUNED_BLOCK = {("oscillating_3d", 32, "list"): 256}
-# the same for the batched workload (one engine of 512 cases): 256 threads
-# 1.513-1.515e9 against 1.497-1.500e9 with 128, the work-list variant
-# 1.443e9 against 1.394e9; its cases stepped one by one stay at the
-# library's default (676 against 666 M particle-substeps/s at 256)
+# the same for the batched workload (one engine of 512 cases).  It was the
+# faster one (1.515e9 against 1.500e9 with 128); since the sweeps of a batch
+# hold the cases' constants in registers 128 threads are (a step of 497 ms
+# against 507), and 256 is kept so that the line stays comparable; its cases
+# stepped one by one stay at the library's default
 BATCH_BLOCK = 256
 
 

@@ -370,7 +370,7 @@ __device__ __forceinline__ void moved_offset(uint32_t e, const V4<T> &si, const 
 // How a sweep gathers its neighbours (U of walk_list), by measurement at 1M and
 // 64k particles in 3D and 37k in 2D (FP32; us per launch, PLAIN against the
 // choice):  C 237 -> 213, 33 -> 25 (AHEAD), 16.0 -> 12.7 (4, in 2D);
-// V + M 977 -> 822, 134 -> 107; A 19.3 -> 14.6; S 72 -> 63, 31 -> 27 (4).
+// V + M 977 -> 822, 134 -> 107 (745 at 1M since they hold the case's constants); A 19.3 -> 14.6; S 72 -> 63, 31 -> 27 (4).
 // Sweep B at 1M particles stays PLAIN (250 against 271-300): its arithmetic
 // leaves no registers for a neighbour in flight at the warps it needs.
 constexpr int PLAIN = 1, AHEAD = -1;
@@ -1803,10 +1803,10 @@ struct BandEntry {
 // operations, so list and walk hold the same pairs: in FP32 for the few that
 // the first test cannot settle, in FP64 for its hits, a sixth of the
 // candidates: the FP64
-// pipe is 64 times narrower.  It is bound by instruction issue (about 18
+// pipe is 64 times narrower.  It is bound by instruction issue (about 21
 // instructions per 32 candidates of a slot).  Measured, rebuild of an
-// advection step: 1M fluid particles in FP32 1.71 -> 1.09 ms, 64k 0.56 ->
-// 0.18 ms, 6.9M 11.6 -> 6.7 ms, 43k in FP64 1.17 -> 0.31 ms, against a thread
+// advection step: 1M fluid particles in FP32 1.71 -> 1.13 ms, 64k 0.56 ->
+// 0.18 ms, 6.9M 11.6 -> 7.1 ms, 43k in FP64 1.17 -> 0.31 ms, against a thread
 // per particle that walked its cells alone (lanes in different cells, the
 // ordered cells of each lane in local memory) and a separate pass over all
 // lists for the band; a warp per cell with the slots in its inner loop took
